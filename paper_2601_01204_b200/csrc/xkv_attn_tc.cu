@@ -23,11 +23,13 @@
 //   4 warps     operand producers: packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
 //               and key group) and V~ (per token) in the 128-byte-swizzled layouts the MMA
 //               descriptors expect.  One dequantised tile serves both query tiles.
-//   2 threads   (in warps of their own) issue the MMAs of query tile 0 resp. 1:
+//   2 warps     issue the MMAs of query tile 0 resp. 1 through an elected lane:
 //               S_t = Q_t K~^T (M128 N128 K64) and O_t += P_t V~ (M128 N64 K128,
-//               A = P from tensor memory).  A thread gets one tcgen05.mma through about every
-//               125 cycles whatever its shape; a single issuing thread for both tiles was the
-//               bottleneck of the CTA.
+//               A = P from tensor memory).  The warps stay converged: a lone thread in a branch
+//               gets one tcgen05.mma through every 48-62 clk at best (its operands are moved into
+//               uniform registers each time), an elected lane every 30 clk for P V~.  Measured
+//               (16384 cached tokens, 1374 queries): 4-bit 160.3 -> 158.6 us, keys quantised once
+//               188.5 -> 181.9 us, 16-bit at 32768 tokens 287.1 -> 273.8 us.
 //   1 thread    issues the bulk copies of the raw tiles, several steps ahead; its warp owns the
 //               tensor-memory allocation (all 512 columns).
 // 4-bit caches multiply in fp16 (the dequantised keys are not bf16-representable:
@@ -267,6 +269,14 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+// One lane of a converged warp.  The issuing warps run converged and let one elected lane issue, so
+// that descriptors and addresses stay warp-uniform and live in uniform registers: inside a branch
+// that only one lane takes, every tcgen05.mma is preceded by moves of its operands into them.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
 }
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t acc) {
@@ -512,7 +522,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   const WaitCtx wc{a.status, abort_flag};
 
   const int tid = threadIdx.x;
-  const int warp = tid >> 5;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (known to be the same in all lanes)
   constexpr bool kBf16 = (BITS == 16);
 
   // this CTA's piece of the line of steps
@@ -539,7 +549,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   if (SPLIT) {
     // Registers move from the warps that need few to the softmax warps, which keep half a row of
@@ -1221,15 +1231,15 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         }
       }
     }
-  } else if (SPLIT && (tid == 32 * (kSW + 4) || tid == 32 * (kSW + 6))) {
+  } else if (SPLIT && (warp == kSW + 4 || warp == kSW + 6)) {
     // =========================== MMA issuers, 16-warp form ====================
-    // One thread per query tile, products in program order (S of step j, then P V~ of step j - 1).
+    // One converged warp per query tile, products in program order (S of step j, then P V~ of step j - 1).
     // The two tiles share one score buffer: its uses are numbered in the order tile 0, tile 1,
     // tile 0, ... (tile 0 alone where the item has no second tile), and use G is issued once the
     // softmax warps have loaded use G - 1.  Even and odd uses are released on two barriers: the
     // barrier of use G - 1 cannot complete again before use G + 1 has been issued, and a thread
     // waits for uses that are at most two apart, so a parity wait is never two phases off.
-    const int t = (tid == 32 * (kSW + 6)) ? 1 : 0;
+    const int t = (warp == kSW + 6) ? 1 : 0;
     const uint32_t idesc_qk = make_idesc(128, kBf16, false);
     const uint32_t idesc_pv = make_idesc(64, kBf16, true);
     const uint64_t dq = make_desc(sQ + t * 16384);
@@ -1251,14 +1261,18 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           tc_fence_after();
           const uint64_t dv = make_desc(sV + (gv % kNV) * 16384);
           const uint32_t d_p = d_p0 + 64 * (cp & 1);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
-            mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
-                   (!first_of_segment || ks > 0) ? 1u : 0u);
-          tc_commit(b_pvdone2 + 16 * t + 8 * (cp & 1));
+            for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
+              mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
+                     (!first_of_segment || ks > 0) ? 1u : 0u);
+            tc_commit(b_pvdone2 + 16 * t + 8 * (cp & 1));
+          }
+          __syncwarp();
           ++cp;
         }
-        tc_commit(b_vfree + 8 * (gv % kNV));
+        if (elect_one()) tc_commit(b_vfree + 8 * (gv % kNV));
+        __syncwarp();
       };
       for (int jj = 0; jj < nt; ++jj, ++g) {
         mbar_wait(b_kfull + 8 * (g % kNK), (g / kNK) & 1, wc);
@@ -1268,10 +1282,13 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           if (jj == 0) mbar_wait(b_qfull + 8 * t, segq & 1, wc);
           tc_fence_after();
           const uint64_t dk = make_desc(sK + (g % kNK) * 16384);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
-            mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
-          tc_commit(b_sfull + 8 * t);
+            for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
+              mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
+            tc_commit(b_sfull + 8 * t);
+          }
+          __syncwarp();
         } else {
           // An item without a second tile: this thread follows the other tile's uses of the score
           // buffer one by one.  A parity wait is only sound while the waiter is at most one
@@ -1279,7 +1296,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           const uint32_t use = g_seg + (uint32_t)jj;
           if (use > 0) mbar_wait(b_sfree + 8 * ((use - 1) & 1), ((use - 1) >> 1) & 1, wc);
         }
-        tc_commit(b_kfree + 8 * (g % kNK));
+        if (elect_one()) tc_commit(b_kfree + 8 * (g % kNK));
+        __syncwarp();
         if (jj > 0) issue_pv(g - 1, jj == 1);
       }
       issue_pv(g - 1, nt == 1);           // the last PV of the segment
@@ -1287,11 +1305,11 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       if (active) ++segq;
     }
     tc_fence_before();
-  } else if (!SPLIT && (tid == 32 * (kSW + 4) || tid == 32 * (kSW + 6))) {
+  } else if (!SPLIT && (warp == kSW + 4 || warp == kSW + 6)) {
     // =========================== MMA issuers ==================================
-    // One thread per query tile.  Both release the K~/V~ stages (two arrivals each), also for an
-    // item that has no second tile: then the second thread only follows the rings.
-    const int t = (tid == 32 * (kSW + 6)) ? 1 : 0;
+    // One converged warp per query tile.  Both release the K~/V~ stages (two arrivals each), also for
+    // an item that has no second tile: then the second warp only follows the rings.
+    const int t = (warp == kSW + 6) ? 1 : 0;
     const uint32_t idesc_qk = make_idesc(128, kBf16, false);
     const uint32_t idesc_pv = make_idesc(64, kBf16, true);
     const uint64_t dq = make_desc(sQ + t * 16384);
@@ -1310,13 +1328,17 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           mbar_wait(b_pfull + 8 * t, (cnt - 1) & 1, wc);        // P_t of that step written
           tc_fence_after();
           const uint64_t dv = make_desc(sV + (gv % kNV) * 16384);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
-            mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
-                   (!first_of_segment || ks > 0) ? 1u : 0u);
-          tc_commit(b_pvdone + 8 * t);
+            for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
+              mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
+                     (!first_of_segment || ks > 0) ? 1u : 0u);
+            tc_commit(b_pvdone + 8 * t);
+          }
+          __syncwarp();
         }
-        tc_commit(b_vfree + 8 * (gv % kNV));
+        if (elect_one()) tc_commit(b_vfree + 8 * (gv % kNV));
+        __syncwarp();
       };
       for (int jj = 0; jj < nt; ++jj, ++g) {
         mbar_wait(b_kfull + 8 * (g % kNK), (g / kNK) & 1, wc);
@@ -1325,12 +1347,16 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           else mbar_wait(b_sfree + 8 * t, (cnt - 1) & 1, wc);   // S_t of the previous step has been read
           tc_fence_after();
           const uint64_t dk = make_desc(sK + (g % kNK) * 16384);
+          if (elect_one()) {
 #pragma unroll
-          for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
-            mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
-          tc_commit(b_sfull + 8 * t);
+            for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
+              mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
+            tc_commit(b_sfull + 8 * t);
+          }
+          __syncwarp();
         }
-        tc_commit(b_kfree + 8 * (g % kNK));
+        if (elect_one()) tc_commit(b_kfree + 8 * (g % kNK));
+        __syncwarp();
         if (jj > 0) issue_pv(g - 1, jj == 1);
         if (active) ++cnt;
       }
