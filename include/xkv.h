@@ -276,7 +276,7 @@ XKV_API int attn_packed_causal_static(xkv_cache* cache, const void* q, void* out
  * k = max(0, L_max - T_first - total) middle tokens, kv_quant_pack packs - and then this call
  * attends frame-causally: the queries of the chunk's frame f see every cached token that is older
  * than the chunk and the chunk's frames 0..f (the cache keeps arrival order, so that is a prefix
- * of it; one launch of the tensor-core kernel per frame).  q, out: the chunk's tensors,
+ * of it; the tensor-core kernel takes all frames in one launch).  q, out: the chunk's tensors,
  * [H][total][d] with the given strides; frame_tokens: HOST array of n_frames sizes that add up to
  * the appended total.  A chunk of one frame is attn_packed_causal.  State and errors as attn_packed_causal. */
 XKV_API int attn_packed_frame_causal(xkv_cache* cache, const void* q, void* out, const int32_t* frame_tokens,
@@ -324,12 +324,12 @@ XKV_API int xkv_set_unquantised_tail(xkv_cache* cache, int32_t on);
  * above with softmax_scale = 1/sqrt(head_dim).  q, k, v, out are HOST arrays of
  * n_layers DEVICE pointers.  Stops at the first error and returns it; the layer that failed
  * may then be left between two of its four calls, and the only way on is xkv_reset.
- * Within a layer kv_append runs on a stream of the library's own (created on
- * first use, one per device) beside kv_score_evict, which does not depend on it;
- * both are ordered after everything already in `stream` and before the layer's
- * kv_quant_pack, and a layer starts only after the previous layer's attention.
- * After kv_quant_pack the step also computes, on that stream and beside the
- * attention, the head means of the cached keys (Eq. 4) into the cache's workspace;
+ * Layers that do not depend on one another are taken together (up to 28 per launch): the maintenance
+ * of all of them, then the attention of all of them.  A layer whose tensors overlap an earlier layer's
+ * output (or whose output overlaps what an earlier layer still reads), or whose cache has come before,
+ * starts after the layers before it, so the results are always those of the layers one after the other.
+ * After kv_quant_pack the step also computes, on a stream of the library's own (created on
+ * first use, one per device) and beside the attention, the head means of the cached keys (Eq. 4) into the cache's workspace;
  * the next frame's scoring of the same cache starts from them (same bits as
  * kv_score_evict computes).  `stream` waits for these kernels at the end of the call.
  * The library's stream and its events are shared by every cache on the device:

@@ -36,8 +36,8 @@
 // rounding them to bf16 alone costs ~1e-2 relative L2 with outlier channels);
 // 16-bit caches hold bf16 and multiply in bf16.  Accumulation is fp32.
 //
-// Every mbarrier wait is bounded (one second of running time): when the bound is hit the thread records
-// XKV_E_TIMEOUT in the cache's status word and carries on without waiting, so the
+// Every mbarrier wait is bounded (one second of running time): when the bound is hit the CTA carries on
+// without waiting and records XKV_E_TIMEOUT in the status words of the caches of the launch, so the
 // kernel always terminates, drains its copies and frees its tensor memory.
 #include <mutex>
 #include <stdlib.h>
@@ -112,42 +112,77 @@ constexpr int kTmemCols = 512;
 constexpr size_t kSlotFloats = 2 * 128 * 64;
 constexpr size_t kSlotBytes = kSlotFloats * sizeof(float) + 2 * 128 * sizeof(float2);
 
-struct Args {
+// One cache (or a prefix of one) and the queries that attend to it.
+struct Job {
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
-  int n;
-  int64_t ts, hs;
   const uint8_t* k;
   const float2* kpar;
   const uint8_t* v;
   const float2* vpar;
-  int cap, t_first, t_phys;
-  float scale_log2;
-  int n_tiles;          // key tiles of the cache
-  int q_tiles;          // 128-row query tiles of the frame
-  int n_pairs;          // ceil(q_tiles / 2)
-  long long total;      // items * n_tiles
-  float* part_o;        // [2 * grid][2][128][64]
-  float2* part_ml;      // [2 * grid][2][128]
   int* status;
   // Newest frame unquantised (Eq. 1 read literally): when k_tail is set, the key slots
   // [tail_lo, t_phys) take K~, V~ from these bf16 tensors ([head][token][64] with the strides
-  // below, token = slot - tail_lo) instead of the packed rows.
+  // of Args, token = slot - tail_lo) instead of the packed rows.
   const __nv_bfloat16* k_tail;
   const __nv_bfloat16* v_tail;
-  int64_t tail_ts, tail_hs;
-  int tail_lo;
   // Quantise-once mode: every token refers to the parameter-table slot of its key group
   // (kslot [cap]); ktab16 [slot][n_heads][8][12] holds, per 8-channel word, the four fp16 pairs
   // of scales, offsets and constants that dequant_word_h takes.
   const int32_t* kslot;
   const uint32_t* ktab16;
-  int n_heads;
+  int n, cap, t_first, t_phys, tail_lo, n_heads;
+  int n_tiles;          // key tiles of the cache
+  int q_tiles;          // 128-row query tiles of the frame
+  int n_pairs;          // ceil(q_tiles / 2)
+  uint32_t step_lo, step_hi;   // its steps on the line: n_heads * n_pairs items of n_tiles steps
 };
 
-__device__ __forceinline__ long long piece_start(long long total, int grid, int b) {
-  return (total * (long long)b) / (long long)grid;
+// Layers of a stack or frames of a chunk in one launch: fewer pieces are cut (an item that is cut
+// costs its queries, first scores and epilogue once more, about 3.3 steps, and a merge), and the
+// multiprocessors run out of work together once per launch.  The table travels in the kernel's
+// parameters, whose classic limit of 4 KB it stays below.
+constexpr int kMaxJobs = kMaxLayers;
+struct Args {
+  int64_t ts, hs;       // strides of q, out, k_tail and v_tail
+  float scale_log2;
+  int n_jobs;
+  int grid;             // pieces that the line of all steps is cut into: the first `longer` of them have
+  uint32_t piece, longer;      // piece + 1 steps, the others `piece`
+  float* part_o;        // [2 * grid][2][128][64]
+  float2* part_ml;      // [2 * grid][2][128]
+  Job job[kMaxJobs];
+};
+
+__device__ __forceinline__ uint32_t piece_start(const Args& a, int b) {
+  return (uint32_t)b * a.piece + min((uint32_t)b, a.longer);
 }
+
+// A CTA's walk along the line: the parts of items that its piece covers, one after the other.
+struct Walk {
+  uint32_t pos, end;
+  int job;
+  // of the current segment
+  int h, pair, tile_lo, nt;
+  __device__ __forceinline__ Walk(const Args& a) {
+    pos = piece_start(a, blockIdx.x);
+    end = piece_start(a, blockIdx.x + 1);
+    job = 0;
+  }
+  __device__ __forceinline__ bool next(const Args& a) {
+    if (pos >= end) return false;
+    while (pos >= a.job[job].step_hi) ++job;
+    const uint32_t tiles = (uint32_t)a.job[job].n_tiles, pairs = (uint32_t)a.job[job].n_pairs;
+    const uint32_t rel = pos - a.job[job].step_lo;
+    const uint32_t item = rel / tiles, head = item / pairs;
+    tile_lo = (int)(rel - item * tiles);
+    nt = (int)min(tiles - (uint32_t)tile_lo, end - pos);
+    h = (int)head;
+    pair = (int)(item - head * pairs);
+    pos += (uint32_t)nt;
+    return true;
+  }
+};
 
 // ---- PTX wrappers -----------------------------------------------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -197,9 +232,9 @@ __device__ __forceinline__ uint64_t global_ns() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Bounded wait.  On exhaustion the failure is recorded (device status word and a
-// per-CTA flag); once the flag is up every later wait of the CTA gives up at once.
-struct WaitCtx { int* status; volatile int* abort_flag; };
+// Bounded wait.  On exhaustion a per-CTA flag goes up, and every later wait of the CTA gives up at
+// once; at its end the CTA records the failure in the status words of the launch's caches.
+struct WaitCtx { volatile int* abort_flag; };
 // Threads on the critical chain (softmax warps, MMA issuers: SLEEP_NS below 128) retry at once, each
 // try suspended by the hardware for a short while: their wake-up latency is part of every step.
 // Threads that wait long and have slack (operand producers, the copy thread) sleep SLEEP_NS between
@@ -227,7 +262,10 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const W
     }
   } while (++rounds < kWaitMinRounds || global_ns() - t0 < kWaitLimitNs);
   *wc.abort_flag = 1;
-  atomicExch(wc.status, (int)XKV_E_TIMEOUT);
+}
+// A wait of the CTA ran out: the results of every cache in the launch are void.
+__device__ __forceinline__ void report_timeout(const Args& a) {
+  for (int j = 0; j < a.n_jobs; ++j) atomicExch(a.job[j].status, (int)XKV_E_TIMEOUT);
 }
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -499,7 +537,7 @@ __device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, 128;
 // ONCE: the keys' dequantisation constants are looked up per token (quantise-once mode) instead of
 // per 64-slot run.
 template <int BITS, bool TAIL = false, bool ONCE = false, bool SPLIT = false>
-__global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_kernel(const Args a) {
+__global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_kernel(const __grid_constant__ Args a) {
   using C = Cfg<BITS>;
   constexpr int kSW = SPLIT ? 16 : 8;        // softmax warps
   constexpr uint32_t kRowThreads = SPLIT ? 256 : 128;   // threads that work on one query tile
@@ -519,18 +557,14 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   const uint32_t b_pvdone2 = b_sfree + 16;             // [2 tiles][2 P buffers], 16-warp form
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sgen + kOffBar + kBarBytes - 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + kOffBar + kBarBytes - 12);
-  const WaitCtx wc{a.status, abort_flag};
+  const WaitCtx wc{abort_flag};
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (known to be the same in all lanes)
   constexpr bool kBf16 = (BITS == 16);
 
-  // this CTA's piece of the line of steps
-  const long long step_lo = piece_start(a.total, gridDim.x, blockIdx.x);
-  const long long step_hi = piece_start(a.total, gridDim.x, blockIdx.x + 1);
-
   if (tid == 0) {
-    *abort_flag = (*reinterpret_cast<volatile int*>(a.status) == (int)XKV_E_TIMEOUT) ? 1 : 0;   // an earlier CTA already gave up
+    *abort_flag = (*reinterpret_cast<volatile int*>(a.job[0].status) == (int)XKV_E_TIMEOUT) ? 1 : 0;   // an earlier CTA already gave up
     for (int i = 0; i < kNK; ++i) { mbar_init(b_kfull + 8 * i, 128); mbar_init(b_kfree + 8 * i, 2); }
     for (int i = 0; i < kNV; ++i) { mbar_init(b_vfull + 8 * i, 128); mbar_init(b_vfree + 8 * i, 2); }
     for (int i = 0; i < C::kNR; ++i) { mbar_init(b_rfull + 8 * i, 1); mbar_init(b_rfree + 8 * i, 128); }
@@ -577,7 +611,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const uint32_t colS = lane_addr + kColS1 + 64 * hf, colP0 = lane_addr + kColP2 + 128 * t + 32 * hf;
     const uint32_t colO = lane_addr + kColO + 64 * t + 32 * hf;
     const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 8 * t, pvdone2 = b_pvdone2 + 16 * t;
-    const int pad_tile = (a.t_first & 127) ? (a.t_first >> 7) : -1;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
     const int pair_bar = 2 + (warp & 7);     // named barrier of the two warps with these rows
     volatile float* xmine = reinterpret_cast<volatile float*>(sgen + kOffX) + ((t * 2 + hf) * 128 + r);
@@ -595,23 +628,22 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
     uint32_t g_seg = 0;                      // uses of the score buffer (both tiles) before this segment
     int seg_idx = 0;
-    for (long long pos = step_lo; pos < step_hi; ++seg_idx) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int h = item / a.n_pairs, pair = item - h * a.n_pairs;
-      const int qt = 2 * pair + t;
-      const uint32_t per_step = (2 * pair + 1 < a.q_tiles) ? 2u : 1u;   // tiles that use the score buffer
+    for (Walk walk(a); walk.next(a); ++seg_idx) {
+      const Job& job = a.job[walk.job];
+      const int h = walk.h, tile_lo = walk.tile_lo, nt = walk.nt;
+      const int qt = 2 * walk.pair + t;
+      // steps whose tile has masked columns: the pad slots after the first frame, the end
+      const int jj_pad = (job.t_first & 127) ? (job.t_first >> 7) - tile_lo : -1, jj_last = job.n_tiles - 1 - tile_lo;
+      const uint32_t per_step = (2 * walk.pair + 1 < job.q_tiles) ? 2u : 1u;   // tiles that use the score buffer
       const uint32_t use0 = g_seg + (uint32_t)t;     // this tile's uses: use0 + jj * per_step
       g_seg += (uint32_t)nt * per_step;
-      if (qt >= a.q_tiles) continue;          // the pair has no second tile
+      if (qt >= job.q_tiles) continue;          // the pair has no second tile
       // ---- Q tile: half of row r, bf16 -> operand type, into the swizzled K-major layout ----
       const int row = qt * kQRows + r;
       {
         uint4 u[4];
-        if (row < a.n) {
-          const __nv_bfloat16* qp = a.q + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
+        if (row < job.n) {
+          const __nv_bfloat16* qp = job.q + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
 #pragma unroll
           for (int c = 0; c < 4; ++c) u[c] = *reinterpret_cast<const uint4*>(qp + 8 * c);
         } else {
@@ -634,17 +666,16 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           }
           *reinterpret_cast<uint4*>(sgen + kOffQ + t * 16384 + swz_off(r, 4 * hf + c)) = o;
         }
-        if (q_bad) report_range(a.status);
+        if (q_bad) report_range(job.status);
         fence_proxy_async();
         mbar_arrive(b_qfull + 8 * t);
       }
       float m_ref = -INFINITY;   // reference maximum of the row (scaled, log2 units; the same in both halves)
       uint64_t l2 = 0ull, l2b = 0ull;   // four partial sums of this half of the row (two packed fp32 pairs)
       for (int jj = 0; jj < nt; ++jj, ++cnt) {
-        const int tile = tile_lo + jj;
-        int lim = 128;           // columns [lim, 128) are masked (pad slots after the first frame, the tail)
-        if (tile == pad_tile) lim = a.t_first & 127;
-        if (tile == a.n_tiles - 1) lim = min(lim, a.t_phys - tile * 128);
+        int lim = 128;           // columns [lim, 128) are masked
+        if (jj == jj_pad) lim = job.t_first & 127;
+        if (jj == jj_last) lim = min(lim, job.t_phys - (tile_lo + jj) * 128);
         mbar_wait(sfull, cnt & 1, wc);
         __syncwarp();            // the waits may leave the warp diverged; tcgen05.ld/st are warp-collective
         tc_fence_after();
@@ -729,14 +760,14 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       const float l_half = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
       const float l_peer = exchange(l_half);
       const float l = hf ? (l_peer + l_half) : (l_half + l_peer);     // the same sum in both halves
-      const bool whole = (tile_lo == 0 && nt == a.n_tiles);
+      const bool whole = (tile_lo == 0 && nt == job.n_tiles);
       uint32_t ro[32];
       XKV_TMEM_LD32(colO, ro);
       tc_wait_ld();
       if (whole) {
         const float inv_l = 1.f / l;
-        if (row < a.n) {
-          __nv_bfloat16* op = a.out + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
+        if (row < job.n) {
+          __nv_bfloat16* op = job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             uint32_t o[4];
@@ -766,24 +797,22 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const uint32_t colS = lane_addr + kColS + 128 * t, colP = lane_addr + kColP + 64 * t;
     const uint32_t colO = lane_addr + kColO + 64 * t;
     const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 8 * t, pvdone = b_pvdone + 8 * t, sfree = b_sfree + 8 * t;
-    const int pad_tile = (a.t_first & 127) ? (a.t_first >> 7) : -1;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
     uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
     int seg_idx = 0;
-    for (long long pos = step_lo; pos < step_hi; ++seg_idx) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int h = item / a.n_pairs, pair = item - h * a.n_pairs;
-      const int qt = 2 * pair + t;
-      if (qt >= a.q_tiles) continue;          // the pair has no second tile
+    for (Walk walk(a); walk.next(a); ++seg_idx) {
+      const Job& job = a.job[walk.job];
+      const int h = walk.h, tile_lo = walk.tile_lo, nt = walk.nt;
+      const int qt = 2 * walk.pair + t;
+      // steps whose tile has masked columns: the pad slots after the first frame, the end
+      const int jj_pad = (job.t_first & 127) ? (job.t_first >> 7) - tile_lo : -1, jj_last = job.n_tiles - 1 - tile_lo;
+      if (qt >= job.q_tiles) continue;          // the pair has no second tile
       // ---- Q tile: row r, bf16 -> operand type, into the swizzled K-major layout ----
       const int row = qt * kQRows + r;
       {
         uint4 u[8];
-        if (row < a.n) {
-          const __nv_bfloat16* qp = a.q + (int64_t)h * a.hs + (int64_t)row * a.ts;
+        if (row < job.n) {
+          const __nv_bfloat16* qp = job.q + (int64_t)h * a.hs + (int64_t)row * a.ts;
 #pragma unroll
           for (int c = 0; c < 8; ++c) u[c] = *reinterpret_cast<const uint4*>(qp + 8 * c);
         } else {
@@ -806,17 +835,16 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           }
           *reinterpret_cast<uint4*>(sgen + kOffQ + t * 16384 + swz_off(r, c)) = o;
         }
-        if (q_bad) report_range(a.status);
+        if (q_bad) report_range(job.status);
         fence_proxy_async();
         mbar_arrive(b_qfull + 8 * t);
       }
       float m_ref = -INFINITY;   // reference maximum (scaled, log2 units) used for the exponentials
       uint64_t l2 = 0ull;        // two partial row sums (packed fp32 pair)
       for (int jj = 0; jj < nt; ++jj, ++cnt) {
-        const int tile = tile_lo + jj;
-        int lim = 128;           // columns [lim, 128) are masked (pad slots after the first frame, the tail)
-        if (tile == pad_tile) lim = a.t_first & 127;
-        if (tile == a.n_tiles - 1) lim = min(lim, a.t_phys - tile * 128);
+        int lim = 128;           // columns [lim, 128) are masked
+        if (jj == jj_pad) lim = job.t_first & 127;
+        if (jj == jj_last) lim = min(lim, job.t_phys - (tile_lo + jj) * 128);
         mbar_wait(sfull, cnt & 1, wc);
         __syncwarp();            // the spin loops may leave the warp diverged; tcgen05.ld/st are warp-collective
         tc_fence_after();
@@ -968,7 +996,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       __syncwarp();
       tc_fence_after();
       const float l = f2_lo(l2) + f2_hi(l2);
-      const bool whole = (tile_lo == 0 && nt == a.n_tiles);
+      const bool whole = (tile_lo == 0 && nt == job.n_tiles);
       if (whole) {
         const float inv_l = 1.f / l;
 #pragma unroll 1
@@ -976,8 +1004,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           uint32_t ra[32];
           XKV_TMEM_LD32(colO + c0, ra);
           tc_wait_ld();
-          if (row < a.n) {
-            __nv_bfloat16* op = a.out + (int64_t)h * a.hs + (int64_t)row * a.ts + c0;
+          if (row < job.n) {
+            __nv_bfloat16* op = job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + c0;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               uint32_t o[4];
@@ -1013,32 +1041,30 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const int kb = t >> 3;        // keys kb + 16 i
     const uint32_t row_off = (uint32_t)((kb >> 3) * 1024 + (kb & 7) * 128 + ((w ^ (kb & 7)) << 4));
     uint32_t g = 0;               // steps so far (ring positions)
-    for (long long pos = step_lo; pos < step_hi;) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int h = item / a.n_pairs;
+    for (Walk walk(a); walk.next(a);) {
+      const Job& job = a.job[walk.job];
+      const int tile_lo = walk.tile_lo, nt = walk.nt;
+      const int h = walk.h;
       for (int jj = 0; jj < nt; ++jj, ++g) {
         // keys of this tile that belong to the unquantised newest frame (none without a tail)
         const int slot0 = (tile_lo + jj) * 128 + kb;              // this thread's keys: slot0 + 16 i
-        const bool tail_tile = TAIL && BITS == 4 && (tile_lo + jj) * 128 + 127 >= a.tail_lo;
-        const int64_t tail_off = (int64_t)h * a.tail_hs + 8 * w;
+        const bool tail_tile = TAIL && BITS == 4 && (tile_lo + jj) * 128 + 127 >= job.tail_lo;
+        const int64_t tail_off = (int64_t)h * a.hs + 8 * w;
         const uint32_t rs = g % C::kNR, ru = g / C::kNR;
         const uint32_t kbuf = g % kNK, ku = g / kNK;
         const uint32_t vbuf = g % kNV, vu = g / kNV;
         const uint8_t* raw = sgen + kOffRaw + rs * C::kRawStage;
         mbar_wait<256>(b_rfull + 8 * rs, ru & 1, wc);
-        if (TAIL && BITS == 4 && (tile_lo + jj) * 128 >= a.tail_lo && (tile_lo + jj) * 128 + 127 < a.t_phys) {
+        if (TAIL && BITS == 4 && (tile_lo + jj) * 128 >= job.tail_lo && (tile_lo + jj) * 128 + 127 < job.t_phys) {
           // ---- a tile that lies in the unquantised frame as a whole: K~ and V~ are the caller's
           // bf16 rows converted to fp16, the packed codes of the stage are not looked at ----
           bool bad = false;
 #pragma unroll
           for (int kv = 0; kv < 2; ++kv) {
-            const __nv_bfloat16* src = (kv ? a.v_tail : a.k_tail) + tail_off + (int64_t)(slot0 - a.tail_lo) * a.tail_ts;
+            const __nv_bfloat16* src = (kv ? job.v_tail : job.k_tail) + tail_off + (int64_t)(slot0 - job.tail_lo) * a.ts;
             uint4 u[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) u[i] = *reinterpret_cast<const uint4*>(src + (int64_t)(16 * i) * a.tail_ts);
+            for (int i = 0; i < 8; ++i) u[i] = *reinterpret_cast<const uint4*>(src + (int64_t)(16 * i) * a.ts);
             if (kv == 0) mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
             else mbar_wait<256>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
             uint8_t* dst = sgen + (kv ? kOffV + vbuf * 16384 : kOffK + kbuf * 16384) + row_off;
@@ -1051,7 +1077,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             fence_proxy_async();
             mbar_arrive(kv ? b_vfull + 8 * vbuf : b_kfull + 8 * kbuf);
           }
-          if (bad) report_range(a.status);
+          if (bad) report_range(job.status);
           mbar_arrive(b_rfree + 8 * rs);
           continue;
         }
@@ -1076,7 +1102,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             *reinterpret_cast<uint4*>(tab + 768 + 16 * t) =
                 make_uint4(pack_h2(vp.x, vp.x), pack_h2(vl, vl), pack_h2(vh, vh), pack_h2(vc, vc));
             // largest magnitude a code of this group / token can dequantise to
-            if (k_bad || beyond_fp16(fabsf(vp.x) * (fabsf(vp.y) + 15.f))) report_range(a.status);
+            if (k_bad || beyond_fp16(fabsf(vp.x) * (fabsf(vp.y) + 15.f))) report_range(job.status);
           }
           producer_sync();
           // ---- keys ----
@@ -1090,7 +1116,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             const uint8_t* slp = raw + C::kRawK + C::kRawV + 4 * kb;      // group references of keys kb + 16 i
             auto entry = [&](int i) {
               const int sl = *reinterpret_cast<const int*>(slp + 64 * i);
-              return reinterpret_cast<const uint4*>(a.ktab16 + (((size_t)sl * a.n_heads + h) * 8 + w) * 12);
+              return reinterpret_cast<const uint4*>(job.ktab16 + (((size_t)sl * job.n_heads + h) * 8 + w) * 12);
             };
             uint4 sv[2], zv[2], cv[2];
 #pragma unroll
@@ -1130,7 +1156,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           }
           }
           if (TAIL && tail_tile)
-            tail_rows_over(sgen + kOffK + kbuf * 16384 + row_off, a.k_tail + tail_off, a.tail_ts, slot0, a.tail_lo, a.t_phys, a.status);
+            tail_rows_over(sgen + kOffK + kbuf * 16384 + row_off, job.k_tail + tail_off, a.ts, slot0, job.tail_lo, job.t_phys, job.status);
           fence_proxy_async();
           mbar_arrive(b_kfull + 8 * kbuf);
           // ---- values ----
@@ -1146,7 +1172,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             *reinterpret_cast<uint4*>(sgen + kOffV + vbuf * 16384 + row_off + i * 2048) = o;
           }
           if (TAIL && tail_tile)
-            tail_rows_over(sgen + kOffV + vbuf * 16384 + row_off, a.v_tail + tail_off, a.tail_ts, slot0, a.tail_lo, a.t_phys, a.status);
+            tail_rows_over(sgen + kOffV + vbuf * 16384 + row_off, job.v_tail + tail_off, a.ts, slot0, job.tail_lo, job.t_phys, job.status);
           fence_proxy_async();
           mbar_arrive(b_vfull + 8 * vbuf);
           // The raw stage is released only here, after the words read from it have been used and
@@ -1161,7 +1187,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             float vl, vh, vc;
             dequant_consts(vp.x, vp.y, vl, vh, vc);
             *reinterpret_cast<uint4*>(tab + 768 + 16 * t) = make_uint4(pack_h2(vp.x, vp.x), pack_h2(vl, vl), 0u, pack_h2(vc, vc));
-            if (beyond_fp16(fabsf(vp.x) * (fabsf(vp.y) + 255.f))) report_range(a.status);
+            if (beyond_fp16(fabsf(vp.x) * (fabsf(vp.y) + 255.f))) report_range(job.status);
           }
           producer_sync();
           uint2 wd8[8];
@@ -1170,7 +1196,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           const uint8_t* slp = raw + C::kRawK + C::kRawV + 4 * kb;      // group references of keys kb + 16 i
           auto entry = [&](int i) {
             const int sl = *reinterpret_cast<const int*>(slp + 64 * i);
-            return reinterpret_cast<const uint4*>(a.ktab16 + (((size_t)sl * a.n_heads + h) * 8 + w) * 12);
+            return reinterpret_cast<const uint4*>(job.ktab16 + (((size_t)sl * job.n_heads + h) * 8 + w) * 12);
           };
           uint4 sv[2], zv[2], cv[2];
 #pragma unroll
@@ -1246,14 +1272,11 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const uint32_t d_s = tmem + kColS1, d_p0 = tmem + kColP2 + 128 * t, d_o = tmem + kColO + 64 * t;
     uint32_t g = 0, cp = 0, segq = 0;
     uint32_t g_seg = 0;              // score-buffer uses before this segment
-    for (long long pos = step_lo; pos < step_hi;) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int pair = item % a.n_pairs;
-      const bool active = 2 * pair + t < a.q_tiles;
-      const uint32_t per_step = (2 * pair + 1 < a.q_tiles) ? 2u : 1u;     // tiles that use the score buffer
+    for (Walk walk(a); walk.next(a);) {
+      const Job& job = a.job[walk.job];
+      const int nt = walk.nt;
+      const bool active = 2 * walk.pair + t < job.q_tiles;
+      const uint32_t per_step = (2 * walk.pair + 1 < job.q_tiles) ? 2u : 1u;     // tiles that use the score buffer
       auto issue_pv = [&](uint32_t gv, bool first_of_segment) {
         mbar_wait(b_vfull + 8 * (gv % kNV), (gv / kNV) & 1, wc);
         if (active) {
@@ -1315,13 +1338,10 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const uint64_t dq = make_desc(sQ + t * 16384);
     const uint32_t d_s = tmem + kColS + 128 * t, d_p = tmem + kColP + 64 * t, d_o = tmem + kColO + 64 * t;
     uint32_t g = 0, cnt = 0, segq = 0;
-    for (long long pos = step_lo; pos < step_hi;) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int pair = item % a.n_pairs;
-      const bool active = 2 * pair + t < a.q_tiles;
+    for (Walk walk(a); walk.next(a);) {
+      const Job& job = a.job[walk.job];
+      const int nt = walk.nt;
+      const bool active = 2 * walk.pair + t < job.q_tiles;
       auto issue_pv = [&](uint32_t gv, bool first_of_segment) {
         mbar_wait(b_vfull + 8 * (gv % kNV), (gv / kNV) & 1, wc);
         if (active) {
@@ -1369,13 +1389,11 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   } else if (tid == 32 * (kSW + 5)) {
     // =========================== TMA loader ===================================
     uint32_t g = 0;
-    for (long long pos = step_lo; pos < step_hi;) {
-      const int item = (int)(pos / a.n_tiles);
-      const int tile_lo = (int)(pos - (long long)item * a.n_tiles);
-      const int nt = (int)min((long long)(a.n_tiles - tile_lo), step_hi - pos);
-      pos += nt;
-      const int h = item / a.n_pairs;
-      const size_t head_slot = (size_t)h * a.cap;
+    for (Walk walk(a); walk.next(a);) {
+      const Job& job = a.job[walk.job];
+      const int tile_lo = walk.tile_lo, nt = walk.nt;
+      const int h = walk.h;
+      const size_t head_slot = (size_t)h * job.cap;
       for (int jj = 0; jj < nt; ++jj, ++g) {
         const int tile = tile_lo + jj;
         const uint32_t rs = g % C::kNR, ru = g / C::kNR;
@@ -1385,19 +1403,19 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         mbar_expect_tx(bar, C::kRawStage - C::kRawKP + kp_bytes);
         const size_t slot0 = head_slot + (size_t)tile * 128;
         if (BITS == 4) {
-          tma_load_1d(dst, a.k + slot0 * 32, C::kRawK, bar);
-          tma_load_1d(dst + C::kRawK, a.v + slot0 * 32, C::kRawV, bar);
-          if (ONCE) tma_load_1d(dst + C::kRawK + C::kRawV, a.kslot + (size_t)tile * 128, kp_bytes, bar);
-          else tma_load_1d(dst + C::kRawK + C::kRawV, a.kpar + ((size_t)h * (a.cap >> 6) + 2 * tile) * 64, C::kRawKP, bar);
-          tma_load_1d(dst + C::kRawK + C::kRawV + C::kRawKP, a.vpar + slot0, C::kRawVP, bar);
+          tma_load_1d(dst, job.k + slot0 * 32, C::kRawK, bar);
+          tma_load_1d(dst + C::kRawK, job.v + slot0 * 32, C::kRawV, bar);
+          if (ONCE) tma_load_1d(dst + C::kRawK + C::kRawV, job.kslot + (size_t)tile * 128, kp_bytes, bar);
+          else tma_load_1d(dst + C::kRawK + C::kRawV, job.kpar + ((size_t)h * (job.cap >> 6) + 2 * tile) * 64, C::kRawKP, bar);
+          tma_load_1d(dst + C::kRawK + C::kRawV + C::kRawKP, job.vpar + slot0, C::kRawVP, bar);
         } else if (BITS == 8) {
-          tma_load_1d(dst, a.k + slot0 * 64, C::kRawK, bar);
-          tma_load_1d(dst + C::kRawK, a.v + slot0 * 64, C::kRawV, bar);
-          tma_load_1d(dst + C::kRawK + C::kRawV, a.kslot + (size_t)tile * 128, kp_bytes, bar);
-          tma_load_1d(dst + C::kRawK + C::kRawV + C::kRawKP, a.vpar + slot0, C::kRawVP, bar);
+          tma_load_1d(dst, job.k + slot0 * 64, C::kRawK, bar);
+          tma_load_1d(dst + C::kRawK, job.v + slot0 * 64, C::kRawV, bar);
+          tma_load_1d(dst + C::kRawK + C::kRawV, job.kslot + (size_t)tile * 128, kp_bytes, bar);
+          tma_load_1d(dst + C::kRawK + C::kRawV + C::kRawKP, job.vpar + slot0, C::kRawVP, bar);
         } else {
-          tma_load_1d(dst, a.k + slot0 * 128, C::kRawK, bar);
-          tma_load_1d(dst + C::kRawK, a.v + slot0 * 128, C::kRawV, bar);
+          tma_load_1d(dst, job.k + slot0 * 128, C::kRawK, bar);
+          tma_load_1d(dst + C::kRawK, job.v + slot0 * 128, C::kRawV, bar);
         }
       }
     }
@@ -1412,6 +1430,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     }
   }
   __syncthreads();
+  if (tid == 0 && *abort_flag) report_timeout(a);
   if (warp == kSW + 5) {
     __syncwarp();
     tc_fence_after();
@@ -1421,40 +1440,36 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
 
 // ---------------------------------------------------------------------------
 // Merge of the partial results of the items that were cut between CTAs:
-// out = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.  Thread = (item, query
-// tile, row, 8-channel chunk); items that one CTA covered alone were written by it.
+// out = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s.  Eight blocks per cut of the line (the start
+// of a piece); the first cut inside an item does the whole item, the others have nothing to do.
+// Thread = (row, 8-channel chunk) of a query tile.  Items that one CTA covered alone were
+// written by it.
 // ---------------------------------------------------------------------------
-// IDX = uint32_t when total * grid fits 32 bits (the divisions are then cheap), else uint64_t.
-template <typename IDX>
 __global__ void __launch_bounds__(256)
-attn_combine_kernel(const float* __restrict__ part_o, const float2* __restrict__ part_ml, int grid_i, long long total_ll,
-                    int n_tiles, int n_pairs, int q_tiles, int n, __nv_bfloat16* __restrict__ out, int64_t ts,
-                    int64_t hs) {
-  const IDX grid = (IDX)grid_i, total = (IDX)total_ll;
-  const long long gidx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int ch = (int)(gidx & 7);
-  const int r = (int)((gidx >> 3) & 127);
-  const int t = (int)((gidx >> 10) & 1);
-  const IDX item = (IDX)(gidx >> 11);
-  if ((long long)item * n_tiles >= total_ll) return;
-  const int h = (int)(item / (IDX)n_pairs), pair = (int)(item - (IDX)h * (IDX)n_pairs);
+attn_combine_kernel(const __grid_constant__ Args a) {
+  const int cut = (int)(blockIdx.x >> 3) + 1, t = (int)(blockIdx.x >> 2) & 1;
+  const int r = (int)(blockIdx.x & 3) * 32 + (int)(threadIdx.x >> 3), ch = (int)(threadIdx.x & 7);
+  const uint32_t at = piece_start(a, cut), before = piece_start(a, cut - 1);
+  int jn = 0;
+  while (at >= a.job[jn].step_hi) ++jn;
+  const Job& job = a.job[jn];
+  const uint32_t tiles = (uint32_t)job.n_tiles, pairs = (uint32_t)job.n_pairs;
+  const uint32_t item = (at - job.step_lo) / tiles;
+  const uint32_t lo = job.step_lo + item * tiles, hi = lo + tiles;
+  if (at == lo || before > lo) return;           // between two items; not the item's first cut
+  const int h = (int)(item / pairs), pair = (int)(item % pairs);
   const int qt = 2 * pair + t;
   const int row = qt * 128 + r;
-  if (qt >= q_tiles || row >= n) return;
-  const IDX lo = item * (IDX)n_tiles, hi = lo + (IDX)n_tiles;
-  // CTA that holds step x: the largest b with piece_start(b) <= x
-  const int b_first = (int)(((lo + 1) * grid - 1) / total);
-  const int b_last = (int)((hi * grid - 1) / total);
-  if (b_first == b_last) return;                 // one CTA covered the whole item and wrote the result
-  // a piece's first segment (slot 0) is this item iff the piece starts inside it: only the first
-  // piece of the item can start before it
-  const bool first_is_second_slot = (total * (IDX)b_first) / grid < lo;
+  if (qt >= job.q_tiles || row >= job.n) return;
+  const int b_first = cut - 1;
+  // the piece before the cut holds the item in its second slot if it began with another item
+  const bool first_is_second_slot = before < lo;
   // The partials are fetched four at a time, all loads before the first use (an item is cut into
   // two or three pieces unless the cache is very long); the running maximum and the weights are
   // those of the online softmax, in the fixed order of the pieces.
   float m = -INFINITY, l = 0.f;
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int b0 = b_first; b0 <= b_last; b0 += 4) {
+  for (int b0 = b_first; b0 < a.grid && (b0 == b_first || piece_start(a, b0) < hi); b0 += 4) {
     float2 ml[4];
     float4 x[4], y[4];
 #pragma unroll
@@ -1462,11 +1477,11 @@ attn_combine_kernel(const float* __restrict__ part_o, const float2* __restrict__
       const int b = b0 + j;
       ml[j] = make_float2(-INFINITY, 0.f);
       x[j] = y[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (b <= b_last) {
+      if (b < a.grid && (b == b_first || piece_start(a, b) < hi)) {
         const size_t slot = (size_t)2 * b + ((b == b_first && first_is_second_slot) ? 1 : 0);
         const size_t prow = (slot * 2 + t) * 128 + r;
-        ml[j] = part_ml[prow];
-        const float4* po = reinterpret_cast<const float4*>(part_o + prow * 64 + 8 * ch);
+        ml[j] = a.part_ml[prow];
+        const float4* po = reinterpret_cast<const float4*>(a.part_o + prow * 64 + 8 * ch);
         x[j] = po[0];
         y[j] = po[1];
       }
@@ -1489,15 +1504,10 @@ attn_combine_kernel(const float* __restrict__ part_o, const float2* __restrict__
   uint32_t o[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) o[i] = pack_bf2(acc[2 * i] * inv, acc[2 * i + 1] * inv);
-  *reinterpret_cast<uint4*>(out + (int64_t)h * hs + (int64_t)row * ts + 8 * ch) = make_uint4(o[0], o[1], o[2], o[3]);
+  *reinterpret_cast<uint4*>(job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + 8 * ch) = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 size_t attn_tc_scratch_bytes(const xkv_params*) { return (size_t)2 * kMaxGrid * kSlotBytes + 512; }
-
-// `part` holds the partial slots: accumulators float [slots][2][128][64], then (max, sum) float2
-// [slots][2][128], slots = part_bytes / kSlotBytes.  The grid is the SM count, capped by the slots
-// available (two per CTA) and by the number of steps.
-struct TailArgs { const void* k; const void* v; int64_t ts, hs; };
 
 // Per device, on first use with that device current: the SM count, and the opt-in to more than
 // 48 KB of dynamic shared memory for the attention kernels (a per-device function attribute).
@@ -1551,56 +1561,51 @@ static cudaError_t attn_device_setup(int* sm_count) {
   return cudaSuccess;
 }
 
-static cudaError_t launch_attn_tc_on(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs,
-                                     float scale, float* part, size_t part_bytes, cudaStream_t st,
-                                     const TailArgs* tail = nullptr, int prefix = 0) {
-  int sm_count = 0;
-  {
-    const cudaError_t e = attn_device_setup(&sm_count);
-    if (e != cudaSuccess) return e;
-  }
-  Args a;
-  a.q = reinterpret_cast<const __nv_bfloat16*>(q);
-  a.out = reinterpret_cast<__nv_bfloat16*>(out);
-  a.n = n; a.ts = ts; a.hs = hs;
+static void fill_job(Job* j, const AttnCall& call) {
+  const xkv_cache* c = call.cache;
   const BufSet& b = c->buf[c->cur];
-  a.k = b.k; a.kpar = b.kpar; a.v = b.v; a.vpar = b.vpar;
-  a.cap = c->cap; a.t_first = c->T_first;
-  a.t_phys = c->rest_base + (c->T - c->T_first);
-  if (c->T == c->T_first) a.t_phys = c->T_first;          // only the first frame: no pad tile beyond it
-  if (prefix > 0 && prefix < c->T) {
+  j->q = reinterpret_cast<const __nv_bfloat16*>(call.q);
+  j->out = reinterpret_cast<__nv_bfloat16*>(call.out);
+  j->k = b.k; j->kpar = b.kpar; j->v = b.v; j->vpar = b.vpar;
+  j->kslot = b.kslot; j->ktab16 = c->ktab16;
+  j->status = c->status;
+  j->n = call.n; j->cap = c->cap; j->n_heads = c->p.n_heads;
+  j->t_first = c->T_first;
+  j->t_phys = c->rest_base + (c->T - c->T_first);
+  if (c->T == c->T_first) j->t_phys = c->T_first;         // only the first frame: no pad tile beyond it
+  if (call.prefix > 0 && call.prefix < c->T) {
     // a prefix of the cache in logical order: inside the first frame it ends the first segment,
     // after it the rest segment
-    if (prefix <= c->T_first) { a.t_first = prefix; a.t_phys = prefix; }
-    else a.t_phys = c->rest_base + (prefix - c->T_first);
+    if (call.prefix <= c->T_first) { j->t_first = call.prefix; j->t_phys = call.prefix; }
+    else j->t_phys = c->rest_base + (call.prefix - c->T_first);
   }
-  a.scale_log2 = scale * 1.4426950408889634f;
-  a.n_tiles = (a.t_phys + 127) / 128;
-  a.q_tiles = (n + kQRows - 1) / kQRows;
-  a.n_pairs = (a.q_tiles + 1) / 2;
-  const int H = c->p.n_heads;
-  a.total = (long long)H * a.n_pairs * a.n_tiles;
+  j->k_tail = j->v_tail = nullptr;
+  j->tail_lo = j->t_phys;
+  if (call.k_tail && c->p.kv_bits == 4) {      // a 16-bit cache holds the frame exactly as it arrived
+    j->k_tail = reinterpret_cast<const __nv_bfloat16*>(call.k_tail);
+    j->v_tail = reinterpret_cast<const __nv_bfloat16*>(call.v_tail);
+    j->tail_lo = j->t_phys - call.n;           // the newest frame holds the last n slots
+  }
+  j->n_tiles = (j->t_phys + 127) / 128;
+  j->q_tiles = (call.n + kQRows - 1) / kQRows;
+  j->n_pairs = (j->q_tiles + 1) / 2;
+}
+
+// One launch (and its merge) for the jobs in `a`.  `part` holds the partial slots: accumulators float
+// [slots][2][128][64], then (max, sum) float2 [slots][2][128], slots = part_bytes / kSlotBytes.  The
+// grid is the SM count, capped by the slots available (two per CTA) and by the number of steps.
+static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail, float* part, size_t part_bytes, int sm_count, cudaStream_t st) {
   const size_t slots = part_bytes / kSlotBytes;
   long long grid = sm_count;
   if (grid > (long long)(slots / 2)) grid = (long long)(slots / 2);
   if (c->attn_max_blocks > 0 && grid > c->attn_max_blocks) grid = c->attn_max_blocks;
-  if (grid > a.total) grid = a.total;
+  if (grid > (long long)total) grid = total;
   if (grid < 1) return cudaErrorMemoryAllocation;
+  a.grid = (int)grid;
+  a.piece = total / (uint32_t)grid;
+  a.longer = total % (uint32_t)grid;
   a.part_o = part;
   a.part_ml = reinterpret_cast<float2*>(part + slots * kSlotFloats);
-  a.status = c->status;
-  a.kslot = b.kslot; a.ktab16 = c->ktab16; a.n_heads = H;
-  a.k_tail = a.v_tail = nullptr;
-  a.tail_ts = a.tail_hs = 0;
-  a.tail_lo = a.t_phys;
-  if (tail && c->p.kv_bits == 8) return cudaErrorNotSupported;      // (the unquantised tail is built for 4-bit caches)
-  if (tail && c->p.kv_bits == 4) {      // a 16-bit cache holds the frame exactly as it arrived
-    a.k_tail = reinterpret_cast<const __nv_bfloat16*>(tail->k);
-    a.v_tail = reinterpret_cast<const __nv_bfloat16*>(tail->v);
-    a.tail_ts = tail->ts;
-    a.tail_hs = tail->hs;
-    a.tail_lo = a.t_phys - n;           // the newest frame holds the last n slots
-  }
   {
     LaunchScope ls(c, XKV_PROF_ATTN, st);
     const bool once = c->p.key_mode == XKV_KEYS_ONCE;
@@ -1610,36 +1615,57 @@ static cudaError_t launch_attn_tc_on(xkv_cache* c, const void* q, void* out, int
     const int T = kThreadsSplit;
     if (c->p.kv_bits == 16) attn_tc_kernel<16, false, false, true><<<(int)grid, T, smem_bytes<16, true>(), st>>>(a);
     else if (c->p.kv_bits == 8) attn_tc_kernel<8, false, true><<<(int)grid, kThreads, smem_bytes<8>(), st>>>(a);
-    else if (a.k_tail && once) attn_tc_kernel<4, true, true><<<(int)grid, kThreads, smem_bytes<4>(), st>>>(a);
-    else if (a.k_tail) attn_tc_kernel<4, true, false, true><<<(int)grid, T, smem_bytes<4, true>(), st>>>(a);
+    else if (tail && once) attn_tc_kernel<4, true, true><<<(int)grid, kThreads, smem_bytes<4>(), st>>>(a);
+    else if (tail) attn_tc_kernel<4, true, false, true><<<(int)grid, T, smem_bytes<4, true>(), st>>>(a);
     else if (once) attn_tc_kernel<4, false, true><<<(int)grid, kThreads, smem_bytes<4>(), st>>>(a);
     else attn_tc_kernel<4, false, false, true><<<(int)grid, T, smem_bytes<4, true>(), st>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  {
+  if (grid > 1) {
     LaunchScope ls(c, XKV_PROF_COMBINE, st);
-    const long long threads = (long long)H * a.n_pairs * 2048;
-    const int blocks = (int)((threads + 255) / 256);
-    if ((a.total + 1) * grid < (1ll << 31))
-      attn_combine_kernel<uint32_t><<<blocks, 256, 0, st>>>(a.part_o, a.part_ml, (int)grid, a.total, a.n_tiles,
-                                                            a.n_pairs, a.q_tiles, n, a.out, ts, hs);
-    else
-      attn_combine_kernel<uint64_t><<<blocks, 256, 0, st>>>(a.part_o, a.part_ml, (int)grid, a.total, a.n_tiles,
-                                                            a.n_pairs, a.q_tiles, n, a.out, ts, hs);
+    attn_combine_kernel<<<(int)(grid - 1) * 8, 256, 0, st>>>(a);
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_attn_tc(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs, float scale,
-                           cudaStream_t st, int prefix) {
-  return launch_attn_tc_on(c, q, out, n, ts, hs, scale, c->attn_part, c->attn_part_bytes, st, nullptr, prefix);
+static cudaError_t launch_attn_tc_on(const AttnCall* calls, int count, int64_t ts, int64_t hs, float scale, float* part,
+                                     size_t part_bytes, cudaStream_t st) {
+  int sm_count = 0;
+  {
+    const cudaError_t e = attn_device_setup(&sm_count);
+    if (e != cudaSuccess) return e;
+  }
+  xkv_cache* lead = calls[0].cache;
+  const bool tail = calls[0].k_tail && lead->p.kv_bits == 4;
+  if (calls[0].k_tail && lead->p.kv_bits == 8) return cudaErrorNotSupported;      // (the unquantised tail is built for 4-bit caches)
+  Args a;
+  a.ts = ts; a.hs = hs;
+  a.scale_log2 = scale * 1.4426950408889634f;
+  for (int i = 0; i < count;) {
+    a.n_jobs = 0;
+    uint32_t total = 0;
+    for (; i < count && a.n_jobs < kMaxJobs; ++i) {
+      Job* j = &a.job[a.n_jobs];
+      fill_job(j, calls[i]);
+      const uint64_t steps = (uint64_t)j->n_heads * j->n_pairs * j->n_tiles;
+      if (total + steps >= (1ull << 32)) {
+        if (a.n_jobs > 0) break;
+        return cudaErrorNotSupported;          // (no workspace of that size fits a GPU)
+      }
+      j->step_lo = total;
+      total += (uint32_t)steps;
+      j->step_hi = total;
+      a.n_jobs++;
+    }
+    const cudaError_t e = launch_jobs(lead, a, total, tail, part, part_bytes, sm_count, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
-cudaError_t launch_attn_tc_tail(xkv_cache* c, const void* q, const void* k_t, const void* v_t, void* out, int n,
-                                int64_t ts, int64_t hs, float scale, cudaStream_t st) {
-  const TailArgs tail{k_t, v_t, ts, hs};
-  return launch_attn_tc_on(c, q, out, n, ts, hs, scale, c->attn_part, c->attn_part_bytes, st, &tail);
+cudaError_t launch_attn_tc(const AttnCall* calls, int count, int64_t ts, int64_t hs, float scale, cudaStream_t st) {
+  return launch_attn_tc_on(calls, count, ts, hs, scale, calls[0].cache->attn_part, calls[0].cache->attn_part_bytes, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -1654,8 +1680,7 @@ static __device__ __align__(256) unsigned char g_static_partials[XKV_STATIC_SCRA
 static std::mutex g_static_mutex;
 static void* g_static_addr[kMaxDevices] = {nullptr};
 
-cudaError_t launch_attn_tc_static(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs,
-                                  float scale, cudaStream_t st) {
+cudaError_t launch_attn_tc_static(const AttnCall& call, int64_t ts, int64_t hs, float scale, cudaStream_t st) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -1671,14 +1696,13 @@ cudaError_t launch_attn_tc_static(xkv_cache* c, const void* q, void* out, int n,
     }
     addr = g_static_addr[dev];
   }
-  return launch_attn_tc_on(c, q, out, n, ts, hs, scale, reinterpret_cast<float*>(addr),
-                           (size_t)XKV_STATIC_SCRATCH_BYTES, st);
+  return launch_attn_tc_on(&call, 1, ts, hs, scale, reinterpret_cast<float*>(addr), (size_t)XKV_STATIC_SCRATCH_BYTES, st);
 }
 
 // ---------------------------------------------------------------------------
 // Test hook: the bounded wait of the attention kernel on a barrier that nothing completes.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(32) timeout_probe_kernel(int* status) {
+__global__ void __launch_bounds__(32) timeout_probe_kernel(const __grid_constant__ Args a) {
   __shared__ __align__(8) unsigned long long bar;
   __shared__ int abort_flag;
   if (threadIdx.x == 0) {
@@ -1687,14 +1711,19 @@ __global__ void __launch_bounds__(32) timeout_probe_kernel(int* status) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const WaitCtx wc{status, &abort_flag};
+  const WaitCtx wc{&abort_flag};
   if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, wc);     // phase 0 never completes: runs into the limit
   __syncthreads();
   mbar_wait(smem_u32(&bar), 0, wc);                           // the flag is up: every later wait returns at once
+  __syncthreads();
+  if (threadIdx.x == 0 && abort_flag) report_timeout(a);
 }
 
 cudaError_t launch_timeout_probe(xkv_cache* c, cudaStream_t st) {
-  timeout_probe_kernel<<<1, 32, 0, st>>>(c->status);
+  Args a;
+  a.n_jobs = 1;
+  a.job[0].status = c->status;
+  timeout_probe_kernel<<<1, 32, 0, st>>>(a);
   c->launches++;
   return cudaGetLastError();
 }

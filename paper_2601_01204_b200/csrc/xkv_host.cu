@@ -383,7 +383,7 @@ int kv_quant_pack(xkv_cache* c, xkv_stream stream) {
   MaintArgs a;
   maint_args(c, &a);
   if (c->p.kv_bits == 4 && !keys_once(c)) {
-    if (launch_regroup(c, a, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return XKV_E_CUDA;
+    if (launch_regroup(&c, &a, 1, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return XKV_E_CUDA;
   } else if (c->kk_pending > 0 || (keys_once(c) && c->rold_pending > 0)) {   // survivors to move, or table slots to release
     a.phases = kPhPack;
     if (launch_maint(c, a, XKV_PROF_PACK, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return XKV_E_CUDA;
@@ -405,7 +405,8 @@ int attn_packed_causal(xkv_cache* c, const void* q, void* out, int32_t n, int64_
   if (impl == 1) {
     e = launch_attn_simple(c, q, out, n, ts, hs, softmax_scale, st);
   } else {
-    e = launch_attn_tc(c, q, out, n, ts, hs, softmax_scale, st);
+    const AttnCall call{c, q, out, n, 0, nullptr, nullptr};
+    e = launch_attn_tc(&call, 1, ts, hs, softmax_scale, st);
     if (e == cudaErrorNotSupported) return XKV_E_UNSUPPORTED;
   }
   if (e != cudaSuccess) return XKV_E_CUDA;
@@ -420,8 +421,8 @@ int attn_packed_causal_tail(xkv_cache* c, const void* q, const void* k_t, const 
   if (n < 1 || n != c->n_pending || !aligned16(q) || !aligned16(k_t) || !aligned16(v_t) || !aligned16(out) ||
       !strides_ok(ts, hs) || !(softmax_scale > 0.f))
     return XKV_E_INVALID;
-  const cudaError_t e =
-      launch_attn_tc_tail(c, q, k_t, v_t, out, n, ts, hs, softmax_scale, reinterpret_cast<cudaStream_t>(stream));
+  const AttnCall call{c, q, out, n, 0, k_t, v_t};
+  const cudaError_t e = launch_attn_tc(&call, 1, ts, hs, softmax_scale, reinterpret_cast<cudaStream_t>(stream));
   if (e == cudaErrorNotSupported) return XKV_E_UNSUPPORTED;
   if (e != cudaSuccess) return XKV_E_CUDA;
   c->stage = 0;
@@ -440,19 +441,20 @@ int attn_packed_frame_causal(xkv_cache* c, const void* q, void* out, const int32
     total += frame_tokens[f];
   }
   if (total != c->n_pending) return XKV_E_INVALID;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const int before = c->T - c->n_pending;              // cached tokens older than the chunk
+  std::vector<AttnCall> calls;                         // the frames' attentions, in one launch
+  try { calls.reserve(n_frames); } catch (const std::bad_alloc&) { return XKV_E_NOMEM; }
   int r0 = 0;
   for (int f = 0; f < n_frames; ++f) {
     const int nf = frame_tokens[f];
-    const __nv_bfloat16* qf = reinterpret_cast<const __nv_bfloat16*>(q) + (int64_t)r0 * ts;
-    __nv_bfloat16* of = reinterpret_cast<__nv_bfloat16*>(out) + (int64_t)r0 * ts;
     // (strides are multiples of 8 elements, so every frame's first row is 16-byte aligned)
-    const cudaError_t e = launch_attn_tc(c, qf, of, nf, ts, hs, softmax_scale, st, before + r0 + nf);
-    if (e == cudaErrorNotSupported) return XKV_E_UNSUPPORTED;
-    if (e != cudaSuccess) return XKV_E_CUDA;
+    calls.push_back({c, reinterpret_cast<const __nv_bfloat16*>(q) + (int64_t)r0 * ts,
+                     reinterpret_cast<__nv_bfloat16*>(out) + (int64_t)r0 * ts, nf, before + r0 + nf, nullptr, nullptr});
     r0 += nf;
   }
+  const cudaError_t e = launch_attn_tc(calls.data(), n_frames, ts, hs, softmax_scale, reinterpret_cast<cudaStream_t>(stream));
+  if (e == cudaErrorNotSupported) return XKV_E_UNSUPPORTED;
+  if (e != cudaSuccess) return XKV_E_CUDA;
   c->stage = 0;
   return XKV_OK;
 }
@@ -487,7 +489,8 @@ int attn_packed_causal_static(xkv_cache* c, const void* q, void* out, int32_t n,
   if (n < 1 || n > c->p.max_frame_tokens || !aligned16(q) || !aligned16(out) || !strides_ok(ts, hs) ||
       !(softmax_scale > 0.f))
     return XKV_E_INVALID;
-  const cudaError_t e = launch_attn_tc_static(c, q, out, n, ts, hs, softmax_scale, reinterpret_cast<cudaStream_t>(stream));
+  const AttnCall call{c, q, out, n, 0, nullptr, nullptr};
+  const cudaError_t e = launch_attn_tc_static(call, ts, hs, softmax_scale, reinterpret_cast<cudaStream_t>(stream));
   if (e == cudaErrorMemoryAllocation) return XKV_E_LIMIT;
   if (e == cudaErrorNotSupported) return XKV_E_UNSUPPORTED;
   if (e != cudaSuccess) return XKV_E_CUDA;
@@ -504,7 +507,8 @@ struct HostStepPipe {
   cudaStream_t up2 = nullptr;                     // a second host -> device stream (two copy engines: 49 GB/s against
                                                   // 31 GB/s for 2.8 MB copies on one stream)
   cudaEvent_t up2_done[2] = {nullptr, nullptr};
-  cudaStream_t side = nullptr;                    // kv_append of a layer, beside its scoring
+  cudaStream_t side = nullptr;                    // head means of the keys, beside the attention
+  bool side_busy = false;                         // started there and not yet ordered before the caller's stream
   cudaEvent_t fork = nullptr, join = nullptr;
   cudaEvent_t start = nullptr;                    // the caller's stream at entry
   cudaEvent_t up_done[2] = {nullptr, nullptr};    // inputs of the layer in slot s are on the device
@@ -538,85 +542,103 @@ HostStepPipe* host_step_pipe() {
   return &p;
 }
 
-// One layer, one frame: the three maintenance calls as one launch, then -- on the library's side
-// stream, beside the attention -- the head means of the keys of the cache just built (Eq. 4), from
-// which the next frame's scoring starts.
-int run_layer(HostStepPipe* pipe, xkv_cache* c, const void* q, const void* k, const void* v, void* out, int32_t n,
-              int64_t ts, int64_t hs, cudaStream_t st) {
-  xkv_stream stream = reinterpret_cast<xkv_stream>(st);
+// The maintenance of one layer for one frame as one launch's arguments; the cache's host state moves
+// to "frame pending".
+int prepare_layer(xkv_cache* c, const void* q, const void* k, const void* v, void* out, int32_t n, int64_t ts, int64_t hs,
+                  MaintArgs* a) {
+  if (!c) return XKV_E_INVALID;
   if (c->stage != 0) return XKV_E_STATE;
-  if (n < 1 || n > c->p.max_frame_tokens || !aligned16(k) || !aligned16(v) || !aligned16(q) || !strides_ok(ts, hs))
+  if (n < 1 || n > c->p.max_frame_tokens || !aligned16(k) || !aligned16(v) || !aligned16(q) || !aligned16(out) || !strides_ok(ts, hs))
     return XKV_E_INVALID;
   FramePlan plan;
-  int rc = plan_frame(c, n, &plan);
+  const int rc = plan_frame(c, n, &plan);
   if (rc != XKV_OK) return rc;
   set_pending(c, n, plan);
   note_scored(c);
-  MaintArgs a;
-  maint_args(c, &a);
+  maint_args(c, a);
   const bool once = keys_once(c);
-  a.phases = kPhAppend;
-  if ((c->p.kv_bits == 16 && c->kk_pending > 0) || (once && (c->kk_pending > 0 || c->rold_pending > 0))) a.phases |= kPhPack;
+  a->phases = kPhAppend;
+  if ((c->p.kv_bits == 16 && c->kk_pending > 0) || (once && (c->kk_pending > 0 || c->rold_pending > 0))) a->phases |= kPhPack;
   if (selecting(c)) {
-    a.phases |= kPhPool | kPhScore | kPhSel;
-    if (once) {
-      // the head means travel with the tokens; those of the frame before were computed beside its attention
-      if (c->kbar_frames == c->frames && cudaStreamWaitEvent(st, c->kbar_done, 0) != cudaSuccess) return XKV_E_CUDA;
-    } else if (kbar_fresh(c)) {
-      if (cudaStreamWaitEvent(st, c->kbar_done, 0) != cudaSuccess) return XKV_E_CUDA;
-    } else {
-      a.phases |= kPhKbar;
-      a.kbar_on_other = 0; a.kbar_lo = 0; a.kbar_hi = c->rold_pending;
+    // (the head means: those of the last step were computed beside its attention, and its caller's
+    // stream has waited for them; in quantise-once mode they travel with the tokens)
+    a->phases |= kPhPool | kPhScore | kPhSel;
+    if (!once && !kbar_fresh(c)) {
+      a->phases |= kPhKbar;
+      a->kbar_on_other = 0; a->kbar_lo = 0; a->kbar_hi = c->rold_pending;
     }
   }
-  a.q = reinterpret_cast<const __nv_bfloat16*>(q);
-  a.k = reinterpret_cast<const __nv_bfloat16*>(k);
-  a.v = reinterpret_cast<const __nv_bfloat16*>(v);
-  a.ts_q = a.ts_kv = ts; a.hs_q = a.hs_kv = hs;
-  if (launch_maint(c, a, XKV_PROF_MAINT, st) != cudaSuccess) return XKV_E_CUDA;
-  if (once) c->pop_base += (uint32_t)((n + 63) / 64);
-  if (c->p.kv_bits == 4 && !once && launch_regroup(c, a, st) != cudaSuccess) return XKV_E_CUDA;
-  note_packed(c);
-  c->stage = 3;
-  // Head means of the keys (Eq. 4), needed by the next frame's scoring only: on the side stream,
-  // beside the attention.  The side stream forks here (after the packing) but its kernel is
-  // launched after the attention has been enqueued, so that the attention's blocks get the
-  // multiprocessors first and the head means fill in as they retire.
-  const bool want_kbar = once ? !plan.first : (c->T > c->T_first);
-  if (want_kbar && !(cudaEventRecord(pipe->fork, st) == cudaSuccess &&
-                     cudaStreamWaitEvent(pipe->side, pipe->fork, 0) == cudaSuccess))
+  a->q = reinterpret_cast<const __nv_bfloat16*>(q);
+  a->k = reinterpret_cast<const __nv_bfloat16*>(k);
+  a->v = reinterpret_cast<const __nv_bfloat16*>(v);
+  a->ts_q = a->ts_kv = ts; a->hs_q = a->hs_kv = hs;
+  return XKV_OK;
+}
+
+struct Range { uintptr_t lo, hi; };
+bool overlap(const Range& x, const Range& y) { return x.lo < y.hi && y.lo < x.hi; }
+
+// One frame through `count` layers whose work does not depend on one another (one launch each of the
+// maintenance, the key regroup and the attention for all of them), then, on the library's side stream
+// beside the attention, the head means of the keys of the caches just built (Eq. 4), from which the
+// next frame's scoring starts.
+int run_layers(HostStepPipe* pipe, xkv_cache* const* cs, MaintArgs* as, int count, const void* const* q, const void* const* k,
+               const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st) {
+  const bool once = keys_once(cs[0]);
+  if (launch_maint(cs, as, count, XKV_PROF_MAINT, st) != cudaSuccess) return XKV_E_CUDA;
+  if (cs[0]->p.kv_bits == 4 && !once && launch_regroup(cs, as, count, st) != cudaSuccess) return XKV_E_CUDA;
+  xkv_cache* kc[kMaxLayers];
+  AttnCall calls[kMaxLayers];
+  int n_kbar = 0;
+  for (int i = 0; i < count; ++i) {
+    xkv_cache* c = cs[i];
+    const bool first = c->first_pending != 0;
+    if (once) c->pop_base += (uint32_t)((n + 63) / 64);
+    note_packed(c);
+    calls[i] = {c, q[i], out[i], n, 0, c->tail_mode ? k[i] : nullptr, c->tail_mode ? v[i] : nullptr};
+    if (once ? !first : (c->T > c->T_first)) {
+      // of the frame just quantised (the rest travels with the tokens), or of the whole cache after the
+      // first frame (re-quantisation changed the keys)
+      MaintArgs b = as[i];
+      if (once) {
+        b.phases = kPhKbarNew;
+      } else {
+        maint_args(c, &b);
+        b.phases = kPhKbar;
+        b.kbar_on_other = 0; b.kbar_lo = 0; b.kbar_hi = c->T - c->T_first;
+      }
+      as[n_kbar] = b;
+      kc[n_kbar++] = c;
+    }
+  }
+  // The side stream forks here (after the packing) but its kernel is launched after the attention has
+  // been enqueued, so that the attention's blocks get the multiprocessors first and the head means
+  // fill in as they retire.
+  if (n_kbar && !(cudaEventRecord(pipe->fork, st) == cudaSuccess && cudaStreamWaitEvent(pipe->side, pipe->fork, 0) == cudaSuccess))
     return XKV_E_CUDA;
-  const float scale = 1.0f / sqrtf((float)c->p.head_dim);
-  rc = c->tail_mode ? attn_packed_causal_tail(c, q, k, v, out, n, ts, hs, scale, stream)
-                    : attn_packed_causal(c, q, out, n, ts, hs, scale, 0, stream);
-  if (want_kbar && rc == XKV_OK) {
-    MaintArgs b;
-    if (once) {               // of the frame just quantised (the rest travelled with their tokens)
-      b = a;
-      b.phases = kPhKbarNew;
-    } else {                  // of the whole cache after the first frame: re-quantisation changed the keys
-      maint_args(c, &b);
-      b.phases = kPhKbar;
-      b.kbar_on_other = 0; b.kbar_lo = 0; b.kbar_hi = c->T - c->T_first;
-    }
-    const bool launched = launch_maint(c, b, XKV_PROF_KBAR, pipe->side) == cudaSuccess;
-    const bool ok = cudaEventRecord(c->kbar_done, pipe->side) == cudaSuccess;
-    // (the caller's stream waits for it at the end of the stream-step call, and at the next
-    // frame's scoring)
-    if (!launched || !ok) return XKV_E_CUDA;
-    c->kbar_T = c->T; c->kbar_cur = c->cur; c->kbar_frames = c->frames;
+  const cudaError_t e = launch_attn_tc(calls, count, ts, hs, 1.0f / sqrtf((float)cs[0]->p.head_dim), st);
+  if (e != cudaSuccess) {
+    for (int i = 0; i < count; ++i) cs[i]->stage = 3;
+    return e == cudaErrorNotSupported ? XKV_E_UNSUPPORTED : XKV_E_CUDA;
   }
-  return rc;
+  if (n_kbar) {
+    bool ok = launch_maint(kc, as, n_kbar, XKV_PROF_KBAR, pipe->side) == cudaSuccess;
+    for (int i = 0; i < n_kbar; ++i) {
+      ok = cudaEventRecord(kc[i]->kbar_done, pipe->side) == cudaSuccess && ok;
+      kc[i]->kbar_T = kc[i]->T; kc[i]->kbar_cur = kc[i]->cur; kc[i]->kbar_frames = kc[i]->frames;
+    }
+    pipe->side_busy = true;
+    if (!ok) return XKV_E_CUDA;
+  }
+  return XKV_OK;
 }
 
 // Everything a stream-step call started on the side stream is ordered before what the caller
-// enqueues next: the caller's stream waits for the head-mean kernels of all layers.
-bool join_side_work(xkv_cache* const* layers, int n_layers, cudaStream_t st) {
-  bool ok = true;
-  for (int l = 0; l < n_layers; ++l)
-    if (layers[l] && layers[l]->kbar_frames == layers[l]->frames && layers[l]->kbar_frames > 0)
-      ok = cudaStreamWaitEvent(st, layers[l]->kbar_done, 0) == cudaSuccess && ok;
-  return ok;
+// enqueues next.
+bool join_side_work(HostStepPipe* pipe, cudaStream_t st) {
+  if (!pipe->side_busy) return true;
+  pipe->side_busy = false;
+  return cudaEventRecord(pipe->join, pipe->side) == cudaSuccess && cudaStreamWaitEvent(st, pipe->join, 0) == cudaSuccess;
 }
 
 }  // namespace
@@ -627,13 +649,44 @@ int xkv_stream_step(xkv_cache* const* layers, int32_t n_layers, const void* cons
   if (!layers || !q || !k || !v || !out || n_layers < 1) return XKV_E_INVALID;
   HostStepPipe* pipe = host_step_pipe();
   if (!pipe) return XKV_E_CUDA;
-  for (int l = 0; l < n_layers; ++l) {
-    xkv_cache* c = layers[l];
-    if (!c) return XKV_E_INVALID;
-    const int rc = run_layer(pipe, c, q[l], k[l], v[l], out[l], n, ts, hs, reinterpret_cast<cudaStream_t>(stream));
-    if (rc != XKV_OK) { join_side_work(layers, l + 1, reinterpret_cast<cudaStream_t>(stream)); return rc; }
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  int rc = XKV_OK;
+  for (int l0 = 0; l0 < n_layers && rc == XKV_OK;) {
+    // The next layers that can go together: the same form of cache, no cache twice, and no layer's
+    // output in memory that a later one reads or writes, nor in a query (or, with the unquantised
+    // tail, key or value) of an earlier one, whose attention runs in the same launch.
+    MaintArgs as[kMaxLayers];
+    Range rq[kMaxLayers], rk[kMaxLayers], rv[kMaxLayers], ro[kMaxLayers];
+    int count = 0;
+    while (l0 + count < n_layers && count < kMaxLayers) {
+      const int l = l0 + count;
+      xkv_cache* c = layers[l];
+      if (c && n >= 1 && ts >= 0 && hs >= 0) {
+        const size_t span = ((size_t)(c->p.n_heads - 1) * (size_t)hs + (size_t)(n - 1) * (size_t)ts + kHeadDim) * sizeof(__nv_bfloat16);
+        auto range = [&](const void* p) { const uintptr_t b = reinterpret_cast<uintptr_t>(p); return Range{b, b + span}; };
+        rq[count] = range(q[l]); rk[count] = range(k[l]); rv[count] = range(v[l]); ro[count] = range(out[l]);
+        const xkv_cache* lead = layers[l0];
+        bool together = count == 0 || (c->p.kv_bits == lead->p.kv_bits && c->p.key_mode == lead->p.key_mode &&
+                                       c->p.n_heads == lead->p.n_heads && c->tail_mode == lead->tail_mode &&
+                                       c->attn_max_blocks == lead->attn_max_blocks);
+        for (int i = 0; i < count && together; ++i)
+          together = layers[l0 + i] != c && !overlap(ro[i], rq[count]) && !overlap(ro[i], rk[count]) && !overlap(ro[i], rv[count]) &&
+                     !overlap(ro[i], ro[count]) && !overlap(ro[count], rq[i]) &&
+                     !(c->tail_mode && (overlap(ro[count], rk[i]) || overlap(ro[count], rv[i])));
+        if (!together) break;
+      }
+      rc = prepare_layer(c, q[l], k[l], v[l], out[l], n, ts, hs, &as[count]);
+      if (rc != XKV_OK) break;
+      ++count;
+    }
+    if (count > 0) {
+      const int e = run_layers(pipe, layers + l0, as, count, q + l0, k + l0, v + l0, out + l0, n, ts, hs, st);
+      if (e != XKV_OK) rc = e;
+    }
+    l0 += count;
   }
-  return join_side_work(layers, n_layers, reinterpret_cast<cudaStream_t>(stream)) ? XKV_OK : XKV_E_CUDA;
+  if (!join_side_work(pipe, st) && rc == XKV_OK) rc = XKV_E_CUDA;
+  return rc;
 }
 
 size_t xkv_stream_step_host_bytes(const xkv_params* params, int32_t n) {
@@ -693,7 +746,10 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
     ck(cudaStreamWaitEvent(st, pipe->up2_done[sl], 0));
     if (l >= 2) ck(cudaStreamWaitEvent(st, pipe->down_done[sl], 0));
     if (!cuda_ok) break;
-    rc = run_layer(pipe, c, dq, dk, dv, dout, n, ts, hs, st);
+    MaintArgs a;
+    const void* cq = dq; const void* ck_ = dk; const void* cv = dv;
+    rc = prepare_layer(c, dq, dk, dv, dout, n, ts, hs, &a);
+    if (rc == XKV_OK) rc = run_layers(pipe, &c, &a, 1, &cq, &ck_, &cv, &dout, n, ts, hs, st);
     ck(cudaEventRecord(pipe->comp_done[sl], st));
     if (rc != XKV_OK) break;
     // output
@@ -702,7 +758,7 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
     ck(cudaEventRecord(pipe->down_done[sl], pipe->down));
   }
   // everything started above ends before the call returns, also after an error
-  if (!join_side_work(layers, n_layers, st)) cuda_ok = false;
+  if (!join_side_work(pipe, st)) cuda_ok = false;
   ck(cudaStreamSynchronize(pipe->up));
   ck(cudaStreamSynchronize(pipe->up2));
   ck(cudaStreamSynchronize(st));

@@ -52,7 +52,7 @@ struct MaintArgs {
   float* stats_next;               // the next selecting launch's (cleared by this one)
   int32_t* kept;
   unsigned int* hist;
-  unsigned int* run_hi;            // [cap / 64] sure keeps of every 64-token run
+  unsigned int* run_hi;            // [cap / 64] sure keeps of every run of the selection
   unsigned long long* cand;        // [cap] candidates (key << 32 | ~position)
   unsigned int* cand_count;        // counter of this launch
   unsigned int* cand_count_next;   // counter of the next selecting launch (cleared by this one)
@@ -169,28 +169,40 @@ struct LaunchScope {
 // ---- launchers implemented in the kernel translation units -------------------
 // All return cudaError_t of the launch (cudaGetLastError) and count launches.
 
-// The maintenance kernel with the phases in a.phases (cooperative when it has a grid barrier).
+// Most layers that one launch takes (the attention's job table fits the classic 4 KB of parameters).
+constexpr int kMaxLayers = 28;
+// The maintenance kernel with the phases in a[i].phases on the caches c[i], count <= kMaxLayers, all
+// of the same storage form (cooperative when it has a grid barrier).
 // Fills in the barrier and status fields of `a`; everything else is the caller's.
-cudaError_t launch_maint(xkv_cache* c, MaintArgs& a, int prof_cat, cudaStream_t st);
+cudaError_t launch_maint(xkv_cache* const* c, MaintArgs* a, int count, int prof_cat, cudaStream_t st);
+inline cudaError_t launch_maint(xkv_cache* c, MaintArgs& a, int prof_cat, cudaStream_t st) {
+  return launch_maint(&c, &a, 1, prof_cat, st);
+}
 // Quantise-once mode: fills the ring of free parameter-table slots (after the workspace was zeroed).
 cudaError_t launch_once_init(xkv_cache* c, cudaStream_t st);
 // kv_quant_pack of a 4-bit cache: key regroup + re-quantisation fused with the survivor gather.
-cudaError_t launch_regroup(xkv_cache* c, const MaintArgs& a, cudaStream_t st);
+// Of `count` <= kMaxLayers caches with the same number of heads, in one launch.
+cudaError_t launch_regroup(xkv_cache* const* c, const MaintArgs* a, int count, cudaStream_t st);
 cudaError_t launch_attn_simple(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs,
                                float scale, cudaStream_t st);
-// Returns cudaErrorNotSupported when the tensor-core kernel cannot take the call.
-// prefix > 0: only the first `prefix` tokens of the cache (logical order) are visible to these queries
-// (frame-causal attention inside a chunk of frames); 0: all of them.
-cudaError_t launch_attn_tc(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs,
-                           float scale, cudaStream_t st, int prefix = 0);
-// Same kernel with the newest frame's keys and values taken unquantised from k_t, v_t (the tensors
-// given to kv_append, same strides as q).
-cudaError_t launch_attn_tc_tail(xkv_cache* c, const void* q, const void* k_t, const void* v_t, void* out, int n,
-                                int64_t ts, int64_t hs, float scale, cudaStream_t st);
+// Queries that attend to a cache with the tensor-core kernel.
+struct AttnCall {
+  xkv_cache* cache;
+  const void* q; void* out;
+  int n;                // queries
+  int prefix;           // > 0: only the first `prefix` tokens of the cache (logical order) are visible to these
+                        // queries (frame-causal attention inside a chunk of frames); 0: all of them
+  const void* k_tail;   // not null: the newest frame's keys and values are taken unquantised from these
+  const void* v_tail;   // (the tensors given to kv_append, same strides as q)
+};
+// `count` of them, in as few launches as possible (the frames of a chunk, the layers of a stack).
+// They share the strides and the form: kv_bits, key mode, block cap, tail or none are those of
+// calls[0], whose workspace holds the partial results.  cudaErrorNotSupported when the kernel cannot
+// take the call.
+cudaError_t launch_attn_tc(const AttnCall* calls, int count, int64_t ts, int64_t hs, float scale, cudaStream_t st);
 // Same kernel, split-KV partials in the library's fixed device array; cudaErrorMemoryAllocation
 // when the launch would need more than XKV_STATIC_SCRATCH_BYTES.
-cudaError_t launch_attn_tc_static(xkv_cache* c, const void* q, void* out, int n, int64_t ts, int64_t hs,
-                                  float scale, cudaStream_t st);
+cudaError_t launch_attn_tc_static(const AttnCall& call, int64_t ts, int64_t hs, float scale, cudaStream_t st);
 size_t attn_tc_scratch_bytes(const xkv_params* p);
 // One small block running the attention kernel's bounded wait on a barrier nobody completes.
 cudaError_t launch_timeout_probe(xkv_cache* c, cudaStream_t st);

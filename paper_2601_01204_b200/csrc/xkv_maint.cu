@@ -239,15 +239,19 @@ __device__ __forceinline__ unsigned int block_sum(unsigned int v, unsigned int* 
   return t;
 }
 
-// Grid-wide barrier.  Every block arrives once per barrier; the counter only grows (the host
+// The blocks that work on one layer: every layer of a launch has its own, which run through the phases
+// independently of the other layers' (their barriers included).
+struct Blocks { int index, count; };
+
+// Barrier of a layer's blocks.  Every block arrives once per barrier; the counter only grows (the host
 // passes the value it had when the kernel was launched).  The wait is bounded: when it runs out
 // the block records XKV_E_TIMEOUT and the kernel winds down without touching anything further.
-__device__ __forceinline__ bool grid_barrier(const MaintArgs& a, uint32_t& epoch, Shared& sh) {
+__device__ __forceinline__ bool grid_barrier(const MaintArgs& a, const Blocks& B, uint32_t& epoch, Shared& sh) {
   __syncthreads();
   if (threadIdx.x == 0 && !sh.abort_flag) {
     __threadfence();
     atomicAdd(a.bar, 1u);
-    const uint32_t target = a.bar_base + (epoch + 1u) * gridDim.x;
+    const uint32_t target = a.bar_base + (epoch + 1u) * (uint32_t)B.count;
     uint32_t it = 0;
     while ((int)(ld_acquire_u32(a.bar) - target) < 0) {
       if (++it > kBarSpin) {
@@ -271,14 +275,14 @@ __device__ __forceinline__ bool grid_barrier(const MaintArgs& a, uint32_t& epoch
 // slot (16-bit).
 // ---------------------------------------------------------------------------
 template <int BITS, bool ONCE>
-__device__ __forceinline__ void phase_append(const MaintArgs& a) {
+__device__ __forceinline__ void phase_append(const MaintArgs& a, const Blocks& B) {
   const long long items = (long long)a.H * a.n * 8;
   const int passes = (int)((items + kMT - 1) / kMT);
   const BufSet& d0 = a.oth;
   const BufSet& d1 = a.cur;
   const bool two = a.first != 0;
   // pass p goes to block G - 1 - (p mod G): the blocks that hold no pooled row start first
-  for (int p = (int)gridDim.x - 1 - (int)blockIdx.x; p < passes; p += gridDim.x) {
+  for (int p = B.count - 1 - B.index; p < passes; p += B.count) {
     const long long g = (long long)p * kMT + threadIdx.x;
     const int w = (int)(g & 7);
     const long long th = g >> 3;
@@ -347,10 +351,10 @@ __device__ __forceinline__ void phase_append(const MaintArgs& a) {
 // heads in order and scale by 1/H.  Loads are issued in batches ahead of the
 // (ordered) additions.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void phase_pool(const MaintArgs& a, Shared& sh) {
+__device__ __forceinline__ void phase_pool(const MaintArgs& a, const Blocks& B, Shared& sh) {
   const int c = threadIdx.x & 63;
   const int hslot = threadIdx.x >> 6;      // 0..7
-  for (int i = blockIdx.x; i < a.n_pooled; i += gridDim.x) {
+  for (int i = B.index; i < a.n_pooled; i += B.count) {
     int ta, tb;
     if (i < a.n_special) { ta = i; tb = i + 1; }
     else { ta = a.n_special + (i - a.n_special) * a.pool_g; tb = min(ta + a.pool_g, a.n_q); }
@@ -534,9 +538,9 @@ __device__ __forceinline__ void kbar_run(const MaintArgs& a, Shared& sh, const B
 // KBAR over the rest-local positions [0, hi) of the buffer set `b` (re-quantising mode and 16-bit):
 // one run per 64-slot key group (the rest segment starts on a 128-slot boundary).
 template <int BITS>
-__device__ __forceinline__ void phase_kbar(const MaintArgs& a, Shared& sh, const BufSet& b, int lo, int hi) {
+__device__ __forceinline__ void phase_kbar(const MaintArgs& a, const Blocks& B, Shared& sh, const BufSet& b, int lo, int hi) {
   const int g_lo = lo >> 6, g_hi = (hi + 63) >> 6;
-  for (int gb = g_lo + blockIdx.x; gb < g_hi; gb += gridDim.x) {
+  for (int gb = g_lo + B.index; gb < g_hi; gb += B.count) {
     const int grp = (a.rest_base >> 6) + gb;
     kbar_run<BITS>(a, sh, b, b.kpar + (size_t)grp * 64, (size_t)(a.cap >> 6) * 64, a.rest_base + gb * 64, gb * 64,
                    min(64, hi - gb * 64));
@@ -556,7 +560,7 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
 }
 
 template <int BITS>
-__device__ __forceinline__ void phase_quant_keys_once(const MaintArgs& a, Shared& sh) {
+__device__ __forceinline__ void phase_quant_keys_once(const MaintArgs& a, const Blocks& B, Shared& sh) {
   constexpr float kQmax = (BITS == 8) ? 255.f : 15.f;
   const BufSet& d0 = a.oth;
   const BufSet& d1 = a.cur;
@@ -566,7 +570,7 @@ __device__ __forceinline__ void phase_quant_keys_once(const MaintArgs& a, Shared
   const int hl = tid >> 7, t = tid & 127, w = t & 7, tq = t >> 3, wih = t >> 5;
   const int n_groups = (n + 63) >> 6, n_quads = (H + 3) >> 2;
   const int items = n_groups * n_quads;
-  for (int item = blockIdx.x; item < items; item += gridDim.x) {
+  for (int item = B.index; item < items; item += B.count) {
     const int gamma = item / n_quads, quad = item - gamma * n_quads;
     const int h = quad * 4 + hl;
     const bool head_ok = h < H;
@@ -668,10 +672,10 @@ __device__ __forceinline__ void phase_quant_keys_once(const MaintArgs& a, Shared
 // Quantise-once mode: head means (Eq. 4) of the frame just quantised, into the destination's
 // array: one run per arrival group, whose parameters sit in the group's table slot.
 template <int BITS>
-__device__ __forceinline__ void phase_kbar_new_once(const MaintArgs& a, Shared& sh) {
+__device__ __forceinline__ void phase_kbar_new_once(const MaintArgs& a, const Blocks& B, Shared& sh) {
   const int n_groups = (a.n + 63) >> 6;
   const BufSet& d = a.oth;
-  for (int gamma = blockIdx.x; gamma < n_groups; gamma += gridDim.x) {
+  for (int gamma = B.index; gamma < n_groups; gamma += B.count) {
     const int slot = __ldcg(&d.kslot[a.dst_slot + gamma * 64]);
     kbar_run<BITS>(a, sh, d, a.ktab32 + (size_t)slot * a.H * 64, 64, a.dst_slot + gamma * 64,
                    a.dst_slot - a.rest_base + gamma * 64, min(64, a.n - gamma * 64));
@@ -681,14 +685,14 @@ __device__ __forceinline__ void phase_kbar_new_once(const MaintArgs& a, Shared& 
 // Quantise-once mode, PACK: the survivors' key and value code rows, value parameters, group
 // references, origins and head means move to their new places in the other buffer set.
 template <int BITS>
-__device__ __forceinline__ void phase_gather_once(const MaintArgs& a) {
+__device__ __forceinline__ void phase_gather_once(const MaintArgs& a, const Blocks& B) {
   constexpr int kRow = (BITS == 8) ? 64 : 32;       // bytes of a code row
   constexpr int kRC = kRow / 16;                    // 16-byte chunks of a row
   const BufSet& src = a.cur;
   const BufSet& dst = a.oth;
   const int32_t* kept = a.identity ? nullptr : a.kept;
-  const long long stride = (long long)gridDim.x * kMT;
-  const long long first = (long long)blockIdx.x * kMT + threadIdx.x;
+  const long long stride = (long long)B.count * kMT;
+  const long long first = (long long)B.index * kMT + threadIdx.x;
   if (a.kk == 0) {
     // the budget leaves no room for the middle (k = 0): every token after the first frame leaves,
     // without a selection; their key groups give their table slots back
@@ -764,10 +768,10 @@ __device__ __forceinline__ void phase_gather_once(const MaintArgs& a) {
 // by xor-shuffle), Eq. 5-6.  Thread = (token, 8-channel word); block b takes the
 // 64-token runs b, b + G, ...
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void phase_score(const MaintArgs& a, Shared& sh) {
+__device__ __forceinline__ void phase_score(const MaintArgs& a, const Blocks& B, Shared& sh) {
   const int tid = threadIdx.x;
   const int n_runs = (a.r_old + 63) >> 6;
-  if ((int)blockIdx.x >= n_runs && blockIdx.x != 0) return;
+  if (B.index >= n_runs && B.index != 0) return;
   // the pooled rows come through shared memory, 120 at a time (one round trip), and one thread
   // per channel adds them in order -- unless the caller supplied the row mean
   for (int r0 = 0; a.w_in == nullptr && r0 < a.n_pooled; r0 += kPoolRows) {
@@ -791,42 +795,54 @@ __device__ __forceinline__ void phase_score(const MaintArgs& a, Shared& sh) {
   if (tid < 64) {
     const float wv = a.w_in ? a.w_in[tid] : __fdiv_rn(sh.u.score.w[tid], (float)a.n_pooled);
     sh.u.score.w[tid] = wv;
-    if (blockIdx.x == 0) a.qvec[tid] = wv;
+    if (B.index == 0) a.qvec[tid] = wv;
   }
   __syncthreads();
   const int w = tid & 7, tok = tid >> 3;
   float wq[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) wq[j] = sh.u.score.w[8 * w + j];
-  for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
-    const int i = run * 64 + tok;
-    const bool valid = i < a.r_old;
-    const float4* src = reinterpret_cast<const float4*>(a.cur.kbar + (size_t)(valid ? i : 0) * 64 + 8 * w);
-    const float4 x = __ldcg(src), y = __ldcg(src + 1);
-    const float kb[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
-    float p[8];
+  float s1 = 0.f, s2 = 0.f;       // sum of S and of S^2 (for budget policies)
+  constexpr int kU = 2;           // runs whose loads are in flight together
+  for (int run0 = B.index; run0 < n_runs; run0 += kU * B.count) {
+    float4 x[kU], y[kU];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) p[j] = __fmul_rn(kb[j], wq[j]);
-    float t0 = __fadd_rn(p[0], p[1]), t1 = __fadd_rn(p[2], p[3]);
-    float t2 = __fadd_rn(p[4], p[5]), t3 = __fadd_rn(p[6], p[7]);
-    t0 = __fadd_rn(t0, t1);
-    t2 = __fadd_rn(t2, t3);
-    float s = __fadd_rn(t0, t2);
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
-    if (valid && w == 0) {
-      __stcg(&a.scores[i], s);
-      atomicAdd(&a.hist[(blockIdx.x & (kHistCopies - 1)) * kSelBins + (order_key(s) >> 20)], 1u);
+    for (int u = 0; u < kU; ++u) {
+      const int i = (run0 + u * B.count) * 64 + tok;
+      const float4* src = reinterpret_cast<const float4*>(a.cur.kbar + (size_t)(i < a.r_old ? i : 0) * 64 + 8 * w);
+      x[u] = __ldcg(src);
+      y[u] = __ldcg(src + 1);
     }
-    // statistics of the scores (for budget policies): block sums, then one atomic per block
-    float s1 = (valid && w == 0) ? s : 0.f, s2 = s1 * s1;
 #pragma unroll
-    for (int o = 8; o < 32; o <<= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
-    if ((tid & 31) == 0) { atomicAdd(&sh.fsum[0], s1); atomicAdd(&sh.fsum[1], s2); }
-    __syncthreads();
-    if (tid == 0) { atomicAdd(&a.stats[0], sh.fsum[0]); atomicAdd(&a.stats[1], sh.fsum[1]); sh.fsum[0] = sh.fsum[1] = 0.f; }
-    __syncthreads();
+    for (int u = 0; u < kU; ++u) {
+      const int i = (run0 + u * B.count) * 64 + tok;
+      const bool valid = i < a.r_old;
+      const float kb[8] = {x[u].x, x[u].y, x[u].z, x[u].w, y[u].x, y[u].y, y[u].z, y[u].w};
+      float p[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) p[j] = __fmul_rn(kb[j], wq[j]);
+      float t0 = __fadd_rn(p[0], p[1]), t1 = __fadd_rn(p[2], p[3]);
+      float t2 = __fadd_rn(p[4], p[5]), t3 = __fadd_rn(p[6], p[7]);
+      t0 = __fadd_rn(t0, t1);
+      t2 = __fadd_rn(t2, t3);
+      float s = __fadd_rn(t0, t2);
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+      if (valid && w == 0) {
+        __stcg(&a.scores[i], s);
+        atomicAdd(&a.hist[(B.index & (kHistCopies - 1)) * kSelBins + (order_key(s) >> 20)], 1u);
+        s1 += s;
+        s2 += s * s;
+      }
+    }
   }
+  // statistics of the scores: block sums, then one atomic per block
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1) { s1 += __shfl_xor_sync(0xffffffffu, s1, o); s2 += __shfl_xor_sync(0xffffffffu, s2, o); }
+  if ((tid & 31) == 0) { atomicAdd(&sh.fsum[0], s1); atomicAdd(&sh.fsum[1], s2); }
+  __syncthreads();
+  if (tid == 0) { atomicAdd(&a.stats[0], sh.fsum[0]); atomicAdd(&a.stats[1], sh.fsum[1]); sh.fsum[0] = sh.fsum[1] = 0.f; }
+  __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -838,15 +854,21 @@ __device__ __forceinline__ unsigned long long composite(uint32_t key, int pos) {
   return ((unsigned long long)key << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)pos);
 }
 
-__device__ __forceinline__ void phase_sel1(const MaintArgs& a, Shared& sh) {
+// Tokens of one pass of the selection phases: 64 when the layer has a block for every 64 tokens (then
+// the latency of a pass counts), else one per thread (then the number of passes does).
+__device__ __forceinline__ int sel_width(const MaintArgs& a, const Blocks& B) {
+  return ((a.r_old + 63) >> 6) <= B.count ? 64 : kMT;
+}
+
+__device__ __forceinline__ void phase_sel1(const MaintArgs& a, const Blocks& B, Shared& sh) {
   const int tid = threadIdx.x;
-  const int n_runs = (a.r_old + 63) >> 6;
-  if (blockIdx.x == gridDim.x - 1) {                 // the next selecting launch's counter and sub-histogram:
+  const int width = sel_width(a, B), n_runs = (a.r_old + width - 1) / width;
+  if (B.index == B.count - 1) {                 // the next selecting launch's counter and sub-histogram:
     if (tid == 0) *a.cand_count_next = 0u;           // nobody uses them in this launch
     if (tid < kSubBins) a.hist2_next[tid] = 0u;
     if (tid < 4) a.stats_next[tid] = 0.f;
   }
-  if ((int)blockIdx.x >= n_runs) return;
+  if (B.index >= n_runs) return;
   // thread t owns the bins 4095 - 8t - 7 .. 4095 - 8t; walked from the top
   unsigned int hb[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
   {
@@ -878,10 +900,10 @@ __device__ __forceinline__ void phase_sel1(const MaintArgs& a, Shared& sh) {
   }
   __syncthreads();
   const uint32_t bin = sh.bin;
-  for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
-    const int i = run * 64 + tid;
+  for (int run = B.index; run < n_runs; run += B.count) {
+    const int i = run * width + tid;
     bool hi = false;
-    if (tid < 64 && i < a.r_old) {
+    if (tid < width && i < a.r_old) {
       const uint32_t key = order_key(__ldcg(&a.scores[i]));
       hi = (key >> 20) > bin;
       if ((key >> 20) == bin) {
@@ -896,13 +918,13 @@ __device__ __forceinline__ void phase_sel1(const MaintArgs& a, Shared& sh) {
 }
 
 template <bool ONCE>
-__device__ __forceinline__ void phase_sel2(const MaintArgs& a, Shared& sh) {
+__device__ __forceinline__ void phase_sel2(const MaintArgs& a, const Blocks& B, Shared& sh) {
   const int tid = threadIdx.x;
-  const int n_runs = (a.r_old + 63) >> 6;
-  if (blockIdx.x == gridDim.x - 1) {                 // every block has read the histogram: ready for the next step
+  const int width = sel_width(a, B), n_runs = (a.r_old + width - 1) / width;
+  if (B.index == B.count - 1) {                 // every block has read the histogram: ready for the next step
     for (int e = tid; e < kSelBins * kHistCopies; e += kMT) a.hist[e] = 0u;
   }
-  if ((int)blockIdx.x >= n_runs) return;
+  if (B.index >= n_runs) return;
   const uint32_t bin = sh.bin;
   const unsigned int need = sh.need;
   const unsigned int ncand = __ldcg(a.cand_count);
@@ -959,34 +981,34 @@ __device__ __forceinline__ void phase_sel2(const MaintArgs& a, Shared& sh) {
     }
   }
   const unsigned long long tau = prefix;             // kept candidates: composite >= tau (exactly `need` of them)
-  if (blockIdx.x == 0 && tid == 0) {                 // the k-th largest score itself, for the statistics
+  if (B.index == 0 && tid == 0) {                 // the k-th largest score itself, for the statistics
     const uint32_t key = (uint32_t)(tau >> 32);
     a.stats[2] = __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
   }
-  for (int run = blockIdx.x; run < n_runs; run += gridDim.x) {
+  for (int run = B.index; run < n_runs; run += B.count) {
     // survivors before this run: the sure keeps of the runs before it plus the kept candidates at
     // lower positions
     unsigned int part = 0u;
     for (int r = tid; r < run; r += kMT) part += __ldcg(&a.run_hi[r]);
-    const uint32_t below = 0xFFFFFFFFu - (uint32_t)(run * 64);         // position part of position run * 64
+    const uint32_t below = 0xFFFFFFFFu - (uint32_t)(run * width);      // position part of the run's first position
     for (unsigned int e = tid; e < ncand; e += kMT) {
       const unsigned long long cv = cand_at(e);
       part += (cv >= tau) && ((uint32_t)cv > below);                   // larger low word = lower position
     }
     const unsigned int base = block_sum(part, &sh.acc);
-    const int i = run * 64 + tid;
+    const int i = run * width + tid;
     bool keep = false;
-    if (tid < 64 && i < a.r_old) {
+    if (tid < width && i < a.r_old) {
       const uint32_t key = order_key(__ldcg(&a.scores[i]));
       keep = (key >> 20) > bin || ((key >> 20) == bin && composite(key, i) >= tau);
     }
-    if (tid < 64) {
-      const unsigned int m = __ballot_sync(0xffffffffu, keep);
-      if (tid == 31) sh.warp[0] = __popc(m);
-      const unsigned int rank = __popc(m & ((1u << (tid & 31)) - 1u));
-      asm volatile("bar.sync 2, 64;" ::: "memory");
-      const unsigned int off = (tid >= 32) ? sh.warp[0] : 0u;
-      if (keep) __stcg(&a.kept[base + off + rank], i);
+    const unsigned int m = __ballot_sync(0xffffffffu, keep);
+    if ((tid & 31) == 0) sh.warp[tid >> 5] = __popc(m);
+    __syncthreads();
+    if (tid < width) {
+      unsigned int off = base + __popc(m & ((1u << (tid & 31)) - 1u));
+      for (int wp = 0; wp < (tid >> 5); ++wp) off += sh.warp[wp];
+      if (keep) __stcg(&a.kept[off], i);
       if (ONCE && i < a.r_old && !keep) {
         // the token leaves: its key group loses a member and gives its table slot back when empty
         const int slot = __ldcg(&a.cur.kslot[a.rest_base + i]);
@@ -1011,10 +1033,27 @@ __device__ __forceinline__ void phase_sel2(const MaintArgs& a, Shared& sh) {
 // ---------------------------------------------------------------------------
 constexpr int kRgHeads = 4;
 
-__global__ void __launch_bounds__(128 * kRgHeads, 2)
-regroup_k_kernel(BufSet src, BufSet dst, BufSet dst2, bool two, int H, int cap, int max_n, int base_slot, int kk,
-                 int r_new, const int32_t* __restrict__ kept, const __nv_bfloat16* __restrict__ kstage,
-                 int force_plain) {
+struct RegroupArgs {
+  BufSet src, dst;                // (the first frame goes to both buffer sets)
+  bool two;
+  int force_plain;
+  int cap, max_n, base_slot, kk, r_new;
+  const int32_t* kept;
+  const __nv_bfloat16* kstage;
+};
+template <int MAX> struct RegroupBatch { RegroupArgs layer[MAX]; };
+
+template <int MAX>
+__global__ void __launch_bounds__(128 * kRgHeads, 2) regroup_k_kernel(const __grid_constant__ RegroupBatch<MAX> batch, const int H) {
+  const RegroupArgs& a = batch.layer[MAX == 1 ? 0 : blockIdx.z];
+  if ((int)blockIdx.x * 64 >= a.r_new) return;
+  const BufSet& src = a.src;
+  const BufSet& dst = a.dst;
+  const BufSet& dst2 = a.src;
+  const bool two = a.two;
+  const int cap = a.cap, max_n = a.max_n, base_slot = a.base_slot, kk = a.kk, r_new = a.r_new, force_plain = a.force_plain;
+  const int32_t* __restrict__ kept = a.kept;
+  const __nv_bfloat16* __restrict__ kstage = a.kstage;
   __shared__ int s_old[64];                      // source position (rest-local) of each token, -1 = new key
   __shared__ float s_mn[kRgHeads][4][64];
   __shared__ float s_mx[kRgHeads][4][64];
@@ -1159,17 +1198,17 @@ regroup_k_kernel(BufSet src, BufSet dst, BufSet dst2, bool two, int H, int cap, 
   // one thread per channel finishes the reduction and derives the group's parameters
   int slow = force_plain;
   if (t < 64) {
-    float a = s_mn[hl][0][t], b = s_mx[hl][0][t];
+    float lo = s_mn[hl][0][t], up = s_mx[hl][0][t];
 #pragma unroll
-    for (int r = 1; r < 4; ++r) { a = fminf(a, s_mn[hl][r][t]); b = fmaxf(b, s_mx[hl][r][t]); }
+    for (int r = 1; r < 4; ++r) { lo = fminf(lo, s_mn[hl][r][t]); up = fmaxf(up, s_mx[hl][r][t]); }
     float sc, inv, z;
-    quant_params(a, b, sc, inv, z);
+    quant_params(lo, up, sc, inv, z);
     s_iz[hl][t] = make_float2(inv, z);
     if (head_ok) {
       dst.kpar[dgrp + t] = make_float2(sc, z);
       if (two) dst2.kpar[dgrp + t] = make_float2(sc, z);
       // the conversion-free quantiser needs |x * inv| < 2^21 and |z| < 2^22
-      const float ymax = __fmul_rn(fmaxf(fabsf(a), fabsf(b)), inv);
+      const float ymax = __fmul_rn(fmaxf(fabsf(lo), fabsf(up)), inv);
       slow |= !(ymax < 2097152.f) || !(fabsf(z) < kZLimit);
     }
   }
@@ -1223,12 +1262,12 @@ regroup_k_kernel(BufSet src, BufSet dst, BufSet dst2, bool two, int H, int cap, 
 // buffer set to the other, preserving order.  Thread-item = (head, survivor,
 // 16-byte chunk).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void phase_gather16(const MaintArgs& a) {
+__device__ __forceinline__ void phase_gather16(const MaintArgs& a, const Blocks& B) {
   const BufSet& src = a.cur;
   const BufSet& dst = a.oth;
   const int32_t* kept = a.identity ? nullptr : a.kept;
   const long long items = (long long)a.H * a.kk * 8;
-  for (long long g = (long long)blockIdx.x * kMT + threadIdx.x; g < items; g += (long long)gridDim.x * kMT) {
+  for (long long g = (long long)B.index * kMT + threadIdx.x; g < items; g += (long long)B.count * kMT) {
     const int ch = (int)(g & 7);
     const long long r = g >> 3;
     const int i = (int)(r % a.kk);
@@ -1247,40 +1286,49 @@ __device__ __forceinline__ void phase_gather16(const MaintArgs& a) {
 // ---------------------------------------------------------------------------
 // The kernel.
 // ---------------------------------------------------------------------------
-template <int BITS, bool ONCE>
-__global__ void __launch_bounds__(kMT, kBlocksPerSM) maint_kernel(const __grid_constant__ MaintArgs a) {
+// A launch takes up to MAX layers: block b works on layer b mod n.  (A layer alone leaves the chip
+// waiting: at 1374 tokens and 16384 cached ones its phases are chains of round trips that move
+// 16 MB in 30 us.)  The form for one layer keeps its parameters directly addressable.
+template <int MAX> struct MaintBatch { int n; MaintArgs layer[MAX]; };
+
+template <int BITS, bool ONCE, int MAX>
+__global__ void __launch_bounds__(kMT, kBlocksPerSM) maint_kernel(const __grid_constant__ MaintBatch<MAX> batch) {
   __shared__ Shared sh;
   if (threadIdx.x == 0) { sh.abort_flag = 0; sh.acc = 0u; sh.bin = 0u; sh.need = 0u; sh.fsum[0] = sh.fsum[1] = 0.f; }
   __syncthreads();
+  const int which = (MAX == 1) ? 0 : (int)blockIdx.x % batch.n;
+  const Blocks B{(MAX == 1) ? (int)blockIdx.x : (int)blockIdx.x / batch.n,
+                 (MAX == 1) ? (int)gridDim.x : ((int)gridDim.x - which + batch.n - 1) / batch.n};
+  const MaintArgs& a = batch.layer[which];
   uint32_t epoch = 0;
   const uint32_t ph = a.phases;
   bool ran = false;                 // something has run since the last barrier
 
   if (ph & kPhAppend) {
-    phase_append<BITS, ONCE>(a);
-    if (ONCE) phase_quant_keys_once<BITS>(a, sh);
+    phase_append<BITS, ONCE>(a, B);
+    if (ONCE) phase_quant_keys_once<BITS>(a, B, sh);
     ran = true;
   }
-  if (ph & kPhPool) { phase_pool(a, sh); ran = true; }
-  if (ph & kPhKbar) { phase_kbar<BITS>(a, sh, a.kbar_on_other ? a.oth : a.cur, a.kbar_lo, a.kbar_hi); ran = true; }
+  if (ph & kPhPool) { phase_pool(a, B, sh); ran = true; }
+  if (ph & kPhKbar) { phase_kbar<BITS>(a, B, sh, a.kbar_on_other ? a.oth : a.cur, a.kbar_lo, a.kbar_hi); ran = true; }
 
   if (ph & (kPhScore | kPhKbarNew)) {
-    if (ran && !grid_barrier(a, epoch, sh)) return;
-    if (ONCE && (ph & kPhKbarNew)) phase_kbar_new_once<BITS>(a, sh);
-    if (ph & kPhScore) phase_score(a, sh);
+    if (ran && !grid_barrier(a, B, epoch, sh)) return;
+    if (ONCE && (ph & kPhKbarNew)) phase_kbar_new_once<BITS>(a, B, sh);
+    if (ph & kPhScore) phase_score(a, B, sh);
     ran = true;
   }
   if (ph & kPhSel) {
-    if (ran && !grid_barrier(a, epoch, sh)) return;
-    phase_sel1(a, sh);
-    if (!grid_barrier(a, epoch, sh)) return;
-    phase_sel2<ONCE>(a, sh);
+    if (ran && !grid_barrier(a, B, epoch, sh)) return;
+    phase_sel1(a, B, sh);
+    if (!grid_barrier(a, B, epoch, sh)) return;
+    phase_sel2<ONCE>(a, B, sh);
     ran = true;
   }
   if (ph & kPhPack) {
-    if (ran && !grid_barrier(a, epoch, sh)) return;
-    if (ONCE) phase_gather_once<BITS>(a);
-    else if (BITS == 16 && a.kk > 0) phase_gather16(a);
+    if (ran && !grid_barrier(a, B, epoch, sh)) return;
+    if (ONCE) phase_gather_once<BITS>(a, B);
+    else if (BITS == 16 && a.kk > 0) phase_gather16(a, B);
   }
 }
 
@@ -1311,6 +1359,13 @@ static int maint_barriers(uint32_t ph) {
 static std::mutex g_maint_mutex;
 static int g_maint_grid[64] = {0};
 
+template <int MAX> static const void* maint_fn(int bits, bool once) {
+  return (bits == 16) ? (const void*)maint_kernel<16, false, MAX>
+         : (bits == 8) ? (const void*)maint_kernel<8, true, MAX>
+         : once        ? (const void*)maint_kernel<4, true, MAX>
+                       : (const void*)maint_kernel<4, false, MAX>;
+}
+
 static cudaError_t maint_grid(int* grid) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
@@ -1321,8 +1376,9 @@ static cudaError_t maint_grid(int* grid) {
     int sms = 0, per_sm = kBlocksPerSM;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const void* fns[4] = {(const void*)maint_kernel<4, false>, (const void*)maint_kernel<16, false>,
-                          (const void*)maint_kernel<4, true>, (const void*)maint_kernel<8, true>};
+    const void* fns[8] = {maint_fn<1>(4, false), maint_fn<1>(16, false), maint_fn<1>(4, true), maint_fn<1>(8, true),
+                          maint_fn<kMaxLayers>(4, false), maint_fn<kMaxLayers>(16, false),
+                          maint_fn<kMaxLayers>(4, true), maint_fn<kMaxLayers>(8, true)};
     for (const void* fn : fns) {
       int nb = 0;
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, kMT, 0);
@@ -1336,46 +1392,63 @@ static cudaError_t maint_grid(int* grid) {
   return cudaSuccess;
 }
 
-cudaError_t launch_regroup(xkv_cache* c, const MaintArgs& a, cudaStream_t st) {
-  const dim3 grid((a.r_new + 63) / 64, (a.H + kRgHeads - 1) / kRgHeads);
-  LaunchScope ls(c, XKV_PROF_PACK, st);
-  regroup_k_kernel<<<grid, 128 * kRgHeads, 0, st>>>(a.cur, a.oth, a.cur, a.first != 0, a.H, a.cap, a.max_n,
-                                                   a.first ? 0 : a.rest_base, a.kk, a.r_new,
-                                                   a.identity ? nullptr : a.kept, a.kstage, a.force_plain);
+template <int MAX>
+static cudaError_t launch_regroup_n(xkv_cache* const* c, const MaintArgs* a, int count, cudaStream_t st) {
+  RegroupBatch<MAX> b;
+  int groups = 0;
+  for (int i = 0; i < count; ++i) {
+    b.layer[i] = {a[i].cur, a[i].oth, a[i].first != 0, a[i].force_plain, a[i].cap, a[i].max_n, a[i].first ? 0 : a[i].rest_base,
+                  a[i].kk, a[i].r_new, a[i].identity ? nullptr : a[i].kept, a[i].kstage};
+    const int g = (a[i].r_new + 63) / 64;
+    if (g > groups) groups = g;
+  }
+  const dim3 grid(groups, (a[0].H + kRgHeads - 1) / kRgHeads, count);
+  LaunchScope ls(c[0], XKV_PROF_PACK, st);
+  regroup_k_kernel<MAX><<<grid, 128 * kRgHeads, 0, st>>>(b, a[0].H);
   return cudaGetLastError();
 }
 
-cudaError_t launch_maint(xkv_cache* c, MaintArgs& a, int prof_cat, cudaStream_t st) {
+cudaError_t launch_regroup(xkv_cache* const* c, const MaintArgs* a, int count, cudaStream_t st) {
+  return count == 1 ? launch_regroup_n<1>(c, a, 1, st) : launch_regroup_n<kMaxLayers>(c, a, count, st);
+}
+
+template <int MAX>
+static cudaError_t launch_maint_n(xkv_cache* const* c, MaintArgs* as, int count, cudaStream_t st) {
   int grid = 0;
   cudaError_t e = maint_grid(&grid);
   if (e != cudaSuccess) return e;
-  const int nb = maint_barriers(a.phases);
-  a.bar = c->counters;
-  a.bar_base = c->bar_base;
-  a.status = c->status;
-  a.cand_count = c->counters + 2 + c->sel_parity;
-  a.cand_count_next = c->counters + 2 + (c->sel_parity ^ 1);
-  a.hist2 = c->counters + 64 + 256 * c->sel_parity;
-  a.hist2_next = c->counters + 64 + 256 * (c->sel_parity ^ 1);
-  a.stats = reinterpret_cast<float*>(c->counters + 16 + 4 * c->sel_parity);
-  a.stats_next = reinterpret_cast<float*>(c->counters + 16 + 4 * (c->sel_parity ^ 1));
-  if (a.phases & kPhSel) c->stats_parity = c->sel_parity;
-  if (a.phases & kPhSel) c->sel_parity ^= 1;
-  LaunchScope ls(c, prof_cat, st);
-  void* params[1] = {(void*)&a};
-  a.push_pos = c->counters + 8;
-  const void* fn = (c->p.kv_bits == 16) ? (const void*)maint_kernel<16, false>
-                   : (c->p.kv_bits == 8) ? (const void*)maint_kernel<8, true>
-                   : c->p.key_mode == XKV_KEYS_ONCE ? (const void*)maint_kernel<4, true>
-                                                    : (const void*)maint_kernel<4, false>;
-  if (nb > 0) {
-    e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kMT), params, 0, st);
-    c->bar_base += (uint32_t)nb * (uint32_t)grid;
-  } else {
-    e = cudaLaunchKernel(fn, dim3(grid), dim3(kMT), params, 0, st);
+  MaintBatch<MAX> batch;
+  batch.n = count;
+  bool barriers = false;
+  for (int i = 0; i < count; ++i) {
+    MaintArgs& a = as[i];
+    xkv_cache* ci = c[i];
+    const int nb = maint_barriers(a.phases);
+    a.bar = ci->counters;
+    a.bar_base = ci->bar_base;
+    a.status = ci->status;
+    a.cand_count = ci->counters + 2 + ci->sel_parity;
+    a.cand_count_next = ci->counters + 2 + (ci->sel_parity ^ 1);
+    a.hist2 = ci->counters + 64 + 256 * ci->sel_parity;
+    a.hist2_next = ci->counters + 64 + 256 * (ci->sel_parity ^ 1);
+    a.stats = reinterpret_cast<float*>(ci->counters + 16 + 4 * ci->sel_parity);
+    a.stats_next = reinterpret_cast<float*>(ci->counters + 16 + 4 * (ci->sel_parity ^ 1));
+    a.push_pos = ci->counters + 8;
+    if (a.phases & kPhSel) { ci->stats_parity = ci->sel_parity; ci->sel_parity ^= 1; }
+    if (nb > 0) barriers = true;
+    ci->bar_base += (uint32_t)nb * (uint32_t)((grid - i + count - 1) / count);      // blocks of this layer
+    batch.layer[i] = a;
   }
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  void* params[1] = {(void*)&batch};
+  const void* fn = maint_fn<MAX>(c[0]->p.kv_bits, c[0]->p.key_mode == XKV_KEYS_ONCE);
+  e = barriers ? cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kMT), params, 0, st)
+               : cudaLaunchKernel(fn, dim3(grid), dim3(kMT), params, 0, st);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_maint(xkv_cache* const* c, MaintArgs* a, int count, int prof_cat, cudaStream_t st) {
+  LaunchScope ls(c[0], prof_cat, st);
+  return count == 1 ? launch_maint_n<1>(c, a, 1, st) : launch_maint_n<kMaxLayers>(c, a, count, st);
 }
 
 }  // namespace xkv

@@ -1,0 +1,123 @@
+"""Layers of one stream step (and frames of one chunk) that share their launches: the cache state of
+every layer is that of the per-call entry points bit for bit, its output within the attention's
+tolerance of theirs (the items are cut at other places, so partial results are merged elsewhere)."""
+import numpy as np
+import pytest
+
+from paper_2601_01204_b200 import synth
+from xkv_testlib import bf16_tensor_to_f32, check_attention, compare_state, oracle_params, to_device_bf16
+
+pytestmark = pytest.mark.gpu
+
+H, D = 3, 64
+
+
+@pytest.fixture(scope="module")
+def xkv():
+    import torch
+    assert torch.cuda.is_available()
+    import paper_2601_01204_b200.xkv as m
+    return m
+
+
+def frame(layer, t, n):
+    return [to_device_bf16(b) for b in synth.gen_frame(70 + layer, layer, t, H, n, D)]
+
+
+def per_call(cache, q, k, v, tail):
+    cache.kv_append(k, v)
+    cache.kv_score_evict(q)
+    cache.kv_quant_pack()
+    return cache.attn_packed_causal_tail(q, k, v) if tail else cache.attn_packed_causal(q)
+
+
+@pytest.mark.parametrize("layers, n, budget, bits, once, tail", [
+    (2, 130, 300, 4, 0, False),
+    (29, 97, 260, 4, 0, False),          # one more than a launch takes
+    (5, 257, 1200, 4, 0, True),
+    (5, 140, 700, 4, 1, False),
+    (3, 97, 300, 8, 1, False),
+    (24, 257, 1030, 16, 0, False),
+    (3, 1, 4, 4, 0, False),
+])
+def test_layers_of_one_step_match_the_calls(xkv, layers, n, budget, bits, once, tail):
+    import torch
+    p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=bits, key_mode=once)
+    together, alone = ([xkv.Cache(p) for _ in range(layers)] for _ in range(2))
+    for c in together:
+        c.xkv_set_unquantised_tail(tail)
+    for t in range(7):
+        q, k, v = zip(*(frame(l, t, n) for l in range(layers)))
+        out = [torch.empty_like(x) for x in q]
+        xkv.xkv_stream_step(together, q, k, v, out)
+        for l in range(layers):
+            ref = per_call(alone[l], q[l], k[l], v[l], tail)
+            if l in (0, 1, layers - 1):
+                check_attention(bf16_tensor_to_f32(out[l]), bf16_tensor_to_f32(ref), f"frame {t} layer {l}")
+                compare_state(together[l].export(), alone[l].export(), f"frame {t} layer {l}")
+    assert all(c.xkv_poll_status() == 0 for c in together)
+
+
+def test_step_with_layers_of_different_forms_and_lengths(xkv):
+    """Neighbours that cannot share a launch, and layers whose caches have different lengths."""
+    import torch
+    forms = [(300, 4, 0), (500, 4, 0), (500, 16, 0), (400, 16, 0), (300, 4, 1), (300, 8, 1), (260, 4, 0)]
+    mk = lambda: [xkv.Cache(xkv.Params(n_heads=H, budget=b, max_frame_tokens=130, kv_bits=bits, key_mode=o)) for b, bits, o in forms]
+    together, alone = mk(), mk()
+    for t, n in enumerate([130, 64, 129, 130, 1, 130]):
+        q, k, v = zip(*(frame(l, t, n) for l in range(len(forms))))
+        out = [torch.empty_like(x) for x in q]
+        xkv.xkv_stream_step(together, q, k, v, out)
+        for l, c in enumerate(alone):
+            ref = per_call(c, q[l], k[l], v[l], False)
+            check_attention(bf16_tensor_to_f32(out[l]), bf16_tensor_to_f32(ref), f"frame {t} layer {l}")
+            compare_state(together[l].export(), c.export(), f"frame {t} layer {l}")
+
+
+def test_step_keeps_the_order_of_layers_that_share_memory(xkv):
+    """A layer's output that is a later layer's input, one output buffer for all layers, and the same
+    cache twice: the results are those of the layers one after the other."""
+    import torch
+    n = 130
+    p = xkv.Params(n_heads=H, budget=300, max_frame_tokens=n, kv_bits=4)
+    a, b = [xkv.Cache(p) for _ in range(2)], [xkv.Cache(p) for _ in range(2)]
+    for t in range(5):
+        (q0, k0, v0), (_, k1, v1), (q2, k2, v2) = (frame(l, t, n) for l in range(3))
+        mid, last = torch.empty_like(q0), torch.empty_like(q0)
+        xkv.xkv_stream_step([a[0], a[1], a[1]], [q0, mid, q2], [k0, k1, k2], [v0, v1, v2], [mid, last, last])
+        m = per_call(b[0], q0, k0, v0, False)
+        per_call(b[1], m, k1, v1, False)
+        ref = per_call(b[1], q2, k2, v2, False)
+        assert torch.equal(mid, m) and torch.equal(last, ref)
+        for x, y in zip(a, b):
+            compare_state(x.export(), y.export(), f"frame {t}")
+
+
+def test_step_stops_at_the_first_bad_layer(xkv):
+    import torch
+    n = 64
+    p = xkv.Params(n_heads=H, budget=300, max_frame_tokens=n, kv_bits=4)
+    caches = [xkv.Cache(p) for _ in range(3)]
+    q, k, v = zip(*(frame(l, 0, n) for l in range(3)))
+    out = [torch.zeros_like(x) for x in q]
+    caches[1].kv_append(k[1], v[1])                       # out of order for a step
+    with pytest.raises(xkv.XkvError) as e:
+        xkv.xkv_stream_step(caches, q, k, v, out)
+    assert e.value.status == xkv.XKV_E_STATE
+    assert [c.xkv_get_info().frames for c in caches] == [1, 0, 0]
+    assert out[0].abs().max() > 0 and out[2].abs().max() == 0
+
+
+def test_chunk_of_more_frames_than_a_launch_takes(xkv):
+    from oracle import xkv_oracle as xo
+    sizes = [9] * 27 + [1, 30, 7]
+    n = sum(sizes)
+    p = xkv.Params(n_heads=H, budget=700, max_frame_tokens=n, kv_bits=4)
+    cache, ora = xkv.Cache(p), xo.OracleLayer(oracle_params(p))
+    for t in range(4):
+        bits = synth.gen_frame(5, 0, t, H, n, D)
+        got = cache.xkv_prefill_chunk(*(to_device_bf16(b) for b in bits), sizes)
+        cuts = np.cumsum(sizes)[:-1]
+        ref = ora.step_chunk(*(np.split(synth.bf16_bits_to_f32(b), cuts, axis=1) for b in bits))
+        check_attention(bf16_tensor_to_f32(got).transpose(1, 0, 2), np.concatenate(ref), f"chunk {t}")
+        compare_state(cache.export(), ora.export(), f"chunk {t}")
