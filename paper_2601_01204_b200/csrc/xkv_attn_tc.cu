@@ -18,8 +18,9 @@
 //               lane quarter, each takes 64 of the 128 key columns; a thread loads its half row
 //               of scores into registers at once and releases the score columns, the maximum
 //               is taken from the registers.  Registers move to these warps with setmaxnreg.
-//               Tensor memory: ONE score buffer of 128 columns that the two tiles use in turn,
-//               P 2 x 2 x 64 (two buffers per tile), O 2 x 64.
+//               Tensor memory (see the columns below): 16-bit caches ONE score buffer of 128 columns
+//               that the two tiles use in turn, P 2 x 2 x 64 (two buffers per tile), O 2 x 64; 4-bit
+//               caches scores of their own for each tile, P over them, O 2 x 64.
 //   4 warps     operand producers: packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
 //               and key group) and V~ (per token) in the 128-byte-swizzled layouts the MMA
 //               descriptors expect.  One dequantised tile serves both query tiles.
@@ -52,8 +53,8 @@ constexpr int kMaxDevices = 64;
 constexpr int kThreads = 480;
 // 16-warp form: registers per thread after the reallocation (softmax warps kSplitRegsSoftmax)
 constexpr int kSplitRegsSoftmax = 96;
-__host__ __device__ constexpr int split_regs_producers(bool once, bool tail) { return (once || tail) ? 56 : 40; }
-__host__ __device__ constexpr int split_regs_misc(bool once, bool tail) { return (once || tail) ? 40 : 48; }   // MMA issuers, copy thread
+__host__ __device__ constexpr int split_regs_producers(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 56 : 48; }
+__host__ __device__ constexpr int split_regs_misc(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 40 : 48; }   // MMA issuers, copy thread
 constexpr int kThreadsSplit = 768;      // 16 softmax warps, 4 producers, 4 for the MMA issuers and the copies
 constexpr int kQRows = 128;
 constexpr int kMaxGrid = 160;                 // CTAs the scratch is sized for (>= SM count of the part)
@@ -94,7 +95,7 @@ constexpr int kTabBytes = 768 + 2048;
 constexpr int kOffBar = kOffTab + 2 * kTabBytes;  // barriers, tmem base, abort flag
 constexpr int kBarBytes = 512;
 constexpr int kOffRaw = kOffBar + kBarBytes;      // raw stages (16-byte aligned)
-constexpr int kXchgBytes = 4096;                  // split softmax: values exchanged between the two halves of a row
+constexpr int kXchgBytes = 6144;                  // split softmax: values exchanged between the two halves of a row
 template <int BITS, bool SPLIT = false> constexpr int smem_bytes() {
   return kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + (SPLIT ? kXchgBytes : 0) + 1024;
 }
@@ -103,9 +104,16 @@ template <int BITS, bool SPLIT = false> constexpr int smem_bytes() {
 constexpr int kColS = 0;      // + 128 t : 128 fp32 columns per query tile
 constexpr int kColP = 256;    // + 64 t  : 64 columns of packed 16-bit pairs
 constexpr int kColO = 384;    // + 64 t  : 64 fp32 columns
-// 16-warp form: one score buffer for both tiles, two P buffers per tile
+// 16-warp form, one score buffer for both tiles, two P buffers per tile:
 constexpr int kColS1 = 0;     // 128 fp32 columns
 constexpr int kColP2 = 128;   // + 128 t + 64 b
+// 16-warp form, scores of their own for each tile (4-bit caches): a query tile has three blocks of 64
+// columns, B0 B1 B2.  In even steps its scores take B0 B1 and P goes over B0 once the scores are in
+// registers; in odd steps the scores take B1 B2 and P goes over B2.  So the scores of a step are
+// computed during the softmax of the step before, whose P they do not touch, and P never waits for
+// the P V~ before.  24 layers at 16384 tokens: 3226 -> 3138 us.  16-bit caches, with twice the bytes a
+// tile, measured the other way (32768 tokens: 6500 -> 7000 us) and keep the shared buffer.
+constexpr int kColTile = 192;      // * t
 constexpr int kTmemCols = 512;
 
 // one partial slot: two query tiles x 128 rows x (64 accumulators + max + sum)
@@ -234,7 +242,15 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 // Bounded wait.  On exhaustion a per-CTA flag goes up, and every later wait of the CTA gives up at
 // once; at its end the CTA records the failure in the status words of the launch's caches.
-struct WaitCtx { volatile int* abort_flag; };
+struct WaitCtx { uint32_t abort_flag; };      // address in shared memory
+__device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.volatile.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 // Threads on the critical chain (softmax warps, MMA issuers: SLEEP_NS below 128) retry at once, each
 // try suspended by the hardware for a short while: their wake-up latency is part of every step.
 // Threads that wait long and have slack (operand producers, the copy thread) sleep SLEEP_NS between
@@ -247,7 +263,7 @@ constexpr uint32_t kWaitMinRounds = 1u << 12;         // ... and this many round
 template <int SLEEP_NS = 32>
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& wc) {
   if (mbar_try(bar, parity)) return;          // the common case costs one instruction
-  if (*wc.abort_flag) return;
+  if (ld_shared_u32(wc.abort_flag)) return;
   const uint64_t t0 = global_ns();
   uint32_t rounds = 0;
   do {
@@ -261,7 +277,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const W
       return;
     }
   } while (++rounds < kWaitMinRounds || global_ns() - t0 < kWaitLimitNs);
-  *wc.abort_flag = 1;
+  st_shared_u32(wc.abort_flag, 1u);
 }
 // A wait of the CTA ran out: the results of every cache in the launch are void.
 __device__ __forceinline__ void report_timeout(const Args& a) {
@@ -540,9 +556,11 @@ template <int BITS, bool TAIL = false, bool ONCE = false, bool SPLIT = false>
 __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_kernel(const __grid_constant__ Args a) {
   using C = Cfg<BITS>;
   constexpr int kSW = SPLIT ? 16 : 8;        // softmax warps
+  constexpr bool kOwnS = SPLIT && BITS == 4; // scores of their own for each tile
   constexpr uint32_t kRowThreads = SPLIT ? 256 : 128;   // threads that work on one query tile
   constexpr int kOffX = kOffRaw + C::kNR * C::kRawStage;   // exchange area of the split softmax
-  constexpr int kRegProd = split_regs_producers(ONCE, TAIL), kRegMisc = split_regs_misc(ONCE, TAIL);
+  static_assert(kOffX % 1024 == 0, "the halves' places differ in one address bit");
+  constexpr int kRegProd = split_regs_producers(BITS, ONCE, TAIL), kRegMisc = split_regs_misc(BITS, ONCE, TAIL);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
@@ -554,10 +572,13 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   const uint32_t b_rfull = b_vfree + 8 * kNV, b_rfree = b_rfull + 8 * C::kNR;
   const uint32_t b_qfull = b_rfree + 8 * C::kNR;      // [2]
   const uint32_t b_sfull = b_qfull + 16, b_pfull = b_sfull + 16, b_pvdone = b_pfull + 16, b_sfree = b_pvdone + 16;
-  const uint32_t b_pvdone2 = b_sfree + 16;             // [2 tiles][2 P buffers], 16-warp form
+  // 16-warp form, [2 tiles][2], even and odd steps: P V~ done, P written.  The warps of a tile may be
+  // almost a step apart (the next scores are there early), so arrivals of a step and of the next one
+  // need barriers of their own.
+  const uint32_t b_pvdone2 = b_sfree + 16, b_pfull2 = b_pvdone2 + 32;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sgen + kOffBar + kBarBytes - 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + kOffBar + kBarBytes - 12);
-  const WaitCtx wc{abort_flag};
+  const WaitCtx wc{sbase + kOffBar + kBarBytes - 12};
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (known to be the same in all lanes)
@@ -572,6 +593,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       mbar_init(b_qfull + 8 * t, kRowThreads); mbar_init(b_sfull + 8 * t, 1);
       mbar_init(b_pfull + 8 * t, kRowThreads); mbar_init(b_pvdone + 8 * t, 1); mbar_init(b_sfree + 8 * t, kRowThreads);
       mbar_init(b_pvdone2 + 16 * t, 1); mbar_init(b_pvdone2 + 16 * t + 8, 1);
+      mbar_init(b_pfull2 + 16 * t, kRowThreads); mbar_init(b_pfull2 + 16 * t + 8, kRowThreads);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -588,8 +610,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   if (SPLIT) {
     // Registers move from the warps that need few to the softmax warps, which keep half a row of
     // scores in registers.  The pool is what the CTA was launched with (per scheduler 6 warps x 80
-    // registers per lane = 480); afterwards 4 x 96 + 40 + 48 (or 56 + 40 where the producers look up
-    // per-token constants) of them are in use: 472 or 480.
+    // registers per lane = 480); afterwards 4 x 96 + 48 + 48 (or 56 + 40 where the producers hold more)
+    // of them are in use: all 480.
     if (warp < 16) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSplitRegsSoftmax));
     else if (warp < 20) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegProd));
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegMisc));
@@ -606,24 +628,22 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const int hf = warp >> 3;                // half of the key columns
     const int r = (warp & 3) * 32 + (tid & 31);   // row of the tile = TMEM lane
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    // tensor memory of this form: one score buffer that the two tiles use in turn (a tile holds it
-    // only from its MMAs to its loads), two P buffers per tile, one accumulator per tile
-    const uint32_t colS = lane_addr + kColS1 + 64 * hf, colP0 = lane_addr + kColP2 + 128 * t + 32 * hf;
+    // (shared buffer: the two tiles use it in turn, a tile holds it only from its MMAs to its loads)
+    const uint32_t colS0 = lane_addr + (kOwnS ? kColTile * t : kColS1) + 64 * hf;
+    const uint32_t colP0 = lane_addr + (kOwnS ? kColTile * t : kColP2 + 128 * t) + 32 * hf;
     const uint32_t colO = lane_addr + kColO + 64 * t + 32 * hf;
-    const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 8 * t, pvdone2 = b_pvdone2 + 16 * t;
+    const uint32_t sfull = b_sfull + 8 * t, pfull2 = b_pfull2 + 16 * t, pvdone2 = b_pvdone2 + 16 * t;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
     const int pair_bar = 2 + (warp & 7);     // named barrier of the two warps with these rows
-    volatile float* xmine = reinterpret_cast<volatile float*>(sgen + kOffX) + ((t * 2 + hf) * 128 + r);
-    volatile float* xpeer = reinterpret_cast<volatile float*>(sgen + kOffX) + ((t * 2 + (hf ^ 1)) * 128 + r);
-    uint32_t xc = 0;
-    // One value per thread to the thread of the other half with the same row.  Two buffers in turn:
-    // a value is overwritten two exchanges later, after a barrier the reader has passed since.
-    auto exchange = [&](float v) -> float {
-      const uint32_t o = (xc++ & 1) * 512;
-      xmine[o] = v;
+    const uint32_t xmine = sbase + kOffX + 4 * ((t * 2 + hf) * 128 + r);
+    // One value per thread to the thread of the other half with the same row.  Two buffers in turn for
+    // the steps, a third for the end of a segment: a value is overwritten after a barrier that its
+    // reader has passed.
+    auto exchange = [&](float v, uint32_t buf) -> float {
+      st_shared_u32(xmine + buf * 2048, __float_as_uint(v));
       __syncwarp();
       asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      return xpeer[o];
+      return __uint_as_float(ld_shared_u32((xmine ^ 512u) + buf * 2048));
     };
     uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
     uint32_t g_seg = 0;                      // uses of the score buffer (both tiles) before this segment
@@ -682,11 +702,13 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         // ---- this half of the scores (64 columns) into registers; after that the score columns
         // may take the next tile's scores ----
         uint32_t ra[32], rb[32];
+        const uint32_t colS = colS0 + (kOwnS ? 64 * (cnt & 1) : 0);
         XKV_TMEM_LD32(colS, ra);
         XKV_TMEM_LD32(colS + 32, rb);
         tc_wait_ld();
         tc_fence_before();
-        mbar_arrive(b_sfree + 8 * ((use0 + (uint32_t)jj * per_step) & 1));    // uses alternate between two barriers
+        if (kOwnS) mbar_arrive(b_sfree + 8 * t);
+        else mbar_arrive(b_sfree + 8 * ((use0 + (uint32_t)jj * per_step) & 1));    // uses alternate between two barriers
         if (lim < 128) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -701,7 +723,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           mx2 = max3(mx2, __uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
         }
         float mx = fmaxf(mx1, mx2);
-        mx = fmaxf(mx, exchange(mx)) * a.scale_log2;
+        mx = fmaxf(mx, exchange(mx, cnt & 1)) * a.scale_log2;
         // The reference maximum moves only when the row maximum grew by more than 2^kGrow over it;
         // then the sums and (at the end of the step, when the registers are free) the accumulator
         // are rescaled.  Every tile has a column that is not masked, so mx is finite.
@@ -714,7 +736,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           l2b = mul_f2(l2b, pack_f2(alpha, alpha));
         }
         const uint64_t nm2 = pack_f2(-m_ref, -m_ref);
-        const uint32_t colP = colP0 + 64 * (cnt & 1);
+        // (own scores: P goes over scores of both halves; the exchange above has made sure that both hold theirs)
+        const uint32_t colP = colP0 + (kOwnS ? 128 : 64) * (cnt & 1);
         // exponentials of 16 columns against the reference; P (16-bit pairs) -> TMEM
         auto chunk16 = [&](const uint32_t* rr, int c) {
           uint64_t x[8];
@@ -731,7 +754,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             pk[i] = kBf16 ? pack_bf2(f2_lo(x[i]), f2_hi(x[i])) : pack_h2(f2_lo(x[i]), f2_hi(x[i]));
             pk[i + 1] = kBf16 ? pack_bf2(f2_lo(x[i + 1]), f2_hi(x[i + 1])) : pack_h2(f2_lo(x[i + 1]), f2_hi(x[i + 1]));
           }
-          if (c == 0 && cnt >= 2) {  // this P buffer's previous contents (two steps ago) consumed
+          if (!kOwnS && c == 0 && cnt >= 2) {  // this P buffer's previous contents (two steps ago) consumed
             mbar_wait(pvdone2 + 8 * (cnt & 1), ((cnt >> 1) - 1) & 1, wc);
             __syncwarp();
             tc_fence_after();
@@ -751,14 +774,14 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         }
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(pfull);
+        mbar_arrive(pfull2 + 8 * (cnt & 1));
       }
       // ---- epilogue of the segment: 32 channels of the row per thread ----
       mbar_wait(pvdone2 + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);    // the last PV (they complete in order)
       __syncwarp();
       tc_fence_after();
       const float l_half = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
-      const float l_peer = exchange(l_half);
+      const float l_peer = exchange(l_half, 2);
       const float l = hf ? (l_peer + l_half) : (l_half + l_peer);     // the same sum in both halves
       const bool whole = (tile_lo == 0 && nt == job.n_tiles);
       uint32_t ro[32];
@@ -1257,7 +1280,76 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         }
       }
     }
-  } else if (SPLIT && (warp == kSW + 4 || warp == kSW + 6)) {
+  } else if (kOwnS && (warp == kSW + 4 || warp == kSW + 6)) {
+    // =========================== MMA issuers, 16-warp form, own scores =========
+    // One converged warp per query tile; an elected lane issues.  Step j: S = Q K~_j^T as soon as
+    // the softmax warps hold the scores of step j - 1 in registers, then O += P V~_(j-1) as soon as
+    // P is there: the scores are a whole step ahead of the softmax.  Both warps release the K~/V~
+    // stages (two arrivals each), also for an item that has no second tile.
+    const uint32_t t = (warp == kSW + 4) ? 0u : 1u;
+    const uint32_t idesc_qk = make_idesc(128, kBf16, false);
+    const uint32_t idesc_pv = make_idesc(64, kBf16, true);
+    const uint64_t dq = make_desc(sQ + t * 16384), dk0 = make_desc(sK), dv0 = make_desc(sV);
+    const uint32_t d_tile = tmem + kColTile * t, d_o = tmem + kColO + 64 * t;
+    uint32_t kb = 0, kph = 0, vb = 0, vph = 0;      // ring positions and their parities
+    uint32_t cs = 0, cq = 0;                        // scores and query tiles so far
+    for (Walk walk(a); walk.next(a);) {
+      const int nt = walk.nt;
+      const bool active = 2 * walk.pair + (int)t < a.job[walk.job].q_tiles;
+#pragma unroll 1
+      for (int jj = 0; jj <= nt; ++jj) {
+        if (jj < nt) {
+          mbar_wait(b_kfull + 8 * kb, kph, wc);
+          if (active) {
+            // The scores of the step before are in registers, P of the one before that is consumed.  At
+            // the start of a segment Q is written after the epilogue of the segment before, so
+            // everything earlier has completed.  (Asking for an older phase would be wrong there: its
+            // parity comes round again.)
+            if (jj == 0) mbar_wait(b_qfull + 8 * t, cq & 1, wc); else mbar_wait(b_sfree + 8 * t, (cs - 1) & 1, wc);
+            if (jj > 1) mbar_wait(b_pvdone2 + 16 * t + 8 * (cs & 1), ((cs >> 1) - 1) & 1, wc);
+          }
+          __syncwarp();
+          tc_fence_after();
+          if (elect_one()) {
+            if (active) {
+              const uint64_t dk = dk0 + (uint64_t)(kb * (16384 >> 4));
+              const uint32_t d_s = d_tile + 64 * (cs & 1);
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
+                mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
+              tc_commit(b_sfull + 8 * t);
+            }
+            tc_commit(b_kfree + 8 * kb);
+          }
+          __syncwarp();
+          if (active) ++cs;
+          if (++kb == (uint32_t)kNK) { kb = 0; kph ^= 1; }
+        }
+        if (jj > 0) {
+          const uint32_t c = cs - ((jj < nt) ? 2u : 1u);       // the step whose P V~ this is
+          mbar_wait(b_vfull + 8 * vb, vph, wc);
+          if (active) mbar_wait(b_pfull2 + 16 * t + 8 * (c & 1), (c >> 1) & 1, wc);
+          __syncwarp();
+          tc_fence_after();
+          if (elect_one()) {
+            if (active) {
+              const uint64_t dv = dv0 + (uint64_t)(vb * (16384 >> 4));
+              const uint32_t d_p = d_tile + 128 * (c & 1);
+#pragma unroll
+              for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
+                mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv, (jj > 1 || ks > 0) ? 1u : 0u);
+              tc_commit(b_pvdone2 + 16 * t + 8 * (c & 1));
+            }
+            tc_commit(b_vfree + 8 * vb);
+          }
+          __syncwarp();
+          if (++vb == (uint32_t)kNV) { vb = 0; vph ^= 1; }
+        }
+      }
+      if (active) ++cq;
+    }
+    tc_fence_before();
+  } else if (SPLIT && !kOwnS && (warp == kSW + 4 || warp == kSW + 6)) {
     // =========================== MMA issuers, 16-warp form ====================
     // One converged warp per query tile, products in program order (S of step j, then P V~ of step j - 1).
     // The two tiles share one score buffer: its uses are numbered in the order tile 0, tile 1,
@@ -1280,7 +1372,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       auto issue_pv = [&](uint32_t gv, bool first_of_segment) {
         mbar_wait(b_vfull + 8 * (gv % kNV), (gv / kNV) & 1, wc);
         if (active) {
-          mbar_wait(b_pfull + 8 * t, cp & 1, wc);               // P_t of that step written
+          mbar_wait(b_pfull2 + 16 * t + 8 * (cp & 1), (cp >> 1) & 1, wc);               // P_t of that step written
           tc_fence_after();
           const uint64_t dv = make_desc(sV + (gv % kNV) * 16384);
           const uint32_t d_p = d_p0 + 64 * (cp & 1);
@@ -1518,12 +1610,12 @@ static int g_sm_count[kMaxDevices] = {0};       // 0: not set up yet
 // what the CTA was launched with.  If a compiler ever gave the kernel fewer registers at launch
 // than the reallocation needs, setmaxnreg.inc would wait for ever: refuse to run instead.
 template <typename K>
-static cudaError_t check_register_pool(K kernel, bool once, bool tail) {
+static cudaError_t check_register_pool(K kernel, int bits, bool once, bool tail) {
   cudaFuncAttributes fa;
   const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
   const int warps_per_scheduler = kThreadsSplit / 32 / 4;
-  return (fa.numRegs * warps_per_scheduler >= 4 * kSplitRegsSoftmax + split_regs_producers(once, tail) + split_regs_misc(once, tail)) ? cudaSuccess
+  return (fa.numRegs * warps_per_scheduler >= 4 * kSplitRegsSoftmax + split_regs_producers(bits, once, tail) + split_regs_misc(bits, once, tail)) ? cudaSuccess
                                                                                     : cudaErrorLaunchOutOfResources;
 }
 
@@ -1549,11 +1641,11 @@ static cudaError_t attn_device_setup(int* sm_count) {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(attn_tc_kernel<8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<8>());
     if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<4, false, false, true>, false, false);
+    e = check_register_pool(attn_tc_kernel<4, false, false, true>, 4, false, false);
     if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<16, false, false, true>, false, false);
+    e = check_register_pool(attn_tc_kernel<16, false, false, true>, 16, false, false);
     if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<4, true, false, true>, false, true);
+    e = check_register_pool(attn_tc_kernel<4, true, false, true>, 4, false, true);
     if (e != cudaSuccess) return e;
     g_sm_count[dev] = sms;
   }
@@ -1704,14 +1796,14 @@ cudaError_t launch_attn_tc_static(const AttnCall& call, int64_t ts, int64_t hs, 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(32) timeout_probe_kernel(const __grid_constant__ Args a) {
   __shared__ __align__(8) unsigned long long bar;
-  __shared__ int abort_flag;
+  __shared__ volatile int abort_flag;
   if (threadIdx.x == 0) {
     abort_flag = 0;
     mbar_init(smem_u32(&bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  const WaitCtx wc{&abort_flag};
+  const WaitCtx wc{smem_u32((const void*)&abort_flag)};
   if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, wc);     // phase 0 never completes: runs into the limit
   __syncthreads();
   mbar_wait(smem_u32(&bar), 0, wc);                           // the flag is up: every later wait returns at once
