@@ -8,19 +8,13 @@
 // not cover an item completely leaves partial results (accumulator, running max
 // and sum) in a scratch slot; a second kernel merges them.
 //
-// One CTA.  The roles are the same in both forms of the kernel; the softmax comes in two:
-//   softmax, 8 warps (SPLIT = false, 15 warps in all): warps 0-3 query tile 0, warps 4-7 query
-//               tile 1; thread r owns query row r = TMEM lane r.  Reads S from tensor memory
-//               chunk by chunk, online max/sum in one pass, writes P (16-bit) back to tensor
-//               memory, rescales O only when the running maximum grew by more than 2^14.
-//               Tensor memory: S 2 x 128 columns, P 2 x 64, O 2 x 64.
-//   softmax, 16 warps (SPLIT = true, 24 warps in all): warps w and w + 8 share the rows of a
-//               lane quarter, each takes 64 of the 128 key columns; a thread loads its half row
-//               of scores into registers at once and releases the score columns, the maximum
-//               is taken from the registers.  Registers move to these warps with setmaxnreg.
-//               Tensor memory (see the columns below): 16-bit caches ONE score buffer of 128 columns
-//               that the two tiles use in turn, P 2 x 2 x 64 (two buffers per tile), O 2 x 64; 4-bit
-//               caches scores of their own for each tile, P over them, O 2 x 64.
+// One CTA.  24 warps:
+//   16 warps    softmax: warps w and w + 8 share the rows of a TMEM lane quarter, each takes 64 of a key
+//               tile's 128 score columns, the matching 32 columns of P and 32 of the accumulator; a
+//               thread loads its half row of scores into registers at once, takes the maximum from
+//               them, exchanges it with the other half, and writes P (16-bit) back to tensor memory.
+//               O is rescaled only when the running maximum grew by more than 2^14.  Registers move to
+//               these warps with setmaxnreg.
 //   4 warps     operand producers: packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
 //               and key group) and V~ (per token) in the 128-byte-swizzled layouts the MMA
 //               descriptors expect.  One dequantised tile serves both query tiles.
@@ -50,12 +44,13 @@ namespace xkv {
 namespace {
 
 constexpr int kMaxDevices = 64;
-constexpr int kThreads = 480;
-// 16-warp form: registers per thread after the reallocation (softmax warps kSplitRegsSoftmax)
-constexpr int kSplitRegsSoftmax = 96;
-__host__ __device__ constexpr int split_regs_producers(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 56 : 48; }
-__host__ __device__ constexpr int split_regs_misc(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 40 : 48; }   // MMA issuers, copy thread
-constexpr int kThreadsSplit = 768;      // 16 softmax warps, 4 producers, 4 for the MMA issuers and the copies
+// Warps: 0-15 softmax, 16-19 producers, 20 and 22 issue the MMAs of query tile 0 resp. 1, 21 issues the
+// copies and owns the tensor memory; 23 only completes the warpgroup that setmaxnreg needs.
+constexpr int kThreads = 768;
+// registers per thread after the reallocation (setmaxnreg)
+constexpr int kRegsSoftmax = 96;
+__host__ __device__ constexpr int regs_producers(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 56 : 48; }
+__host__ __device__ constexpr int regs_misc(int bits, bool once, bool tail) { return (once || tail || bits == 16) ? 40 : 48; }   // MMA issuers, copy thread
 constexpr int kQRows = 128;
 constexpr int kMaxGrid = 160;                 // CTAs the scratch is sized for (>= SM count of the part)
 constexpr uint32_t kSpinLimit = 1u << 22;
@@ -96,24 +91,16 @@ constexpr int kOffBar = kOffTab + 2 * kTabBytes;  // barriers, tmem base, abort 
 constexpr int kBarBytes = 512;
 constexpr int kOffRaw = kOffBar + kBarBytes;      // raw stages (16-byte aligned)
 constexpr int kXchgBytes = 6144;                  // split softmax: values exchanged between the two halves of a row
-template <int BITS, bool SPLIT = false> constexpr int smem_bytes() {
-  return kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + (SPLIT ? kXchgBytes : 0) + 1024;
+template <int BITS> constexpr int smem_bytes() {
+  return kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + kXchgBytes + 1024;
 }
 
-// tensor memory columns (all 512)
-constexpr int kColS = 0;      // + 128 t : 128 fp32 columns per query tile
-constexpr int kColP = 256;    // + 64 t  : 64 columns of packed 16-bit pairs
-constexpr int kColO = 384;    // + 64 t  : 64 fp32 columns
-// 16-warp form, one score buffer for both tiles, two P buffers per tile:
-constexpr int kColS1 = 0;     // 128 fp32 columns
-constexpr int kColP2 = 128;   // + 128 t + 64 b
-// 16-warp form, scores of their own for each tile (4-bit caches): a query tile has three blocks of 64
-// columns, B0 B1 B2.  In even steps its scores take B0 B1 and P goes over B0 once the scores are in
-// registers; in odd steps the scores take B1 B2 and P goes over B2.  So the scores of a step are
-// computed during the softmax of the step before, whose P they do not touch, and P never waits for
-// the P V~ before.  24 layers at 16384 tokens: 3226 -> 3138 us.  16-bit caches, with twice the bytes a
-// tile, measured the other way (32768 tokens: 6500 -> 7000 us) and keep the shared buffer.
+// Tensor memory columns (all 512).  A query tile has three blocks of 64 columns, B0 B1 B2.  In even
+// steps its scores take B0 B1 and P (16-bit pairs) goes over B0 once the scores are in registers; in
+// odd steps the scores take B1 B2 and P goes over B2.  So the scores of a step are computed during the
+// softmax of the step before, whose P they do not touch, and P never waits for the P V~ before.
 constexpr int kColTile = 192;      // * t
+constexpr int kColO = 384;         // + 64 t : 64 fp32 columns, the accumulator
 constexpr int kTmemCols = 512;
 
 // one partial slot: two query tiles x 128 rows x (64 accumulators + max + sum)
@@ -370,23 +357,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b_d
         "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),          \
         "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory")
 
-#define XKV_TMEM_ST16(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "                                                \
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"                                    \
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
-        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), \
-        "r"(r[15]) : "memory")
-
-#define XKV_TMEM_LD16(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "                                                      \
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"                              \
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), \
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),     \
-        "=r"(r[15])                                                                                  \
-      : "r"(taddr) : "memory")
-
 #define XKV_TMEM_ST8(taddr, r)                                                                       \
   asm volatile(                                                                                      \
       "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"                       \
@@ -463,8 +433,8 @@ __device__ __forceinline__ uint4 dequant_word_h(uint32_t w, const uint32_t (&s2)
 // The same for eight 8-bit codes (two words, channels 4i..4i+3 as c0 | c2<<8 | c1<<16 | c3<<24):
 // (w & 0x00FF00FF) | 0x6400 is the fp16 pair (1024 + c0, 1024 + c1), the word shifted by 8 gives
 // (1024 + c2, 1024 + c3); every pair carries the bias 1024.
-__device__ __forceinline__ uint4 dequant_words8_h(uint2 w, const uint32_t (&s2)[4], const uint32_t (&zo)[4],
-                                                  const uint32_t (&c2)[4]) {
+__device__ __forceinline__ uint4 dequant_word_h(uint2 w, const uint32_t (&s2)[4], const uint32_t (&zo)[4],
+                                                const uint32_t (&c2)[4]) {
   const uint32_t a0 = (w.x & 0x00FF00FFu) | 0x64006400u;
   const uint32_t a1 = ((w.x >> 8) & 0x00FF00FFu) | 0x64006400u;
   const uint32_t a2 = (w.y & 0x00FF00FFu) | 0x64006400u;
@@ -496,29 +466,34 @@ __device__ __forceinline__ uint4 bf16x8_to_h8(const uint4& u) {
 }
 
 // Rows of the unquantised newest frame over the dequantised rows of a K~ or V~ tile: keys
-// slot0 + 16 i of the tile that lie in [tail_lo, t_phys) are replaced by the caller's bf16 rows
-// (src already points at this thread's head and 8-channel chunk).  A real call, so that the
-// producers' loop carries none of this code.
-__device__ __noinline__ void tail_rows_over(uint8_t* tile_row, const __nv_bfloat16* src, int64_t ts, int slot0,
+// row0 + STEP i of the tile (whose first slot is `base`) that lie in [tail_lo, t_phys) are replaced by
+// the caller's bf16 rows (src already points at this thread's head and 8-channel chunk w).  The rows
+// are those that the same thread has dequantised.  A real call, so that the producers' loop carries
+// none of this code.
+template <int STEP>
+__device__ __noinline__ void tail_rows_over(uint8_t* tile, const __nv_bfloat16* src, int64_t ts, int base, int row0, int w,
                                             int tail_lo, int t_phys, int* status) {
-  uint4 u[8];
+  bool bad = false;       // something beyond fp16
+#pragma unroll 1
+  for (int i0 = 0; i0 < 8; i0 += 4) {
+    uint4 u[4];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int slot = slot0 + 16 * i;
-    u[i] = make_uint4(0, 0, 0, 0);
-    if (slot >= tail_lo && slot < t_phys) u[i] = *reinterpret_cast<const uint4*>(src + (int64_t)(slot - tail_lo) * ts);
-  }
-  uint32_t seen = 0u;       // exponent bits of everything written: all ones somewhere = beyond fp16
+    for (int i = 0; i < 4; ++i) {
+      const int slot = base + row0 + STEP * (i0 + i);
+      u[i] = make_uint4(0, 0, 0, 0);
+      if (slot >= tail_lo && slot < t_phys) u[i] = *reinterpret_cast<const uint4*>(src + (int64_t)(slot - tail_lo) * ts);
+    }
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const int slot = slot0 + 16 * i;
-    if (slot >= tail_lo && slot < t_phys) {
-      const uint4 hv = bf16x8_to_h8(u[i]);
-      *reinterpret_cast<uint4*>(tile_row + i * 2048) = hv;
-      seen |= (h2_not_finite(hv.x) || h2_not_finite(hv.y) || h2_not_finite(hv.z) || h2_not_finite(hv.w)) ? 1u : 0u;
+    for (int i = 0; i < 4; ++i) {
+      const int row = row0 + STEP * (i0 + i), slot = base + row;
+      if (slot >= tail_lo && slot < t_phys) {
+        const uint4 hv = bf16x8_to_h8(u[i]);
+        *reinterpret_cast<uint4*>(tile + swz_off(row, w)) = hv;
+        bad |= h2_not_finite(hv.x) || h2_not_finite(hv.y) || h2_not_finite(hv.z) || h2_not_finite(hv.w);
+      }
     }
   }
-  if (seen) report_range(status);
+  if (bad) report_range(status);
 }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
@@ -529,6 +504,35 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void tma_load_1d(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// Keys quantised once: the rows of one K~ tile.  Thread t = (8-channel word, eight consecutive keys);
+// the constants of a key's group come from the table in global memory, and only where the group
+// changes: neighbours mostly belong to the same one, so a thread fetches them once or twice instead
+// of eight times (keys 16 apart, two at a time, took 4650 clk a tile in this kernel).
+// WORD: the codes of eight channels (uint32_t: 4-bit, uint2: 8-bit).
+template <typename WORD>
+__device__ __forceinline__ void once_keys(const uint8_t* codes, const uint8_t* refs, uint8_t* tile, const uint32_t* ktab16,
+                                          int n_heads, int h, int t, uint32_t b_free, uint32_t parity, const WaitCtx& wc) {
+  const int w = t & 7, k0 = (t >> 3) * 8;
+  const int4 ra = *reinterpret_cast<const int4*>(refs + 4 * k0), rb = *reinterpret_cast<const int4*>(refs + 4 * k0 + 16);
+  const int ref[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+  const uint4* table = reinterpret_cast<const uint4*>(ktab16) + (h * 8 + w) * 3;
+  uint4 sv, zv, cv;
+  auto fetch = [&](int r) {
+    const uint4* e = table + (size_t)r * n_heads * 24;
+    sv = __ldg(e); zv = __ldg(e + 1); cv = __ldg(e + 2);
+  };
+  fetch(ref[0]);
+  WORD wd[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const WORD*>(codes + (k0 + i) * (8 * sizeof(WORD)) + w * sizeof(WORD));
+  mbar_wait<256>(b_free, parity, wc);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (i > 0 && ref[i] != ref[i - 1]) fetch(ref[i]);
+    const uint32_t s2[4] = {sv.x, sv.y, sv.z, sv.w}, zo[4] = {zv.x, zv.y, zv.z, zv.w}, c2[4] = {cv.x, cv.y, cv.z, cv.w};
+    *reinterpret_cast<uint4*>(tile + (k0 + i) * 128 + ((w ^ i) << 4)) = dequant_word_h(wd[i], s2, zo, c2);
+  }
 }
 // O[row][0..63] *= alpha for the 32 rows (TMEM lanes) of the calling warp; a real call, to keep its
 // registers out of the softmax loop.  Warp-collective.
@@ -552,15 +556,14 @@ __device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, 128;
 // instantiation, so that the kernel without a tail carries none of its code).
 // ONCE: the keys' dequantisation constants are looked up per token (quantise-once mode) instead of
 // per 64-slot run.
-template <int BITS, bool TAIL = false, bool ONCE = false, bool SPLIT = false>
-__global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_kernel(const __grid_constant__ Args a) {
+template <int BITS, bool TAIL = false, bool ONCE = false>
+__global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_constant__ Args a) {
   using C = Cfg<BITS>;
-  constexpr int kSW = SPLIT ? 16 : 8;        // softmax warps
-  constexpr bool kOwnS = SPLIT && BITS == 4; // scores of their own for each tile
-  constexpr uint32_t kRowThreads = SPLIT ? 256 : 128;   // threads that work on one query tile
+  constexpr int kSW = 16;                    // softmax warps
+  constexpr uint32_t kRowThreads = 256;      // threads that work on one query tile
   constexpr int kOffX = kOffRaw + C::kNR * C::kRawStage;   // exchange area of the split softmax
   static_assert(kOffX % 1024 == 0, "the halves' places differ in one address bit");
-  constexpr int kRegProd = split_regs_producers(BITS, ONCE, TAIL), kRegMisc = split_regs_misc(BITS, ONCE, TAIL);
+  constexpr int kRegProd = regs_producers(BITS, ONCE, TAIL), kRegMisc = regs_misc(BITS, ONCE, TAIL);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
@@ -571,11 +574,12 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   const uint32_t b_vfull = b_kfree + 8 * kNK, b_vfree = b_vfull + 8 * kNV;
   const uint32_t b_rfull = b_vfree + 8 * kNV, b_rfree = b_rfull + 8 * C::kNR;
   const uint32_t b_qfull = b_rfree + 8 * C::kNR;      // [2]
-  const uint32_t b_sfull = b_qfull + 16, b_pfull = b_sfull + 16, b_pvdone = b_pfull + 16, b_sfree = b_pvdone + 16;
-  // 16-warp form, [2 tiles][2], even and odd steps: P V~ done, P written.  The warps of a tile may be
-  // almost a step apart (the next scores are there early), so arrivals of a step and of the next one
-  // need barriers of their own.
-  const uint32_t b_pvdone2 = b_sfree + 16, b_pfull2 = b_pvdone2 + 32;
+  const uint32_t b_sfull = b_qfull + 16, b_sfree = b_sfull + 16;
+  // [2 tiles][2], even and odd steps: P V~ done, P written.  A parity wait is only sound while the
+  // waiter is at most one completion away from the barrier; and the warps of a tile may be almost a
+  // step apart (the next scores are there early), so arrivals of a step and of the next one need
+  // barriers of their own.
+  const uint32_t b_pvdone = b_sfree + 16, b_pfull = b_pvdone + 32;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sgen + kOffBar + kBarBytes - 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + kOffBar + kBarBytes - 12);
   const WaitCtx wc{sbase + kOffBar + kBarBytes - 12};
@@ -591,9 +595,9 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     for (int i = 0; i < C::kNR; ++i) { mbar_init(b_rfull + 8 * i, 1); mbar_init(b_rfree + 8 * i, 128); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(b_qfull + 8 * t, kRowThreads); mbar_init(b_sfull + 8 * t, 1);
-      mbar_init(b_pfull + 8 * t, kRowThreads); mbar_init(b_pvdone + 8 * t, 1); mbar_init(b_sfree + 8 * t, kRowThreads);
-      mbar_init(b_pvdone2 + 16 * t, 1); mbar_init(b_pvdone2 + 16 * t + 8, 1);
-      mbar_init(b_pfull2 + 16 * t, kRowThreads); mbar_init(b_pfull2 + 16 * t + 8, kRowThreads);
+      mbar_init(b_sfree + 8 * t, kRowThreads);
+      mbar_init(b_pvdone + 16 * t, 1); mbar_init(b_pvdone + 16 * t + 8, 1);
+      mbar_init(b_pfull + 16 * t, kRowThreads); mbar_init(b_pfull + 16 * t + 8, kRowThreads);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -607,17 +611,17 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-  if (SPLIT) {
+  {
     // Registers move from the warps that need few to the softmax warps, which keep half a row of
     // scores in registers.  The pool is what the CTA was launched with (per scheduler 6 warps x 80
     // registers per lane = 480); afterwards 4 x 96 + 48 + 48 (or 56 + 40 where the producers hold more)
     // of them are in use: all 480.
-    if (warp < 16) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSplitRegsSoftmax));
+    if (warp < 16) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
     else if (warp < 20) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegProd));
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegMisc));
   }
 
-  if (SPLIT && warp < 16) {
+  if (warp < 16) {
     // ============== softmax warps, two per 32 rows of a query tile ==============
     // Warps w and w + 8 work on the same rows: each takes 64 of a key tile's 128 score columns, the
     // matching 32 columns of P and 32 of the accumulator.  A thread reads its half row of scores
@@ -628,11 +632,10 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
     const int hf = warp >> 3;                // half of the key columns
     const int r = (warp & 3) * 32 + (tid & 31);   // row of the tile = TMEM lane
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    // (shared buffer: the two tiles use it in turn, a tile holds it only from its MMAs to its loads)
-    const uint32_t colS0 = lane_addr + (kOwnS ? kColTile * t : kColS1) + 64 * hf;
-    const uint32_t colP0 = lane_addr + (kOwnS ? kColTile * t : kColP2 + 128 * t) + 32 * hf;
+    const uint32_t colS0 = lane_addr + kColTile * t + 64 * hf;
+    const uint32_t colP0 = lane_addr + kColTile * t + 32 * hf;
     const uint32_t colO = lane_addr + kColO + 64 * t + 32 * hf;
-    const uint32_t sfull = b_sfull + 8 * t, pfull2 = b_pfull2 + 16 * t, pvdone2 = b_pvdone2 + 16 * t;
+    const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 16 * t, pvdone = b_pvdone + 16 * t;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
     const int pair_bar = 2 + (warp & 7);     // named barrier of the two warps with these rows
     const uint32_t xmine = sbase + kOffX + 4 * ((t * 2 + hf) * 128 + r);
@@ -646,7 +649,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       return __uint_as_float(ld_shared_u32((xmine ^ 512u) + buf * 2048));
     };
     uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
-    uint32_t g_seg = 0;                      // uses of the score buffer (both tiles) before this segment
     int seg_idx = 0;
     for (Walk walk(a); walk.next(a); ++seg_idx) {
       const Job& job = a.job[walk.job];
@@ -654,9 +656,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       const int qt = 2 * walk.pair + t;
       // steps whose tile has masked columns: the pad slots after the first frame, the end
       const int jj_pad = (job.t_first & 127) ? (job.t_first >> 7) - tile_lo : -1, jj_last = job.n_tiles - 1 - tile_lo;
-      const uint32_t per_step = (2 * walk.pair + 1 < job.q_tiles) ? 2u : 1u;   // tiles that use the score buffer
-      const uint32_t use0 = g_seg + (uint32_t)t;     // this tile's uses: use0 + jj * per_step
-      g_seg += (uint32_t)nt * per_step;
       if (qt >= job.q_tiles) continue;          // the pair has no second tile
       // ---- Q tile: half of row r, bf16 -> operand type, into the swizzled K-major layout ----
       const int row = qt * kQRows + r;
@@ -702,13 +701,12 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         // ---- this half of the scores (64 columns) into registers; after that the score columns
         // may take the next tile's scores ----
         uint32_t ra[32], rb[32];
-        const uint32_t colS = colS0 + (kOwnS ? 64 * (cnt & 1) : 0);
+        const uint32_t colS = colS0 + 64 * (cnt & 1);
         XKV_TMEM_LD32(colS, ra);
         XKV_TMEM_LD32(colS + 32, rb);
         tc_wait_ld();
         tc_fence_before();
-        if (kOwnS) mbar_arrive(b_sfree + 8 * t);
-        else mbar_arrive(b_sfree + 8 * ((use0 + (uint32_t)jj * per_step) & 1));    // uses alternate between two barriers
+        mbar_arrive(b_sfree + 8 * t);
         if (lim < 128) {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
@@ -736,8 +734,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           l2b = mul_f2(l2b, pack_f2(alpha, alpha));
         }
         const uint64_t nm2 = pack_f2(-m_ref, -m_ref);
-        // (own scores: P goes over scores of both halves; the exchange above has made sure that both hold theirs)
-        const uint32_t colP = colP0 + (kOwnS ? 128 : 64) * (cnt & 1);
+        // (P goes over scores of both halves; the exchange above has made sure that both hold theirs)
+        const uint32_t colP = colP0 + 128 * (cnt & 1);
         // exponentials of 16 columns against the reference; P (16-bit pairs) -> TMEM
         auto chunk16 = [&](const uint32_t* rr, int c) {
           uint64_t x[8];
@@ -754,11 +752,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             pk[i] = kBf16 ? pack_bf2(f2_lo(x[i]), f2_hi(x[i])) : pack_h2(f2_lo(x[i]), f2_hi(x[i]));
             pk[i + 1] = kBf16 ? pack_bf2(f2_lo(x[i + 1]), f2_hi(x[i + 1])) : pack_h2(f2_lo(x[i + 1]), f2_hi(x[i + 1]));
           }
-          if (!kOwnS && c == 0 && cnt >= 2) {  // this P buffer's previous contents (two steps ago) consumed
-            mbar_wait(pvdone2 + 8 * (cnt & 1), ((cnt >> 1) - 1) & 1, wc);
-            __syncwarp();
-            tc_fence_after();
-          }
           XKV_TMEM_ST8(colP + 8 * c, pk);
         };
         chunk16(ra, 0);
@@ -767,17 +760,17 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         chunk16(rb + 16, 3);
         if (jj > 0 && __any_sync(0xffffffffu, grow)) {
           // the accumulator is quiescent once the previous step's PV has completed
-          mbar_wait(pvdone2 + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);
+          mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);
           __syncwarp();
           tc_fence_after();
           rescale_rows(colO, alpha, 32);
         }
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(pfull2 + 8 * (cnt & 1));
+        mbar_arrive(pfull + 8 * (cnt & 1));
       }
       // ---- epilogue of the segment: 32 channels of the row per thread ----
-      mbar_wait(pvdone2 + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);    // the last PV (they complete in order)
+      mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);    // the last PV (they complete in order)
       __syncwarp();
       tc_fence_after();
       const float l_half = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
@@ -809,251 +802,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           dst[c] = make_float4(__uint_as_float(ro[4 * c]), __uint_as_float(ro[4 * c + 1]),
                                __uint_as_float(ro[4 * c + 2]), __uint_as_float(ro[4 * c + 3]));
         if (hf == 0) a.part_ml[prow] = make_float2(m_ref, l);
-      }
-      tc_fence_before();
-    }
-  } else if (!SPLIT && warp < 8) {
-    // =========================== softmax warps ===============================
-    const int t = warp >> 2;                 // query tile of the pair
-    const int r = tid & 127;                 // row of the tile = TMEM lane
-    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t colS = lane_addr + kColS + 128 * t, colP = lane_addr + kColP + 64 * t;
-    const uint32_t colO = lane_addr + kColO + 64 * t;
-    const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 8 * t, pvdone = b_pvdone + 8 * t, sfree = b_sfree + 8 * t;
-    const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
-    uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
-    int seg_idx = 0;
-    for (Walk walk(a); walk.next(a); ++seg_idx) {
-      const Job& job = a.job[walk.job];
-      const int h = walk.h, tile_lo = walk.tile_lo, nt = walk.nt;
-      const int qt = 2 * walk.pair + t;
-      // steps whose tile has masked columns: the pad slots after the first frame, the end
-      const int jj_pad = (job.t_first & 127) ? (job.t_first >> 7) - tile_lo : -1, jj_last = job.n_tiles - 1 - tile_lo;
-      if (qt >= job.q_tiles) continue;          // the pair has no second tile
-      // ---- Q tile: row r, bf16 -> operand type, into the swizzled K-major layout ----
-      const int row = qt * kQRows + r;
-      {
-        uint4 u[8];
-        if (row < job.n) {
-          const __nv_bfloat16* qp = job.q + (int64_t)h * a.hs + (int64_t)row * a.ts;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) u[c] = *reinterpret_cast<const uint4*>(qp + 8 * c);
-        } else {
-#pragma unroll
-          for (int c = 0; c < 8; ++c) u[c] = make_uint4(0, 0, 0, 0);
-        }
-        bool q_bad = false;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          uint4 o = u[c];
-          if (!kBf16) {
-            const uint32_t rr[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
-            uint32_t hh[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              hh[i] = pack_h2(__uint_as_float(rr[i] << 16), __uint_as_float(rr[i] & 0xFFFF0000u));
-              q_bad |= h2_not_finite(hh[i]);
-            }
-            o = make_uint4(hh[0], hh[1], hh[2], hh[3]);
-          }
-          *reinterpret_cast<uint4*>(sgen + kOffQ + t * 16384 + swz_off(r, c)) = o;
-        }
-        if (q_bad) report_range(job.status);
-        fence_proxy_async();
-        mbar_arrive(b_qfull + 8 * t);
-      }
-      float m_ref = -INFINITY;   // reference maximum (scaled, log2 units) used for the exponentials
-      uint64_t l2 = 0ull;        // two partial row sums (packed fp32 pair)
-      for (int jj = 0; jj < nt; ++jj, ++cnt) {
-        int lim = 128;           // columns [lim, 128) are masked
-        if (jj == jj_pad) lim = job.t_first & 127;
-        if (jj == jj_last) lim = min(lim, job.t_phys - (tile_lo + jj) * 128);
-        mbar_wait(sfull, cnt & 1, wc);
-        __syncwarp();            // the spin loops may leave the warp diverged; tcgen05.ld/st are warp-collective
-        tc_fence_after();
-        bool pv_waited = (jj == 0);   // P of the previous step consumed, O quiescent (its PV completed)
-        auto wait_pv = [&]() {
-          if (!pv_waited) {
-            mbar_wait(pvdone, (cnt - 1) & 1, wc);
-            __syncwarp();
-            tc_fence_after();
-            pv_waited = true;
-          }
-        };
-        // The reference maximum m_ref moves only when the row maximum grew by more than 2^14 over
-        // it: then the row sum and the accumulator are rescaled.
-        auto apply_max = [&](float mx_scaled) {
-          float alpha = 1.f;
-          const bool grow = mx_scaled > m_ref + kGrow;
-          if (grow) {
-            alpha = exp2f(m_ref - mx_scaled);      // 0 on the first tile (m_ref = -inf)
-            m_ref = mx_scaled;
-            l2 = mul_f2(l2, pack_f2(alpha, alpha));
-          }
-          if (jj > 0) {
-            wait_pv();
-            if (__any_sync(0xffffffffu, grow)) rescale_rows(colO, alpha);
-          }
-        };
-        if (lim >= 128) {
-          // ---- full tile.  Exponentials against the current reference in one pass over S.  The
-          // pass is valid when no exponential exceeded 2^kGrow; that is checked on the row sum of
-          // the first 96 columns and the maximum of the last 32.  Otherwise (always on the first
-          // tile of a segment, rarely afterwards) the row maximum is taken first, the reference
-          // moves, and the pass is repeated. ----
-          uint64_t lt2;
-#pragma unroll 1
-          for (int attempt = 0; attempt < 2; ++attempt) {
-            if (jj == 0 || attempt == 1) {
-              float mx = -INFINITY;
-#pragma unroll 1
-              for (int c0 = 0; c0 < 128; c0 += 32) {
-                uint32_t ra[32];
-                XKV_TMEM_LD32(colS + c0, ra);
-                tc_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) mx = max3(mx, __uint_as_float(ra[i]), __uint_as_float(ra[i + 1]));
-              }
-              apply_max(mx * a.scale_log2);
-            }
-            const bool last_attempt = (jj == 0 || attempt == 1);
-            const uint64_t nm2 = pack_f2(-m_ref, -m_ref);
-            lt2 = 0ull;
-            bool redo = false;
-            uint32_t ra[32], rb[32];
-            // exponentials of 32 columns against the reference; P (16-bit pairs) -> TMEM
-            // Written in three sweeps over the chunk (scale and shift, exponentials, sums and
-            // conversion), each of 16 or 32 independent operations, so that the latency of the
-            // special-function unit is covered inside one warp.
-            auto chunk = [&](uint32_t (&rr)[32], int c) {
-              uint64_t x[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i)
-                x[i] = fma_f2(pack_f2(__uint_as_float(rr[2 * i]), __uint_as_float(rr[2 * i + 1])), sc2, nm2);
-#pragma unroll
-              for (int i = 0; i < 16; ++i) x[i] = pack_f2(fast_exp2(f2_lo(x[i])), fast_exp2(f2_hi(x[i])));
-              uint32_t pk[16];
-              uint64_t s0 = 0ull, s1 = 0ull;
-#pragma unroll
-              for (int i = 0; i < 16; i += 2) {
-                s0 = add_f2(s0, x[i]);
-                s1 = add_f2(s1, x[i + 1]);
-                pk[i] = kBf16 ? pack_bf2(f2_lo(x[i]), f2_hi(x[i])) : pack_h2(f2_lo(x[i]), f2_hi(x[i]));
-                pk[i + 1] = kBf16 ? pack_bf2(f2_lo(x[i + 1]), f2_hi(x[i + 1])) : pack_h2(f2_lo(x[i + 1]), f2_hi(x[i + 1]));
-              }
-              lt2 = add_f2(lt2, add_f2(s0, s1));
-              if (c == 0) wait_pv();
-              XKV_TMEM_ST16(colP + 16 * c, pk);
-            };
-            XKV_TMEM_LD32(colS, ra);
-            tc_wait_ld();
-#pragma unroll 1
-            for (int c = 0; c < 4; c += 2) {
-              XKV_TMEM_LD32(colS + 32 * (c + 1), rb);          // in flight while chunk c is processed
-              chunk(ra, c);
-              tc_wait_ld();
-              if (c == 0) {
-                XKV_TMEM_LD32(colS + 64, ra);
-              } else {
-                // all of S is in registers: unless the pass has to be repeated, the score columns
-                // can take the next tile's scores already
-                if (!last_attempt) {
-                  float mxl = -INFINITY;
-#pragma unroll
-                  for (int i = 0; i < 32; i += 2) mxl = max3(mxl, __uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
-                  const float part = f2_lo(lt2) + f2_hi(lt2);
-                  const bool bad = !(part < 16384.f) || (mxl * a.scale_log2 > m_ref + kGrow);
-                  redo = __any_sync(0xffffffffu, bad);
-                }
-                if (!redo) { tc_fence_before(); mbar_arrive(sfree); }
-              }
-              chunk(rb, c + 1);
-              if (c == 0) tc_wait_ld();
-            }
-            if (!redo) break;
-            tc_wait_st();
-          }
-          l2 = add_f2(l2, lt2);
-        } else {
-          // ---- masked tile (pad slots after the first frame, the tail): two plain passes ----
-          float mx = -INFINITY;
-#pragma unroll 1
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            uint32_t ra[32];
-            XKV_TMEM_LD32(colS + c0, ra);
-            tc_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const float x = (c0 + i < lim) ? __uint_as_float(ra[i]) : -INFINITY;
-              mx = fmaxf(mx, x);
-            }
-          }
-          apply_max(mx * a.scale_log2);
-          wait_pv();
-#pragma unroll 1
-          for (int c0 = 0; c0 < 128; c0 += 32) {
-            uint32_t ra[32];
-            XKV_TMEM_LD32(colS + c0, ra);
-            tc_wait_ld();
-            uint32_t pk[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              float p0 = fast_exp2(fmaf(__uint_as_float(ra[2 * i]), a.scale_log2, -m_ref));
-              float p1 = fast_exp2(fmaf(__uint_as_float(ra[2 * i + 1]), a.scale_log2, -m_ref));
-              if (c0 + 2 * i >= lim) p0 = 0.f;
-              if (c0 + 2 * i + 1 >= lim) p1 = 0.f;
-              l2 = add_f2(l2, pack_f2(p0, p1));
-              pk[i] = kBf16 ? pack_bf2(p0, p1) : pack_h2(p0, p1);
-            }
-            XKV_TMEM_ST16(colP + (c0 >> 1), pk);
-          }
-          tc_fence_before();
-          mbar_arrive(sfree);
-        }
-        tc_wait_st();
-        tc_fence_before();
-        mbar_arrive(pfull);
-      }
-      // ---- epilogue of the segment ----
-      mbar_wait(pvdone, (cnt - 1) & 1, wc);
-      __syncwarp();
-      tc_fence_after();
-      const float l = f2_lo(l2) + f2_hi(l2);
-      const bool whole = (tile_lo == 0 && nt == job.n_tiles);
-      if (whole) {
-        const float inv_l = 1.f / l;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          uint32_t ra[32];
-          XKV_TMEM_LD32(colO + c0, ra);
-          tc_wait_ld();
-          if (row < job.n) {
-            __nv_bfloat16* op = job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + c0;
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              uint32_t o[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i)
-                o[i] = pack_bf2(__uint_as_float(ra[8 * c + 2 * i]) * inv_l, __uint_as_float(ra[8 * c + 2 * i + 1]) * inv_l);
-              *reinterpret_cast<uint4*>(op + 8 * c) = make_uint4(o[0], o[1], o[2], o[3]);
-            }
-          }
-        }
-      } else {
-        const size_t slot = (size_t)2 * blockIdx.x + (seg_idx == 0 ? 0 : 1);
-        const size_t prow = (slot * 2 + t) * 128 + r;
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          uint32_t ra[32];
-          XKV_TMEM_LD32(colO + c0, ra);
-          tc_wait_ld();
-          float4* dst = reinterpret_cast<float4*>(a.part_o + prow * 64 + c0);
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            dst[c] = make_float4(__uint_as_float(ra[4 * c]), __uint_as_float(ra[4 * c + 1]),
-                                 __uint_as_float(ra[4 * c + 2]), __uint_as_float(ra[4 * c + 3]));
-        }
-        a.part_ml[prow] = make_float2(m_ref, l);
       }
       tc_fence_before();
     }
@@ -1130,39 +878,12 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           producer_sync();
           // ---- keys ----
           uint32_t wd[8];
+          if (ONCE) {
+            once_keys<uint32_t>(raw, raw + C::kRawK + C::kRawV, sgen + kOffK + kbuf * 16384, job.ktab16, job.n_heads, h, t,
+                                b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
+          } else {
 #pragma unroll
           for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const uint32_t*>(raw + (kb + 16 * i) * 32 + 4 * w);
-          if (ONCE) {
-            // constants of each token's own key group, from the table in global memory (the tokens of
-            // a group mostly sit next to each other, so the lines are shared); two tokens at a time,
-            // the next two fetched while these are dequantised
-            const uint8_t* slp = raw + C::kRawK + C::kRawV + 4 * kb;      // group references of keys kb + 16 i
-            auto entry = [&](int i) {
-              const int sl = *reinterpret_cast<const int*>(slp + 64 * i);
-              return reinterpret_cast<const uint4*>(job.ktab16 + (((size_t)sl * job.n_heads + h) * 8 + w) * 12);
-            };
-            uint4 sv[2], zv[2], cv[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) { const uint4* e = entry(i); sv[i] = __ldg(e); zv[i] = __ldg(e + 1); cv[i] = __ldg(e + 2); }
-            mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
-#pragma unroll
-            for (int q2 = 0; q2 < 4; ++q2) {
-              uint4 o[2];
-#pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                const uint32_t s2[4] = {sv[i].x, sv[i].y, sv[i].z, sv[i].w}, zo[4] = {zv[i].x, zv[i].y, zv[i].z, zv[i].w};
-                const uint32_t c2[4] = {cv[i].x, cv[i].y, cv[i].z, cv[i].w};
-                o[i] = dequant_word_h(wd[2 * q2 + i], s2, zo, c2);
-              }
-              if (q2 < 3) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) { const uint4* e = entry(2 * q2 + 2 + i); sv[i] = __ldg(e); zv[i] = __ldg(e + 1); cv[i] = __ldg(e + 2); }
-              }
-#pragma unroll
-              for (int i = 0; i < 2; ++i)
-                *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + (2 * q2 + i) * 2048) = o[i];
-            }
-          } else {
           mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
 #pragma unroll
           for (int grp = 0; grp < 2; ++grp) {
@@ -1179,7 +900,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           }
           }
           if (TAIL && tail_tile)
-            tail_rows_over(sgen + kOffK + kbuf * 16384 + row_off, job.k_tail + tail_off, a.ts, slot0, job.tail_lo, job.t_phys, job.status);
+            tail_rows_over<ONCE ? 1 : 16>(sgen + kOffK + kbuf * 16384, job.k_tail + tail_off, a.ts, slot0 - kb, ONCE ? (t >> 3) * 8 : kb, w, job.tail_lo,
+                                          job.t_phys, job.status);
           fence_proxy_async();
           mbar_arrive(b_kfull + 8 * kbuf);
           // ---- values ----
@@ -1195,7 +917,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             *reinterpret_cast<uint4*>(sgen + kOffV + vbuf * 16384 + row_off + i * 2048) = o;
           }
           if (TAIL && tail_tile)
-            tail_rows_over(sgen + kOffV + vbuf * 16384 + row_off, job.v_tail + tail_off, a.ts, slot0, job.tail_lo, job.t_phys, job.status);
+            tail_rows_over<16>(sgen + kOffV + vbuf * 16384, job.v_tail + tail_off, a.ts, slot0 - kb, kb, w, job.tail_lo, job.t_phys, job.status);
           fence_proxy_async();
           mbar_arrive(b_vfull + 8 * vbuf);
           // The raw stage is released only here, after the words read from it have been used and
@@ -1214,34 +936,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
           }
           producer_sync();
           uint2 wd8[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) wd8[i] = *reinterpret_cast<const uint2*>(raw + (kb + 16 * i) * 64 + 8 * w);
-          const uint8_t* slp = raw + C::kRawK + C::kRawV + 4 * kb;      // group references of keys kb + 16 i
-          auto entry = [&](int i) {
-            const int sl = *reinterpret_cast<const int*>(slp + 64 * i);
-            return reinterpret_cast<const uint4*>(job.ktab16 + (((size_t)sl * job.n_heads + h) * 8 + w) * 12);
-          };
-          uint4 sv[2], zv[2], cv[2];
-#pragma unroll
-          for (int i = 0; i < 2; ++i) { const uint4* e = entry(i); sv[i] = __ldg(e); zv[i] = __ldg(e + 1); cv[i] = __ldg(e + 2); }
-          mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
-#pragma unroll
-          for (int q2 = 0; q2 < 4; ++q2) {
-            uint4 o[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-              const uint32_t s2[4] = {sv[i].x, sv[i].y, sv[i].z, sv[i].w}, zo[4] = {zv[i].x, zv[i].y, zv[i].z, zv[i].w};
-              const uint32_t c2[4] = {cv[i].x, cv[i].y, cv[i].z, cv[i].w};
-              o[i] = dequant_words8_h(wd8[2 * q2 + i], s2, zo, c2);
-            }
-            if (q2 < 3) {
-#pragma unroll
-              for (int i = 0; i < 2; ++i) { const uint4* e = entry(2 * q2 + 2 + i); sv[i] = __ldg(e); zv[i] = __ldg(e + 1); cv[i] = __ldg(e + 2); }
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-              *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + (2 * q2 + i) * 2048) = o[i];
-          }
+          once_keys<uint2>(raw, raw + C::kRawK + C::kRawV, sgen + kOffK + kbuf * 16384, job.ktab16, job.n_heads, h, t,
+                           b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
           fence_proxy_async();
           mbar_arrive(b_kfull + 8 * kbuf);
 #pragma unroll
@@ -1252,7 +948,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             const uint4 pv = *reinterpret_cast<const uint4*>(tab + 768 + 16 * (kb + 16 * i));
             const uint32_t s2[4] = {pv.x, pv.x, pv.x, pv.x}, zo[4] = {pv.y, pv.y, pv.y, pv.y};
             const uint32_t c2[4] = {pv.w, pv.w, pv.w, pv.w};
-            const uint4 o = dequant_words8_h(wd8[i], s2, zo, c2);
+            const uint4 o = dequant_word_h(wd8[i], s2, zo, c2);
             *reinterpret_cast<uint4*>(sgen + kOffV + vbuf * 16384 + row_off + i * 2048) = o;
           }
           fence_proxy_async();
@@ -1280,8 +976,8 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         }
       }
     }
-  } else if (kOwnS && (warp == kSW + 4 || warp == kSW + 6)) {
-    // =========================== MMA issuers, 16-warp form, own scores =========
+  } else if (warp == kSW + 4 || warp == kSW + 6) {
+    // =========================== MMA issuers ==================================
     // One converged warp per query tile; an elected lane issues.  Step j: S = Q K~_j^T as soon as
     // the softmax warps hold the scores of step j - 1 in registers, then O += P V~_(j-1) as soon as
     // P is there: the scores are a whole step ahead of the softmax.  Both warps release the K~/V~
@@ -1306,7 +1002,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
             // everything earlier has completed.  (Asking for an older phase would be wrong there: its
             // parity comes round again.)
             if (jj == 0) mbar_wait(b_qfull + 8 * t, cq & 1, wc); else mbar_wait(b_sfree + 8 * t, (cs - 1) & 1, wc);
-            if (jj > 1) mbar_wait(b_pvdone2 + 16 * t + 8 * (cs & 1), ((cs >> 1) - 1) & 1, wc);
+            if (jj > 1) mbar_wait(b_pvdone + 16 * t + 8 * (cs & 1), ((cs >> 1) - 1) & 1, wc);
           }
           __syncwarp();
           tc_fence_after();
@@ -1328,7 +1024,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
         if (jj > 0) {
           const uint32_t c = cs - ((jj < nt) ? 2u : 1u);       // the step whose P V~ this is
           mbar_wait(b_vfull + 8 * vb, vph, wc);
-          if (active) mbar_wait(b_pfull2 + 16 * t + 8 * (c & 1), (c >> 1) & 1, wc);
+          if (active) mbar_wait(b_pfull + 16 * t + 8 * (c & 1), (c >> 1) & 1, wc);
           __syncwarp();
           tc_fence_after();
           if (elect_one()) {
@@ -1338,7 +1034,7 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
 #pragma unroll
               for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
                 mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv, (jj > 1 || ks > 0) ? 1u : 0u);
-              tc_commit(b_pvdone2 + 16 * t + 8 * (c & 1));
+              tc_commit(b_pvdone + 16 * t + 8 * (c & 1));
             }
             tc_commit(b_vfree + 8 * vb);
           }
@@ -1348,135 +1044,6 @@ __global__ void __launch_bounds__(SPLIT ? kThreadsSplit : kThreads, 1) attn_tc_k
       }
       if (active) ++cq;
     }
-    tc_fence_before();
-  } else if (SPLIT && !kOwnS && (warp == kSW + 4 || warp == kSW + 6)) {
-    // =========================== MMA issuers, 16-warp form ====================
-    // One converged warp per query tile, products in program order (S of step j, then P V~ of step j - 1).
-    // The two tiles share one score buffer: its uses are numbered in the order tile 0, tile 1,
-    // tile 0, ... (tile 0 alone where the item has no second tile), and use G is issued once the
-    // softmax warps have loaded use G - 1.  Even and odd uses are released on two barriers: the
-    // barrier of use G - 1 cannot complete again before use G + 1 has been issued, and a thread
-    // waits for uses that are at most two apart, so a parity wait is never two phases off.
-    const int t = (warp == kSW + 6) ? 1 : 0;
-    const uint32_t idesc_qk = make_idesc(128, kBf16, false);
-    const uint32_t idesc_pv = make_idesc(64, kBf16, true);
-    const uint64_t dq = make_desc(sQ + t * 16384);
-    const uint32_t d_s = tmem + kColS1, d_p0 = tmem + kColP2 + 128 * t, d_o = tmem + kColO + 64 * t;
-    uint32_t g = 0, cp = 0, segq = 0;
-    uint32_t g_seg = 0;              // score-buffer uses before this segment
-    for (Walk walk(a); walk.next(a);) {
-      const Job& job = a.job[walk.job];
-      const int nt = walk.nt;
-      const bool active = 2 * walk.pair + t < job.q_tiles;
-      const uint32_t per_step = (2 * walk.pair + 1 < job.q_tiles) ? 2u : 1u;     // tiles that use the score buffer
-      auto issue_pv = [&](uint32_t gv, bool first_of_segment) {
-        mbar_wait(b_vfull + 8 * (gv % kNV), (gv / kNV) & 1, wc);
-        if (active) {
-          mbar_wait(b_pfull2 + 16 * t + 8 * (cp & 1), (cp >> 1) & 1, wc);               // P_t of that step written
-          tc_fence_after();
-          const uint64_t dv = make_desc(sV + (gv % kNV) * 16384);
-          const uint32_t d_p = d_p0 + 64 * (cp & 1);
-          if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
-              mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
-                     (!first_of_segment || ks > 0) ? 1u : 0u);
-            tc_commit(b_pvdone2 + 16 * t + 8 * (cp & 1));
-          }
-          __syncwarp();
-          ++cp;
-        }
-        if (elect_one()) tc_commit(b_vfree + 8 * (gv % kNV));
-        __syncwarp();
-      };
-      for (int jj = 0; jj < nt; ++jj, ++g) {
-        mbar_wait(b_kfull + 8 * (g % kNK), (g / kNK) & 1, wc);
-        if (active) {
-          const uint32_t use = g_seg + (uint32_t)jj * per_step + (uint32_t)t;
-          if (use > 0) mbar_wait(b_sfree + 8 * ((use - 1) & 1), ((use - 1) >> 1) & 1, wc);   // use - 1 is in registers
-          if (jj == 0) mbar_wait(b_qfull + 8 * t, segq & 1, wc);
-          tc_fence_after();
-          const uint64_t dk = make_desc(sK + (g % kNK) * 16384);
-          if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
-              mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
-            tc_commit(b_sfull + 8 * t);
-          }
-          __syncwarp();
-        } else {
-          // An item without a second tile: this thread follows the other tile's uses of the score
-          // buffer one by one.  A parity wait is only sound while the waiter is at most one
-          // completion ahead of the barrier, so no use may be skipped.
-          const uint32_t use = g_seg + (uint32_t)jj;
-          if (use > 0) mbar_wait(b_sfree + 8 * ((use - 1) & 1), ((use - 1) >> 1) & 1, wc);
-        }
-        if (elect_one()) tc_commit(b_kfree + 8 * (g % kNK));
-        __syncwarp();
-        if (jj > 0) issue_pv(g - 1, jj == 1);
-      }
-      issue_pv(g - 1, nt == 1);           // the last PV of the segment
-      g_seg += (uint32_t)nt * per_step;
-      if (active) ++segq;
-    }
-    tc_fence_before();
-  } else if (!SPLIT && (warp == kSW + 4 || warp == kSW + 6)) {
-    // =========================== MMA issuers ==================================
-    // One converged warp per query tile.  Both release the K~/V~ stages (two arrivals each), also for
-    // an item that has no second tile: then the second warp only follows the rings.
-    const int t = (warp == kSW + 6) ? 1 : 0;
-    const uint32_t idesc_qk = make_idesc(128, kBf16, false);
-    const uint32_t idesc_pv = make_idesc(64, kBf16, true);
-    const uint64_t dq = make_desc(sQ + t * 16384);
-    const uint32_t d_s = tmem + kColS + 128 * t, d_p = tmem + kColP + 64 * t, d_o = tmem + kColO + 64 * t;
-    uint32_t g = 0, cnt = 0, segq = 0;
-    for (Walk walk(a); walk.next(a);) {
-      const Job& job = a.job[walk.job];
-      const int nt = walk.nt;
-      const bool active = 2 * walk.pair + t < job.q_tiles;
-      auto issue_pv = [&](uint32_t gv, bool first_of_segment) {
-        mbar_wait(b_vfull + 8 * (gv % kNV), (gv / kNV) & 1, wc);
-        if (active) {
-          mbar_wait(b_pfull + 8 * t, (cnt - 1) & 1, wc);        // P_t of that step written
-          tc_fence_after();
-          const uint64_t dv = make_desc(sV + (gv % kNV) * 16384);
-          if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)   // 16 keys per step: 2 swizzle atoms = 2048 B of V~, 8 columns of P
-              mma_ts(d_o, d_p + 8 * ks, dv + (uint64_t)((ks * 2048) >> 4), idesc_pv,
-                     (!first_of_segment || ks > 0) ? 1u : 0u);
-            tc_commit(b_pvdone + 8 * t);
-          }
-          __syncwarp();
-        }
-        if (elect_one()) tc_commit(b_vfree + 8 * (gv % kNV));
-        __syncwarp();
-      };
-      for (int jj = 0; jj < nt; ++jj, ++g) {
-        mbar_wait(b_kfull + 8 * (g % kNK), (g / kNK) & 1, wc);
-        if (active) {
-          if (jj == 0) mbar_wait(b_qfull + 8 * t, segq & 1, wc);
-          else mbar_wait(b_sfree + 8 * t, (cnt - 1) & 1, wc);   // S_t of the previous step has been read
-          tc_fence_after();
-          const uint64_t dk = make_desc(sK + (g % kNK) * 16384);
-          if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)   // 16 channels per step: 32 B inside the swizzle span
-              mma_ss(d_s, dq + (uint64_t)(ks * 2), dk + (uint64_t)(ks * 2), idesc_qk, ks > 0 ? 1u : 0u);
-            tc_commit(b_sfull + 8 * t);
-          }
-          __syncwarp();
-        }
-        if (elect_one()) tc_commit(b_kfree + 8 * (g % kNK));
-        __syncwarp();
-        if (jj > 0) issue_pv(g - 1, jj == 1);
-        if (active) ++cnt;
-      }
-      issue_pv(g - 1, nt == 1);           // the last PV of the segment
-      if (active) ++segq;
-    }
-    // all MMAs must be done before the CTA may free tensor memory: the softmax warps have waited
-    // for every PV (pvdone) before their epilogues, and every QK (sfull) before that.
     tc_fence_before();
   } else if (tid == 32 * (kSW + 5)) {
     // =========================== TMA loader ===================================
@@ -1606,17 +1173,20 @@ size_t attn_tc_scratch_bytes(const xkv_params*) { return (size_t)2 * kMaxGrid * 
 static std::mutex g_setup_mutex;
 static int g_sm_count[kMaxDevices] = {0};       // 0: not set up yet
 
-// The 16-warp form moves registers between its warps with setmaxnreg; the pool they move in is
-// what the CTA was launched with.  If a compiler ever gave the kernel fewer registers at launch
-// than the reallocation needs, setmaxnreg.inc would wait for ever: refuse to run instead.
-template <typename K>
-static cudaError_t check_register_pool(K kernel, int bits, bool once, bool tail) {
-  cudaFuncAttributes fa;
-  const cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+// The kernel moves registers between its warps with setmaxnreg; the pool they move in is what the CTA
+// was launched with.  If a compiler ever gave the kernel fewer registers at launch than the
+// reallocation needs, setmaxnreg.inc would wait for ever: refuse to run instead.
+template <int BITS, bool TAIL, bool ONCE>
+static cudaError_t prepare_kernel() {
+  const auto kernel = attn_tc_kernel<BITS, TAIL, ONCE>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<BITS>());
   if (e != cudaSuccess) return e;
-  const int warps_per_scheduler = kThreadsSplit / 32 / 4;
-  return (fa.numRegs * warps_per_scheduler >= 4 * kSplitRegsSoftmax + split_regs_producers(bits, once, tail) + split_regs_misc(bits, once, tail)) ? cudaSuccess
-                                                                                    : cudaErrorLaunchOutOfResources;
+  cudaFuncAttributes fa;
+  e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  const int warps_per_scheduler = kThreads / 32 / 4;
+  return (fa.numRegs * warps_per_scheduler >= 4 * kRegsSoftmax + regs_producers(BITS, ONCE, TAIL) + regs_misc(BITS, ONCE, TAIL))
+             ? cudaSuccess : cudaErrorLaunchOutOfResources;
 }
 
 static cudaError_t attn_device_setup(int* sm_count) {
@@ -1629,23 +1199,12 @@ static cudaError_t attn_device_setup(int* sm_count) {
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<4, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<4, true>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<16, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<16, true>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<4, true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<4, true>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<4, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<4>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<4, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<4>());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_tc_kernel<8, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<8>());
-    if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<4, false, false, true>, 4, false, false);
-    if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<16, false, false, true>, 16, false, false);
-    if (e != cudaSuccess) return e;
-    e = check_register_pool(attn_tc_kernel<4, true, false, true>, 4, false, true);
+    e = prepare_kernel<4, false, false>();
+    if (e == cudaSuccess) e = prepare_kernel<4, true, false>();
+    if (e == cudaSuccess) e = prepare_kernel<4, false, true>();
+    if (e == cudaSuccess) e = prepare_kernel<4, true, true>();
+    if (e == cudaSuccess) e = prepare_kernel<8, false, true>();
+    if (e == cudaSuccess) e = prepare_kernel<16, false, false>();
     if (e != cudaSuccess) return e;
     g_sm_count[dev] = sms;
   }
@@ -1701,16 +1260,13 @@ static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail,
   {
     LaunchScope ls(c, XKV_PROF_ATTN, st);
     const bool once = c->p.key_mode == XKV_KEYS_ONCE;
-    // The 16-warp softmax where the producers have registers to spare for it; with per-token
-    // constants (keys quantised once, 8-bit codes) the producers need theirs and the 8-warp
-    // softmax measured faster.
-    const int T = kThreadsSplit;
-    if (c->p.kv_bits == 16) attn_tc_kernel<16, false, false, true><<<(int)grid, T, smem_bytes<16, true>(), st>>>(a);
-    else if (c->p.kv_bits == 8) attn_tc_kernel<8, false, true><<<(int)grid, kThreads, smem_bytes<8>(), st>>>(a);
-    else if (tail && once) attn_tc_kernel<4, true, true><<<(int)grid, kThreads, smem_bytes<4>(), st>>>(a);
-    else if (tail) attn_tc_kernel<4, true, false, true><<<(int)grid, T, smem_bytes<4, true>(), st>>>(a);
-    else if (once) attn_tc_kernel<4, false, true><<<(int)grid, kThreads, smem_bytes<4>(), st>>>(a);
-    else attn_tc_kernel<4, false, false, true><<<(int)grid, T, smem_bytes<4, true>(), st>>>(a);
+    const int g = (int)grid;
+    if (c->p.kv_bits == 16) attn_tc_kernel<16><<<g, kThreads, smem_bytes<16>(), st>>>(a);
+    else if (c->p.kv_bits == 8) attn_tc_kernel<8, false, true><<<g, kThreads, smem_bytes<8>(), st>>>(a);
+    else if (tail && once) attn_tc_kernel<4, true, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
+    else if (tail) attn_tc_kernel<4, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
+    else if (once) attn_tc_kernel<4, false, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
+    else attn_tc_kernel<4><<<g, kThreads, smem_bytes<4>(), st>>>(a);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
