@@ -116,6 +116,17 @@ __device__ __forceinline__ void dequant8_magic(uint32_t word, const float2 (&par
   }
 }
 
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // Two fp32 numbers in one 64-bit register and the packed forms of the IEEE operations (each half
 // is rounded exactly like the scalar operation, so results do not change; one instruction does two).
 __device__ __forceinline__ uint64_t pk2(float lo, float hi) {
@@ -1022,8 +1033,6 @@ __device__ __forceinline__ void phase_sel2(const MaintArgs& a, const Blocks& B, 
 // ---------------------------------------------------------------------------
 // kv_quant_pack, 4-bit: a kernel of its own (one thread block per item, placed by the
 // hardware scheduler; the arithmetic needs more registers than the phases above).
-// Item = (new 64-slot key group, four heads); 128 threads per head, thread =
-// (8-channel word, four tokens 16 apart).
 // Keys: survivors are dequantised with the parameters of the group they came
 // from (Eq. 10), new keys come from the bf16 staging buffer; per-channel min/max
 // over the group's tokens; new parameters and codes (Eq. 7-8).  A complete group
@@ -1031,7 +1040,9 @@ __device__ __forceinline__ void phase_sel2(const MaintArgs& a, const Blocks& B, 
 // Values: the survivors' code rows and parameters, and the origins, move to
 // their new slots in the other buffer set (they were quantised on arrival).
 // ---------------------------------------------------------------------------
-constexpr int kRgHeads = 4;
+constexpr int kTpt = 4;                          // tokens per thread
+constexpr int kRgLanes = 64 / kTpt;              // token lanes
+constexpr int kRgThreads = 8 * kRgLanes;
 
 struct RegroupArgs {
   BufSet src, dst;                // (the first frame goes to both buffer sets)
@@ -1043,197 +1054,192 @@ struct RegroupArgs {
 };
 template <int MAX> struct RegroupBatch { RegroupArgs layer[MAX]; };
 
+// Block = (64-slot group, head), thread = (four consecutive tokens, 8-channel word).  Bound by
+// instruction issue and latency: consecutive tokens rarely change the source group (its parameters are
+// 40 instructions), and the per-channel extremes go through shared memory instead of 32 shuffles a
+// thread.  24 layers at 16384 tokens: 584 us with four heads a block, tokens 16 apart and shuffles; eight tokens
+// a thread 414 (80 registers, spills) and 447 us (117 registers, too few warps); four tokens, four
+// heads a block 436, two heads 396, one head 369 us (small blocks wait for less at their barriers).
 template <int MAX>
-__global__ void __launch_bounds__(128 * kRgHeads, 2) regroup_k_kernel(const __grid_constant__ RegroupBatch<MAX> batch, const int H) {
+__global__ void __launch_bounds__(kRgThreads, 8) regroup_k_kernel(const __grid_constant__ RegroupBatch<MAX> batch) {
   const RegroupArgs& a = batch.layer[MAX == 1 ? 0 : blockIdx.z];
   if ((int)blockIdx.x * 64 >= a.r_new) return;
-  const BufSet& src = a.src;
-  const BufSet& dst = a.dst;
-  const BufSet& dst2 = a.src;
-  const bool two = a.two;
-  const int cap = a.cap, max_n = a.max_n, base_slot = a.base_slot, kk = a.kk, r_new = a.r_new, force_plain = a.force_plain;
-  const int32_t* __restrict__ kept = a.kept;
-  const __nv_bfloat16* __restrict__ kstage = a.kstage;
-  __shared__ int s_old[64];                      // source position (rest-local) of each token, -1 = new key
-  __shared__ float s_mn[kRgHeads][4][64];
-  __shared__ float s_mx[kRgHeads][4][64];
-  __shared__ float2 s_iz[kRgHeads][64];
+  const int cap = a.cap, base_slot = a.base_slot, kk = a.kk, r_new = a.r_new;
+  __shared__ __align__(16) int s_old[64];        // source position (rest-local) of each token, -1 = new key, -2 = none
+  __shared__ __align__(16) float s_mn[kRgLanes][64];   // per token lane; channel 8w + 4k + e at 32k + 4w + e
+  __shared__ __align__(16) float s_mx[kRgLanes][64];
+  __shared__ __align__(16) float2 s_iz[64];     // 1/s and z - magic (int); channel 8w + 2v + e at (8v + w) 2 + e
+  __shared__ float s_z[64];                     // z, for the plain forms
   const int tid = threadIdx.x;
   const int gamma = blockIdx.x;
-  const int hl = tid >> 7;                       // head within the CTA
-  const int h = blockIdx.y * kRgHeads + hl;
-  const int t = tid & 127;
-  const int w = t & 7;
-  const int tq = t >> 3;                         // tokens tq + 16 u
-  const int wih = t >> 5;                        // warp within the head
-  const bool head_ok = h < H;
+  const int h = blockIdx.y;
+  const int w = tid & 7, tq = tid >> 3;              // tokens kTpt tq + u
   if (tid < 64) {
     const int i = gamma * 64 + tid;
-    s_old[tid] = (i < kk) ? (kept ? kept[i] : i) : -1;
+    s_old[tid] = (i < kk) ? (a.kept ? a.kept[i] : i) : (i < r_new) ? -1 : -2;
   }
   __syncthreads();
+  const size_t head_slot = (size_t)h * cap + base_slot;
 
-  // ---- values, parameters and origins of the survivors (first frame: nothing to move): the row is
-  // fetched here and stored after the key loads below have been issued, so that the two round
-  // trips overlap (thread = (head, token, half row): exactly one item per thread) ----
+  // ---- values, parameters and origins of the survivors (first frame: nothing to move): half a
+  // token's row is fetched here and stored after the key loads below have been issued, so that the two
+  // round trips overlap ----
   uint4 v_row = make_uint4(0, 0, 0, 0);
   float2 v_par = make_float2(0.f, 0.f);
   int v_org = 0;
-  size_t v_dst = 0;
-  bool v_move = false, o_move = false;
-  {
-    const int half = tid & 1, tok = (tid >> 1) & 63, hh = blockIdx.y * kRgHeads + (tid >> 7);
-    const int i = gamma * 64 + tok;
-    if (kk > 0 && hh < H && i < kk) {
-      const size_t s_slot = (size_t)hh * cap + base_slot + s_old[tok];
-      v_dst = (size_t)hh * cap + base_slot + i;
-      v_row = *reinterpret_cast<const uint4*>(src.v + s_slot * 32 + 16 * half);
-      if (half == 0) v_par = src.vpar[s_slot];
-      v_move = true;
-    }
-    if (kk > 0 && blockIdx.y == 0 && tid < 64 && gamma * 64 + tid < kk) {
-      v_org = src.origin[base_slot + s_old[tid]];
-      o_move = true;
-    }
+  const int v_tok = tid >> 1, v_half = tid & 1;
+  const int v_old = s_old[v_tok];
+  const bool v_move = v_old >= 0, o_move = v_move && h == 0 && v_half == 0;
+  if (v_move) {
+    v_row = *(reinterpret_cast<const uint4*>(a.src.v + (head_slot + v_old) * 32) + v_half);
+    if (v_half == 0) v_par = a.src.vpar[head_slot + v_old];
   }
+  if (o_move) v_org = a.src.origin[base_slot + v_old];
   auto store_values = [&]() {
     if (v_move) {
-      *reinterpret_cast<uint4*>(dst.v + v_dst * 32 + 16 * (tid & 1)) = v_row;
-      if ((tid & 1) == 0) dst.vpar[v_dst] = v_par;
+      *(reinterpret_cast<uint4*>(a.dst.v + (head_slot + gamma * 64 + v_tok) * 32) + v_half) = v_row;
+      if (v_half == 0) a.dst.vpar[head_slot + gamma * 64 + v_tok] = v_par;
     }
-    if (o_move) dst.origin[base_slot + gamma * 64 + tid] = v_org;
+    if (o_move) a.dst.origin[base_slot + gamma * 64 + v_tok] = v_org;
   };
 
   // ---- keys ----
   const int last = gamma * 64 + 63;
   const bool carried = (last < kk) && (s_old[63] == last);
   const size_t dgrp = ((size_t)h * (cap >> 6) + (base_slot >> 6) + gamma) * 64;
+  const size_t drow = (head_slot + gamma * 64 + kTpt * tq) * 32 + 4 * w;      // this thread's first word in the destination
   if (carried) {
     store_values();
-    if (head_ok) {
+    {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const size_t dslot = (size_t)h * cap + base_slot + gamma * 64 + tq + 16 * u;
-        const uint32_t word = *reinterpret_cast<const uint32_t*>(src.k + dslot * 32 + 4 * w);
-        *reinterpret_cast<uint32_t*>(dst.k + dslot * 32 + 4 * w) = word;
-        if (two) *reinterpret_cast<uint32_t*>(dst2.k + dslot * 32 + 4 * w) = word;
+      for (int u = 0; u < kTpt; ++u) {
+        const uint32_t word = *reinterpret_cast<const uint32_t*>(a.src.k + drow + 32 * u);
+        *reinterpret_cast<uint32_t*>(a.dst.k + drow + 32 * u) = word;
+        if (a.two) *reinterpret_cast<uint32_t*>(a.src.k + drow + 32 * u) = word;
       }
-      if (t < 64) {
-        const float2 sz = src.kpar[dgrp + t];
-        dst.kpar[dgrp + t] = sz;
-        if (two) dst2.kpar[dgrp + t] = sz;
+      if (tid < 64) {
+        const float2 sz = a.src.kpar[dgrp + tid];
+        a.dst.kpar[dgrp + tid] = sz;
+        if (a.two) a.src.kpar[dgrp + tid] = sz;
       }
     }
     return;
   }
-  float x[4][8];
-  uint32_t word[4];
-  uint4 fresh[4];
-  int old[4];
+  int old[kTpt];
+  {
+    const int4 o = *reinterpret_cast<const int4*>(&s_old[kTpt * tq]);
+    old[0] = o.x; old[1] = o.y; old[2] = o.z; old[3] = o.w;
+  }
+  uint32_t word[kTpt];
+  {
+    const uint8_t* kp = a.src.k + head_slot * 32 + 4 * w;
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int tok = tq + 16 * u;
-    const int i = gamma * 64 + tok;
-    old[u] = (i < r_new) ? s_old[tok] : -2;      // -2: beyond the segment
-    word[u] = 0u;
-    fresh[u] = make_uint4(0, 0, 0, 0);
-    if (head_ok && old[u] >= 0)
-      word[u] = *reinterpret_cast<const uint32_t*>(src.k + ((size_t)h * cap + base_slot + old[u]) * 32 + 4 * w);
-    else if (head_ok && old[u] == -1)
-      fresh[u] = *reinterpret_cast<const uint4*>(kstage + ((size_t)h * max_n + (i - kk)) * 64 + 8 * w);
+    for (int u = 0; u < kTpt; ++u) {
+      word[u] = 0u;
+      if (old[u] >= 0) word[u] = *reinterpret_cast<const uint32_t*>(kp + (size_t)old[u] * 32);
+    }
   }
   store_values();
-  int par_grp = -1;
-  const float2* par_src = nullptr; // the group's (s, z) in global memory (the plain path reads them there)
-  uint64_t s2[4], mz2[4];          // fast path: (s, s) and (magic + z, magic + z) of the channel pairs
-  bool par_plain = false;
+  float x[kTpt][8];
+  {
+    int par_grp = -1;
+    const float2* par_src = nullptr; // the group's (s, z) in global memory (the plain path reads them there)
+    uint64_t s2[4], mz2[4];          // fast path: (s, s) and (magic + z, magic + z) of the channel pairs
+    bool par_plain = false;
+    const float2* par0 = a.src.kpar + ((size_t)h * (cap >> 6) + (base_slot >> 6)) * 64 + 8 * w;   // (base_slot is a multiple of 64)
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (old[u] >= 0) {
-      const int g = (base_slot + old[u]) >> 6;
-      if (g != par_grp && head_ok) {
-        const float4* pp = reinterpret_cast<const float4*>(src.kpar + ((size_t)h * (cap >> 6) + g) * 64 + 8 * w);
-        float zmax = 0.f;
+    for (int u = 0; u < kTpt; ++u) {
+      if (old[u] >= 0) {
+        const int g = old[u] >> 6;
+        if (g != par_grp) {
+          const float4* pp = reinterpret_cast<const float4*>(par0 + (size_t)g * 64);
+          float zmax = 0.f;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          const float4 q4 = __ldg(pp + v);
-          zmax = fmaxf(zmax, fmaxf(fabsf(q4.y), fabsf(q4.w)));
-          s2[v] = pk2(q4.x, q4.z);
-          mz2[v] = pk2(__fadd_rn(magic_val(2 * v), q4.y), __fadd_rn(magic_val(2 * v), q4.w));
+          for (int v = 0; v < 4; ++v) {
+            const float4 q4 = __ldg(pp + v);
+            zmax = fmaxf(zmax, fmaxf(fabsf(q4.y), fabsf(q4.w)));
+            s2[v] = pk2(q4.x, q4.z);
+            mz2[v] = pk2(__fadd_rn(magic_val(2 * v), q4.y), __fadd_rn(magic_val(2 * v), q4.w));
+          }
+          par_plain = !(zmax < kZLimit) || a.force_plain;
+          par_src = reinterpret_cast<const float2*>(pp);
+          par_grp = g;
         }
-        par_plain = !(zmax < kZLimit) || force_plain;
-        par_src = reinterpret_cast<const float2*>(pp);
-        par_grp = g;
+        if (par_plain) dequant8_plain(word[u], par_src, x[u]);
+        else dequant8_magic2(word[u], s2, mz2, x[u]);
+      } else {
+        uint4 fresh = make_uint4(0, 0, 0, 0);
+        if (old[u] == -1)
+          fresh = *reinterpret_cast<const uint4*>(a.kstage + ((size_t)h * a.max_n + (gamma * 64 + kTpt * tq + u - kk)) * 64 + 8 * w);
+        bf16x8_to_float(fresh, x[u]);
       }
-      if (par_plain) dequant8_plain(word[u], par_src, x[u]);
-      else dequant8_magic2(word[u], s2, mz2, x[u]);
+    }
+  }
+  {
+    float mn[8], mx[8];
+    if (old[kTpt - 1] != -2) {        // all tokens there
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        mn[j] = min3(x[0][j], x[1][j], fminf(x[2][j], x[3][j]));
+        mx[j] = max3(x[0][j], x[1][j], fmaxf(x[2][j], x[3][j]));
+      }
     } else {
-      bf16x8_to_float(fresh[u], x[u]);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { mn[j] = INFINITY; mx[j] = -INFINITY; }
+#pragma unroll
+      for (int u = 0; u < kTpt - 1; ++u) {
+        if (old[u] != -2) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) { mn[j] = fminf(mn[j], x[u][j]); mx[j] = fmaxf(mx[j], x[u][j]); }
+        }
+      }
     }
-  }
-  float mn[8], mx[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) { mn[j] = INFINITY; mx[j] = -INFINITY; }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    if (old[u] != -2) {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { mn[j] = fminf(mn[j], x[u][j]); mx[j] = fmaxf(mx[j], x[u][j]); }
+    for (int k = 0; k < 2; ++k) {
+      *reinterpret_cast<float4*>(&s_mn[tq][32 * k + 4 * w]) = make_float4(mn[4 * k], mn[4 * k + 1], mn[4 * k + 2], mn[4 * k + 3]);
+      *reinterpret_cast<float4*>(&s_mx[tq][32 * k + 4 * w]) = make_float4(mx[4 * k], mx[4 * k + 1], mx[4 * k + 2], mx[4 * k + 3]);
     }
-  }
-  // tokens of a warp: lanes with equal (lane & 7) hold the same channels
-#pragma unroll
-  for (int o = 8; o < 32; o <<= 1) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      mn[j] = fminf(mn[j], __shfl_xor_sync(0xffffffffu, mn[j], o));
-      mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], o));
-    }
-  }
-  if ((t & 31) < 8) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { s_mn[hl][wih][8 * w + j] = mn[j]; s_mx[hl][wih][8 * w + j] = mx[j]; }
   }
   __syncthreads();
   // one thread per channel finishes the reduction and derives the group's parameters
-  int slow = force_plain;
-  if (t < 64) {
-    float lo = s_mn[hl][0][t], up = s_mx[hl][0][t];
+  int slow = a.force_plain;
+  if (tid < 64) {
+    float lo = s_mn[0][tid], up = s_mx[0][tid];
 #pragma unroll
-    for (int r = 1; r < 4; ++r) { lo = fminf(lo, s_mn[hl][r][t]); up = fmaxf(up, s_mx[hl][r][t]); }
+    for (int r = 1; r < kRgLanes; ++r) { lo = fminf(lo, s_mn[r][tid]); up = fmaxf(up, s_mx[r][tid]); }
     float sc, inv, z;
     quant_params(lo, up, sc, inv, z);
-    s_iz[hl][t] = make_float2(inv, z);
-    if (head_ok) {
-      dst.kpar[dgrp + t] = make_float2(sc, z);
-      if (two) dst2.kpar[dgrp + t] = make_float2(sc, z);
+    const int ch = ((tid >> 2) & 7) * 8 + (tid >> 5) * 4 + (tid & 3);
+    s_iz[(((ch & 7) >> 1) * 8 + (ch >> 3)) * 2 + (ch & 1)] = make_float2(inv, __int_as_float((int)z - (int)0x4B400000));
+    s_z[ch] = z;
+    {
+      a.dst.kpar[dgrp + ch] = make_float2(sc, z);
+      if (a.two) a.src.kpar[dgrp + ch] = make_float2(sc, z);
       // the conversion-free quantiser needs |x * inv| < 2^21 and |z| < 2^22
       const float ymax = __fmul_rn(fmaxf(fabsf(lo), fabsf(up)), inv);
       slow |= !(ymax < 2097152.f) || !(fabsf(z) < kZLimit);
     }
   }
   slow = __syncthreads_or(slow);
-  if (!head_ok) return;
-  float2 iz[8];
+  float inv[8];
   int zadj[8];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    const float4 q4 = *reinterpret_cast<const float4*>(&s_iz[(8 * v + w) * 2]);
+    inv[2 * v] = q4.x; inv[2 * v + 1] = q4.z;
+    zadj[2 * v] = __float_as_int(q4.y); zadj[2 * v + 1] = __float_as_int(q4.w);
+  }
   uint64_t inv2[4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    iz[j] = s_iz[hl][8 * w + j];
-    zadj[j] = slow ? 0 : (int)iz[j].y - (int)0x4B400000;
-  }
+  for (int p = 0; p < 4; ++p) inv2[p] = pk2(inv[2 * p], inv[2 * p + 1]);
 #pragma unroll
-  for (int p = 0; p < 4; ++p) inv2[p] = pk2(iz[2 * p].x, iz[2 * p + 1].x);
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
+  for (int u = 0; u < kTpt; ++u) {
     if (old[u] == -2) continue;
-    uint32_t packed;
+    uint32_t packed = 0u;
     if (slow) {
-      packed = 0u;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) packed |= quant_code_call(x[u][j], iz[j].x, iz[j].y) << nib_shift(j);
+      for (int j = 0; j < 8; ++j) packed |= quant_code_call(x[u][j], inv[j], s_z[8 * w + j]) << nib_shift(j);
     } else {
-      packed = 0u;
 #pragma unroll
       for (int p = 0; p < 4; ++p) {
         // x * inv for two channels at once; the addition of 1.5 * 2^23 stays scalar: a packed
@@ -1251,9 +1257,8 @@ __global__ void __launch_bounds__(128 * kRgHeads, 2) regroup_k_kernel(const __gr
         packed = (uint32_t)qo * (1u << nib_shift(2 * p + 1)) + packed;
       }
     }
-    const size_t dslot = (size_t)h * cap + base_slot + gamma * 64 + tq + 16 * u;
-    *reinterpret_cast<uint32_t*>(dst.k + dslot * 32 + 4 * w) = packed;
-    if (two) *reinterpret_cast<uint32_t*>(dst2.k + dslot * 32 + 4 * w) = packed;
+    *reinterpret_cast<uint32_t*>(a.dst.k + drow + 32 * u) = packed;
+    if (a.two) *reinterpret_cast<uint32_t*>(a.src.k + drow + 32 * u) = packed;
   }
 }
 
@@ -1402,9 +1407,9 @@ static cudaError_t launch_regroup_n(xkv_cache* const* c, const MaintArgs* a, int
     const int g = (a[i].r_new + 63) / 64;
     if (g > groups) groups = g;
   }
-  const dim3 grid(groups, (a[0].H + kRgHeads - 1) / kRgHeads, count);
+  const dim3 grid(groups, a[0].H, count);
   LaunchScope ls(c[0], XKV_PROF_PACK, st);
-  regroup_k_kernel<MAX><<<grid, 128 * kRgHeads, 0, st>>>(b, a[0].H);
+  regroup_k_kernel<MAX><<<grid, kRgThreads, 0, st>>>(b);
   return cudaGetLastError();
 }
 
