@@ -504,16 +504,17 @@ namespace {
 struct HostStepPipe {
   bool ready = false;
   cudaStream_t up = nullptr, down = nullptr;      // host -> device, device -> host
-  cudaStream_t up2 = nullptr;                     // a second host -> device stream (two copy engines: 49 GB/s against
-                                                  // 31 GB/s for 2.8 MB copies on one stream)
-  cudaEvent_t up2_done[2] = {nullptr, nullptr};
+  cudaStream_t up2 = nullptr, up3 = nullptr;      // more host -> device streams (two copy engines: 49 GB/s against
+                                                  // 31 GB/s for 2.8 MB copies on one): keys, values, queries
+  cudaEvent_t up2_done = nullptr, up3_done = nullptr;
   cudaStream_t side = nullptr;                    // head means of the keys, beside the attention
   bool side_busy = false;                         // started there and not yet ordered before the caller's stream
   cudaEvent_t fork = nullptr, join = nullptr;
   cudaEvent_t start = nullptr;                    // the caller's stream at entry
-  cudaEvent_t up_done[2] = {nullptr, nullptr};    // inputs of the layer in slot s are on the device
-  cudaEvent_t comp_done[2] = {nullptr, nullptr};  // the layer in slot s has run: inputs free, output ready
-  cudaEvent_t down_done[2] = {nullptr, nullptr};  // output of slot s is in host memory: output buffer free
+  cudaEvent_t up_done = nullptr;                  // inputs of a group of layers are on the device
+  cudaEvent_t kv_free[2] = {nullptr, nullptr};    // keys and values of a half of the staging buffer have been taken
+  cudaEvent_t comp_done = nullptr;                // a group has run: outputs ready
+  cudaEvent_t down_done[2] = {nullptr, nullptr};  // outputs are in host memory: their buffers (the queries') free
 };
 std::mutex g_pipe_mutex;
 HostStepPipe g_pipe[64];
@@ -527,14 +528,17 @@ HostStepPipe* host_step_pipe() {
     bool ok = cudaStreamCreateWithFlags(&p.up, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.down, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.up2, cudaStreamNonBlocking) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&p.up3, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.side, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&p.join, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming) == cudaSuccess;
+              cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p.up_done, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p.up2_done, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p.up3_done, cudaEventDisableTiming) == cudaSuccess &&
+              cudaEventCreateWithFlags(&p.comp_done, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; i < 2 && ok; ++i)
-      ok = cudaEventCreateWithFlags(&p.up_done[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&p.up2_done[i], cudaEventDisableTiming) == cudaSuccess &&
-           cudaEventCreateWithFlags(&p.comp_done[i], cudaEventDisableTiming) == cudaSuccess &&
+      ok = cudaEventCreateWithFlags(&p.kv_free[i], cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&p.down_done[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) return nullptr;
     p.ready = true;
@@ -575,17 +579,26 @@ int prepare_layer(xkv_cache* c, const void* q, const void* k, const void* v, voi
   return XKV_OK;
 }
 
+// Caches that one launch of each kernel can take together.
+bool same_form(const xkv_cache* a, const xkv_cache* b) {
+  return a->p.kv_bits == b->p.kv_bits && a->p.key_mode == b->p.key_mode && a->p.n_heads == b->p.n_heads &&
+         a->tail_mode == b->tail_mode && a->attn_max_blocks == b->attn_max_blocks;
+}
+
 struct Range { uintptr_t lo, hi; };
 bool overlap(const Range& x, const Range& y) { return x.lo < y.hi && y.lo < x.hi; }
 
 // One frame through `count` layers whose work does not depend on one another (one launch each of the
 // maintenance, the key regroup and the attention for all of them), then, on the library's side stream
 // beside the attention, the head means of the keys of the caches just built (Eq. 4), from which the
-// next frame's scoring starts.
+// next frame's scoring starts.  kv_taken: recorded once k and v have been read (not with the tail).
 int run_layers(HostStepPipe* pipe, xkv_cache* const* cs, MaintArgs* as, int count, const void* const* q, const void* const* k,
-               const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st) {
+               const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st,
+               const cudaEvent_t* kv_taken = nullptr, int n_taken = 0) {
   const bool once = keys_once(cs[0]);
   if (launch_maint(cs, as, count, XKV_PROF_MAINT, st) != cudaSuccess) return XKV_E_CUDA;
+  for (int i = 0; i < n_taken; ++i)
+    if (cudaEventRecord(kv_taken[i], st) != cudaSuccess) return XKV_E_CUDA;
   if (cs[0]->p.kv_bits == 4 && !once && launch_regroup(cs, as, count, st) != cudaSuccess) return XKV_E_CUDA;
   xkv_cache* kc[kMaxLayers];
   AttnCall calls[kMaxLayers];
@@ -665,10 +678,7 @@ int xkv_stream_step(xkv_cache* const* layers, int32_t n_layers, const void* cons
         const size_t span = ((size_t)(c->p.n_heads - 1) * (size_t)hs + (size_t)(n - 1) * (size_t)ts + kHeadDim) * sizeof(__nv_bfloat16);
         auto range = [&](const void* p) { const uintptr_t b = reinterpret_cast<uintptr_t>(p); return Range{b, b + span}; };
         rq[count] = range(q[l]); rk[count] = range(k[l]); rv[count] = range(v[l]); ro[count] = range(out[l]);
-        const xkv_cache* lead = layers[l0];
-        bool together = count == 0 || (c->p.kv_bits == lead->p.kv_bits && c->p.key_mode == lead->p.key_mode &&
-                                       c->p.n_heads == lead->p.n_heads && c->tail_mode == lead->tail_mode &&
-                                       c->attn_max_blocks == lead->attn_max_blocks);
+        bool together = count == 0 || same_form(c, layers[l0]);
         for (int i = 0; i < count && together; ++i)
           together = layers[l0 + i] != c && !overlap(ro[i], rq[count]) && !overlap(ro[i], rk[count]) && !overlap(ro[i], rv[count]) &&
                      !overlap(ro[i], ro[count]) && !overlap(ro[count], rq[i]) &&
@@ -696,8 +706,19 @@ size_t xkv_stream_step_host_bytes(const xkv_params* params, int32_t n) {
   return 2 * 4 * ((t + kAlign - 1) / kAlign * kAlign);
 }
 
-// The layers run on the caller's stream; the inputs of layer l + 1 are copied to the other half of
-// the staging buffer on a copy stream while layer l runs, and outputs go back on a third stream.
+// Cached tokens from which the kernels of a layer take about as long as the copies of its inputs (the
+// ratio does not depend on the frame size): with shorter caches the copies are the limit, and a layer
+// at a time leaves no gap between them (24 x 1374 tokens at 4096: 4.49 ms, in pairs 4.70).
+constexpr int kPairTokens = 10240;
+
+// The layers run on the caller's stream, two at a time where the caches are long (the first and the
+// last alone, so that the copies before and after all work are short).  The staging buffer is eight
+// tensors: keys and values of two layers, which are free again once the maintenance has read them, and twice the queries of two
+// layers, over which the outputs are written (a block reads an item's queries before it writes them,
+// and the merge comes after all).  So the copies of the next two layers' inputs run beside the
+// attention of these two, and their outputs go back beside the next two layers.  One layer at a time
+// took 5.74 ms for a frame of 24 layers of 1374 tokens: beside copies every short kernel is half as
+// fast, and two layers' maintenance costs little more than one's.
 int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void* const* q,
                          const void* const* k, const void* const* v, void* const* out, int32_t n,
                          void* dev_staging, size_t staging_bytes, xkv_stream stream) {
@@ -721,46 +742,65 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
   ck(cudaEventRecord(pipe->start, st));
   ck(cudaStreamWaitEvent(pipe->up, pipe->start, 0));
   ck(cudaStreamWaitEvent(pipe->up2, pipe->start, 0));
+  ck(cudaStreamWaitEvent(pipe->up3, pipe->start, 0));
   ck(cudaStreamWaitEvent(pipe->down, pipe->start, 0));
-  int l = 0;
-  for (; l < n_layers && cuda_ok && rc == XKV_OK; ++l) {
-    xkv_cache* c = layers[l];
-    const int sl = l & 1;
-    uint8_t* s = base + (size_t)sl * 4 * slot;
-    void* dq = s;
-    void* dk = s + slot;
-    void* dv = s + 2 * slot;
-    void* dout = s + 3 * slot;
-    // inputs: once the layer that used this half two layers ago has run
-    if (l >= 2) {
-      ck(cudaStreamWaitEvent(pipe->up, pipe->comp_done[sl], 0));
-      ck(cudaStreamWaitEvent(pipe->up2, pipe->comp_done[sl], 0));
+  bool kv_used[2] = {false, false}, qo_used[2] = {false, false};      // halves of the staging buffer in use before
+  for (int l = 0, group = 0; l < n_layers && cuda_ok && rc == XKV_OK; ++group) {
+    int count = 1;
+    if (l > 0 && l + 2 < n_layers && !layers[l]->tail_mode && layers[l]->T >= kPairTokens && layers[l] != layers[l + 1] &&
+        same_form(layers[l], layers[l + 1]))
+      count = 2;
+    const int par = group & 1;
+    void *dq[2], *dk[2], *dv[2];
+    int half[2];
+    for (int i = 0; i < count; ++i) {
+      half[i] = (count == 2) ? i : par;
+      dk[i] = base + (size_t)(2 * half[i]) * slot;
+      dv[i] = base + (size_t)(2 * half[i] + 1) * slot;
+      dq[i] = base + (size_t)(4 + 2 * par + i) * slot;
+      if (kv_used[half[i]]) {
+        ck(cudaStreamWaitEvent(pipe->up, pipe->kv_free[half[i]], 0));
+        ck(cudaStreamWaitEvent(pipe->up2, pipe->kv_free[half[i]], 0));
+      }
+      ck(cudaMemcpyAsync(dk[i], k[l + i], t, cudaMemcpyHostToDevice, pipe->up));
+      ck(cudaMemcpyAsync(dv[i], v[l + i], t, cudaMemcpyHostToDevice, pipe->up2));
     }
-    ck(cudaMemcpyAsync(dk, k[l], t, cudaMemcpyHostToDevice, pipe->up));
-    ck(cudaMemcpyAsync(dq, q[l], t, cudaMemcpyHostToDevice, pipe->up2));
-    ck(cudaMemcpyAsync(dv, v[l], t, cudaMemcpyHostToDevice, pipe->up));
-    ck(cudaEventRecord(pipe->up_done[sl], pipe->up));
-    ck(cudaEventRecord(pipe->up2_done[sl], pipe->up2));
-    // the layer: inputs present, and the output of two layers ago copied out of this half
-    ck(cudaStreamWaitEvent(st, pipe->up_done[sl], 0));
-    ck(cudaStreamWaitEvent(st, pipe->up2_done[sl], 0));
-    if (l >= 2) ck(cudaStreamWaitEvent(st, pipe->down_done[sl], 0));
+    if (qo_used[par]) ck(cudaStreamWaitEvent(pipe->up3, pipe->down_done[par], 0));
+    for (int i = 0; i < count; ++i) ck(cudaMemcpyAsync(dq[i], q[l + i], t, cudaMemcpyHostToDevice, pipe->up3));
+    ck(cudaEventRecord(pipe->up_done, pipe->up));
+    ck(cudaEventRecord(pipe->up2_done, pipe->up2));
+    ck(cudaEventRecord(pipe->up3_done, pipe->up3));
+    ck(cudaStreamWaitEvent(st, pipe->up3_done, 0));
+    ck(cudaStreamWaitEvent(st, pipe->up_done, 0));
+    ck(cudaStreamWaitEvent(st, pipe->up2_done, 0));
     if (!cuda_ok) break;
-    MaintArgs a;
-    const void* cq = dq; const void* ck_ = dk; const void* cv = dv;
-    rc = prepare_layer(c, dq, dk, dv, dout, n, ts, hs, &a);
-    if (rc == XKV_OK) rc = run_layers(pipe, &c, &a, 1, &cq, &ck_, &cv, &dout, n, ts, hs, st);
-    ck(cudaEventRecord(pipe->comp_done[sl], st));
-    if (rc != XKV_OK) break;
-    // output
-    ck(cudaStreamWaitEvent(pipe->down, pipe->comp_done[sl], 0));
-    ck(cudaMemcpyAsync(out[l], dout, t, cudaMemcpyDeviceToHost, pipe->down));
-    ck(cudaEventRecord(pipe->down_done[sl], pipe->down));
+    MaintArgs as[2];
+    int ready = 0;
+    for (; ready < count && rc == XKV_OK; ++ready) {
+      rc = prepare_layer(layers[l + ready], dq[ready], dk[ready], dv[ready], dq[ready], n, ts, hs, &as[ready]);
+      if (rc != XKV_OK) break;
+    }
+    if (ready > 0) {
+      const bool tail = layers[l]->tail_mode != 0;
+      const int e = run_layers(pipe, layers + l, as, ready, dq, dk, dv, dq, n, ts, hs, st, &pipe->kv_free[half[0]],
+                               tail ? 0 : count);
+      if (e != XKV_OK) rc = e;
+      if (tail) ck(cudaEventRecord(pipe->kv_free[half[0]], st));
+      for (int i = 0; i < ready; ++i) kv_used[half[i]] = true;
+    }
+    if (rc != XKV_OK && ready == 0) break;
+    ck(cudaEventRecord(pipe->comp_done, st));
+    ck(cudaStreamWaitEvent(pipe->down, pipe->comp_done, 0));
+    for (int i = 0; i < ready; ++i) ck(cudaMemcpyAsync(out[l + i], dq[i], t, cudaMemcpyDeviceToHost, pipe->down));
+    ck(cudaEventRecord(pipe->down_done[par], pipe->down));
+    qo_used[par] = true;
+    l += count;
   }
   // everything started above ends before the call returns, also after an error
   if (!join_side_work(pipe, st)) cuda_ok = false;
   ck(cudaStreamSynchronize(pipe->up));
   ck(cudaStreamSynchronize(pipe->up2));
+  ck(cudaStreamSynchronize(pipe->up3));
   ck(cudaStreamSynchronize(st));
   ck(cudaStreamSynchronize(pipe->down));
   if (rc != XKV_OK) return rc;
