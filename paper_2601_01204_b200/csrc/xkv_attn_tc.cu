@@ -247,6 +247,7 @@ __device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t v) {
 // descheduled for a while (a GPU shared between processes) does not time out on the clock alone.
 constexpr uint64_t kWaitLimitNs = 1000000000ull;      // one second ...
 constexpr uint32_t kWaitMinRounds = 1u << 12;         // ... and this many rounds, then XKV_E_TIMEOUT
+constexpr int kSlack = 1000;     // sleep of the producers and the copy thread (256: 16-bit at 32768 tokens 6440 instead of 6290 us)
 template <int SLEEP_NS = 32>
 __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& wc) {
   if (mbar_try(bar, parity)) return;          // the common case costs one instruction
@@ -362,6 +363,14 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b_d
       "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"                       \
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
         "r"(r[7]) : "memory")
+
+#define XKV_TMEM_ST16(taddr, r)                                                                      \
+  asm volatile(                                                                                      \
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "                                                \
+      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"                                    \
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
+        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), \
+        "r"(r[15]) : "memory")
 
 // Shared-memory matrix descriptor, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
@@ -526,7 +535,7 @@ __device__ __forceinline__ void once_keys(const uint8_t* codes, const uint8_t* r
   WORD wd[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const WORD*>(codes + (k0 + i) * (8 * sizeof(WORD)) + w * sizeof(WORD));
-  mbar_wait<256>(b_free, parity, wc);
+  mbar_wait<kSlack>(b_free, parity, wc);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     if (i > 0 && ref[i] != ref[i - 1]) fetch(ref[i]);
@@ -736,28 +745,29 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const uint64_t nm2 = pack_f2(-m_ref, -m_ref);
         // (P goes over scores of both halves; the exchange above has made sure that both hold theirs)
         const uint32_t colP = colP0 + 128 * (cnt & 1);
-        // exponentials of 16 columns against the reference; P (16-bit pairs) -> TMEM
-        auto chunk16 = [&](const uint32_t* rr, int c) {
-          uint64_t x[8];
+        // Exponentials against the reference; P (16-bit pairs) -> TMEM.  32 columns at a time, or 16 where
+        // the producers fetch constants per token (24 layers at 16384: 4-bit 3157 -> 3100 us with 32, keys
+        // quantised once 3693 -> 3727).
+        auto columns = [&](const uint32_t* rr, uint32_t* pk, int pairs) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            x[i] = fma_f2(pack_f2(__uint_as_float(rr[2 * i]), __uint_as_float(rr[2 * i + 1])), sc2, nm2);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) x[i] = pack_f2(fast_exp2(f2_lo(x[i])), fast_exp2(f2_hi(x[i])));
-          uint32_t pk[8];
-#pragma unroll
-          for (int i = 0; i < 8; i += 2) {
-            l2 = add_f2(l2, x[i]);
-            l2b = add_f2(l2b, x[i + 1]);
-            pk[i] = kBf16 ? pack_bf2(f2_lo(x[i]), f2_hi(x[i])) : pack_h2(f2_lo(x[i]), f2_hi(x[i]));
-            pk[i + 1] = kBf16 ? pack_bf2(f2_lo(x[i + 1]), f2_hi(x[i + 1])) : pack_h2(f2_lo(x[i + 1]), f2_hi(x[i + 1]));
+          for (int i = 0; i < pairs; ++i) {
+            const uint64_t x = fma_f2(pack_f2(__uint_as_float(rr[2 * i]), __uint_as_float(rr[2 * i + 1])), sc2, nm2);
+            const float e0 = fast_exp2(f2_lo(x)), e1 = fast_exp2(f2_hi(x));
+            if (i & 1) l2b = add_f2(l2b, pack_f2(e0, e1)); else l2 = add_f2(l2, pack_f2(e0, e1));
+            pk[i] = kBf16 ? pack_bf2(e0, e1) : pack_h2(e0, e1);
           }
-          XKV_TMEM_ST8(colP + 8 * c, pk);
         };
-        chunk16(ra, 0);
-        chunk16(ra + 16, 1);
-        chunk16(rb, 2);
-        chunk16(rb + 16, 3);
+        if (ONCE) {
+          uint32_t pk[8];
+          columns(ra, pk, 8);      XKV_TMEM_ST8(colP, pk);
+          columns(ra + 16, pk, 8); XKV_TMEM_ST8(colP + 8, pk);
+          columns(rb, pk, 8);      XKV_TMEM_ST8(colP + 16, pk);
+          columns(rb + 16, pk, 8); XKV_TMEM_ST8(colP + 24, pk);
+        } else {
+          uint32_t pk[16];
+          columns(ra, pk, 16); XKV_TMEM_ST16(colP, pk);
+          columns(rb, pk, 16); XKV_TMEM_ST16(colP + 16, pk);
+        }
         if (jj > 0 && __any_sync(0xffffffffu, grow)) {
           // the accumulator is quiescent once the previous step's PV has completed
           mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);
@@ -825,7 +835,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const uint32_t kbuf = g % kNK, ku = g / kNK;
         const uint32_t vbuf = g % kNV, vu = g / kNV;
         const uint8_t* raw = sgen + kOffRaw + rs * C::kRawStage;
-        mbar_wait<256>(b_rfull + 8 * rs, ru & 1, wc);
+        mbar_wait<kSlack>(b_rfull + 8 * rs, ru & 1, wc);
         if (TAIL && BITS == 4 && (tile_lo + jj) * 128 >= job.tail_lo && (tile_lo + jj) * 128 + 127 < job.t_phys) {
           // ---- a tile that lies in the unquantised frame as a whole: K~ and V~ are the caller's
           // bf16 rows converted to fp16, the packed codes of the stage are not looked at ----
@@ -836,8 +846,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             uint4 u[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) u[i] = *reinterpret_cast<const uint4*>(src + (int64_t)(16 * i) * a.ts);
-            if (kv == 0) mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
-            else mbar_wait<256>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
+            if (kv == 0) mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
+            else mbar_wait<kSlack>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
             uint8_t* dst = sgen + (kv ? kOffV + vbuf * 16384 : kOffK + kbuf * 16384) + row_off;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -884,7 +894,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           } else {
 #pragma unroll
           for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const uint32_t*>(raw + (kb + 16 * i) * 32 + 4 * w);
-          mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
+          mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
 #pragma unroll
           for (int grp = 0; grp < 2; ++grp) {
             const uint4 sv = *reinterpret_cast<const uint4*>(tab + grp * 128 + 16 * w);
@@ -907,7 +917,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           // ---- values ----
 #pragma unroll
           for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const uint32_t*>(raw + C::kRawK + (kb + 16 * i) * 32 + 4 * w);
-          mbar_wait<256>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
+          mbar_wait<kSlack>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const uint4 pv = *reinterpret_cast<const uint4*>(tab + 768 + 16 * (kb + 16 * i));
@@ -942,7 +952,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           mbar_arrive(b_kfull + 8 * kbuf);
 #pragma unroll
           for (int i = 0; i < 8; ++i) wd8[i] = *reinterpret_cast<const uint2*>(raw + C::kRawK + (kb + 16 * i) * 64 + 8 * w);
-          mbar_wait<256>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
+          mbar_wait<kSlack>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const uint4 pv = *reinterpret_cast<const uint4*>(tab + 768 + 16 * (kb + 16 * i));
@@ -958,7 +968,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           uint4 rowk[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) rowk[i] = *reinterpret_cast<const uint4*>(raw + (kb + 16 * i) * 128 + 16 * w);
-          mbar_wait<256>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
+          mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + i * 2048) = rowk[i];
@@ -966,7 +976,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           mbar_arrive(b_kfull + 8 * kbuf);
 #pragma unroll
           for (int i = 0; i < 8; ++i) rowk[i] = *reinterpret_cast<const uint4*>(raw + C::kRawK + (kb + 16 * i) * 128 + 16 * w);
-          mbar_wait<256>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
+          mbar_wait<kSlack>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             *reinterpret_cast<uint4*>(sgen + kOffV + vbuf * 16384 + row_off + i * 2048) = rowk[i];
@@ -1056,7 +1066,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       for (int jj = 0; jj < nt; ++jj, ++g) {
         const int tile = tile_lo + jj;
         const uint32_t rs = g % C::kNR, ru = g / C::kNR;
-        mbar_wait<256>(b_rfree + 8 * rs, (ru & 1) ^ 1, wc);
+        mbar_wait<kSlack>(b_rfree + 8 * rs, (ru & 1) ^ 1, wc);
         const uint32_t dst = sRaw + rs * C::kRawStage, bar = b_rfull + 8 * rs;
         const uint32_t kp_bytes = ONCE ? 512u : (uint32_t)C::kRawKP;    // 128 group references instead of 2 x 64 parameters
         mbar_expect_tx(bar, C::kRawStage - C::kRawKP + kp_bytes);
