@@ -693,6 +693,40 @@ __device__ __forceinline__ void phase_kbar_new_once(const MaintArgs& a, const Bl
   }
 }
 
+// The survivor gathers.  Tile = (head, kMT / PIECES consecutive survivors), thread = (survivor,
+// 16-byte piece ch of PIECES): one division per tile and thread, where an index of (head, survivor,
+// piece) split by 64-bit divisions cost more than the copies.  Several tiles are in flight per thread: the kept
+// indices, then the rows, then the stores.
+template <int PIECES>
+struct GatherTiles {
+  static constexpr int kTokens = kMT / PIECES;
+  int ch, tok, per_head, count;
+  __device__ __forceinline__ GatherTiles(const MaintArgs& a, const Blocks&) {
+    ch = (int)threadIdx.x % PIECES;
+    tok = (int)threadIdx.x / PIECES;
+    per_head = (a.kk + kTokens - 1) / kTokens;
+    count = a.H * per_head;
+  }
+  // slots that this thread's survivor of a tile comes from and goes to; false if there is none
+  __device__ __forceinline__ bool rows(const MaintArgs& a, int tile, size_t* from, size_t* to) const {
+    const int h = tile / per_head, i = (tile - h * per_head) * kTokens + tok;
+    const bool ok = tile < count && i < a.kk;
+    const int old = (ok && !a.identity) ? __ldcg(&a.kept[i]) : i;
+    const size_t base = (size_t)h * a.cap + a.rest_base;
+    *from = base + old;
+    *to = base + i;
+    return ok;
+  }
+};
+// Origins (and, quantise-once mode, group references) of the survivors.
+__device__ __forceinline__ void gather_origins(const MaintArgs& a, const Blocks& B) {
+  for (int i = B.index * kMT + (int)threadIdx.x; i < a.kk; i += B.count * kMT) {
+    const int old = a.identity ? i : __ldcg(&a.kept[i]);
+    a.oth.origin[a.rest_base + i] = a.cur.origin[a.rest_base + old];
+    if (a.cur.kslot) a.oth.kslot[a.rest_base + i] = a.cur.kslot[a.rest_base + old];
+  }
+}
+
 // Quantise-once mode, PACK: the survivors' key and value code rows, value parameters, group
 // references, origins and head means move to their new places in the other buffer set.
 template <int BITS>
@@ -713,35 +747,28 @@ __device__ __forceinline__ void phase_gather_once(const MaintArgs& a, const Bloc
     }
     return;
   }
-  // four items per thread and pass: the kept indices, then the rows, then the stores
-  const long long items = (long long)a.H * a.kk * (2 * kRC);         // (head, survivor, 16-byte chunk of K | V codes)
-  for (long long g0 = first; g0 < items; g0 += 4 * stride) {
-    int old[4]; size_t so[4], dd[4]; int chn[4]; bool ok[4];
+  const GatherTiles<2 * kRC> tiles(a, B);                            // the 16-byte pieces of K codes, then of V codes
+  constexpr int kU = 4;
+  const int piece = 16 * (tiles.ch % kRC);
+  const uint8_t* from_base = (tiles.ch < kRC ? src.k : src.v) + piece;
+  uint8_t* to_base = (tiles.ch < kRC ? dst.k : dst.v) + piece;
+  for (int t0 = B.index; t0 < tiles.count; t0 += kU * B.count) {
+    size_t from[kU], to[kU];
+    bool ok[kU];
+    uint4 row[kU];
+    float2 vp[kU];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const long long g = g0 + u * stride;
-      ok[u] = g < items;
-      chn[u] = (int)(g % (2 * kRC));
-      const long long r = ok[u] ? (g / (2 * kRC)) : 0;
-      const int i = (int)(r % a.kk), h = (int)(r / a.kk);
-      old[u] = kept ? __ldcg(&kept[i]) : i;
-      dd[u] = (size_t)h * a.cap + a.rest_base + i;
-      so[u] = (size_t)h * a.cap + a.rest_base;
-    }
-    uint4 row[4]; float2 vp[4];
+    for (int u = 0; u < kU; ++u) ok[u] = tiles.rows(a, t0 + u * B.count, &from[u], &to[u]);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const size_t s = so[u] + old[u];
-      const uint8_t* base = chn[u] < kRC ? src.k : src.v;
-      row[u] = ok[u] ? *reinterpret_cast<const uint4*>(base + s * kRow + 16 * (chn[u] % kRC)) : make_uint4(0, 0, 0, 0);
-      vp[u] = (ok[u] && chn[u] == kRC) ? src.vpar[s] : make_float2(0.f, 0.f);
+    for (int u = 0; u < kU; ++u) {
+      row[u] = ok[u] ? *reinterpret_cast<const uint4*>(from_base + from[u] * kRow) : make_uint4(0, 0, 0, 0);
+      vp[u] = (ok[u] && tiles.ch == kRC) ? src.vpar[from[u]] : make_float2(0.f, 0.f);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kU; ++u) {
       if (!ok[u]) continue;
-      uint8_t* base = chn[u] < kRC ? dst.k : dst.v;
-      *reinterpret_cast<uint4*>(base + dd[u] * kRow + 16 * (chn[u] % kRC)) = row[u];
-      if (chn[u] == kRC) dst.vpar[dd[u]] = vp[u];
+      *reinterpret_cast<uint4*>(to_base + to[u] * kRow) = row[u];
+      if (tiles.ch == kRC) dst.vpar[to[u]] = vp[u];
     }
   }
   const long long rows = (long long)a.kk * 16;                       // (survivor, 16-byte chunk of its head-mean row)
@@ -753,24 +780,17 @@ __device__ __forceinline__ void phase_gather_once(const MaintArgs& a, const Bloc
       ok[u] = g < rows;
       old[u] = ok[u] ? (kept ? __ldcg(&kept[(int)(g >> 4)]) : (int)(g >> 4)) : 0;
     }
-    float4 row[4]; int org[4], ks[4];
+    float4 row[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      row[u] = ok[u] ? __ldcg(reinterpret_cast<const float4*>(src.kbar + (size_t)old[u] * 64) + ((g0 + u * stride) & 15)) : make_float4(0, 0, 0, 0);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const long long g = g0 + u * stride;
-      const int ch = (int)(g & 15);
-      row[u] = ok[u] ? __ldcg(reinterpret_cast<const float4*>(src.kbar + (size_t)old[u] * 64) + ch) : make_float4(0, 0, 0, 0);
-      org[u] = (ok[u] && ch == 0) ? src.origin[a.rest_base + old[u]] : 0;
-      ks[u] = (ok[u] && ch == 0) ? src.kslot[a.rest_base + old[u]] : 0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const long long g = g0 + u * stride;
-      if (!ok[u]) continue;
-      const int ch = (int)(g & 15), i = (int)(g >> 4);
-      reinterpret_cast<float4*>(dst.kbar + (size_t)i * 64)[ch] = row[u];
-      if (ch == 0) { dst.origin[a.rest_base + i] = org[u]; dst.kslot[a.rest_base + i] = ks[u]; }
+      if (ok[u]) reinterpret_cast<float4*>(dst.kbar + (size_t)(g >> 4) * 64)[g & 15] = row[u];
     }
   }
+  gather_origins(a, B);
 }
 
 // ---------------------------------------------------------------------------
@@ -1270,20 +1290,30 @@ __global__ void __launch_bounds__(kRgThreads, 8) regroup_k_kernel(const __grid_c
 __device__ __forceinline__ void phase_gather16(const MaintArgs& a, const Blocks& B) {
   const BufSet& src = a.cur;
   const BufSet& dst = a.oth;
-  const int32_t* kept = a.identity ? nullptr : a.kept;
-  const long long items = (long long)a.H * a.kk * 8;
-  for (long long g = (long long)B.index * kMT + threadIdx.x; g < items; g += (long long)B.count * kMT) {
-    const int ch = (int)(g & 7);
-    const long long r = g >> 3;
-    const int i = (int)(r % a.kk);
-    const int h = (int)(r / a.kk);
-    const int old = kept ? __ldcg(&kept[i]) : i;
-    const size_t s = (size_t)h * a.cap + a.rest_base + old;
-    const size_t d = (size_t)h * a.cap + a.rest_base + i;
-    *reinterpret_cast<uint4*>(dst.v + d * 128 + 16 * ch) = *reinterpret_cast<const uint4*>(src.v + s * 128 + 16 * ch);
-    *reinterpret_cast<uint4*>(dst.k + d * 128 + 16 * ch) = *reinterpret_cast<const uint4*>(src.k + s * 128 + 16 * ch);
-    if (h == 0 && ch == 0) dst.origin[a.rest_base + i] = src.origin[a.rest_base + old];
+  const GatherTiles<8> tiles(a, B);
+  constexpr int kU = 3;
+  for (int t0 = B.index; t0 < tiles.count; t0 += kU * B.count) {
+    size_t from[kU], to[kU];
+    bool ok[kU];
+    uint4 k[kU], v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) ok[u] = tiles.rows(a, t0 + u * B.count, &from[u], &to[u]);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      k[u] = v[u] = make_uint4(0, 0, 0, 0);
+      if (ok[u]) {
+        k[u] = *reinterpret_cast<const uint4*>(src.k + from[u] * 128 + 16 * tiles.ch);
+        v[u] = *reinterpret_cast<const uint4*>(src.v + from[u] * 128 + 16 * tiles.ch);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      if (!ok[u]) continue;
+      *reinterpret_cast<uint4*>(dst.k + to[u] * 128 + 16 * tiles.ch) = k[u];
+      *reinterpret_cast<uint4*>(dst.v + to[u] * 128 + 16 * tiles.ch) = v[u];
+    }
   }
+  gather_origins(a, B);
 }
 
 }  // namespace
