@@ -618,6 +618,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_dependency_wait();        // the cache and the queries (all of the above ran beside the kernel before)
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   {
@@ -1116,6 +1117,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
 attn_combine_kernel(const __grid_constant__ Args a) {
+  grid_dependency_wait();
   const int cut = (int)(blockIdx.x >> 3) + 1, t = (int)(blockIdx.x >> 2) & 1;
   const int r = (int)(blockIdx.x & 3) * 32 + (int)(threadIdx.x >> 3), ch = (int)(threadIdx.x & 7);
   const uint32_t at = piece_start(a, cut), before = piece_start(a, cut - 1);
@@ -1270,19 +1272,23 @@ static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail,
   {
     LaunchScope ls(c, XKV_PROF_ATTN, st);
     const bool once = c->p.key_mode == XKV_KEYS_ONCE;
-    const int g = (int)grid;
-    if (c->p.kv_bits == 16) attn_tc_kernel<16><<<g, kThreads, smem_bytes<16>(), st>>>(a);
-    else if (c->p.kv_bits == 8) attn_tc_kernel<8, false, true><<<g, kThreads, smem_bytes<8>(), st>>>(a);
-    else if (tail && once) attn_tc_kernel<4, true, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
-    else if (tail) attn_tc_kernel<4, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
-    else if (once) attn_tc_kernel<4, false, true><<<g, kThreads, smem_bytes<4>(), st>>>(a);
-    else attn_tc_kernel<4><<<g, kThreads, smem_bytes<4>(), st>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    const void* fn;
+    int smem = smem_bytes<4>();
+    if (c->p.kv_bits == 16) { fn = (const void*)attn_tc_kernel<16>; smem = smem_bytes<16>(); }
+    else if (c->p.kv_bits == 8) { fn = (const void*)attn_tc_kernel<8, false, true>; smem = smem_bytes<8>(); }
+    else if (tail && once) fn = (const void*)attn_tc_kernel<4, true, true>;
+    else if (tail) fn = (const void*)attn_tc_kernel<4, true>;
+    else if (once) fn = (const void*)attn_tc_kernel<4, false, true>;
+    else fn = (const void*)attn_tc_kernel<4>;
+    void* params[1] = {(void*)&a};
+    const cudaError_t e = launch_overlapped(fn, dim3((unsigned)grid), dim3(kThreads), params, (size_t)smem, st);
     if (e != cudaSuccess) return e;
   }
   if (grid > 1) {
     LaunchScope ls(c, XKV_PROF_COMBINE, st);
-    attn_combine_kernel<<<(int)(grid - 1) * 8, 256, 0, st>>>(a);
+    void* params[1] = {(void*)&a};
+    const cudaError_t e = launch_overlapped((const void*)attn_combine_kernel, dim3((unsigned)(grid - 1) * 8), dim3(256), params, 0, st);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }

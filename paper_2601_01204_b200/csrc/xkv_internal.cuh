@@ -166,6 +166,28 @@ struct LaunchScope {
   }
 };
 
+#ifdef __CUDACC__
+// Kernels of a stream overlap at their ends (programmatic dependent launch): a kernel launched with
+// launch_overlapped may be set up while its predecessor still runs, and every such kernel waits, first of all,
+// until the predecessor has completed and its writes are visible.  Without the trigger a
+// predecessor lets its successor start when it ends.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
+inline cudaError_t launch_overlapped(const void* fn, dim3 grid, dim3 block, void** params, size_t smem, cudaStream_t st) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, fn, params);
+}
+
 // ---- launchers implemented in the kernel translation units -------------------
 // All return cudaError_t of the launch (cudaGetLastError) and count launches.
 

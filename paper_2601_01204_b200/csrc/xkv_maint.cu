@@ -260,8 +260,8 @@ struct Blocks { int index, count; };
 __device__ __forceinline__ bool grid_barrier(const MaintArgs& a, const Blocks& B, uint32_t& epoch, Shared& sh) {
   __syncthreads();
   if (threadIdx.x == 0 && !sh.abort_flag) {
-    __threadfence();
-    atomicAdd(a.bar, 1u);
+    // (release and acquire by this thread cover the block: the barriers around order the others)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.bar) : "memory");
     const uint32_t target = a.bar_base + (epoch + 1u) * (uint32_t)B.count;
     uint32_t it = 0;
     while ((int)(ld_acquire_u32(a.bar) - target) < 0) {
@@ -270,9 +270,8 @@ __device__ __forceinline__ bool grid_barrier(const MaintArgs& a, const Blocks& B
         atomicExch(a.status, (int)XKV_E_TIMEOUT);
         break;
       }
-      __nanosleep(40);
+      __nanosleep(20);
     }
-    __threadfence();
   }
   ++epoch;
   __syncthreads();
@@ -1082,6 +1081,8 @@ template <int MAX> struct RegroupBatch { RegroupArgs layer[MAX]; };
 // heads a block 436, two heads 396, one head 369 us (small blocks wait for less at their barriers).
 template <int MAX>
 __global__ void __launch_bounds__(kRgThreads, 8) regroup_k_kernel(const __grid_constant__ RegroupBatch<MAX> batch) {
+  grid_dependency_trigger();
+  grid_dependency_wait();
   const RegroupArgs& a = batch.layer[MAX == 1 ? 0 : blockIdx.z];
   if ((int)blockIdx.x * 64 >= a.r_new) return;
   const int cap = a.cap, base_slot = a.base_slot, kk = a.kk, r_new = a.r_new;
@@ -1331,6 +1332,7 @@ __global__ void __launch_bounds__(kMT, kBlocksPerSM) maint_kernel(const __grid_c
   __shared__ Shared sh;
   if (threadIdx.x == 0) { sh.abort_flag = 0; sh.acc = 0u; sh.bin = 0u; sh.need = 0u; sh.fsum[0] = sh.fsum[1] = 0.f; }
   __syncthreads();
+  grid_dependency_wait();
   const int which = (MAX == 1) ? 0 : (int)blockIdx.x % batch.n;
   const Blocks B{(MAX == 1) ? (int)blockIdx.x : (int)blockIdx.x / batch.n,
                  (MAX == 1) ? (int)gridDim.x : ((int)gridDim.x - which + batch.n - 1) / batch.n};
@@ -1439,12 +1441,33 @@ static cudaError_t launch_regroup_n(xkv_cache* const* c, const MaintArgs* a, int
   }
   const dim3 grid(groups, a[0].H, count);
   LaunchScope ls(c[0], XKV_PROF_PACK, st);
-  regroup_k_kernel<MAX><<<grid, kRgThreads, 0, st>>>(b);
-  return cudaGetLastError();
+  void* params[1] = {(void*)&b};
+  const cudaError_t e = launch_overlapped((const void*)regroup_k_kernel<MAX>, grid, dim3(kRgThreads), params, 0, st);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_regroup(xkv_cache* const* c, const MaintArgs* a, int count, cudaStream_t st) {
   return count == 1 ? launch_regroup_n<1>(c, a, 1, st) : launch_regroup_n<kMaxLayers>(c, a, count, st);
+}
+
+// Blocks that have something to do in the busiest phase of a layer (what runs between two barriers
+// counts together).  A layer of 261 tokens fills 87 of 296; the others would only make its barriers
+// longer.
+static int useful_blocks(const xkv_cache* c, const MaintArgs& a) {
+  long long first = 0, later = 1;
+  auto ceil_div = [](long long x, long long y) { return (x + y - 1) / y; };
+  if (a.phases & kPhAppend) first += ceil_div((long long)a.H * a.n * 8, kMT);
+  if ((a.phases & kPhAppend) && c->p.key_mode == XKV_KEYS_ONCE) first += ceil_div(a.n, 64) * ceil_div(a.H, 4);
+  if (a.phases & kPhPool) first += a.n_pooled;
+  if (a.phases & kPhKbar) first += ceil_div(a.kbar_hi - a.kbar_lo, 64) + 1;
+  if (a.phases & kPhKbarNew) later = ceil_div(a.n, 64);
+  if ((a.phases & (kPhScore | kPhSel)) && ceil_div(a.r_old, 64) > later) later = ceil_div(a.r_old, 64);
+  if (a.phases & kPhPack) {
+    const long long bytes = (long long)a.H * (a.kk > 0 ? a.kk : a.r_old) * 2 * c->row_bytes;
+    if (ceil_div(bytes, 16 * kMT) > later) later = ceil_div(bytes, 16 * kMT);
+  }
+  const long long n = first > later ? first : later;
+  return n < 65536 ? (int)n : 65536;
 }
 
 template <int MAX>
@@ -1455,6 +1478,12 @@ static cudaError_t launch_maint_n(xkv_cache* const* c, MaintArgs* as, int count,
   MaintBatch<MAX> batch;
   batch.n = count;
   bool barriers = false;
+  int useful = 1;
+  for (int i = 0; i < count; ++i) {
+    const int u = useful_blocks(c[i], as[i]);
+    if (u > useful) useful = u;
+  }
+  if ((long long)useful * count < grid) grid = useful * count;
   for (int i = 0; i < count; ++i) {
     MaintArgs& a = as[i];
     xkv_cache* ci = c[i];
@@ -1477,7 +1506,7 @@ static cudaError_t launch_maint_n(xkv_cache* const* c, MaintArgs* as, int count,
   void* params[1] = {(void*)&batch};
   const void* fn = maint_fn<MAX>(c[0]->p.kv_bits, c[0]->p.key_mode == XKV_KEYS_ONCE);
   e = barriers ? cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kMT), params, 0, st)
-               : cudaLaunchKernel(fn, dim3(grid), dim3(kMT), params, 0, st);
+               : launch_overlapped(fn, dim3(grid), dim3(kMT), params, 0, st);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
