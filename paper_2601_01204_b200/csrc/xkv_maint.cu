@@ -1347,7 +1347,13 @@ __global__ void __launch_bounds__(kMT, kBlocksPerSM) maint_kernel(const __grid_c
     ran = true;
   }
   if (ph & kPhPool) { phase_pool(a, B, sh); ran = true; }
-  if (ph & kPhKbar) { phase_kbar<BITS>(a, B, sh, a.kbar_on_other ? a.oth : a.cur, a.kbar_lo, a.kbar_hi); ran = true; }
+  if (ph & kPhKbar) {
+    // (from the first block that has no pooled row)
+    const int skip = (ph & kPhPool) ? a.n_pooled % B.count : 0;
+    const Blocks K{B.index >= skip ? B.index - skip : B.index + B.count - skip, B.count};
+    phase_kbar<BITS>(a, K, sh, a.kbar_on_other ? a.oth : a.cur, a.kbar_lo, a.kbar_hi);
+    ran = true;
+  }
 
   if (ph & (kPhScore | kPhKbarNew)) {
     if (ran && !grid_barrier(a, B, epoch, sh)) return;

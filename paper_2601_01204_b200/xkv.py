@@ -143,11 +143,18 @@ def _check(status: int, where: str) -> None:
         raise XkvError(status, where)
 
 
+_current_stream = None
+
+
 def _stream() -> int:
-    import torch
-    if not torch.cuda.is_available():
-        raise RuntimeError("xkv needs a CUDA device; there is no CPU fallback")
-    return torch.cuda.current_stream().cuda_stream
+    # (asking for the device again at every call took as long as a kernel launch)
+    global _current_stream
+    if _current_stream is None:
+        import torch
+        if not torch.cuda.is_available():
+            raise RuntimeError("xkv needs a CUDA device; there is no CPU fallback")
+        _current_stream = torch.cuda.current_stream
+    return _current_stream().cuda_stream
 
 
 def _strides(t) -> tuple[int, int]:
@@ -389,10 +396,7 @@ class Cache:
 
 
 def _ptr_array(tensors) -> "C.Array":
-    arr = (_vp * len(tensors))()
-    for i, t in enumerate(tensors):
-        arr[i] = t if isinstance(t, int) else t.data_ptr()
-    return arr
+    return (_vp * len(tensors))(*[t if isinstance(t, int) else t.data_ptr() for t in tensors])
 
 
 def xkv_stream_step(layers: list[Cache], q: list, k: list, v: list, out: list) -> None:
