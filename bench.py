@@ -27,7 +27,7 @@ WORKLOAD = dict(name="full_stack_24L_1374tok_budget16384_int4", layers=24, n_hea
                 n_tokens=1374, budget=16384, kv_bits=4, n_special=5, pool_g=16, quant_group=64, seed=3)
 METRIC = "stream frames/s (24-layer compressed-KV attention)"
 UNIT = "frames/s"
-# dram__bytes_read.sum + dram__bytes_write.sum of one attention launch, from the ncu capture
+# dram__bytes_read.sum + dram__bytes_write.sum of one attention launch for one layer, from the ncu capture
 # summarised under profiles/ (None until a capture of the current kernel exists).
 ATTN_DRAM_TRAFFIC_BYTES = 23.3e6
 
@@ -319,7 +319,9 @@ def run_xkv(args) -> None:
         peaks = _peaks()
         ms_step = ms_total / K
         attn_ms, attn_cnt = prof.get("attn", (0.0, 0))
-        flops = 4.0 * n * w["budget"] * d * H                     # useful FLOPs of one attention launch
+        # a launch of the stream step serves all layers of a frame (up to 28): its FLOPs and bytes are theirs
+        attn_layers = L * K / max(attn_cnt, 1)
+        flops = 4.0 * n * w["budget"] * d * H * attn_layers       # useful FLOPs of one attention launch
         attn_avg_s = (attn_ms / max(attn_cnt, 1)) * 1e-3
         achieved = flops / attn_avg_s / 1e12 if attn_avg_s > 0 else 0.0
         # the head means run on the library's side stream beside the attention: their event span in
@@ -331,9 +333,9 @@ def run_xkv(args) -> None:
         def entry(ms: float, cnt: int, per: int, key: str | None, **extra) -> dict:
             e = dict(ms_per_step=ms / per, launches_per_step=cnt / per, avg_launch_us=ms / max(cnt, 1) * 1e3, **extra)
             if key in nbytes and ms > 0:
-                sec = ms / cnt * 1e-3
-                e.update(bytes_per_launch=nbytes[key], gb_per_s=nbytes[key] / sec / 1e9,
-                         hbm_frac=nbytes[key] / sec / 1e9 / peaks["hbm_gbs"])
+                sec, moved = ms / cnt * 1e-3, nbytes[key] * L * per / cnt
+                e.update(layers_per_launch=L * per / cnt, bytes_per_launch=moved, gb_per_s=moved / sec / 1e9,
+                         hbm_frac=moved / sec / 1e9 / peaks["hbm_gbs"])
             return e
 
         kernels = {}
@@ -363,8 +365,8 @@ def run_xkv(args) -> None:
                                   peak=peaks["tflops_sustained"], unit="TFLOP/s",
                                   frac=achieved / peaks["tflops_sustained"], peak_source=peaks["source"] + " (sustained)",
                                   frac_of_burst=achieved / peaks["tflops_burst"], flops_per_launch=flops,
-                                  avg_launch_ms=attn_avg_s * 1e3,
-                                  traffic=ATTN_DRAM_TRAFFIC_BYTES if w["name"] == WORKLOAD["name"] else None),
+                                  avg_launch_ms=attn_avg_s * 1e3, layers_per_launch=attn_layers,
+                                  traffic=ATTN_DRAM_TRAFFIC_BYTES * attn_layers if w["name"] == WORKLOAD["name"] else None),
                     kernels=kernels, kernels_per_call=per_call)
         if world == 1 and not args.no_cpu_baseline:
             line["cpu_baseline"] = cpu_baseline(w)
