@@ -45,7 +45,8 @@ namespace {
 
 constexpr int kMaxDevices = 64;
 // Warps: 0-15 softmax, 16-19 producers, 20 and 22 issue the MMAs of query tile 0 resp. 1, 21 issues the
-// copies and owns the tensor memory; 23 only completes the warpgroup that setmaxnreg needs.
+// copies and owns the tensor memory; 23 asks for the key constants ahead of the producers (keys
+// quantised once; else it only completes the warpgroup that setmaxnreg needs).
 constexpr int kThreads = 768;
 // registers per thread after the reallocation (setmaxnreg)
 constexpr int kRegsSoftmax = 96;
@@ -65,6 +66,7 @@ constexpr float kGrow = 14.f;
 // ring depths
 constexpr int kNK = 3;                        // dequantised K~ tiles
 constexpr int kNV = 3;                        // dequantised V~ tiles
+constexpr uint32_t kAhead = 4;        // tiles whose constants are asked for ahead of the producers (keys quantised once)
 
 template <int BITS> struct Cfg;
 template <> struct Cfg<4> {
@@ -594,6 +596,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(sgen + kOffBar + kBarBytes - 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(sgen + kOffBar + kBarBytes - 12);
   const WaitCtx wc{sbase + kOffBar + kBarBytes - 12};
+  const uint32_t s_progress = sbase + kOffBar + kBarBytes - 8;      // tiles that the producers have begun
 
   const int tid = threadIdx.x;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);     // (known to be the same in all lanes)
@@ -601,6 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
 
   if (tid == 0) {
     *abort_flag = (*reinterpret_cast<volatile int*>(a.job[0].status) == (int)XKV_E_TIMEOUT) ? 1 : 0;   // an earlier CTA already gave up
+    st_shared_u32(s_progress, 0u);
     for (int i = 0; i < kNK; ++i) { mbar_init(b_kfull + 8 * i, 128); mbar_init(b_kfree + 8 * i, 2); }
     for (int i = 0; i < kNV; ++i) { mbar_init(b_vfull + 8 * i, 128); mbar_init(b_vfree + 8 * i, 2); }
     for (int i = 0; i < C::kNR; ++i) { mbar_init(b_rfull + 8 * i, 1); mbar_init(b_rfree + 8 * i, 128); }
@@ -838,6 +842,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         const uint32_t kbuf = g % kNK, ku = g / kNK;
         const uint32_t vbuf = g % kNV, vu = g / kNV;
         const uint8_t* raw = sgen + kOffRaw + rs * C::kRawStage;
+        if (ONCE && t == 0) st_shared_u32(s_progress, g + 1);
         mbar_wait<kSlack>(b_rfull + 8 * rs, ru & 1, wc);
         if (TAIL && BITS == 4 && (tile_lo + jj) * 128 >= job.tail_lo && (tile_lo + jj) * 128 + 127 < job.t_phys) {
           // ---- a tile that lies in the unquantised frame as a whole: K~ and V~ are the caller's
@@ -1058,6 +1063,34 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       if (active) ++cq;
     }
     tc_fence_before();
+  } else if (ONCE && warp == kSW + 7) {
+    // =========================== constants, ahead of the producers =============
+    // The constants of a tile's key groups lie anywhere in a table of hundreds of megabytes a layer: a
+    // look-up can miss the L2 and the TLB, and the producers' look-ups depend on one another.  This
+    // warp asks for the lines a few tiles before the producers need them.  (24 layers at 16384, three
+    // streams taking turns: 5216 us a frame without it, 3778 with; 8-bit at 8192 2409 and 1537.)
+    const int lane = tid & 31;
+    uint32_t g = 0;
+    for (Walk walk(a); walk.next(a);) {
+      const Job& job = a.job[walk.job];
+      for (int jj = 0; jj < walk.nt; ++jj, ++g) {
+        for (int it = 0; it < (1 << 16); ++it) {           // (only a pace: nothing depends on it)
+          if (g < ld_shared_u32(s_progress) + kAhead || ld_shared_u32(wc.abort_flag)) break;
+          __nanosleep(500);
+        }
+        const int4 sl = *(reinterpret_cast<const int4*>(job.kslot + (size_t)(walk.tile_lo + jj) * 128) + lane);
+        int before = __shfl_up_sync(0xffffffffu, sl.w, 1);
+        if (lane == 0) before = -1;
+        auto ask = [&](int slot, int prev) {
+          if (slot == prev) return;
+          const uint8_t* e = reinterpret_cast<const uint8_t*>(job.ktab16 + ((size_t)slot * job.n_heads + walk.h) * 96);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) asm volatile("prefetch.global.L2 [%0];" ::"l"(e + min(128 * i, 383)));
+        };
+        ask(sl.x, before); ask(sl.y, sl.x); ask(sl.z, sl.y); ask(sl.w, sl.z);
+        __syncwarp();
+      }
+    }
   } else if (tid == 32 * (kSW + 5)) {
     // =========================== TMA loader ===================================
     uint32_t g = 0;
