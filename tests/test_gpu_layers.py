@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2601_01204_b200 import synth
-from xkv_testlib import bf16_tensor_to_f32, check_attention, compare_state, oracle_params, to_device_bf16
+from xkv_testlib import ATTN_MAXABS, ATTN_RELL2, attn_errors, bf16_tensor_to_f32, check_attention, compare_state, oracle_params, to_device_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -121,3 +121,37 @@ def test_chunk_of_more_frames_than_a_launch_takes(xkv):
         ref = ora.step_chunk(*(np.split(synth.bf16_bits_to_f32(b), cuts, axis=1) for b in bits))
         check_attention(bf16_tensor_to_f32(got).transpose(1, 0, 2), np.concatenate(ref), f"chunk {t}")
         compare_state(cache.export(), ora.export(), f"chunk {t}")
+
+
+@pytest.mark.parametrize("layers, n, budget, bits, once, tail", [
+    (5, 1500, 10500, 4, 0, False),       # one layer, two, one, one
+    (4, 1400, 10300, 16, 0, False),      # one, two, one
+    (6, 1400, 10300, 4, 1, False),
+    (4, 1400, 10300, 4, 0, True),        # the tail needs keys and values to the end: one at a time
+    (5, 130, 300, 4, 0, False),          # short caches: one at a time
+])
+def test_host_buffer_step_in_pairs(xkv, layers, n, budget, bits, once, tail):
+    """Caches long enough that the host-buffer step takes two layers at a time, with its outputs over
+    the queries in the staging buffer, against the step on device tensors."""
+    import torch
+    p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=bits, key_mode=once)
+    host, dev = ([xkv.Cache(p) for _ in range(layers)] for _ in range(2))
+    for c in host + dev:
+        c.xkv_set_unquantised_tail(tail)
+    staging = torch.empty(xkv.xkv_stream_step_host_bytes(p, n), dtype=torch.uint8, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    for t in range(budget // n + 3):
+        q, k, v = ([torch.randn(H, n, D, device="cuda", dtype=torch.bfloat16, generator=gen) for _ in range(layers)] for _ in range(3))
+        out = [torch.empty_like(x) for x in q]
+        xkv.xkv_stream_step(dev, q, k, v, out)
+        hq, hk, hv = ([x.cpu().pin_memory() for x in xs] for xs in (q, k, v))
+        ho = [torch.zeros(H, n, D, dtype=torch.bfloat16).pin_memory() for _ in range(layers)]
+        xkv.xkv_stream_step_host(host, hq, hk, hv, ho, staging)
+        for l in range(layers):
+            # Both are within the tolerance of the exact result, so within twice of it of each other
+            # (16-bit caches round P to bf16 against reference maxima that differ with the cuts).
+            maxabs, rell2 = attn_errors(ho[l].float().numpy(), bf16_tensor_to_f32(out[l]))
+            assert maxabs <= 2 * ATTN_MAXABS and rell2 <= 2 * ATTN_RELL2, (t, l, maxabs, rell2)
+    for l in range(layers):
+        compare_state(host[l].export(), dev[l].export(), f"layer {l}")
+    assert all(c.xkv_poll_status() == 0 for c in host + dev)
