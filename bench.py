@@ -436,7 +436,8 @@ def maintenance_bytes(H: int, n: int, d: int, budget: int, bits: int, key_mode: 
     what it reads plus what it writes, every array once.  prunable = budget - n middle tokens are
     scored, k = budget - 2 n of them survive, n new tokens arrive.  Keys are the profile categories:
     the per-call launches (append, score_evict, pack), the head means (kbar) and the stream step's
-    single launch (maint = append + pooled query + scores + selection + pack)."""
+    single launch (maint = append + pooled query + scores + selection; with keys quantised once it
+    moves the survivors too, while regrouped keys have the pack launch to themselves)."""
     if bits != 4:
         return {}
     row, code, par = d * 2, d // 2, 8                      # bf16 row, packed row, one (scale, zero) pair
@@ -458,7 +459,7 @@ def maintenance_bytes(H: int, n: int, d: int, budget: int, bits: int, key_mode: 
         return {"append": append, "score_evict": pool + score + select, "pack": pack,
                 "maint": append + pool + score + select + pack}
     return {"append": append, "score_evict": pool + kbar + score + select, "pack": pack, "kbar": kbar,
-            "maint": append + pool + score + select + pack}
+            "maint": append + pool + score + select}
 
 
 def main() -> None:
