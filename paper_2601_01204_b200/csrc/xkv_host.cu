@@ -565,7 +565,8 @@ int prepare_layer(xkv_cache* c, const void* q, const void* k, const void* v, voi
   if ((c->p.kv_bits == 16 && c->kk_pending > 0) || (once && (c->kk_pending > 0 || c->rold_pending > 0))) a->phases |= kPhPack;
   if (selecting(c)) {
     // (the head means: those of the last step were computed beside its attention, and its caller's
-    // stream has waited for them; in quantise-once mode they travel with the tokens)
+    // stream has waited for them, as run_layers does for those of this call; in quantise-once mode they
+    // travel with the tokens)
     a->phases |= kPhPool | kPhScore | kPhSel;
     if (!once && !kbar_fresh(c)) {
       a->phases |= kPhKbar;
@@ -588,14 +589,26 @@ bool same_form(const xkv_cache* a, const xkv_cache* b) {
 struct Range { uintptr_t lo, hi; };
 bool overlap(const Range& x, const Range& y) { return x.lo < y.hi && y.lo < x.hi; }
 
-// One frame through `count` layers whose work does not depend on one another (one launch each of the
-// maintenance, the key regroup and the attention for all of them), then, on the library's side stream
-// beside the attention, the head means of the keys of the caches just built (Eq. 4), from which the
-// next frame's scoring starts.  kv_taken: recorded once k and v have been read (not with the tail).
-int run_layers(HostStepPipe* pipe, xkv_cache* const* cs, MaintArgs* as, int count, const void* const* q, const void* const* k,
-               const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st,
+// One frame through the `count` layers from layers[from] on, whose work does not depend on one another (one
+// launch each of the maintenance, the key regroup and the attention for all of them), then, on the
+// library's side stream beside the attention, the head means of the keys of the caches just built
+// (Eq. 4), from which the next frame's scoring starts.  The caller's stream waits for those only at the
+// end of the call, so a cache that has come before in it waits for its own here: its scoring reads
+// them, and with keys quantised once its gather moves them.
+// kv_taken: recorded once k and v have been read (not with the tail).
+int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs* as, int count, const void* const* q,
+               const void* const* k, const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st,
                const cudaEvent_t* kv_taken = nullptr, int n_taken = 0) {
+  xkv_cache* const* cs = layers + from;
   const bool once = keys_once(cs[0]);
+  for (int i = 0; i < count; ++i) {
+    const bool started = cs[i]->kbar_frames == cs[i]->frames;
+    for (int l = 0; started && l < from; ++l) {
+      if (layers[l] != cs[i]) continue;
+      if (cudaStreamWaitEvent(st, cs[i]->kbar_done, 0) != cudaSuccess) return XKV_E_CUDA;
+      break;
+    }
+  }
   if (launch_maint(cs, as, count, XKV_PROF_MAINT, st) != cudaSuccess) return XKV_E_CUDA;
   for (int i = 0; i < n_taken; ++i)
     if (cudaEventRecord(kv_taken[i], st) != cudaSuccess) return XKV_E_CUDA;
@@ -690,7 +703,7 @@ int xkv_stream_step(xkv_cache* const* layers, int32_t n_layers, const void* cons
       ++count;
     }
     if (count > 0) {
-      const int e = run_layers(pipe, layers + l0, as, count, q + l0, k + l0, v + l0, out + l0, n, ts, hs, st);
+      const int e = run_layers(pipe, layers, l0, as, count, q + l0, k + l0, v + l0, out + l0, n, ts, hs, st);
       if (e != XKV_OK) rc = e;
     }
     l0 += count;
@@ -782,7 +795,7 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
     }
     if (ready > 0) {
       const bool tail = layers[l]->tail_mode != 0;
-      const int e = run_layers(pipe, layers + l, as, ready, dq, dk, dv, dq, n, ts, hs, st, &pipe->kv_free[half[0]],
+      const int e = run_layers(pipe, layers, l, as, ready, dq, dk, dv, dq, n, ts, hs, st, &pipe->kv_free[half[0]],
                                tail ? 0 : count);
       if (e != XKV_OK) rc = e;
       if (tail) ck(cudaEventRecord(pipe->kv_free[half[0]], st));
