@@ -847,6 +847,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         if (TAIL && BITS == 4 && (tile_lo + jj) * 128 >= job.tail_lo && (tile_lo + jj) * 128 + 127 < job.t_phys) {
           // ---- a tile that lies in the unquantised frame as a whole: K~ and V~ are the caller's
           // bf16 rows converted to fp16, the packed codes of the stage are not looked at ----
+          // (The parameter tables take turns by step.  A table is filled again once all producers have
+          // passed the step between, which must therefore make them meet although it fills no table.)
+          producer_sync();
           bool bad = false;
 #pragma unroll
           for (int kv = 0; kv < 2; ++kv) {

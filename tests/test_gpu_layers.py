@@ -155,3 +155,30 @@ def test_host_buffer_step_in_pairs(xkv, layers, n, budget, bits, once, tail):
     for l in range(layers):
         compare_state(host[l].export(), dev[l].export(), f"layer {l}")
     assert all(c.xkv_poll_status() == 0 for c in host + dev)
+
+
+@pytest.mark.parametrize("once", [0, 1])
+def test_one_key_tile_inside_the_unquantised_frame(xkv, once):
+    """The newest frame starts inside a key tile, covers the next one and ends inside the one after: only
+    the outer two go through the producers' parameter tables.  Against the oracle, then the same launch
+    again and again, bit for bit."""
+    import torch
+    from oracle import xkv_oracle as xo
+    heads, n, budget = 16, 261, 1500                      # slots 1362 .. 1622: tiles 10 (from 1280), 11, 12
+    p = xkv.Params(n_heads=heads, budget=budget, max_frame_tokens=n, kv_bits=4, key_mode=once)
+    cache, ora = xkv.Cache(p), xo.OracleLayer(oracle_params(p))
+    for t in range(budget // n + 3):
+        bits = synth.gen_frame(17, 0, t, heads, n, D)
+        q, k, v = (to_device_bf16(b) for b in bits)
+        qf, kf, vf = (synth.bf16_bits_to_f32(b) for b in bits)
+        got = per_call(cache, q, k, v, True)
+        ora.append(kf, vf), ora.score_evict(qf), ora.quant_pack()
+        ref = ora.attend(qf, full_precision_tail=True)
+        check_attention(bf16_tensor_to_f32(got).transpose(1, 0, 2), ref, f"frame {t}")
+    info = cache.xkv_get_info()
+    assert (info.T_phys - n) % 128 and info.T_phys % 128 and info.T_phys // 128 - (info.T_phys - n) // 128 == 2
+    first = got.clone()
+    for rep in range(40):
+        cache.xkv_debug_rewind_attention()
+        assert torch.equal(cache.attn_packed_causal_tail(q, k, v, got).view(torch.int16), first.view(torch.int16)), rep
+    assert cache.xkv_poll_status() == 0
