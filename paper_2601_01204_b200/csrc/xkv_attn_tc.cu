@@ -32,7 +32,7 @@
 // 16-bit caches hold bf16 and multiply in bf16.  Accumulation is fp32.
 //
 // Every mbarrier wait is bounded (one second of running time): when the bound is hit the CTA carries on
-// without waiting and records XKV_E_TIMEOUT in the status words of the caches of the launch, so the
+// without waiting and records XKV_E_TIMEOUT in the status words of the caches in its piece, so the
 // kernel always terminates, drains its copies and frees its tensor memory.
 #include <mutex>
 #include <stdlib.h>
@@ -232,7 +232,7 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 // Bounded wait.  On exhaustion a per-CTA flag goes up, and every later wait of the CTA gives up at
-// once; at its end the CTA records the failure in the status words of the launch's caches.
+// once; at its end the CTA records the failure in the status words of the caches that it worked on.
 struct WaitCtx { uint32_t abort_flag; };      // address in shared memory
 __device__ __forceinline__ uint32_t ld_shared_u32(uint32_t addr) {
   uint32_t v;
@@ -271,9 +271,11 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, const W
   } while (++rounds < kWaitMinRounds || global_ns() - t0 < kWaitLimitNs);
   st_shared_u32(wc.abort_flag, 1u);
 }
-// A wait of the CTA ran out: the results of every cache in the launch are void.
+// A wait of the CTA ran out: the results of the caches with steps in its piece are void.
 __device__ __forceinline__ void report_timeout(const Args& a) {
-  for (int j = 0; j < a.n_jobs; ++j) atomicExch(a.job[j].status, (int)XKV_E_TIMEOUT);
+  const uint32_t lo = piece_start(a, blockIdx.x), hi = piece_start(a, blockIdx.x + 1);
+  for (int j = 0; j < a.n_jobs; ++j)
+    if (a.job[j].step_lo < hi && a.job[j].step_hi > lo) atomicExch(a.job[j].status, (int)XKV_E_TIMEOUT);
 }
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;
@@ -603,7 +605,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   constexpr bool kBf16 = (BITS == 16);
 
   if (tid == 0) {
-    *abort_flag = (*reinterpret_cast<volatile int*>(a.job[0].status) == (int)XKV_E_TIMEOUT) ? 1 : 0;   // an earlier CTA already gave up
+    *abort_flag = 0;           // (the status words are older launches' too: they say nothing about this one)
     st_shared_u32(s_progress, 0u);
     for (int i = 0; i < kNK; ++i) { mbar_init(b_kfull + 8 * i, 128); mbar_init(b_kfree + 8 * i, 2); }
     for (int i = 0; i < kNV; ++i) { mbar_init(b_vfull + 8 * i, 128); mbar_init(b_vfree + 8 * i, 2); }
@@ -1424,6 +1426,10 @@ __global__ void __launch_bounds__(32) timeout_probe_kernel(const __grid_constant
 cudaError_t launch_timeout_probe(xkv_cache* c, cudaStream_t st) {
   Args a;
   a.n_jobs = 1;
+  a.piece = 1;                       // one step, all of it this cache's
+  a.longer = 0;
+  a.job[0].step_lo = 0;
+  a.job[0].step_hi = 1;
   a.job[0].status = c->status;
   timeout_probe_kernel<<<1, 32, 0, st>>>(a);
   c->launches++;

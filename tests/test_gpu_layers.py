@@ -182,3 +182,24 @@ def test_one_key_tile_inside_the_unquantised_frame(xkv, once):
         cache.xkv_debug_rewind_attention()
         assert torch.equal(cache.attn_packed_causal_tail(q, k, v, got).view(torch.int16), first.view(torch.int16)), rep
     assert cache.xkv_poll_status() == 0
+
+
+@pytest.mark.parametrize("failed", [0, 2])
+def test_a_failed_cache_does_not_touch_the_others_of_its_launch(xkv, failed):
+    """A cache whose status word holds a time-out from before: the layers that share its launches keep
+    their results and their status."""
+    import torch
+    layers, n, budget = 4, 200, 512
+    p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=4)
+    together, alone = ([xkv.Cache(p) for _ in range(layers)] for _ in range(2))
+    together[failed].xkv_debug_timeout_probe()
+    assert together[failed].xkv_poll_status() == xkv.XKV_E_TIMEOUT
+    for t in range(4):
+        q, k, v = zip(*(frame(l, t, n) for l in range(layers)))
+        out = [torch.empty_like(x) for x in q]
+        xkv.xkv_stream_step(together, q, k, v, out)
+        for l in range(layers):
+            ref = per_call(alone[l], q[l], k[l], v[l], False)
+            check_attention(bf16_tensor_to_f32(out[l]), bf16_tensor_to_f32(ref), f"frame {t} layer {l}")
+            compare_state(together[l].export(), alone[l].export(), f"frame {t} layer {l}")
+    assert [c.xkv_poll_status() for c in together] == [xkv.XKV_E_TIMEOUT if l == failed else 0 for l in range(layers)]
