@@ -601,18 +601,23 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
                const cudaEvent_t* kv_taken = nullptr, int n_taken = 0) {
   xkv_cache* const* cs = layers + from;
   const bool once = keys_once(cs[0]);
+  // after a failed call the caches take no further frame (only xkv_reset goes on)
+  auto fail = [&](int stage) {
+    for (int i = 0; i < count; ++i) cs[i]->stage = stage;
+    return XKV_E_CUDA;
+  };
   for (int i = 0; i < count; ++i) {
     const bool started = cs[i]->kbar_frames == cs[i]->frames;
     for (int l = 0; started && l < from; ++l) {
       if (layers[l] != cs[i]) continue;
-      if (cudaStreamWaitEvent(st, cs[i]->kbar_done, 0) != cudaSuccess) return XKV_E_CUDA;
+      if (cudaStreamWaitEvent(st, cs[i]->kbar_done, 0) != cudaSuccess) return fail(1);
       break;
     }
   }
-  if (launch_maint(cs, as, count, XKV_PROF_MAINT, st) != cudaSuccess) return XKV_E_CUDA;
+  if (launch_maint(cs, as, count, XKV_PROF_MAINT, st) != cudaSuccess) return fail(1);
   for (int i = 0; i < n_taken; ++i)
-    if (cudaEventRecord(kv_taken[i], st) != cudaSuccess) return XKV_E_CUDA;
-  if (cs[0]->p.kv_bits == 4 && !once && launch_regroup(cs, as, count, st) != cudaSuccess) return XKV_E_CUDA;
+    if (cudaEventRecord(kv_taken[i], st) != cudaSuccess) return fail(1);
+  if (cs[0]->p.kv_bits == 4 && !once && launch_regroup(cs, as, count, st) != cudaSuccess) return fail(2);
   xkv_cache* kc[kMaxLayers];
   AttnCall calls[kMaxLayers];
   int n_kbar = 0;
@@ -641,20 +646,20 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
   // been enqueued, so that the attention's blocks get the multiprocessors first and the head means
   // fill in as they retire.
   if (n_kbar && !(cudaEventRecord(pipe->fork, st) == cudaSuccess && cudaStreamWaitEvent(pipe->side, pipe->fork, 0) == cudaSuccess))
-    return XKV_E_CUDA;
+    return fail(3);
   const cudaError_t e = launch_attn_tc(calls, count, ts, hs, 1.0f / sqrtf((float)cs[0]->p.head_dim), st);
   if (e != cudaSuccess) {
-    for (int i = 0; i < count; ++i) cs[i]->stage = 3;
+    fail(3);
     return e == cudaErrorNotSupported ? XKV_E_UNSUPPORTED : XKV_E_CUDA;
   }
   if (n_kbar) {
     bool ok = launch_maint(kc, as, n_kbar, XKV_PROF_KBAR, pipe->side) == cudaSuccess;
-    for (int i = 0; i < n_kbar; ++i) {
-      ok = cudaEventRecord(kc[i]->kbar_done, pipe->side) == cudaSuccess && ok;
-      kc[i]->kbar_T = kc[i]->T; kc[i]->kbar_cur = kc[i]->cur; kc[i]->kbar_frames = kc[i]->frames;
-    }
+    for (int i = 0; i < n_kbar; ++i) ok = cudaEventRecord(kc[i]->kbar_done, pipe->side) == cudaSuccess && ok;
     pipe->side_busy = true;
-    if (!ok) return XKV_E_CUDA;
+    // (means that were never computed don't pass for those of this frame: the next scoring computes them
+    // anew, except with keys quantised once, where they travel with the tokens)
+    if (!ok) return once ? fail(3) : XKV_E_CUDA;
+    for (int i = 0; i < n_kbar; ++i) { kc[i]->kbar_T = kc[i]->T; kc[i]->kbar_cur = kc[i]->cur; kc[i]->kbar_frames = kc[i]->frames; }
   }
   return XKV_OK;
 }

@@ -31,6 +31,7 @@ std::map<const void*, Event> g_events;
 std::vector<Op> g_ops;
 std::string g_report;
 std::string g_fail_name;       // the next operation of this name fails
+std::map<const void*, int> g_means_of;     // head-mean array -> frame of the cache that it was computed for
 int g_epoch = 0;
 uintptr_t g_handles = 0x1000;
 
@@ -96,7 +97,7 @@ XKV_API int fake_ops(const char* name) {
   return n;
 }
 XKV_API void fake_fail_next(const char* name) { g_fail_name = name; }
-XKV_API void fake_clear() { g_report.clear(); g_ops.clear(); g_fail_name.clear(); }
+XKV_API void fake_clear() { g_report.clear(); g_ops.clear(); g_fail_name.clear(); }   // (the clocks go on)
 // From here on a wait on an event that was recorded before is an error, as inside a stream capture.
 XKV_API void fake_begin_capture() { ++g_epoch; }
 
@@ -185,7 +186,11 @@ cudaError_t launch_maint(xkv_cache* const* cs, MaintArgs* as, int count, int cat
       b.reads(a.ktab32, table, "key table");
       head_means(b, c, a.oth, true);
     }
-    if (a.phases & kPhScore) { head_means(b, c, a.cur, false); b.writes(a.scores, 4, "scores"); }
+    if (a.phases & kPhScore) {
+      if (!once && !(a.phases & kPhKbar) && g_means_of[a.cur.kbar] != c->frames) note("scores from head means of another frame");
+      head_means(b, c, a.cur, false);
+      b.writes(a.scores, 4, "scores");
+    }
     if (a.phases & kPhSel) b.writes(a.kept, 4, "kept positions");
     if (a.phases & kPhPack) {
       buffers(b, c, a.cur, false);
@@ -193,7 +198,10 @@ cudaError_t launch_maint(xkv_cache* const* cs, MaintArgs* as, int count, int cat
       if (once) { head_means(b, c, a.cur, false); head_means(b, c, a.oth, true); }
     }
   }
-  return b.run();
+  const cudaError_t e = b.run();
+  for (int i = 0; i < count && e == cudaSuccess; ++i)
+    if (as[i].phases & kPhKbar) g_means_of[as[i].cur.kbar] = cs[i]->frames;
+  return e;
 }
 cudaError_t launch_regroup(xkv_cache* const* cs, const MaintArgs* as, int count, cudaStream_t st) {
   Builder b("regroup", st);

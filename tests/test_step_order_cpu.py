@@ -114,3 +114,24 @@ def test_captured_steps_wait_on_nothing_from_before(lib):
         lib.fake_begin_capture()
         assert s.step([0, 1]) == 0
         assert s.races() == "", form
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("launch", [b"maintenance", b"regroup", b"attention", b"head means"])
+@pytest.mark.parametrize("form", FORMS)
+def test_a_launch_that_fails(lib, form, launch, host):
+    """The caches of a failed launch take no further frame before a reset.  Without their head means, which
+    only the next frame needs, regrouped and 16-bit caches go on and compute them anew."""
+    s = Stack(lib, 2, 1000, 200, **form)
+    for _ in range(7):
+        assert s.step([0, 1], host) == 0
+    if launch == b"regroup" and (form["bits"] != 4 or form["once"]):
+        return
+    lib.fake_fail_next(launch)
+    assert s.step([0, 1], host) == s.xkv.XKV_E_CUDA
+    goes_on = launch == b"head means" and not form["once"]
+    status = s.step([0], host)
+    assert status == (0 if goes_on else s.xkv.XKV_E_STATE)
+    assert lib.xkv_reset(s.caches[0], None) == 0
+    assert s.step([0], host) == 0
+    assert s.races() == ""
