@@ -554,6 +554,7 @@ int prepare_layer(xkv_cache* c, const void* q, const void* k, const void* v, voi
   if (c->stage != 0) return XKV_E_STATE;
   if (n < 1 || n > c->p.max_frame_tokens || !aligned16(k) || !aligned16(v) || !aligned16(q) || !aligned16(out) || !strides_ok(ts, hs))
     return XKV_E_INVALID;
+  if (c->tail_mode && c->p.kv_bits == 8) return XKV_E_UNSUPPORTED;      // (the tail is built for 4-bit and 16-bit caches)
   FramePlan plan;
   const int rc = plan_frame(c, n, &plan);
   if (rc != XKV_OK) return rc;

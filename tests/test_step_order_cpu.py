@@ -102,7 +102,6 @@ def test_steps_of_different_layers_are_ordered(lib, form, host):
         s = Stack(lib, layers, budget, n, **form)
         for _ in range(budget // n + 3 if layers == 6 else 6):
             assert s.step(range(layers), host) == 0
-            s.lib.fake_ops(b"copy")
         assert s.races() == "", (layers, budget, n)
 
 
@@ -134,4 +133,18 @@ def test_a_launch_that_fails(lib, form, launch, host):
     assert status == (0 if goes_on else s.xkv.XKV_E_STATE)
     assert lib.xkv_reset(s.caches[0], None) == 0
     assert s.step([0], host) == 0
+    assert s.races() == ""
+
+
+@pytest.mark.parametrize("host", [False, True])
+def test_a_step_that_is_not_supported_leaves_the_caches_alone(lib, host):
+    """The unquantised tail is not built for 8-bit codes: refused before anything is launched, for every
+    layer that would have shared the launch."""
+    s = Stack(lib, 3, 1000, 200, bits=8, once=1, tail=1)
+    assert s.step([0, 1, 2], host) == s.xkv.XKV_E_UNSUPPORTED
+    assert [(s.info(i).frames, s.info(i).stage) for i in range(3)] == [(0, 0)] * 3
+    assert lib.fake_ops(b"maintenance") == 0
+    for c in s.caches:
+        lib.xkv_set_unquantised_tail(c, 0)
+    assert s.step([0, 1, 2], host) == 0
     assert s.races() == ""
