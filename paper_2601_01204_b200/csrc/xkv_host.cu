@@ -508,8 +508,6 @@ struct HostStepPipe {
                                                   // 31 GB/s for 2.8 MB copies on one): keys, values, queries
   cudaEvent_t up2_done = nullptr, up3_done = nullptr;
   cudaStream_t side = nullptr;                    // head means of the keys, beside the attention
-  bool side_busy = false;                         // started there and not yet ordered before the caller's stream
-  cudaEvent_t fork = nullptr, join = nullptr;
   cudaEvent_t start = nullptr;                    // the caller's stream at entry
   cudaEvent_t up_done = nullptr;                  // inputs of a group of layers are on the device
   cudaEvent_t kv_free[2] = {nullptr, nullptr};    // keys and values of a half of the staging buffer have been taken
@@ -530,8 +528,6 @@ HostStepPipe* host_step_pipe() {
               cudaStreamCreateWithFlags(&p.up2, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.up3, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.side, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&p.fork, cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&p.join, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&p.start, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&p.up_done, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&p.up2_done, cudaEventDisableTiming) == cudaSuccess &&
@@ -595,11 +591,11 @@ bool overlap(const Range& x, const Range& y) { return x.lo < y.hi && y.lo < x.hi
 // library's side stream beside the attention, the head means of the keys of the caches just built
 // (Eq. 4), from which the next frame's scoring starts.  The caller's stream waits for those only at the
 // end of the call, so a cache that has come before in it waits for its own here: its scoring reads
-// them, and with keys quantised once its gather moves them.
-// kv_taken: recorded once k and v have been read (not with the tail).
+// them, and with keys quantised once its gather moves them.  *last_means: the cache whose head means
+// the call started last, if any.  kv_taken: recorded once k and v have been read (not with the tail).
 int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs* as, int count, const void* const* q,
                const void* const* k, const void* const* v, void* const* out, int32_t n, int64_t ts, int64_t hs, cudaStream_t st,
-               const cudaEvent_t* kv_taken = nullptr, int n_taken = 0) {
+               xkv_cache** last_means, const cudaEvent_t* kv_taken = nullptr, int n_taken = 0) {
   xkv_cache* const* cs = layers + from;
   const bool once = keys_once(cs[0]);
   // after a failed call the caches take no further frame (only xkv_reset goes on)
@@ -645,8 +641,9 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
   }
   // The side stream forks here (after the packing) but its kernel is launched after the attention has
   // been enqueued, so that the attention's blocks get the multiprocessors first and the head means
-  // fill in as they retire.
-  if (n_kbar && !(cudaEventRecord(pipe->fork, st) == cudaSuccess && cudaStreamWaitEvent(pipe->side, pipe->fork, 0) == cudaSuccess))
+  // fill in as they retire.  The events are the caches' own, for the fork too: steps of other caches
+  // from other threads share the side stream with this one and nothing else.
+  if (n_kbar && !(cudaEventRecord(kc[0]->kbar_done, st) == cudaSuccess && cudaStreamWaitEvent(pipe->side, kc[0]->kbar_done, 0) == cudaSuccess))
     return fail(3);
   const cudaError_t e = launch_attn_tc(calls, count, ts, hs, 1.0f / sqrtf((float)cs[0]->p.head_dim), st);
   if (e != cudaSuccess) {
@@ -656,7 +653,7 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
   if (n_kbar) {
     bool ok = launch_maint(kc, as, n_kbar, XKV_PROF_KBAR, pipe->side) == cudaSuccess;
     for (int i = 0; i < n_kbar; ++i) ok = cudaEventRecord(kc[i]->kbar_done, pipe->side) == cudaSuccess && ok;
-    pipe->side_busy = true;
+    *last_means = kc[n_kbar - 1];
     // (means that were never computed don't pass for those of this frame: the next scoring computes them
     // anew, except with keys quantised once, where they travel with the tokens)
     if (!ok) return once ? fail(3) : XKV_E_CUDA;
@@ -666,11 +663,9 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
 }
 
 // Everything a stream-step call started on the side stream is ordered before what the caller
-// enqueues next.
-bool join_side_work(HostStepPipe* pipe, cudaStream_t st) {
-  if (!pipe->side_busy) return true;
-  pipe->side_busy = false;
-  return cudaEventRecord(pipe->join, pipe->side) == cudaSuccess && cudaStreamWaitEvent(st, pipe->join, 0) == cudaSuccess;
+// enqueues next (the last of it came last there).
+bool join_side_work(const xkv_cache* last_means, cudaStream_t st) {
+  return !last_means || cudaStreamWaitEvent(st, last_means->kbar_done, 0) == cudaSuccess;
 }
 
 }  // namespace
@@ -683,6 +678,7 @@ int xkv_stream_step(xkv_cache* const* layers, int32_t n_layers, const void* cons
   if (!pipe) return XKV_E_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   int rc = XKV_OK;
+  xkv_cache* last_means = nullptr;
   for (int l0 = 0; l0 < n_layers && rc == XKV_OK;) {
     // The next layers that can go together: the same form of cache, no cache twice, and no layer's
     // output in memory that a later one reads or writes, nor in a query (or, with the unquantised
@@ -709,12 +705,12 @@ int xkv_stream_step(xkv_cache* const* layers, int32_t n_layers, const void* cons
       ++count;
     }
     if (count > 0) {
-      const int e = run_layers(pipe, layers, l0, as, count, q + l0, k + l0, v + l0, out + l0, n, ts, hs, st);
+      const int e = run_layers(pipe, layers, l0, as, count, q + l0, k + l0, v + l0, out + l0, n, ts, hs, st, &last_means);
       if (e != XKV_OK) rc = e;
     }
     l0 += count;
   }
-  if (!join_side_work(pipe, st) && rc == XKV_OK) rc = XKV_E_CUDA;
+  if (!join_side_work(last_means, st) && rc == XKV_OK) rc = XKV_E_CUDA;
   return rc;
 }
 
@@ -763,6 +759,7 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
   ck(cudaStreamWaitEvent(pipe->up2, pipe->start, 0));
   ck(cudaStreamWaitEvent(pipe->up3, pipe->start, 0));
   ck(cudaStreamWaitEvent(pipe->down, pipe->start, 0));
+  xkv_cache* last_means = nullptr;
   bool kv_used[2] = {false, false}, qo_used[2] = {false, false};      // halves of the staging buffer in use before
   for (int l = 0, group = 0; l < n_layers && cuda_ok && rc == XKV_OK; ++group) {
     int count = 1;
@@ -801,7 +798,7 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
     }
     if (ready > 0) {
       const bool tail = layers[l]->tail_mode != 0;
-      const int e = run_layers(pipe, layers, l, as, ready, dq, dk, dv, dq, n, ts, hs, st, &pipe->kv_free[half[0]],
+      const int e = run_layers(pipe, layers, l, as, ready, dq, dk, dv, dq, n, ts, hs, st, &last_means, &pipe->kv_free[half[0]],
                                tail ? 0 : count);
       if (e != XKV_OK) rc = e;
       if (tail) ck(cudaEventRecord(pipe->kv_free[half[0]], st));
@@ -816,7 +813,7 @@ int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void*
     l += count;
   }
   // everything started above ends before the call returns, also after an error
-  if (!join_side_work(pipe, st)) cuda_ok = false;
+  if (!join_side_work(last_means, st)) cuda_ok = false;
   ck(cudaStreamSynchronize(pipe->up));
   ck(cudaStreamSynchronize(pipe->up2));
   ck(cudaStreamSynchronize(pipe->up3));

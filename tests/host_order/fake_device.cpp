@@ -32,6 +32,9 @@ std::vector<Op> g_ops;
 std::string g_report;
 std::string g_fail_name;       // the next operation of this name fails
 std::map<const void*, int> g_means_of;     // head-mean array -> frame of the cache that it was computed for
+std::string g_hook_name;       // before the g_hook_after-th operation of this name, g_hook is called
+int g_hook_after = 0;
+void (*g_hook)() = nullptr;
 int g_epoch = 0;
 uintptr_t g_handles = 0x1000;
 
@@ -46,6 +49,11 @@ struct Builder {
   void reads(const void* p, size_t bytes, const char* what) { add(p, bytes, false, what); }
   void writes(const void* p, size_t bytes, const char* what) { add(p, bytes, true, what); }
   cudaError_t run() {
+    if (g_hook && g_hook_name == op.name && --g_hook_after == 0) {
+      void (*hook)() = g_hook;
+      g_hook = nullptr;
+      hook();
+    }
     std::lock_guard<std::recursive_mutex> lock(g_mutex);
     if (g_fail_name == op.name) { g_fail_name.clear(); return cudaErrorLaunchFailure; }
     Clock& now = g_streams[op.stream];
@@ -97,6 +105,7 @@ XKV_API int fake_ops(const char* name) {
   return n;
 }
 XKV_API void fake_fail_next(const char* name) { g_fail_name = name; }
+XKV_API void fake_hook(const char* name, int nth, void (*fn)()) { g_hook_name = name; g_hook_after = nth; g_hook = fn; }
 XKV_API void fake_clear() { g_report.clear(); g_ops.clear(); g_fail_name.clear(); }   // (the clocks go on)
 // From here on a wait on an event that was recorded before is an error, as inside a stream capture.
 XKV_API void fake_begin_capture() { ++g_epoch; }

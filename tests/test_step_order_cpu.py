@@ -38,15 +38,15 @@ class Stack:
     """Caches on addresses that nobody ever reads."""
     bump = 1 << 40
 
-    def __init__(self, lib, layers, budget, n, bits=4, once=0, tail=0):
+    def __init__(self, lib, layers, budget, n, bits=4, once=0, tail=0, stream=None):
         import paper_2601_01204_b200.xkv as xkv
-        self.lib, self.xkv, self.n = lib, xkv, n
+        self.lib, self.xkv, self.n, self.stream = lib, xkv, n, stream
         self.p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=bits, key_mode=once).c()
         self.caches = []
         for _ in range(layers):
             size = lib.xkv_workspace_bytes(C.byref(self.p))
             h = C.c_void_p()
-            assert lib.xkv_create(C.byref(self.p), Stack.take(size), size, None, C.byref(h)) == 0
+            assert lib.xkv_create(C.byref(self.p), Stack.take(size), size, stream, C.byref(h)) == 0
             assert lib.xkv_set_unquantised_tail(h, tail) == 0
             self.caches.append(h.value)
 
@@ -63,9 +63,9 @@ class Stack:
     def tensors(self, count):
         return [Stack.take(FRAME) for _ in range(count)]
 
-    def step(self, which, host=False, q=None, k=None, v=None, out=None, stream=None):
+    def step(self, which, host=False, q=None, k=None, v=None, out=None):
         """One step of the caches with these numbers, in this order; returns the status."""
-        n = len(which)
+        n, stream = len(which), self.stream
         arr = lambda xs: (C.c_void_p * n)(*xs)
         q, k, v, out = (x or self.tensors(n) for x in (q, k, v, out))
         caches = arr([self.caches[i] for i in which])
@@ -148,3 +148,21 @@ def test_a_step_that_is_not_supported_leaves_the_caches_alone(lib, host):
         lib.xkv_set_unquantised_tail(c, 0)
     assert s.step([0, 1, 2], host) == 0
     assert s.races() == ""
+
+
+@pytest.mark.parametrize("launch", [b"maintenance", b"attention", b"head means"])
+@pytest.mark.parametrize("nth", [1, 2])
+def test_a_step_of_other_caches_in_the_middle_of_one(lib, launch, nth):
+    """As when two threads drive different caches on streams of their own."""
+    ours, theirs = Stack(lib, 1, 1000, 200, stream=0x11), Stack(lib, 2, 1000, 200, stream=0x22)
+    hook = C.CFUNCTYPE(None)(lambda: theirs.step([0, 1]))
+    for _ in range(7):
+        assert ours.step([0]) == 0 and theirs.step([0, 1]) == 0
+        new = Stack(lib, 1, 1000, 200, bits=16, stream=0x11)     # its first frame: no head means behind its attention
+        ours.caches[1:] = new.caches
+        lib.fake_hook(launch, nth, hook)
+        assert ours.step([0, 1]) == 0
+        lib.fake_hook(b"", 0, C.CFUNCTYPE(None)())
+        assert ours.step([0]) == 0
+    assert ours.info(0).last_evicted > 0 and theirs.info(0).last_evicted > 0
+    assert ours.races() == ""
