@@ -246,7 +246,8 @@ def run_xkv(args) -> None:
     t = 0
     for _ in range(fill + W):                       # untimed: fill to steady state, then W warm-up steps
         step(t); t += 1
-    launches0 = sum(c.xkv_get_info().launches for c in caches)
+    # (every launch of a step serves all layers and counts for each of them)
+    launches0 = caches[0].xkv_get_info().launches
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     barrier()
     with ClockSampler(local) as clocks:
@@ -256,7 +257,7 @@ def run_xkv(args) -> None:
         ev1.record()
         barrier()
     ms_total = ev0.elapsed_time(ev1)
-    launches = sum(c.xkv_get_info().launches for c in caches) - launches0
+    launches = caches[0].xkv_get_info().launches - launches0
     ms_total = max_over_ranks(ms_total)
     assert all(c.xkv_get_info().T == w["budget"] for c in caches)
     assert all(c.xkv_poll_status() == 0 for c in caches)

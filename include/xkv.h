@@ -106,7 +106,8 @@ typedef struct {
   int32_t last_prunable;     /* size of the middle segment at the last kv_score_evict    */
   int32_t stage;             /* 0 idle, 1 appended, 2 scored, 3 packed                   */
   int32_t n_pending;         /* tokens of the frame in flight                            */
-  int64_t launches;          /* kernels launched for this cache so far                   */
+  int64_t launches;          /* kernels launched for this cache so far; one that serves  */
+                             /* several layers of a step counts for each of them         */
   uint64_t workspace_bytes;
   int32_t key_table_slots;   /* XKV_KEYS_ONCE: slots of the key parameter table, else 0  */
   int32_t budget;            /* the token budget in force (xkv_set_budget)               */
@@ -402,7 +403,9 @@ XKV_API int xkv_debug_timeout_probe(xkv_cache* cache, xkv_stream stream);
 
 /* Optional per-kernel timing for benchmarks.  While enabled, every kernel the
  * library launches for this cache is bracketed by a pair of CUDA events on the
- * launching stream (a small overhead; leave it off in production).
+ * launching stream (a small overhead; leave it off in production).  A kernel that
+ * serves several layers of a step is recorded once, for the first of them that has
+ * profiling on.
  * xkv_profile_read synchronises `stream`, adds the elapsed time of all launches
  * recorded since the last read to the per-category totals, copies the totals to
  * *out and clears them. */

@@ -1294,10 +1294,12 @@ static void fill_job(Job* j, const AttnCall& call) {
   j->n_pairs = (j->q_tiles + 1) / 2;
 }
 
-// One launch (and its merge) for the jobs in `a`.  `part` holds the partial slots: accumulators float
+// One launch (and its merge) for the jobs in `a`, which are those caches'.  `part` holds the partial slots: accumulators float
 // [slots][2][128][64], then (max, sum) float2 [slots][2][128], slots = part_bytes / kSlotBytes.  The
 // grid is the SM count, capped by the slots available (two per CTA) and by the number of steps.
-static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail, float* part, size_t part_bytes, int sm_count, cudaStream_t st) {
+static cudaError_t launch_jobs(xkv_cache* const* caches, int n_caches, Args& a, uint32_t total, bool tail, float* part,
+                               size_t part_bytes, int sm_count, cudaStream_t st) {
+  const xkv_cache* c = caches[0];
   const size_t slots = part_bytes / kSlotBytes;
   long long grid = sm_count;
   if (grid > (long long)(slots / 2)) grid = (long long)(slots / 2);
@@ -1310,7 +1312,7 @@ static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail,
   a.part_o = part;
   a.part_ml = reinterpret_cast<float2*>(part + slots * kSlotFloats);
   {
-    LaunchScope ls(c, XKV_PROF_ATTN, st);
+    LaunchScope ls(caches, n_caches, XKV_PROF_ATTN, st);
     const bool once = c->p.key_mode == XKV_KEYS_ONCE;
     const void* fn;
     int smem = smem_bytes<4>();
@@ -1325,7 +1327,7 @@ static cudaError_t launch_jobs(xkv_cache* c, Args& a, uint32_t total, bool tail,
     if (e != cudaSuccess) return e;
   }
   if (grid > 1) {
-    LaunchScope ls(c, XKV_PROF_COMBINE, st);
+    LaunchScope ls(caches, n_caches, XKV_PROF_COMBINE, st);
     void* params[1] = {(void*)&a};
     const cudaError_t e = launch_overlapped((const void*)attn_combine_kernel, dim3((unsigned)(grid - 1) * 8), dim3(256), params, 0, st);
     if (e != cudaSuccess) return e;
@@ -1349,6 +1351,8 @@ static cudaError_t launch_attn_tc_on(const AttnCall* calls, int count, int64_t t
   for (int i = 0; i < count;) {
     a.n_jobs = 0;
     uint32_t total = 0;
+    xkv_cache* caches[kMaxJobs];
+    int n_caches = 0;
     for (; i < count && a.n_jobs < kMaxJobs; ++i) {
       Job* j = &a.job[a.n_jobs];
       fill_job(j, calls[i]);
@@ -1361,8 +1365,10 @@ static cudaError_t launch_attn_tc_on(const AttnCall* calls, int count, int64_t t
       total += (uint32_t)steps;
       j->step_hi = total;
       a.n_jobs++;
+      // (the frames of a chunk are jobs of one cache)
+      if (n_caches == 0 || caches[n_caches - 1] != calls[i].cache) caches[n_caches++] = calls[i].cache;
     }
-    const cudaError_t e = launch_jobs(lead, a, total, tail, part, part_bytes, sm_count, st);
+    const cudaError_t e = launch_jobs(caches, n_caches, a, total, tail, part, part_bytes, sm_count, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

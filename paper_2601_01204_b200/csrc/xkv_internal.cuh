@@ -147,13 +147,16 @@ __device__ __forceinline__ void dequant_consts(float s, float z, float& zo_1024,
 }
 #endif
 
-// Brackets one kernel launch with events when profiling is on; counts the launch.
+// Counts one kernel launch for every cache that it serves, and brackets it with events for the first of
+// them that has profiling on (one only, so that sums over caches count a launch once).
 struct LaunchScope {
-  xkv_cache* c; int cat; cudaStream_t st; cudaEvent_t a = nullptr, b = nullptr;
-  LaunchScope(xkv_cache* c_, int cat_, cudaStream_t st_) : c(c_), cat(cat_), st(st_) {
-    c->launches++;
-    Profiler* p = c->prof;
-    if (p && p->on) {
+  Profiler* p = nullptr; int cat; cudaStream_t st; cudaEvent_t a = nullptr, b = nullptr;
+  LaunchScope(xkv_cache* const* cs, int count, int cat_, cudaStream_t st_) : cat(cat_), st(st_) {
+    for (int i = 0; i < count; ++i) {
+      cs[i]->launches++;
+      if (!p && cs[i]->prof && cs[i]->prof->on) p = cs[i]->prof;
+    }
+    if (p) {
       auto get = [&]() { cudaEvent_t e = nullptr;
         if (!p->pool.empty()) { e = p->pool.back(); p->pool.pop_back(); } else cudaEventCreate(&e);
         return e; };
@@ -162,7 +165,7 @@ struct LaunchScope {
     }
   }
   ~LaunchScope() {
-    if (a) { cudaEventRecord(b, st); c->prof->pending.push_back({cat, a, b}); }
+    if (a) { cudaEventRecord(b, st); p->pending.push_back({cat, a, b}); }
   }
 };
 

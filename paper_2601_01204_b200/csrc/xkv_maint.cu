@@ -1446,7 +1446,7 @@ static cudaError_t launch_regroup_n(xkv_cache* const* c, const MaintArgs* a, int
     if (g > groups) groups = g;
   }
   const dim3 grid(groups, a[0].H, count);
-  LaunchScope ls(c[0], XKV_PROF_PACK, st);
+  LaunchScope ls(c, count, XKV_PROF_PACK, st);
   void* params[1] = {(void*)&b};
   const cudaError_t e = launch_overlapped((const void*)regroup_k_kernel<MAX>, grid, dim3(kRgThreads), params, 0, st);
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -1517,7 +1517,7 @@ static cudaError_t launch_maint_n(xkv_cache* const* c, MaintArgs* as, int count,
 }
 
 cudaError_t launch_maint(xkv_cache* const* c, MaintArgs* a, int count, int prof_cat, cudaStream_t st) {
-  LaunchScope ls(c[0], prof_cat, st);
+  LaunchScope ls(c, count, prof_cat, st);
   return count == 1 ? launch_maint_n<1>(c, a, 1, st) : launch_maint_n<kMaxLayers>(c, a, count, st);
 }
 

@@ -203,3 +203,23 @@ def test_a_failed_cache_does_not_touch_the_others_of_its_launch(xkv, failed):
             check_attention(bf16_tensor_to_f32(out[l]), bf16_tensor_to_f32(ref), f"frame {t} layer {l}")
             compare_state(together[l].export(), alone[l].export(), f"frame {t} layer {l}")
     assert [c.xkv_poll_status() for c in together] == [xkv.XKV_E_TIMEOUT if l == failed else 0 for l in range(layers)]
+
+
+def test_launches_of_a_step_count_for_every_layer(xkv):
+    """A launch that serves several layers counts for each of them and is timed for the first one with
+    profiling on, whichever that is."""
+    import torch
+    layers, n, budget = 4, 97, 300
+    caches = [xkv.Cache(xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=4)) for _ in range(layers)]
+    for t in range(5):
+        q, k, v = zip(*(frame(l, t, n) for l in range(layers)))
+        if t == 4:
+            caches[2].xkv_profile_enable(True)
+            caches[3].xkv_profile_enable(True)
+            before = [c.xkv_get_info().launches for c in caches]
+        xkv.xkv_stream_step(caches, q, k, v, [torch.empty_like(x) for x in q])
+    # maintenance, regroup, attention, its merge, head means
+    assert [c.xkv_get_info().launches - b for c, b in zip(caches, before)] == [5] * layers
+    timed, rest = caches[2].xkv_profile_read(), caches[3].xkv_profile_read()
+    assert all(timed[name][1] == 1 and timed[name][0] > 0 for name in ("maint", "pack", "attn", "attn_combine", "kbar"))
+    assert all(count == 0 for _, count in rest.values())
