@@ -1225,9 +1225,10 @@ __global__ void __launch_bounds__(kRgThreads, 8) regroup_k_kernel(const __grid_c
   // one thread per channel finishes the reduction and derives the group's parameters
   int slow = a.force_plain;
   if (tid < 64) {
-    float lo = s_mn[0][tid], up = s_mx[0][tid];
+    // (from the empty extremes: a lane whose tokens are all not numbers has none of its own)
+    float lo = INFINITY, up = -INFINITY;
 #pragma unroll
-    for (int r = 1; r < kRgLanes; ++r) { lo = fminf(lo, s_mn[r][tid]); up = fmaxf(up, s_mx[r][tid]); }
+    for (int r = 0; r < kRgLanes; ++r) { lo = fminf(lo, s_mn[r][tid]); up = fmaxf(up, s_mx[r][tid]); }
     float sc, inv, z;
     quant_params(lo, up, sc, inv, z);
     const int ch = ((tid >> 2) & 7) * 8 + (tid >> 5) * 4 + (tid & 3);

@@ -223,3 +223,28 @@ def test_launches_of_a_step_count_for_every_layer(xkv):
     timed, rest = caches[2].xkv_profile_read(), caches[3].xkv_profile_read()
     assert all(timed[name][1] == 1 and timed[name][0] > 0 for name in ("maint", "pack", "attn", "attn_combine", "kbar"))
     assert all(count == 0 for _, count in rest.values())
+
+
+def test_key_channels_that_are_not_numbers(xkv):
+    """The extremes of a key group pass over what is not a number; a channel without any number has the
+    empty extremes, in full and in ragged groups alike."""
+    import torch
+    n = 100                                               # one group of 64, one of 36
+    k = to_device_bf16(synth.gen_frame(6, 0, 0, H, n, D)[1])
+    some, none = k.clone(), k.clone()
+    some[0, ::3, 5] = float("nan")
+    none[0, ::3, 5] = k[0, 1, 5]                          # the same extremes in both groups ...
+    none[0, 66::3, 5] = k[0, 67, 5]                       # ... from the numbers that are there
+    some[:, :, 3] = float("nan")
+    params = []
+    for x in (some, none):
+        cache = xkv.Cache(xkv.Params(n_heads=H, budget=300, max_frame_tokens=n, kv_bits=4))
+        cache.kv_append(x, x)
+        cache.kv_score_evict(x)
+        cache.kv_quant_pack()
+        e = cache.export()
+        params.append((e["k_s_first"], e["k_z_first"]))
+    (s, z), (s_ref, z_ref) = params
+    rest = [c for c in range(D) if c != 3]
+    assert np.array_equal(s[:, :, rest], s_ref[:, :, rest]) and np.array_equal(z[:, :, rest], z_ref[:, :, rest])
+    assert np.all(s[:, :, 3] == -np.inf)                  # (-inf - inf) / 15
