@@ -248,3 +248,35 @@ def test_key_channels_that_are_not_numbers(xkv):
     rest = [c for c in range(D) if c != 3]
     assert np.array_equal(s[:, :, rest], s_ref[:, :, rest]) and np.array_equal(z[:, :, rest], z_ref[:, :, rest])
     assert np.all(s[:, :, 3] == -np.inf)                  # (-inf - inf) / 15
+
+
+@pytest.mark.parametrize("layers", [1, 5])
+def test_16bit_weights_are_normalised_as_they_are_multiplied(xkv, layers):
+    """The softmax weights of a 16-bit cache are rounded to bf16.  With each rounding error d_i (relative
+    variance r2) the output is off by sum w_i d_i (v_i - out) if the weights are divided by the sum of the
+    rounded ones, by sum w_i d_i v_i if not: for rows that one key dominates next to nothing against as
+    much as the rounding of the output itself.  The bound is the former and the output's rounding, plus
+    10 % for the sample."""
+    import torch
+    heads, n, budget = 8, 211, 6007
+    p = xkv.Params(n_heads=heads, budget=budget, max_frame_tokens=n, kv_bits=16)
+    caches = [xkv.Cache(p) for _ in range(layers)]
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    mk = lambda scale: [(scale * torch.randn(heads, n, D, device="cuda", generator=gen)).to(torch.bfloat16) for _ in range(layers)]
+    for t in range(budget // n + 2):
+        q, k, v = mk(6.0), mk(1.0), mk(1.0)
+        out = [torch.empty_like(x) for x in q]
+        xkv.xkv_stream_step(caches, q, k, v, out)
+    r2 = (2.0 ** -7) ** 2 / 12 * 3 / (8 * np.log(2))      # mean of (ulp^2 / 12) / m^2 over mantissas m, log-uniform in [1, 2)
+    for l in (0, layers - 1):
+        e = caches[l].export()
+        K, V = (torch.from_numpy(e[x]).cuda().double() for x in ("k_val", "v_val"))
+        w = torch.softmax(q[l].double() @ K.transpose(1, 2) / 8.0, dim=-1)
+        ref = w @ V
+        # sum_i w_i^2 |v_i - out|^2 = sum_i w_i^2 (|v_i|^2 - 2 v_i out + |out|^2)
+        w2 = w * w
+        var = (w2 @ (V * V).sum(-1, keepdim=True)).sum() - 2 * ((w2 @ V) * ref).sum() + (w2.sum(-1) * (ref * ref).sum(-1)).sum()
+        rounding = (ref.to(torch.bfloat16).double() - ref).norm() / ref.norm()
+        bound = 1.1 * float(torch.sqrt(rounding ** 2 + r2 * var / ref.norm() ** 2))
+        err = float((out[l].double() - ref).norm() / ref.norm())
+        assert err <= bound, (l, err, bound)
