@@ -12,7 +12,7 @@ import pytest
 
 from oracle import xkv_oracle as xo
 from paper_2601_01204_b200 import synth
-from xkv_testlib import (ATTN_MAXABS, ATTN_RELL2, bf16_tensor_to_f32, compare_state, oracle_params,
+from xkv_testlib import (ATTN_MAXABS, ATTN_RELL2, bf16_tensor_to_f32, compare_state, dequantized, oracle_params,
                          to_device_bf16)
 
 pytestmark = pytest.mark.gpu
@@ -265,3 +265,110 @@ def test_attention_repeated_launches_are_bit_identical(xkv, variant):
         else:
             assert torch.equal(first, bits_out), f"{variant}: launch {rep} differs from launch 0"
     cache.close()
+
+
+def _sampled_attention(out, q, K, V, rng, tag):
+    """24 query rows, the first and the last among them, against the oracle's attention."""
+    n = q.shape[1]
+    rows = np.sort(rng.choice(n, size=24, replace=False))
+    rows[0], rows[-1] = 0, n - 1
+    ref = xo.attention(q[:, rows], K, V, 1.0 / np.sqrt(q.shape[2]))
+    err = out[:, rows].astype(np.float64) - ref
+    assert np.abs(err).max() <= ATTN_MAXABS * np.abs(ref).max(), tag
+    assert np.linalg.norm(err) <= ATTN_RELL2 * np.linalg.norm(ref), tag
+
+
+@pytest.mark.parametrize("bits, once, tail", [(4, 0, False), (4, 1, False), (4, 0, True), (8, 1, False), (16, 0, False)])
+def test_24_layers_in_one_launch_full_size(xkv, bits, once, tail):
+    """The full stack as the benchmark steps it (24 layers, 1374 tokens, budget 16384): two stacks on the
+    same frames give the same bits in every layer of twelve launches on full caches, and layers
+    0, 11 and 23 of the last one agree with the oracle's attention over the cache as exported, whose
+    state is that of the per-call entry points."""
+    import torch
+    L, H, n, d, budget = 24, 16, 1374, 64, 16384
+    p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=bits, key_mode=once)
+    stacks = [[xkv.Cache(p) for _ in range(L)] for _ in range(2)]
+    calls = {l: xkv.Cache(p) for l in (0, 11, 23)}
+    for c in stacks[0] + stacks[1]:
+        c.xkv_set_unquantised_tail(tail)
+    new = lambda: [torch.empty(H, n, d, dtype=torch.bfloat16, device="cuda") for _ in range(L)]
+    q, k, v, outs = new(), new(), new(), (new(), new())
+    frames = budget // n + 12
+    for t in range(frames):
+        for l in range(L):
+            for x, which in ((q, synth.TENSOR_Q), (k, synth.TENSOR_K), (v, synth.TENSOR_V)):
+                xkv.xkv_synth_fill(x[l], 3 + l, l, t, which)
+        for caches, out in zip(stacks, outs):
+            xkv.xkv_stream_step(caches, q, k, v, out)
+        for l, c in calls.items():
+            c.step(q[l], k[l], v[l])
+        if t >= frames - 12:
+            assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(*outs)), f"frame {t}"
+    assert all(c.xkv_poll_status() == 0 and c.xkv_get_info().T == budget for c in stacks[0] + stacks[1])
+    rng = np.random.default_rng(11)
+    for l, c in calls.items():
+        e = stacks[0][l].export()
+        compare_state(e, c.export(), f"layer {l}")
+        K, V = dequantized(e, bits)
+        if tail:
+            K[:, budget - n:], V[:, budget - n:] = bf16_tensor_to_f32(k[l]), bf16_tensor_to_f32(v[l])
+        _sampled_attention(bf16_tensor_to_f32(outs[0][l]), bf16_tensor_to_f32(q[l]), K, V, rng, f"layer {l}")
+
+
+def test_chunk_of_four_full_size_frames_in_one_launch(xkv):
+    """Chunks of four frames of 1004 tokens at a budget of 9000, the third one evicting: every frame's
+    attention on sampled rows against the oracle, then the launch twelve times, bit for bit."""
+    import torch
+    H, n, F, d = 16, 1004, 4, 64
+    p = xkv.Params(n_heads=H, budget=9000, max_frame_tokens=F * n, kv_bits=4)
+    cache, ora = xkv.Cache(p), xo.OracleLayer(oracle_params(p))
+    rng = np.random.default_rng(12)
+    for t in range(3):
+        bits = synth.gen_frame(7, 0, t, H, F * n, d)
+        q, k, v = (to_device_bf16(x) for x in bits)
+        qf, kf, vf = (synth.bf16_bits_to_f32(x) for x in bits)
+        out = cache.xkv_prefill_chunk(q, k, v, [n] * F)
+        ora.append(kf, vf)
+        ora.score_evict(qf[:, -n:])
+        ora.quant_pack()
+        compare_state(cache.export(), ora.export(), f"chunk {t}")
+        K, V = ora.keys_dequantized(), ora.values_dequantized()
+        for f in range(F):
+            seen = ora.T - F * n + (f + 1) * n
+            _sampled_attention(bf16_tensor_to_f32(out)[:, f * n:(f + 1) * n], qf[:, f * n:(f + 1) * n], K[:, :seen], V[:, :seen],
+                               rng, f"chunk {t} frame {f}")
+    info = cache.xkv_get_info()
+    assert info.last_evicted > 0 and info.last_kept > 0
+    first = out.clone()
+    for rep in range(12):
+        cache.xkv_debug_rewind_attention()
+        again = cache.attn_packed_frame_causal(q, [n] * F)
+        assert torch.equal(again.view(torch.int16), first.view(torch.int16)), rep
+    assert cache.xkv_poll_status() == 0
+
+
+@pytest.mark.parametrize("once", [0, 1])
+def test_a_cache_twice_in_one_step_full_size(xkv, once):
+    """[a, b, b]: the second layer on b starts where the head means of the first are still on their way.
+    Scores, kept indices and state are those of the four calls one after the other, fourteen times."""
+    import torch
+    H, n, d, budget = 16, 1374, 64, 16384
+    p = xkv.Params(n_heads=H, budget=budget, max_frame_tokens=n, kv_bits=4, key_mode=once)
+    step, calls = [xkv.Cache(p) for _ in range(2)], [xkv.Cache(p) for _ in range(2)]
+    new = lambda: [torch.empty(H, n, d, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    q, k, v, out = new(), new(), new(), new()
+    for t in range(14):
+        for l in range(3):
+            for x, which in ((q, synth.TENSOR_Q), (k, synth.TENSOR_K), (v, synth.TENSOR_V)):
+                xkv.xkv_synth_fill(x[l], 9 + l, l, t, which)
+        xkv.xkv_stream_step([step[0], step[1], step[1]], q, k, v, out)
+        for l, c in enumerate((calls[0], calls[1], calls[1])):
+            c.step(q[l], k[l], v[l])
+        for a, b in zip(step, calls):
+            info = b.xkv_get_info()
+            if info.last_kept:
+                for buf, size in ((xkv.BUF_SCORES, info.last_prunable), (xkv.BUF_KEPT, info.last_kept)):
+                    assert np.array_equal(a.xkv_debug_export(buf, 4 * size), b.xkv_debug_export(buf, 4 * size)), (t, buf)
+            if t % 4 == 1:
+                compare_state(a.export(), b.export(), f"call {t}")
+    assert step[1].xkv_get_info().last_evicted == n and all(c.xkv_poll_status() == 0 for c in step)

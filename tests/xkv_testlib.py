@@ -44,6 +44,20 @@ def compare_state(gpu: dict, ora: dict, tag: str = "") -> None:
                                  f"gpu {a[tuple(bad[0])]} oracle {b[tuple(bad[0])]}")
 
 
+def dequantized(e: dict, bits: int) -> tuple[np.ndarray, np.ndarray]:
+    """Keys and values [H][T][d] of an exported cache (Eq. 10)."""
+    if bits == 16:
+        return e["k_val"].copy(), e["v_val"].copy()
+    unpack = xo.unpack_nibbles if bits == 4 else xo.unpack_bytes8
+    k, Tf = unpack(e["k_packed"]), e["T_first"]
+    if "k_s_tok" in e:
+        K = xo.dequantize(k, e["k_s_tok"], e["k_z_tok"])
+    else:
+        K = np.concatenate([xo.dequantize_keys(k[:, :Tf], e["k_s_first"], e["k_z_first"], 64),
+                            xo.dequantize_keys(k[:, Tf:], e["k_s_rest"], e["k_z_rest"], 64)], axis=1)
+    return K, xo.dequantize_values(unpack(e["v_packed"]), e["v_s"], e["v_z"])
+
+
 def attn_errors(got: np.ndarray, ref: np.ndarray) -> tuple[float, float]:
     err = got.astype(np.float64) - ref.astype(np.float64)
     return float(np.abs(err).max() / np.abs(ref).max()), float(np.linalg.norm(err) / np.linalg.norm(ref))
