@@ -329,6 +329,10 @@ XKV_API int xkv_set_unquantised_tail(xkv_cache* cache, int32_t on);
  * of all of them, then the attention of all of them.  A layer whose tensors overlap an earlier layer's
  * output (or whose output overlaps what an earlier layer still reads), or whose cache has come before,
  * starts after the layers before it, so the results are always those of the layers one after the other.
+ * The caches (codes, parameters, scores, kept tokens) are the same bit for bit whichever way a frame is
+ * driven: step, host-buffer step or the four calls, alone or with other layers.  Outputs agree to the
+ * attention's accuracy but not bit for bit: where the keys of a head are cut between thread blocks
+ * depends on what shares the launch.  The same call on the same state repeats exactly.
  * After kv_quant_pack the step also computes, on a stream of the library's own (created on
  * first use, one per device) and beside the attention, the head means of the cached keys (Eq. 4) into the cache's workspace;
  * the next frame's scoring of the same cache starts from them (same bits as

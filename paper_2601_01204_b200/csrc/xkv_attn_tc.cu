@@ -27,6 +27,8 @@
 //               188.5 -> 181.9 us, 16-bit at 32768 tokens 287.1 -> 273.8 us.
 //   1 thread    issues the bulk copies of the raw tiles, several steps ahead; its warp owns the
 //               tensor-memory allocation (all 512 columns).
+//   1 warp      with keys quantised once asks for the key constants a few tiles ahead of the producers,
+//               else idle.
 // 4-bit caches multiply in fp16 (the dequantised keys are not bf16-representable:
 // rounding them to bf16 alone costs ~1e-2 relative L2 with outlier channels);
 // 16-bit caches hold bf16 and multiply in bf16.  Accumulation is fp32.
@@ -152,6 +154,7 @@ struct Args {
   float2* part_ml;      // [2 * grid][2][128]
   Job job[kMaxJobs];
 };
+static_assert(sizeof(Args) <= 4096, "the job table");
 
 __device__ __forceinline__ uint32_t piece_start(const Args& a, int b) {
   return (uint32_t)b * a.piece + min((uint32_t)b, a.longer);
@@ -549,18 +552,15 @@ __device__ __forceinline__ void once_keys(const uint8_t* codes, const uint8_t* r
     *reinterpret_cast<uint4*>(tile + (k0 + i) * 128 + ((w ^ i) << 4)) = dequant_word_h(wd[i], s2, zo, c2);
   }
 }
-// O[row][0..63] *= alpha for the 32 rows (TMEM lanes) of the calling warp; a real call, to keep its
+// 32 columns of O *= alpha for the 32 rows (TMEM lanes) of the calling warp; a real call, to keep its
 // registers out of the softmax loop.  Warp-collective.
-__device__ __noinline__ void rescale_rows(uint32_t col_o, float alpha, int cols = 64) {
-#pragma unroll 1
-  for (int c0 = 0; c0 < cols; c0 += 32) {
-    uint32_t ra[32];
-    XKV_TMEM_LD32(col_o + c0, ra);
-    tc_wait_ld();
+__device__ __noinline__ void rescale_rows(uint32_t col_o, float alpha) {
+  uint32_t ra[32];
+  XKV_TMEM_LD32(col_o, ra);
+  tc_wait_ld();
 #pragma unroll
-    for (int i = 0; i < 32; ++i) ra[i] = __float_as_uint(__uint_as_float(ra[i]) * alpha);
-    XKV_TMEM_ST32(col_o + c0, ra);
-  }
+  for (int i = 0; i < 32; ++i) ra[i] = __float_as_uint(__uint_as_float(ra[i]) * alpha);
+  XKV_TMEM_ST32(col_o, ra);
   tc_wait_st();
 }
 __device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -791,7 +791,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);
           __syncwarp();
           tc_fence_after();
-          rescale_rows(colO, alpha, 32);
+          rescale_rows(colO, alpha);
         }
         tc_wait_st();
         tc_fence_before();
@@ -915,21 +915,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
                                 b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
           } else {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const uint32_t*>(raw + (kb + 16 * i) * 32 + 4 * w);
-          mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
+            for (int i = 0; i < 8; ++i) wd[i] = *reinterpret_cast<const uint32_t*>(raw + (kb + 16 * i) * 32 + 4 * w);
+            mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
 #pragma unroll
-          for (int grp = 0; grp < 2; ++grp) {
-            const uint4 sv = *reinterpret_cast<const uint4*>(tab + grp * 128 + 16 * w);
-            const uint4 zv = *reinterpret_cast<const uint4*>(tab + 256 + grp * 128 + 16 * w);
-            const uint4 cv = *reinterpret_cast<const uint4*>(tab + 512 + grp * 128 + 16 * w);
-            const uint32_t s2[4] = {sv.x, sv.y, sv.z, sv.w}, zo[4] = {zv.x, zv.y, zv.z, zv.w};
-            const uint32_t c2[4] = {cv.x, cv.y, cv.z, cv.w};
+            for (int grp = 0; grp < 2; ++grp) {
+              const uint4 sv = *reinterpret_cast<const uint4*>(tab + grp * 128 + 16 * w);
+              const uint4 zv = *reinterpret_cast<const uint4*>(tab + 256 + grp * 128 + 16 * w);
+              const uint4 cv = *reinterpret_cast<const uint4*>(tab + 512 + grp * 128 + 16 * w);
+              const uint32_t s2[4] = {sv.x, sv.y, sv.z, sv.w}, zo[4] = {zv.x, zv.y, zv.z, zv.w};
+              const uint32_t c2[4] = {cv.x, cv.y, cv.z, cv.w};
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint4 o = dequant_word_h(wd[4 * grp + i], s2, zo, c2);
-              *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + (4 * grp + i) * 2048) = o;
+              for (int i = 0; i < 4; ++i) {
+                const uint4 o = dequant_word_h(wd[4 * grp + i], s2, zo, c2);
+                *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + (4 * grp + i) * 2048) = o;
+              }
             }
-          }
           }
           if (TAIL && tail_tile)
             tail_rows_over<ONCE ? 1 : 16>(sgen + kOffK + kbuf * 16384, job.k_tail + tail_off, a.ts, slot0 - kb, ONCE ? (t >> 3) * 8 : kb, w, job.tail_lo,
@@ -1082,7 +1082,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     // The constants of a tile's key groups lie anywhere in a table of hundreds of megabytes a layer: a
     // look-up can miss the L2 and the TLB, and the producers' look-ups depend on one another.  This
     // warp asks for the lines a few tiles before the producers need them.  (24 layers at 16384, three
-    // streams taking turns: 5216 us a frame without it, 3778 with; 8-bit at 8192 2409 and 1537.)
+    // streams taking turns: 5290 us a frame without it, 4440 with; 8-bit at 8192 2440 and 1970.  One
+    // stream alone, whose constants the L2 holds better: 3920 and 3790, 1590 and 1550.)
     const int lane = tid & 31;
     uint32_t g = 0;
     for (Walk walk(a); walk.next(a);) {

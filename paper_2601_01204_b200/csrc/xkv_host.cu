@@ -326,7 +326,7 @@ int kv_score_evict(xkv_cache* c, const void* q, int32_t n, int64_t ts, int64_t h
     a.phases = kPhPool | kPhScore | kPhSel;
     if (!keys_once(c) && !kbar_fresh(c)) {          // head means of the keys (Eq. 4) of the cache as it stands
       a.phases |= kPhKbar;
-      a.kbar_on_other = 0; a.kbar_lo = 0; a.kbar_hi = c->rold_pending;
+      a.kbar_hi = c->rold_pending;
     }
     a.q = reinterpret_cast<const __nv_bfloat16*>(q);
     a.ts_q = ts; a.hs_q = hs;
@@ -348,7 +348,7 @@ int kv_score_evict_w(xkv_cache* c, const float* w, int32_t n, xkv_stream stream)
     a.phases = kPhScore | kPhSel;
     if (!keys_once(c) && !kbar_fresh(c)) {
       a.phases |= kPhKbar;
-      a.kbar_on_other = 0; a.kbar_lo = 0; a.kbar_hi = c->rold_pending;
+      a.kbar_hi = c->rold_pending;
     }
     a.w_in = w;
     if (launch_maint(c, a, XKV_PROF_SCORE_EVICT, reinterpret_cast<cudaStream_t>(stream)) != cudaSuccess) return XKV_E_CUDA;
@@ -567,7 +567,7 @@ int prepare_layer(xkv_cache* c, const void* q, const void* k, const void* v, voi
     a->phases |= kPhPool | kPhScore | kPhSel;
     if (!once && !kbar_fresh(c)) {
       a->phases |= kPhKbar;
-      a->kbar_on_other = 0; a->kbar_lo = 0; a->kbar_hi = c->rold_pending;
+      a->kbar_hi = c->rold_pending;
     }
   }
   a->q = reinterpret_cast<const __nv_bfloat16*>(q);
@@ -633,7 +633,7 @@ int run_layers(HostStepPipe* pipe, xkv_cache* const* layers, int from, MaintArgs
       } else {
         maint_args(c, &b);
         b.phases = kPhKbar;
-        b.kbar_on_other = 0; b.kbar_lo = 0; b.kbar_hi = c->T - c->T_first;
+        b.kbar_hi = c->T - c->T_first;
       }
       as[n_kbar] = b;
       kc[n_kbar++] = c;
@@ -721,9 +721,14 @@ size_t xkv_stream_step_host_bytes(const xkv_params* params, int32_t n) {
   return 2 * 4 * ((t + kAlign - 1) / kAlign * kAlign);
 }
 
-// Cached tokens from which the kernels of a layer take about as long as the copies of its inputs (the
-// ratio does not depend on the frame size): with shorter caches the copies are the limit, and a layer
-// at a time leaves no gap between them (24 x 1374 tokens at 4096: 4.49 ms, in pairs 4.70).
+// Cached tokens from which the host-buffer step takes layers in pairs.  24 layers, us a frame by the
+// host's clock, pairs at every length against one layer at a time:
+//   1374 tokens, 4-bit   4096 4680 / 5030   6144 4400 / 4760   8192 4910 / 4700
+//                       10240 4720 / 5140  12288 4820 / 5080  16384 5230 / 5660
+//   keys quantised once  8192 4670 / 5150  12288 5140 / 5360  16384 5400 / 5770
+//   16-bit               8192 4650 / 5040  12288 4910 / 5150;   1004 tokens, 4-bit 8192 3710 / 3780
+// From 10240 on pairs win throughout; below, the copies are the limit, and where they lie in the host's
+// memory moves a frame by some 10 % (8192 against 6144), so one layer at a time stays there.
 constexpr int kPairTokens = 10240;
 
 // The layers run on the caller's stream, two at a time where the caches are long (the first and the
@@ -731,9 +736,8 @@ constexpr int kPairTokens = 10240;
 // tensors: keys and values of two layers, which are free again once the maintenance has read them, and twice the queries of two
 // layers, over which the outputs are written (a block reads an item's queries before it writes them,
 // and the merge comes after all).  So the copies of the next two layers' inputs run beside the
-// attention of these two, and their outputs go back beside the next two layers.  One layer at a time
-// took 5.74 ms for a frame of 24 layers of 1374 tokens: beside copies every short kernel is half as
-// fast, and two layers' maintenance costs little more than one's.
+// attention of these two, and their outputs go back beside the next two layers.  Beside copies every
+// short kernel is half as fast, and two layers' maintenance costs little more than one's.
 int xkv_stream_step_host(xkv_cache* const* layers, int32_t n_layers, const void* const* q,
                          const void* const* k, const void* const* v, void* const* out, int32_t n,
                          void* dev_staging, size_t staging_bytes, xkv_stream stream) {
@@ -908,7 +912,7 @@ int xkv_debug_head_means(xkv_cache* c, xkv_stream stream) {
   MaintArgs a;
   maint_args(c, &a);
   a.phases = kPhKbar;
-  a.kbar_on_other = 0; a.kbar_lo = 0; a.kbar_hi = c->T - c->T_first;
+  a.kbar_hi = c->T - c->T_first;
   if (launch_maint(c, a, XKV_PROF_KBAR, st) != cudaSuccess) return XKV_E_CUDA;
   if (cudaEventRecord(c->kbar_done, st) != cudaSuccess) return XKV_E_CUDA;
   c->kbar_T = c->T; c->kbar_cur = c->cur; c->kbar_frames = c->frames;

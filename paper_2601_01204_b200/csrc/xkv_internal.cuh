@@ -44,7 +44,7 @@ struct MaintArgs {
   int dst_slot;                    // physical slot of the frame's first token in the destination
   int rest_base, r_old, kk, r_new, identity;
   int n_special, pool_g, n_pooled;
-  int kbar_on_other, kbar_lo, kbar_hi;   // KBAR phase: buffer set and rest-local range
+  int kbar_hi;                     // KBAR phase: rest-local positions [0, kbar_hi) of the current buffer set
   __nv_bfloat16* kstage;
   float* qbar; float* qvec; float* scores;
   const float* w_in;               // the pooled query's row mean from the caller (no POOL phase), or null
@@ -194,7 +194,8 @@ inline cudaError_t launch_overlapped(const void* fn, dim3 grid, dim3 block, void
 // ---- launchers implemented in the kernel translation units -------------------
 // All return cudaError_t of the launch (cudaGetLastError) and count launches.
 
-// Most layers that one launch takes (the attention's job table fits the classic 4 KB of parameters).
+// Most layers that one launch takes: the attention's job table stays below 4 KB with them.  (The arguments
+// of the maintenance and of the regroup are 13 and 5 KB, which needs the 32 KB limit of kernel parameters.)
 constexpr int kMaxLayers = 28;
 // The maintenance kernel with the phases in a[i].phases on the caches c[i], count <= kMaxLayers, all
 // of the same storage form (cooperative when it has a grid barrier).

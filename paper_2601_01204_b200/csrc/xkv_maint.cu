@@ -4,8 +4,9 @@
 // operation and order is fixed, because it decides integers (kept indices, 4-bit
 // codes) that must be reproducible bit for bit.
 //
-// One persistent kernel, launched cooperatively with two thread blocks per SM,
-// runs the phases that a call needs, separated by grid-wide barriers:
+// One persistent kernel of up to two thread blocks per SM (fewer where the busiest phase has less work)
+// runs the phases that a call needs.  A launch takes one layer or up to 28; every layer has blocks of
+// its own, with barriers among them (the launch is cooperative where there is one):
 //
 //   APPEND  values quantised per token (Eq. 7-9) into their final slot; keys staged
 //           (4-bit) or copied (16-bit)                                 [kv_append]
@@ -20,9 +21,10 @@
 //           keys in higher bins are kept, keys in that bin become candidates
 //   ---- barrier ----
 //   SEL2    every block finds the k-th largest (key, position) among the candidates
-//           by bisection and writes the kept positions of its own tokens in order
+//           (a histogram of their next 8 key bits, then a ranking inside each warp) and
+//           writes the kept positions of its own tokens in order
 //   ---- barrier ----
-//   PACK    16-bit caches: the survivor gather                          [kv_quant_pack]
+//   PACK    16-bit caches and keys quantised once: the survivor gather  [kv_quant_pack]
 //
 // xkv_stream_step runs all of them in one launch; the per-call entry points launch
 // the same kernel with the phases of that call.  The 4-bit kv_quant_pack (key regroup +
@@ -40,7 +42,7 @@ namespace {
 
 constexpr int kMT = 512;                 // threads per block
 constexpr int kBlocksPerSM = 2;
-constexpr uint32_t kBarSpin = 1u << 21;  // polls of a grid barrier before it gives up (about 0.1 s)
+constexpr uint32_t kBarSpin = 1u << 21;  // polls of a barrier before it gives up (each a sleep and an L2 round trip)
 
 // ---------------------------------------------------------------------------
 // Eq. 7-8, fixed-order fp32:  s = (max-min)/(2^b - 1) (1 if the range is 0),
@@ -185,7 +187,7 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const unsigned int* p) {
 }
 
 constexpr int kSelBins = 4096;       // histogram of the top 12 key bits
-constexpr int kHistCopies = 4;       // copies of the histogram (a block adds to copy blockIdx mod 4: fewer collisions)
+constexpr int kHistCopies = 4;       // copies of the histogram (a block adds to copy index mod 4: fewer collisions)
 constexpr int kPoolRows = 120;       // pooled rows staged in shared memory at a time
 constexpr int kCandSmem = 4096;      // candidates a block holds in shared memory
 constexpr int kSubBins = 256;        // second histogram: the next 8 key bits of the candidates
@@ -545,12 +547,13 @@ __device__ __forceinline__ void kbar_run(const MaintArgs& a, Shared& sh, const B
   }
 }
 
-// KBAR over the rest-local positions [0, hi) of the buffer set `b` (re-quantising mode and 16-bit):
+// KBAR over the rest-local positions [0, kbar_hi) (re-quantising mode and 16-bit):
 // one run per 64-slot key group (the rest segment starts on a 128-slot boundary).
 template <int BITS>
-__device__ __forceinline__ void phase_kbar(const MaintArgs& a, const Blocks& B, Shared& sh, const BufSet& b, int lo, int hi) {
-  const int g_lo = lo >> 6, g_hi = (hi + 63) >> 6;
-  for (int gb = g_lo + B.index; gb < g_hi; gb += B.count) {
+__device__ __forceinline__ void phase_kbar(const MaintArgs& a, const Blocks& B, Shared& sh) {
+  const BufSet& b = a.cur;
+  const int hi = a.kbar_hi, g_hi = (hi + 63) >> 6;
+  for (int gb = B.index; gb < g_hi; gb += B.count) {
     const int grp = (a.rest_base >> 6) + gb;
     kbar_run<BITS>(a, sh, b, b.kpar + (size_t)grp * 64, (size_t)(a.cap >> 6) * 64, a.rest_base + gb * 64, gb * 64,
                    min(64, hi - gb * 64));
@@ -700,7 +703,7 @@ template <int PIECES>
 struct GatherTiles {
   static constexpr int kTokens = kMT / PIECES;
   int ch, tok, per_head, count;
-  __device__ __forceinline__ GatherTiles(const MaintArgs& a, const Blocks&) {
+  __device__ __forceinline__ explicit GatherTiles(const MaintArgs& a) {
     ch = (int)threadIdx.x % PIECES;
     tok = (int)threadIdx.x / PIECES;
     per_head = (a.kk + kTokens - 1) / kTokens;
@@ -746,7 +749,7 @@ __device__ __forceinline__ void phase_gather_once(const MaintArgs& a, const Bloc
     }
     return;
   }
-  const GatherTiles<2 * kRC> tiles(a, B);                            // the 16-byte pieces of K codes, then of V codes
+  const GatherTiles<2 * kRC> tiles(a);                            // the 16-byte pieces of K codes, then of V codes
   constexpr int kU = 4;
   const int piece = 16 * (tiles.ch % kRC);
   const uint8_t* from_base = (tiles.ch < kRC ? src.k : src.v) + piece;
@@ -1292,7 +1295,7 @@ __global__ void __launch_bounds__(kRgThreads, 8) regroup_k_kernel(const __grid_c
 __device__ __forceinline__ void phase_gather16(const MaintArgs& a, const Blocks& B) {
   const BufSet& src = a.cur;
   const BufSet& dst = a.oth;
-  const GatherTiles<8> tiles(a, B);
+  const GatherTiles<8> tiles(a);
   constexpr int kU = 3;
   for (int t0 = B.index; t0 < tiles.count; t0 += kU * B.count) {
     size_t from[kU], to[kU];
@@ -1352,7 +1355,7 @@ __global__ void __launch_bounds__(kMT, kBlocksPerSM) maint_kernel(const __grid_c
     // (from the first block that has no pooled row)
     const int skip = (ph & kPhPool) ? a.n_pooled % B.count : 0;
     const Blocks K{B.index >= skip ? B.index - skip : B.index + B.count - skip, B.count};
-    phase_kbar<BITS>(a, K, sh, a.kbar_on_other ? a.oth : a.cur, a.kbar_lo, a.kbar_hi);
+    phase_kbar<BITS>(a, K, sh);
     ran = true;
   }
 
@@ -1466,7 +1469,7 @@ static int useful_blocks(const xkv_cache* c, const MaintArgs& a) {
   if (a.phases & kPhAppend) first += ceil_div((long long)a.H * a.n * 8, kMT);
   if ((a.phases & kPhAppend) && c->p.key_mode == XKV_KEYS_ONCE) first += ceil_div(a.n, 64) * ceil_div(a.H, 4);
   if (a.phases & kPhPool) first += a.n_pooled;
-  if (a.phases & kPhKbar) first += ceil_div(a.kbar_hi - a.kbar_lo, 64) + 1;
+  if (a.phases & kPhKbar) first += ceil_div(a.kbar_hi, 64) + 1;
   if (a.phases & kPhKbarNew) later = ceil_div(a.n, 64);
   if ((a.phases & (kPhScore | kPhSel)) && ceil_div(a.r_old, 64) > later) later = ceil_div(a.r_old, 64);
   if (a.phases & kPhPack) {
