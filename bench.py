@@ -27,9 +27,9 @@ WORKLOAD = dict(name="full_stack_24L_1374tok_budget16384_int4", layers=24, n_hea
                 n_tokens=1374, budget=16384, kv_bits=4, n_special=5, pool_g=16, quant_group=64, seed=3)
 METRIC = "stream frames/s (24-layer compressed-KV attention)"
 UNIT = "frames/s"
-# dram__bytes_read.sum + dram__bytes_write.sum of one attention launch for one layer, from the ncu capture
-# summarised under profiles/ (None until a capture of the current kernel exists).
-ATTN_DRAM_TRAFFIC_BYTES = 23.3e6
+# dram__bytes_read.sum + dram__bytes_write.sum of the attention per layer: a quarter of the launch for four
+# layers whose ncu capture is summarised under profiles/.
+ATTN_DRAM_TRAFFIC_BYTES = 31.0e6
 
 
 def _peaks() -> dict:
