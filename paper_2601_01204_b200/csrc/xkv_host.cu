@@ -92,6 +92,14 @@ Layout make_layout(const xkv_params* p) {
 bool strides_ok(int64_t ts, int64_t hs) { return ts >= kHeadDim && (ts % 8) == 0 && hs >= 0 && (hs % 8) == 0; }
 bool aligned16(const void* p) { return p && (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Orders `st` after the head means that the last stream step of the cache started on the library's
+// stream.  If that step was captured its event belongs to the graph and can't be waited for: whoever
+// launches the graph orders it.  (That error must not stay behind for the next launch to find; a fault
+// of the context shows at the next call all the same.)
+void after_head_means(const xkv_cache* c, cudaStream_t st) {
+  if (c->kbar_done && cudaStreamWaitEvent(st, c->kbar_done, 0) != cudaSuccess) cudaGetLastError();
+}
+
 int zero_workspace(xkv_cache* c, cudaStream_t st) {
   if (cudaMemsetAsync(c->ws, 0, c->ws_bytes, st) != cudaSuccess) return XKV_E_CUDA;
   if (c->p.key_mode == XKV_KEYS_ONCE && launch_once_init(c, st) != cudaSuccess) return XKV_E_CUDA;
@@ -183,8 +191,7 @@ int xkv_create(const xkv_params* params, void* dev_workspace, size_t bytes, xkv_
 int xkv_reset(xkv_cache* c, xkv_stream stream) {
   if (!c) return XKV_E_INVALID;
   // a head-mean kernel of the last stream step may still run on the library's stream
-  if (c->kbar_done && cudaStreamWaitEvent(reinterpret_cast<cudaStream_t>(stream), c->kbar_done, 0) != cudaSuccess)
-    return XKV_E_CUDA;
+  after_head_means(c, reinterpret_cast<cudaStream_t>(stream));
   reset_host_state(c);
   return zero_workspace(c, reinterpret_cast<cudaStream_t>(stream));
 }
@@ -196,7 +203,10 @@ int xkv_destroy(xkv_cache* c) {
     for (auto& e : c->prof->pool) cudaEventDestroy(e);
     delete c->prof;
   }
-  if (c->kbar_done) { cudaEventSynchronize(c->kbar_done); cudaEventDestroy(c->kbar_done); }
+  if (c->kbar_done) {
+    if (cudaEventSynchronize(c->kbar_done) != cudaSuccess) cudaGetLastError();      // (as above)
+    cudaEventDestroy(c->kbar_done);
+  }
   delete c;
   return XKV_OK;
 }
@@ -908,7 +918,7 @@ int xkv_debug_head_means(xkv_cache* c, xkv_stream stream) {
   if (c->stage != 0) return XKV_E_STATE;
   if (c->T <= c->T_first || keys_once(c)) return XKV_OK;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  if (c->kbar_done && cudaStreamWaitEvent(st, c->kbar_done, 0) != cudaSuccess) return XKV_E_CUDA;
+  after_head_means(c, st);
   MaintArgs a;
   maint_args(c, &a);
   a.phases = kPhKbar;

@@ -279,3 +279,39 @@ def test_16bit_weights_are_normalised_as_they_are_multiplied(xkv, layers):
         bound = 1.1 * float(torch.sqrt(rounding ** 2 + r2 * var / ref.norm() ** 2))
         err = float((out[l].double() - ref).norm() / ref.norm())
         assert err <= bound, (l, err, bound)
+
+
+@pytest.mark.parametrize("bits, once", [(4, 0), (4, 1), (16, 0)])
+def test_steps_captured_into_graphs(xkv, bits, once):
+    """Every step from the third on captured into a graph of its own and launched once: outputs and state of
+    the plain steps bit for bit.  Afterwards the caches reset, and others are created, as ever."""
+    import torch
+    p = xkv.Params(n_heads=H, budget=700, max_frame_tokens=200, kv_bits=bits, key_mode=once)
+    graphed, plain = ([xkv.Cache(p) for _ in range(3)] for _ in range(2))
+    for t in range(7):
+        q, k, v = zip(*(frame(l, t, 200) for l in range(3)))
+        outs = [[torch.zeros_like(x) for x in q] for _ in range(2)]
+        if t < 3:
+            xkv.xkv_stream_step(graphed, q, k, v, outs[0])
+        else:
+            torch.cuda.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph):
+                xkv.xkv_stream_step(graphed, q, k, v, outs[0])
+            graph.replay()
+        xkv.xkv_stream_step(plain, q, k, v, outs[1])
+        torch.cuda.synchronize()
+        for l in range(3):
+            assert torch.equal(outs[0][l].view(torch.int16), outs[1][l].view(torch.int16)), (t, l)
+            compare_state(graphed[l].export(), plain[l].export(), f"frame {t} layer {l}")
+    assert graphed[0].xkv_get_info().last_evicted > 0
+    graphed[0].xkv_reset()
+    for c in graphed[1:]:
+        c.close()
+    again = [graphed[0], xkv.Cache(p)]
+    fresh = [xkv.Cache(p) for _ in range(2)]
+    q, k, v = zip(*(frame(l, 0, 200) for l in range(2)))
+    for caches in (again, fresh):
+        xkv.xkv_stream_step(caches, q, k, v, [torch.empty_like(x) for x in q])
+    for a, b in zip(again, fresh):
+        compare_state(a.export(), b.export(), "after the graphs")
