@@ -77,8 +77,8 @@ attn_simple_kernel(const __nv_bfloat16* __restrict__ q, __nv_bfloat16* __restric
             vx[j] = vp.x * ((float)((vws[j >> 2] >> sh) & 0xFFu) - vp.y);
           }
         } else {
-          const uint4 ku = *reinterpret_cast<const uint4*>(buf.k + slot * 128 + 16 * w);
-          const uint4 vu = *reinterpret_cast<const uint4*>(buf.v + slot * 128 + 16 * w);
+          const uint4 ku = *reinterpret_cast<const uint4*>(buf.k + slot * 128 + 16 * (w ^ (int)(slot & 7)));
+          const uint4 vu = *reinterpret_cast<const uint4*>(buf.v + slot * 128 + 16 * (w ^ (int)(slot & 7)));
           const uint32_t kr[4] = {ku.x, ku.y, ku.z, ku.w};
           const uint32_t vr[4] = {vu.x, vu.y, vu.z, vu.w};
 #pragma unroll

@@ -15,7 +15,7 @@
 //               them, exchanges it with the other half, and writes P (16-bit) back to tensor memory.
 //               O is rescaled only when the running maximum grew by more than 2^14.  Registers move to
 //               these warps with setmaxnreg.
-//   4 warps     operand producers: packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
+//   4 warps     operand producers (4 and 8 bits): packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
 //               and key group) and V~ (per token) in the 128-byte-swizzled layouts the MMA
 //               descriptors expect.  One dequantised tile serves both query tiles.
 //   2 warps     issue the MMAs of query tile 0 resp. 1 through an elected lane:
@@ -31,7 +31,8 @@
 //               else idle.
 // 4-bit caches multiply in fp16 (the dequantised keys are not bf16-representable:
 // rounding them to bf16 alone costs ~1e-2 relative L2 with outlier channels);
-// 16-bit caches hold bf16 and multiply in bf16.  Accumulation is fp32.
+// 16-bit caches hold bf16 rows in the operands' order, which the copies bring to the operand tiles, and multiply in
+// bf16.  Accumulation is fp32.
 //
 // Every mbarrier wait is bounded (one second of running time): when the bound is hit the CTA carries on
 // without waiting and records XKV_E_TIMEOUT in the status words of the caches in its piece, so the
@@ -54,8 +55,8 @@ constexpr int kThreads = 768;
 constexpr int kRegsSoftmax = 96;
 // (24 layers at 16384 tokens: tail 3535 us with 56 + 40, 3421 with 64 + 32; keys once 3688 with 56 + 40,
 // 3897 with 48 + 48)
-__host__ __device__ constexpr int regs_producers(int bits, bool once, bool tail) { return tail ? 64 : (once || bits == 16) ? 56 : 48; }
-__host__ __device__ constexpr int regs_misc(int bits, bool once, bool tail) { return 96 - regs_producers(bits, once, tail); }   // MMA issuers, copy thread
+__host__ __device__ constexpr int regs_producers(bool once, bool tail) { return tail ? 64 : once ? 56 : 48; }
+__host__ __device__ constexpr int regs_misc(bool once, bool tail) { return 96 - regs_producers(once, tail); }   // MMA issuers, copy thread
 constexpr int kQRows = 128;
 constexpr int kMaxGrid = 160;                 // CTAs the scratch is sized for (>= SM count of the part)
 constexpr uint32_t kSpinLimit = 1u << 22;
@@ -65,40 +66,45 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 // few tiles.
 constexpr float kGrow = 14.f;
 
-// ring depths
-constexpr int kNK = 3;                        // dequantised K~ tiles
-constexpr int kNV = 3;                        // dequantised V~ tiles
 constexpr uint32_t kAhead = 4;        // tiles whose constants are asked for ahead of the producers (keys quantised once)
 
+// ring depths: kNK, kNV operand tiles of K~ and V~, kNR raw stages
 template <int BITS> struct Cfg;
 template <> struct Cfg<4> {
+  static constexpr int kNK = 3, kNV = 3;
   static constexpr int kNR = 4;               // raw stages
   static constexpr int kRawK = 4096, kRawV = 4096, kRawKP = 1024, kRawVP = 1024;
   static constexpr int kRawStage = kRawK + kRawV + kRawKP + kRawVP;
 };
 template <> struct Cfg<8> {                    // 8-bit codes, keys quantised once: K, V rows of 64 bytes,
+  static constexpr int kNK = 3, kNV = 3;
   static constexpr int kNR = 4;               // 128 group references (in the K-parameter region), V parameters
   static constexpr int kRawK = 8192, kRawV = 8192, kRawKP = 1024, kRawVP = 1024;
   static constexpr int kRawStage = kRawK + kRawV + kRawKP + kRawVP;
 };
-template <> struct Cfg<16> {
-  static constexpr int kNR = 2;
+// 16-bit caches: no raw stages and no work for the producers, whose copies within shared memory (64 KB a tile, read and
+// written) cost time and, at the power cap, clock.  24 layers, 1374 tokens at 32768: 8047 -> 7887 us a step.
+template <> struct Cfg<16> {                   // rows are stored as the MMA wants them (BufSet): the copies fill the
+  static constexpr int kNK = 4, kNV = 4;      // operand tiles themselves
+  static constexpr int kNR = 1;               // (no raw stages: two unused barriers)
   static constexpr int kRawK = 16384, kRawV = 16384, kRawKP = 0, kRawVP = 0;
-  static constexpr int kRawStage = kRawK + kRawV;
+  static constexpr int kRawStage = 0;
 };
 
 // shared memory map (offsets from a 1024-byte aligned base)
 constexpr int kOffQ = 0;                          // 2 x 16 KB  Q tiles, K-major, SW128
 constexpr int kOffK = 32768;                      // kNK x 16 KB  K~ tiles
-constexpr int kOffV = kOffK + kNK * 16384;        // kNV x 16 KB  V~ tiles
-constexpr int kOffTab = kOffV + kNV * 16384;      // 2 x (K table 768 B + V table 2048 B) fp16 parameters
-constexpr int kTabBytes = 768 + 2048;
-constexpr int kOffBar = kOffTab + 2 * kTabBytes;  // barriers, tmem base, abort flag
-constexpr int kBarBytes = 512;
-constexpr int kOffRaw = kOffBar + kBarBytes;      // raw stages (16-byte aligned)
+constexpr int kTabBytes = 768 + 2048;             // K table 768 B + V table 2048 B of fp16 parameters
+constexpr int kBarBytes = 512;                    // barriers, tmem base, abort flag
+template <int BITS> struct Map {
+  static constexpr int kOffV = kOffK + Cfg<BITS>::kNK * 16384;          // kNV x 16 KB  V~ tiles
+  static constexpr int kOffTab = kOffV + Cfg<BITS>::kNV * 16384;        // two tables (512 bytes that keep the alignment in 16-bit caches)
+  static constexpr int kOffBar = kOffTab + (BITS == 16 ? 512 : 2 * kTabBytes);
+  static constexpr int kOffRaw = kOffBar + kBarBytes;                   // raw stages (16-byte aligned)
+};
 constexpr int kXchgBytes = 6144;                  // split softmax: values exchanged between the two halves of a row
 template <int BITS> constexpr int smem_bytes() {
-  return kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + kXchgBytes + 1024;
+  return Map<BITS>::kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + kXchgBytes + 1024;
 }
 
 // Tensor memory columns (all 512).  A query tile has three blocks of 64 columns, B0 B1 B2.  In even
@@ -576,9 +582,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   using C = Cfg<BITS>;
   constexpr int kSW = 16;                    // softmax warps
   constexpr uint32_t kRowThreads = 256;      // threads that work on one query tile
+  constexpr int kNK = C::kNK, kNV = C::kNV;
+  constexpr int kOffV = Map<BITS>::kOffV, kOffTab = Map<BITS>::kOffTab, kOffBar = Map<BITS>::kOffBar, kOffRaw = Map<BITS>::kOffRaw;
   constexpr int kOffX = kOffRaw + C::kNR * C::kRawStage;   // exchange area of the split softmax
   static_assert(kOffX % 1024 == 0, "the halves' places differ in one address bit");
-  constexpr int kRegProd = regs_producers(BITS, ONCE, TAIL), kRegMisc = regs_misc(BITS, ONCE, TAIL);
+  constexpr int kRegProd = regs_producers(ONCE, TAIL), kRegMisc = regs_misc(ONCE, TAIL);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t* sgen = smem_raw + (sbase - smem_u32(smem_raw));
@@ -607,8 +615,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   if (tid == 0) {
     *abort_flag = 0;           // (the status words are older launches' too: they say nothing about this one)
     st_shared_u32(s_progress, 0u);
-    for (int i = 0; i < kNK; ++i) { mbar_init(b_kfull + 8 * i, 128); mbar_init(b_kfree + 8 * i, 2); }
-    for (int i = 0; i < kNV; ++i) { mbar_init(b_vfull + 8 * i, 128); mbar_init(b_vfree + 8 * i, 2); }
+    for (int i = 0; i < kNK; ++i) { mbar_init(b_kfull + 8 * i, BITS == 16 ? 1 : 128); mbar_init(b_kfree + 8 * i, 2); }
+    for (int i = 0; i < kNV; ++i) { mbar_init(b_vfull + 8 * i, BITS == 16 ? 1 : 128); mbar_init(b_vfree + 8 * i, 2); }
     for (int i = 0; i < C::kNR; ++i) { mbar_init(b_rfull + 8 * i, 1); mbar_init(b_rfree + 8 * i, 128); }
     for (int t = 0; t < 2; ++t) {
       mbar_init(b_qfull + 8 * t, kRowThreads); mbar_init(b_sfull + 8 * t, 1);
@@ -840,7 +848,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     const int kb = t >> 3;        // keys kb + 16 i
     const uint32_t row_off = (uint32_t)((kb >> 3) * 1024 + (kb & 7) * 128 + ((w ^ (kb & 7)) << 4));
     uint32_t g = 0;               // steps so far (ring positions)
-    for (Walk walk(a); walk.next(a);) {
+    for (Walk walk(a); BITS != 16 && walk.next(a);) {
       const Job& job = a.job[walk.job];
       const int tile_lo = walk.tile_lo, nt = walk.nt;
       const int h = walk.h;
@@ -986,25 +994,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           fence_proxy_async();
           mbar_arrive(b_vfull + 8 * vbuf);
           mbar_arrive(b_rfree + 8 * rs);
-        } else {
-          uint4 rowk[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) rowk[i] = *reinterpret_cast<const uint4*>(raw + (kb + 16 * i) * 128 + 16 * w);
-          mbar_wait<kSlack>(b_kfree + 8 * kbuf, (ku & 1) ^ 1, wc);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(sgen + kOffK + kbuf * 16384 + row_off + i * 2048) = rowk[i];
-          fence_proxy_async();
-          mbar_arrive(b_kfull + 8 * kbuf);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) rowk[i] = *reinterpret_cast<const uint4*>(raw + C::kRawK + (kb + 16 * i) * 128 + 16 * w);
-          mbar_wait<kSlack>(b_vfree + 8 * vbuf, (vu & 1) ^ 1, wc);
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            *reinterpret_cast<uint4*>(sgen + kOffV + vbuf * 16384 + row_off + i * 2048) = rowk[i];
-          fence_proxy_async();
-          mbar_arrive(b_vfull + 8 * vbuf);
-          mbar_arrive(b_rfree + 8 * rs);
         }
       }
     }
@@ -1116,12 +1105,22 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       const size_t head_slot = (size_t)h * job.cap;
       for (int jj = 0; jj < nt; ++jj, ++g) {
         const int tile = tile_lo + jj;
+        const size_t slot0 = head_slot + (size_t)tile * 128;
+        if (BITS == 16) {
+          const uint32_t ks = g % kNK, vs = g % kNV;
+          mbar_wait<kSlack>(b_kfree + 8 * ks, ((g / kNK) & 1) ^ 1, wc);
+          mbar_expect_tx(b_kfull + 8 * ks, C::kRawK);
+          tma_load_1d(sK + ks * 16384, job.k + slot0 * 128, C::kRawK, b_kfull + 8 * ks);
+          mbar_wait<kSlack>(b_vfree + 8 * vs, ((g / kNV) & 1) ^ 1, wc);
+          mbar_expect_tx(b_vfull + 8 * vs, C::kRawV);
+          tma_load_1d(sV + vs * 16384, job.v + slot0 * 128, C::kRawV, b_vfull + 8 * vs);
+          continue;
+        }
         const uint32_t rs = g % C::kNR, ru = g / C::kNR;
         mbar_wait<kSlack>(b_rfree + 8 * rs, (ru & 1) ^ 1, wc);
         const uint32_t dst = sRaw + rs * C::kRawStage, bar = b_rfull + 8 * rs;
         const uint32_t kp_bytes = ONCE ? 512u : (uint32_t)C::kRawKP;    // 128 group references instead of 2 x 64 parameters
         mbar_expect_tx(bar, C::kRawStage - C::kRawKP + kp_bytes);
-        const size_t slot0 = head_slot + (size_t)tile * 128;
         if (BITS == 4) {
           tma_load_1d(dst, job.k + slot0 * 32, C::kRawK, bar);
           tma_load_1d(dst + C::kRawK, job.v + slot0 * 32, C::kRawV, bar);
@@ -1133,21 +1132,21 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           tma_load_1d(dst + C::kRawK, job.v + slot0 * 64, C::kRawV, bar);
           tma_load_1d(dst + C::kRawK + C::kRawV, job.kslot + (size_t)tile * 128, kp_bytes, bar);
           tma_load_1d(dst + C::kRawK + C::kRawV + C::kRawKP, job.vpar + slot0, C::kRawVP, bar);
-        } else {
-          tma_load_1d(dst, job.k + slot0 * 128, C::kRawK, bar);
-          tma_load_1d(dst + C::kRawK, job.v + slot0 * 128, C::kRawV, bar);
         }
       }
     }
     // Drain: every copy this thread started has landed once the last use of each stage completed
     // (bounded, and not cut short by the abort flag, so that nothing is in flight at exit).
     const uint32_t issued = g;
-    for (uint32_t i = 0; i < (uint32_t)C::kNR && i < issued; ++i) {
-      const uint32_t gi = issued - 1 - i;
-      const uint32_t rs = gi % C::kNR, ru = gi / C::kNR;
-      for (uint32_t it = 0; it < kSpinLimit; ++it)
-        if (mbar_try(b_rfull + 8 * rs, ru & 1)) break;
-    }
+    auto drain = [&](uint32_t full, uint32_t stages) {
+      for (uint32_t i = 0; i < stages && i < issued; ++i) {
+        const uint32_t gi = issued - 1 - i;
+        for (uint32_t it = 0; it < kSpinLimit; ++it)
+          if (mbar_try(full + 8 * (gi % stages), (gi / stages) & 1)) break;
+      }
+    };
+    if (BITS == 16) { drain(b_kfull, kNK); drain(b_vfull, kNV); }
+    else drain(b_rfull, C::kNR);
   }
   __syncthreads();
   if (tid == 0 && *abort_flag) report_timeout(a);
@@ -1247,7 +1246,7 @@ static cudaError_t prepare_kernel() {
   e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
   const int warps_per_scheduler = kThreads / 32 / 4;
-  return (fa.numRegs * warps_per_scheduler >= 4 * kRegsSoftmax + regs_producers(BITS, ONCE, TAIL) + regs_misc(BITS, ONCE, TAIL))
+  return (fa.numRegs * warps_per_scheduler >= 4 * kRegsSoftmax + regs_producers(ONCE, TAIL) + regs_misc(ONCE, TAIL))
              ? cudaSuccess : cudaErrorLaunchOutOfResources;
 }
 

@@ -881,6 +881,17 @@ int64_t xkv_debug_export(const xkv_cache* c, int32_t which, void* host_dst, size
     default: return XKV_E_INVALID;
   }
   const size_t nbytes = bytes < avail ? bytes : avail;
+  if (nbytes && c->p.kv_bits == 16 && (which == XKV_BUF_K_CODES || which == XKV_BUF_V_CODES)) {
+    // rows in channel order, whole ones through a buffer of their own (the caller's may end inside one)
+    std::vector<uint8_t> rows;
+    try { rows.resize((nbytes + 127) / 128 * 128); } catch (const std::bad_alloc&) { return XKV_E_NOMEM; }
+    if (cudaMemcpy(rows.data(), src, rows.size(), cudaMemcpyDeviceToHost) != cudaSuccess) return XKV_E_CUDA;
+    for (size_t at = 0; at < nbytes; at += 16) {
+      const size_t row = at / 128, w = at % 128 / 16;
+      memcpy(static_cast<uint8_t*>(host_dst) + at, rows.data() + row * 128 + 16 * (w ^ (row & 7)), nbytes - at < 16 ? nbytes - at : 16);
+    }
+    return (int64_t)nbytes;
+  }
   if (nbytes && cudaMemcpy(host_dst, src, nbytes, cudaMemcpyDeviceToHost) != cudaSuccess) return XKV_E_CUDA;
   return (int64_t)nbytes;
 }

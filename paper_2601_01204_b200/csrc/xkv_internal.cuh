@@ -19,6 +19,8 @@ constexpr int kWordsPerRow = 8;       // 32-bit words of one packed 4-bit row (6
 
 // One of the two buffer sets of a cache (physical layout, see xkv.h).
 struct BufSet {
+  // 16-bit rows (128 bytes): the 16-byte piece of channels 8w..8w+7 of slot s lies at place w ^ (s mod 8), so
+  // that a tile copied as it is has the 128-byte swizzle that the attention's matrix operands want.
   uint8_t* k;        // [H][cap][row_bytes]
   float2* kpar;      // [H][cap/64][64]   (scale, zero)
   uint8_t* v;        // [H][cap][row_bytes]

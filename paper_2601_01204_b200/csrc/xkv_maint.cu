@@ -319,11 +319,12 @@ __device__ __forceinline__ void phase_append(const MaintArgs& a, const Blocks& B
     const size_t slot = (size_t)h * a.cap + a.dst_slot + tok;
     if (BITS == 16) {
       if (valid) {
-        *reinterpret_cast<uint4*>(d0.k + slot * 128 + 16 * w) = kv;
-        *reinterpret_cast<uint4*>(d0.v + slot * 128 + 16 * w) = vv;
+        const size_t at = slot * 128 + 16 * (w ^ (int)(slot & 7));
+        *reinterpret_cast<uint4*>(d0.k + at) = kv;
+        *reinterpret_cast<uint4*>(d0.v + at) = vv;
         if (two) {
-          *reinterpret_cast<uint4*>(d1.k + slot * 128 + 16 * w) = kv;
-          *reinterpret_cast<uint4*>(d1.v + slot * 128 + 16 * w) = vv;
+          *reinterpret_cast<uint4*>(d1.k + at) = kv;
+          *reinterpret_cast<uint4*>(d1.v + at) = vv;
         }
       }
     } else {
@@ -517,7 +518,7 @@ __device__ __forceinline__ void kbar_run(const MaintArgs& a, Shared& sh, const B
         if (BITS == 4) word[u] = 0u; else wide[u] = make_uint4(0, 0, 0, 0);
         if (valid && h < H) {
           if (BITS == 4) word[u] = __ldcg(reinterpret_cast<const uint32_t*>(b.k + ((size_t)h * cap + slot) * 32 + 4 * w));
-          else wide[u] = __ldcg(reinterpret_cast<const uint4*>(b.k + ((size_t)h * cap + slot) * 128 + 16 * w));
+          else wide[u] = __ldcg(reinterpret_cast<const uint4*>(b.k + ((size_t)h * cap + slot) * 128 + 16 * (w ^ (slot & 7))));
         }
       }
 #pragma unroll
@@ -1319,15 +1320,17 @@ __device__ __forceinline__ void phase_gather16(const MaintArgs& a, const Blocks&
     for (int u = 0; u < kU; ++u) {
       k[u] = v[u] = make_uint4(0, 0, 0, 0);
       if (ok[u]) {
-        k[u] = *reinterpret_cast<const uint4*>(src.k + from[u] * 128 + 16 * tiles.ch);
-        v[u] = *reinterpret_cast<const uint4*>(src.v + from[u] * 128 + 16 * tiles.ch);
+        const size_t at = from[u] * 128 + 16 * (tiles.ch ^ (int)(from[u] & 7));
+        k[u] = *reinterpret_cast<const uint4*>(src.k + at);
+        v[u] = *reinterpret_cast<const uint4*>(src.v + at);
       }
     }
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
       if (!ok[u]) continue;
-      *reinterpret_cast<uint4*>(dst.k + to[u] * 128 + 16 * tiles.ch) = k[u];
-      *reinterpret_cast<uint4*>(dst.v + to[u] * 128 + 16 * tiles.ch) = v[u];
+      const size_t at = to[u] * 128 + 16 * (tiles.ch ^ (int)(to[u] & 7));
+      *reinterpret_cast<uint4*>(dst.k + at) = k[u];
+      *reinterpret_cast<uint4*>(dst.v + at) = v[u];
     }
   }
   gather_origins(a, B);
