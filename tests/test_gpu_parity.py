@@ -583,3 +583,46 @@ def test_8bit_ragged_frames_chunks_and_budget_changes(xkv):
             r0 += n
         assert cache.xkv_poll_status() == 0
     assert cache.xkv_get_info().T == ora.T and ora.last_scores is not None
+
+
+# ------------------------------------------------------------------ 16-bit rows, resets
+@pytest.mark.parametrize("n_bytes", [1, 127, 128, 130, 1000, 16 * 128 + 24])
+def test_export_of_16bit_rows_may_end_anywhere(xkv, n_bytes):
+    """The rows of a 16-bit cache are stored in the attention's operand order and exported in channel order, also
+    where the caller's buffer ends inside a row or a 16-byte piece."""
+    p = xkv.Params(n_heads=2, budget=300, max_frame_tokens=70, kv_bits=16)
+    cache, ora, _ = run_stream(xkv, p, 70, 2, seed=9)
+    cap = cache.xkv_get_info().capacity
+    for which in (xkv.BUF_K_CODES, xkv.BUF_V_CODES):
+        whole = cache.xkv_debug_export(which, 2 * cap * 128)
+        part = cache.xkv_debug_export(which, n_bytes)
+        assert np.array_equal(np.asarray(part)[:n_bytes], np.asarray(whole)[:n_bytes])
+
+
+@pytest.mark.parametrize("bits,once", [(4, 0), (4, 1), (8, 1), (16, 0)])
+def test_reset_after_a_stream_of_bad_values(xkv, bits, once):
+    """xkv_reset zeroes what a stream needs zeroed and no more: after a stream of infinities, numbers beyond fp16 and
+    NaN, with longer frames, a cache behaves like a new one."""
+    import torch
+    H, n = 2, 150
+    p = xkv.Params(n_heads=H, budget=400, max_frame_tokens=n, kv_bits=bits, key_mode=once)
+    used, new = xkv.Cache(p), xkv.Cache(p)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    for t in range(6):
+        x = [torch.randn(H, n, 64, device="cuda", generator=gen) * 1e6 for _ in range(3)]
+        x[1][:, ::3], x[2][:, ::3] = float("inf"), float("nan")
+        used.step(*(y.to(torch.bfloat16) for y in x))
+    assert bits == 16 or used.xkv_poll_status() != 0
+    used.xkv_reset()
+    for t, m in enumerate([33, 100, 7, 140, 64, 150]):
+        frame = [to_device_bf16(b) for b in synth.gen_frame(83, 0, t, H, m, 64)]
+        outs = []
+        for c in (used, new):
+            out = torch.empty_like(frame[0])
+            c.kv_append(frame[1], frame[2]); c.kv_score_evict(frame[0]); c.kv_quant_pack()
+            c.attn_packed_causal(frame[0], out)
+            outs.append(out)
+        assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16)), t
+        ea, eb = used.export(), new.export()
+        assert all(np.array_equal(np.asarray(ea[key]), np.asarray(eb[key])) for key in eb), t
+        assert used.xkv_poll_status() == 0 and new.xkv_poll_status() == 0
