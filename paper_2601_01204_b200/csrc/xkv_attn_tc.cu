@@ -9,12 +9,10 @@
 // and sum) in a scratch slot; a second kernel merges them.
 //
 // One CTA.  24 warps:
-//   16 warps    softmax: warps w and w + 8 share the rows of a TMEM lane quarter, each takes 64 of a key
-//               tile's 128 score columns, the matching 32 columns of P and 32 of the accumulator; a
-//               thread loads its half row of scores into registers at once, takes the maximum from
-//               them, exchanges it with the other half, and writes P (16-bit) back to tensor memory.
-//               O is rescaled only when the running maximum grew by more than 2^14.  Registers move to
-//               these warps with setmaxnreg.
+//   16 warps    softmax: a warp takes 16 whole rows of a query tile, half of a TMEM lane quarter; a quad of
+//               lanes holds 128 scores each of two rows, loaded into registers at once, exchanges their
+//               maxima by shuffles and writes P (16-bit) back to tensor memory.  O is rescaled only when
+//               the running maximum grew by more than 2^14.  Registers move to these warps with setmaxnreg.
 //   4 warps     operand producers (4 and 8 bits): packed codes (raw, as copied by TMA) -> fp16 K~ (per channel
 //               and key group) and V~ (per token) in the 128-byte-swizzled layouts the MMA
 //               descriptors expect.  One dequantised tile serves both query tiles.
@@ -102,9 +100,8 @@ template <int BITS> struct Map {
   static constexpr int kOffBar = kOffTab + (BITS == 16 ? 512 : 2 * kTabBytes);
   static constexpr int kOffRaw = kOffBar + kBarBytes;                   // raw stages (16-byte aligned)
 };
-constexpr int kXchgBytes = 6144;                  // split softmax: values exchanged between the two halves of a row
 template <int BITS> constexpr int smem_bytes() {
-  return Map<BITS>::kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + kXchgBytes + 1024;
+  return Map<BITS>::kOffRaw + Cfg<BITS>::kNR * Cfg<BITS>::kRawStage + 1024;
 }
 
 // Tensor memory columns (all 512).  A query tile has three blocks of 64 columns, B0 B1 B2.  In even
@@ -350,42 +347,57 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b_d
       ::"r"(d), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
 
-#define XKV_TMEM_LD32(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "                                                      \
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"                                      \
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"                     \
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), \
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),     \
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),   \
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),   \
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])                                                        \
+// Tensor memory <-> registers, 16 lanes (rows) of the calling warp's quarter.  Of every 8 columns lane l holds, as in
+// the accumulators of a warp-level MMA, columns 2 (l mod 4) and the next of row l / 4 (registers 4g, 4g + 1) and of row
+// l / 4 + 8 (4g + 2, 4g + 3).  A pair of neighbours makes one 32-bit word of 16-bit P, and of every 4 words lane l
+// holds word l mod 4 of the same two rows (2g, 2g + 1).  LD_64, ST_64: 64 columns; ST_P32, ST_P16: 32 and 16 words.
+#define XKV_TMEM_LD_64(taddr, r, o)                                                                 \
+  asm volatile(                                                                                     \
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"                                                    \
+      "%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"                                      \
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"                    \
+      : "=r"(r[(o) + 0]), "=r"(r[(o) + 1]), "=r"(r[(o) + 2]), "=r"(r[(o) + 3]),                     \
+        "=r"(r[(o) + 4]), "=r"(r[(o) + 5]), "=r"(r[(o) + 6]), "=r"(r[(o) + 7]),                     \
+        "=r"(r[(o) + 8]), "=r"(r[(o) + 9]), "=r"(r[(o) + 10]), "=r"(r[(o) + 11]),                   \
+        "=r"(r[(o) + 12]), "=r"(r[(o) + 13]), "=r"(r[(o) + 14]), "=r"(r[(o) + 15]),                 \
+        "=r"(r[(o) + 16]), "=r"(r[(o) + 17]), "=r"(r[(o) + 18]), "=r"(r[(o) + 19]),                 \
+        "=r"(r[(o) + 20]), "=r"(r[(o) + 21]), "=r"(r[(o) + 22]), "=r"(r[(o) + 23]),                 \
+        "=r"(r[(o) + 24]), "=r"(r[(o) + 25]), "=r"(r[(o) + 26]), "=r"(r[(o) + 27]),                 \
+        "=r"(r[(o) + 28]), "=r"(r[(o) + 29]), "=r"(r[(o) + 30]), "=r"(r[(o) + 31])                  \
       : "r"(taddr) : "memory")
 
-#define XKV_TMEM_ST32(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "                                                \
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"                                     \
-      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"                            \
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
-        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), \
-        "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),          \
-        "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]),          \
-        "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory")
+#define XKV_TMEM_ST_64(taddr, r)                                                                    \
+  asm volatile(                                                                                     \
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], {"                                              \
+      "%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"                                     \
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"                           \
+      ::"r"(taddr),                                                                                 \
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),                                                 \
+        "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),                                                 \
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]),                                               \
+        "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),                                             \
+        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),                                             \
+        "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),                                             \
+        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),                                             \
+        "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory")
 
-#define XKV_TMEM_ST8(taddr, r)                                                                       \
-  asm volatile(                                                                                      \
-      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"                       \
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
-        "r"(r[7]) : "memory")
+#define XKV_TMEM_ST_P32(taddr, r)                                                                   \
+  asm volatile(                                                                                     \
+      "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {"                                              \
+      "%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"                                    \
+      ::"r"(taddr),                                                                                 \
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),                                                 \
+        "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),                                                 \
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]),                                               \
+        "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory")
 
-#define XKV_TMEM_ST16(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "                                                \
-      "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"                                    \
-      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]),     \
-        "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), \
-        "r"(r[15]) : "memory")
+#define XKV_TMEM_ST_P16(taddr, r)                                                                   \
+  asm volatile(                                                                                     \
+      "tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {"                                              \
+      "%1,%2,%3,%4,%5,%6,%7,%8};"                                                                   \
+      ::"r"(taddr),                                                                                 \
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),                                                 \
+        "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory")
 
 // Shared-memory matrix descriptor, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
@@ -558,15 +570,15 @@ __device__ __forceinline__ void once_keys(const uint8_t* codes, const uint8_t* r
     *reinterpret_cast<uint4*>(tile + (k0 + i) * 128 + ((w ^ i) << 4)) = dequant_word_h(wd[i], s2, zo, c2);
   }
 }
-// 32 columns of O *= alpha for the 32 rows (TMEM lanes) of the calling warp; a real call, to keep its
-// registers out of the softmax loop.  Warp-collective.
-__device__ __noinline__ void rescale_rows(uint32_t col_o, float alpha) {
-  uint32_t ra[32];
-  XKV_TMEM_LD32(col_o, ra);
+// O *= alpha for the calling warp's 16 rows (two per thread); a real call, to keep its registers out of the
+// softmax loop.  Warp-collective.
+__device__ __noinline__ void rescale_rows(uint32_t col_o, float alpha0, float alpha1) {
+  uint32_t ro[32];
+  XKV_TMEM_LD_64(col_o, ro, 0);
   tc_wait_ld();
 #pragma unroll
-  for (int i = 0; i < 32; ++i) ra[i] = __float_as_uint(__uint_as_float(ra[i]) * alpha);
-  XKV_TMEM_ST32(col_o, ra);
+  for (int i = 0; i < 32; ++i) ro[i] = __float_as_uint(__uint_as_float(ro[i]) * ((i & 2) ? alpha1 : alpha0));
+  XKV_TMEM_ST_64(col_o, ro);
   tc_wait_st();
 }
 __device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
@@ -584,8 +596,6 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   constexpr uint32_t kRowThreads = 256;      // threads that work on one query tile
   constexpr int kNK = C::kNK, kNV = C::kNV;
   constexpr int kOffV = Map<BITS>::kOffV, kOffTab = Map<BITS>::kOffTab, kOffBar = Map<BITS>::kOffBar, kOffRaw = Map<BITS>::kOffRaw;
-  constexpr int kOffX = kOffRaw + C::kNR * C::kRawStage;   // exchange area of the split softmax
-  static_assert(kOffX % 1024 == 0, "the halves' places differ in one address bit");
   constexpr int kRegProd = regs_producers(ONCE, TAIL), kRegMisc = regs_misc(ONCE, TAIL);
   extern __shared__ uint8_t smem_raw[];
   const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -648,32 +658,26 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   }
 
   if (warp < 16) {
-    // ============== softmax warps, two per 32 rows of a query tile ==============
-    // Warps w and w + 8 work on the same rows: each takes 64 of a key tile's 128 score columns, the
-    // matching 32 columns of P and 32 of the accumulator.  A thread reads its half row of scores
-    // into registers at once and releases the score columns, so that the next S = Q K~^T runs while
-    // the exponentials are computed.  What the row needs as a whole (its maximum, its sum) the two
-    // threads exchange through shared memory.
+    // ============== softmax warps, 16 rows of a query tile each ==============
+    // Warps w and w + 8 may access the same quarter of the TMEM lanes and take 16 of its 32 rows each, whole rows:
+    // a quad of lanes holds 128 scores of a row and of the row 8 further, 32 of each per lane.  The scores are
+    // read into registers at once and their columns released, so that the next S = Q K~^T runs while the
+    // exponentials are computed.  What a row needs as a whole (its maximum, its sum) goes around the quad by
+    // shuffles; no warp waits for another one.
+    // (Before, warps w and w + 8 shared 32 rows, 64 columns each, and exchanged maxima through shared memory and
+    // a barrier in every step, 360 of its 2900 clk, which also kept the two in step.  Separate: one layer of
+    // 1374 tokens at 8192, all four calls, 132.3 -> 122.3 us; chunks of four frames, 24 layers, 7016 -> 6359; 24 layers
+    // at 4096 1038 -> 993, at 16384 3607 -> 3576, with the tail 4039 -> 3880; 16-bit at 32768 7481 -> 7398.)
     const int t = (warp >> 2) & 1;           // query tile of the pair
-    const int hf = warp >> 3;                // half of the key columns
-    const int r = (warp & 3) * 32 + (tid & 31);   // row of the tile = TMEM lane
-    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-    const uint32_t colS0 = lane_addr + kColTile * t + 64 * hf;
-    const uint32_t colP0 = lane_addr + kColTile * t + 32 * hf;
-    const uint32_t colO = lane_addr + kColO + 64 * t + 32 * hf;
+    const int hf = warp >> 3;                // half of the quarter's rows
+    const int lane = tid & 31;
+    const int r = (warp & 3) * 32 + 16 * hf + (lane >> 2);        // rows r and r + 8 of the tile
+    const int cq2 = 2 * (lane & 3);          // this thread's columns: cq2 and the next of every 8
+    const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32 + 16 * hf) << 16);
+    const uint32_t col_t = lane_addr + kColTile * t;
+    const uint32_t colO = lane_addr + kColO + 64 * t;
     const uint32_t sfull = b_sfull + 8 * t, pfull = b_pfull + 16 * t, pvdone = b_pvdone + 16 * t;
     const uint64_t sc2 = pack_f2(a.scale_log2, a.scale_log2);
-    const int pair_bar = 2 + (warp & 7);     // named barrier of the two warps with these rows
-    const uint32_t xmine = sbase + kOffX + 4 * ((t * 2 + hf) * 128 + r);
-    // One value per thread to the thread of the other half with the same row.  Two buffers in turn for
-    // the steps, a third for the end of a segment: a value is overwritten after a barrier that its
-    // reader has passed.
-    auto exchange = [&](float v, uint32_t buf) -> float {
-      st_shared_u32(xmine + buf * 2048, __float_as_uint(v));
-      __syncwarp();
-      asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-      return __uint_as_float(ld_shared_u32((xmine ^ 512u) + buf * 2048));
-    };
     uint32_t cnt = 0;                        // steps this tile has been through (barrier phases)
     int seg_idx = 0;
     for (Walk walk(a); walk.next(a); ++seg_idx) {
@@ -683,9 +687,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
       // steps whose tile has masked columns: the pad slots after the first frame, the end
       const int jj_pad = (job.t_first & 127) ? (job.t_first >> 7) - tile_lo : -1, jj_last = job.n_tiles - 1 - tile_lo;
       if (qt >= job.q_tiles) continue;          // the pair has no second tile
-      // ---- Q tile: half of row r, bf16 -> operand type, into the swizzled K-major layout ----
-      const int row = qt * kQRows + r;
+      // ---- Q tile: half a row per thread, bf16 -> operand type, into the swizzled K-major layout ----
       {
+        const int rq = (warp & 3) * 32 + lane, row = qt * kQRows + rq;
         uint4 u[4];
         if (row < job.n) {
           const __nv_bfloat16* qp = job.q + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
@@ -709,14 +713,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             }
             o = make_uint4(hh[0], hh[1], hh[2], hh[3]);
           }
-          *reinterpret_cast<uint4*>(sgen + kOffQ + t * 16384 + swz_off(r, 4 * hf + c)) = o;
+          *reinterpret_cast<uint4*>(sgen + kOffQ + t * 16384 + swz_off(rq, 4 * hf + c)) = o;
         }
         if (q_bad) report_range(job.status);
         fence_proxy_async();
         mbar_arrive(b_qfull + 8 * t);
       }
-      float m_ref = -INFINITY;   // reference maximum of the row (scaled, log2 units; the same in both halves)
-      uint64_t l2 = 0ull, l2b = 0ull;   // four partial sums of this half of the row (two packed fp32 pairs)
+      float m0 = -INFINITY, m1 = -INFINITY;     // reference maxima of the two rows (scaled, log2 units; the same in the quad)
+      uint64_t l0 = 0ull, l1 = 0ull;            // partial sums of this thread's columns (packed fp32 pairs)
       for (int jj = 0; jj < nt; ++jj, ++cnt) {
         int lim = 128;           // columns [lim, 128) are masked
         if (jj == jj_pad) lim = job.t_first & 127;
@@ -724,120 +728,133 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         mbar_wait(sfull, cnt & 1, wc);
         __syncwarp();            // the waits may leave the warp diverged; tcgen05.ld/st are warp-collective
         tc_fence_after();
-        // ---- this half of the scores (64 columns) into registers; after that the score columns
-        // may take the next tile's scores ----
-        uint32_t ra[32], rb[32];
-        const uint32_t colS = colS0 + 64 * (cnt & 1);
-        XKV_TMEM_LD32(colS, ra);
-        XKV_TMEM_LD32(colS + 32, rb);
+        // ---- the scores into registers; after that their columns may take the next tile's scores ----
+        uint32_t sc[64];
+        XKV_TMEM_LD_64(col_t + 64 * (cnt & 1), sc, 0);
+        XKV_TMEM_LD_64(col_t + 64 * (cnt & 1) + 64, sc, 32);
         tc_wait_ld();
         tc_fence_before();
         mbar_arrive(b_sfree + 8 * t);
         if (lim < 128) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            if (64 * hf + i >= lim) ra[i] = 0xff800000u;           // -inf: exponential 0
-            if (64 * hf + 32 + i >= lim) rb[i] = 0xff800000u;
-          }
+          for (int i = 0; i < 64; ++i)
+            if (8 * (i >> 2) + cq2 + (i & 1) >= lim) sc[i] = 0xff800000u;           // -inf: exponential 0
         }
-        float mx1 = -INFINITY, mx2 = -INFINITY;      // two chains of 16, not one of 32
+        float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < 32; i += 2) {
-          mx1 = max3(mx1, __uint_as_float(ra[i]), __uint_as_float(ra[i + 1]));
-          mx2 = max3(mx2, __uint_as_float(rb[i]), __uint_as_float(rb[i + 1]));
+        for (int g = 0; g < 16; ++g) {
+          mx0 = max3(mx0, __uint_as_float(sc[4 * g]), __uint_as_float(sc[4 * g + 1]));
+          mx1 = max3(mx1, __uint_as_float(sc[4 * g + 2]), __uint_as_float(sc[4 * g + 3]));
         }
-        const float mx_half = fmaxf(mx1, mx2);
-        const float mx = fmaxf(mx_half, exchange(mx_half, cnt & 1)) * a.scale_log2;
+        const float own0 = mx0, own1 = mx1;
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) {
+          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+        }
+        mx0 *= a.scale_log2;
+        mx1 *= a.scale_log2;
         // The reference maximum moves only when the row maximum grew by more than 2^kGrow over it;
         // then the sums and (at the end of the step, when the registers are free) the accumulator
-        // are rescaled.  Every tile has a column that is not masked, so mx is finite.
-        float alpha = 1.f;
-        const bool grow = mx > m_ref + kGrow;
+        // are rescaled.  Every tile has a column that is not masked, so the maxima are finite.
+        float alpha0 = 1.f, alpha1 = 1.f;
+        const bool grow = mx0 > m0 + kGrow || mx1 > m1 + kGrow;
         if (grow) {
-          alpha = exp2f(m_ref - mx);      // 0 on the first tile (m_ref = -inf)
-          m_ref = mx;
-          l2 = mul_f2(l2, pack_f2(alpha, alpha));
-          l2b = mul_f2(l2b, pack_f2(alpha, alpha));
+          if (mx0 > m0 + kGrow) {
+            alpha0 = exp2f(m0 - mx0);      // 0 on the first tile (-inf)
+            m0 = mx0;
+            l0 = mul_f2(l0, pack_f2(alpha0, alpha0));
+          }
+          if (mx1 > m1 + kGrow) {
+            alpha1 = exp2f(m1 - mx1);
+            m1 = mx1;
+            l1 = mul_f2(l1, pack_f2(alpha1, alpha1));
+          }
         }
-        const uint64_t nm2 = pack_f2(-m_ref, -m_ref);
+        const uint64_t nm0 = pack_f2(-m0, -m0), nm1 = pack_f2(-m1, -m1);
         if (kBf16) {
           // A weight rounded to bf16 and the sum that it is divided by: where one key dominates a row its
           // rounding error drops out if the sum holds the rounded weight as well.  The largest weight of
-          // these 64 columns is enough (error against float64 as with all of them: 32768 tokens 2.18e-3
+          // these 32 columns is enough (of 64, error against float64 as with all of them: 32768 tokens 2.18e-3
           // -> 1.92e-3, of which the rounding of the output is 1.67e-3); adding up all rounded weights
           // cost 6 % of the step (24 layers at 32768: 7860 -> 8400 us).
-          const float top = fast_exp2(fmaf(mx_half, a.scale_log2, -m_ref));
-          l2 = add_f2(l2, pack_f2(__bfloat162float(__float2bfloat16_rn(top)) - top, 0.f));
+          const float top0 = fast_exp2(fmaf(own0, a.scale_log2, -m0)), top1 = fast_exp2(fmaf(own1, a.scale_log2, -m1));
+          l0 = add_f2(l0, pack_f2(__bfloat162float(__float2bfloat16_rn(top0)) - top0, 0.f));
+          l1 = add_f2(l1, pack_f2(__bfloat162float(__float2bfloat16_rn(top1)) - top1, 0.f));
         }
-        // (P goes over scores of both halves; the exchange above has made sure that both hold theirs)
-        const uint32_t colP = colP0 + 128 * (cnt & 1);
-        // Exponentials against the reference; P (16-bit pairs) -> TMEM.  32 columns at a time, or 16 where
-        // the producers fetch constants per token (24 layers at 16384: 4-bit 3157 -> 3100 us with 32, keys
-        // quantised once 3693 -> 3727).
-        auto columns = [&](const uint32_t* rr, uint32_t* pk, int pairs) {
+        const uint32_t colP = col_t + 128 * (cnt & 1);       // (over scores of these rows only)
+        // Exponentials against the reference; P (16-bit pairs) -> TMEM.  64 columns at a time, or 32 where
+        // the producers fetch constants per token.
+        auto columns = [&](int g0, uint32_t* pk, int groups) {
 #pragma unroll
-          for (int i = 0; i < pairs; ++i) {
-            const uint64_t x = fma_f2(pack_f2(__uint_as_float(rr[2 * i]), __uint_as_float(rr[2 * i + 1])), sc2, nm2);
-            const float e0 = fast_exp2(f2_lo(x)), e1 = fast_exp2(f2_hi(x));
-            if (i & 1) l2b = add_f2(l2b, pack_f2(e0, e1)); else l2 = add_f2(l2, pack_f2(e0, e1));
-            pk[i] = kBf16 ? pack_bf2(e0, e1) : pack_h2(e0, e1);
+          for (int g = 0; g < groups; ++g) {
+            const uint32_t* x = sc + 4 * (g0 + g);
+            const uint64_t x0 = fma_f2(pack_f2(__uint_as_float(x[0]), __uint_as_float(x[1])), sc2, nm0);
+            const uint64_t x1 = fma_f2(pack_f2(__uint_as_float(x[2]), __uint_as_float(x[3])), sc2, nm1);
+            const float e0 = fast_exp2(f2_lo(x0)), e1 = fast_exp2(f2_hi(x0)), e2 = fast_exp2(f2_lo(x1)), e3 = fast_exp2(f2_hi(x1));
+            l0 = add_f2(l0, pack_f2(e0, e1));
+            l1 = add_f2(l1, pack_f2(e2, e3));
+            pk[2 * g] = kBf16 ? pack_bf2(e0, e1) : pack_h2(e0, e1);
+            pk[2 * g + 1] = kBf16 ? pack_bf2(e2, e3) : pack_h2(e2, e3);
           }
         };
         if (ONCE) {
           uint32_t pk[8];
-          columns(ra, pk, 8);      XKV_TMEM_ST8(colP, pk);
-          columns(ra + 16, pk, 8); XKV_TMEM_ST8(colP + 8, pk);
-          columns(rb, pk, 8);      XKV_TMEM_ST8(colP + 16, pk);
-          columns(rb + 16, pk, 8); XKV_TMEM_ST8(colP + 24, pk);
+          columns(0, pk, 4);  XKV_TMEM_ST_P16(colP, pk);
+          columns(4, pk, 4);  XKV_TMEM_ST_P16(colP + 16, pk);
+          columns(8, pk, 4);  XKV_TMEM_ST_P16(colP + 32, pk);
+          columns(12, pk, 4); XKV_TMEM_ST_P16(colP + 48, pk);
         } else {
           uint32_t pk[16];
-          columns(ra, pk, 16); XKV_TMEM_ST16(colP, pk);
-          columns(rb, pk, 16); XKV_TMEM_ST16(colP + 16, pk);
+          columns(0, pk, 8); XKV_TMEM_ST_P32(colP, pk);
+          columns(8, pk, 8); XKV_TMEM_ST_P32(colP + 32, pk);
         }
         if (jj > 0 && __any_sync(0xffffffffu, grow)) {
           // the accumulator is quiescent once the previous step's PV has completed
           mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);
           __syncwarp();
           tc_fence_after();
-          rescale_rows(colO, alpha);
+          rescale_rows(colO, alpha0, alpha1);
         }
         tc_wait_st();
         tc_fence_before();
         mbar_arrive(pfull + 8 * (cnt & 1));
       }
-      // ---- epilogue of the segment: 32 channels of the row per thread ----
+      // ---- epilogue of the segment ----
       mbar_wait(pvdone + 8 * ((cnt - 1) & 1), ((cnt - 1) >> 1) & 1, wc);    // the last PV (they complete in order)
       __syncwarp();
       tc_fence_after();
-      const float l_half = (f2_lo(l2) + f2_hi(l2)) + (f2_lo(l2b) + f2_hi(l2b));
-      const float l_peer = exchange(l_half, 2);
-      const float l = hf ? (l_peer + l_half) : (l_half + l_peer);     // the same sum in both halves
+      float s0 = f2_lo(l0) + f2_hi(l0), s1 = f2_lo(l1) + f2_hi(l1);
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      }
       const bool whole = (tile_lo == 0 && nt == job.n_tiles);
       uint32_t ro[32];
-      XKV_TMEM_LD32(colO, ro);
+      XKV_TMEM_LD_64(colO, ro, 0);
       tc_wait_ld();
       if (whole) {
-        const float inv_l = 1.f / l;
-        if (row < job.n) {
-          __nv_bfloat16* op = job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + 32 * hf;
+        const float inv0 = 1.f / s0, inv1 = 1.f / s1;
+        const int row = qt * kQRows + r;
+        __nv_bfloat16* op = job.out + (int64_t)h * a.hs + (int64_t)row * a.ts + cq2;
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              o[i] = pack_bf2(__uint_as_float(ro[8 * c + 2 * i]) * inv_l, __uint_as_float(ro[8 * c + 2 * i + 1]) * inv_l);
-            *reinterpret_cast<uint4*>(op + 8 * c) = make_uint4(o[0], o[1], o[2], o[3]);
-          }
+        for (int g = 0; g < 8; ++g) {
+          if (row < job.n)
+            *reinterpret_cast<uint32_t*>(op + 8 * g) = pack_bf2(__uint_as_float(ro[4 * g]) * inv0, __uint_as_float(ro[4 * g + 1]) * inv0);
+          if (row + 8 < job.n)
+            *reinterpret_cast<uint32_t*>(op + 8 * a.ts + 8 * g) = pack_bf2(__uint_as_float(ro[4 * g + 2]) * inv1, __uint_as_float(ro[4 * g + 3]) * inv1);
         }
       } else {
         const size_t slot = (size_t)2 * blockIdx.x + (seg_idx == 0 ? 0 : 1);
         const size_t prow = (slot * 2 + t) * 128 + r;
-        float4* dst = reinterpret_cast<float4*>(a.part_o + prow * 64 + 32 * hf);
+        float* dst = a.part_o + prow * 64 + cq2;
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-          dst[c] = make_float4(__uint_as_float(ro[4 * c]), __uint_as_float(ro[4 * c + 1]),
-                               __uint_as_float(ro[4 * c + 2]), __uint_as_float(ro[4 * c + 3]));
-        if (hf == 0) a.part_ml[prow] = make_float2(m_ref, l);
+        for (int g = 0; g < 8; ++g) {
+          *reinterpret_cast<float2*>(dst + 8 * g) = make_float2(__uint_as_float(ro[4 * g]), __uint_as_float(ro[4 * g + 1]));
+          *reinterpret_cast<float2*>(dst + 512 + 8 * g) = make_float2(__uint_as_float(ro[4 * g + 2]), __uint_as_float(ro[4 * g + 3]));
+        }
+        if ((lane & 3) == 0) { a.part_ml[prow] = make_float2(m0, s0); a.part_ml[prow + 8] = make_float2(m1, s1); }
       }
       tc_fence_before();
     }
