@@ -350,7 +350,7 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b_d
 // Tensor memory <-> registers, 16 lanes (rows) of the calling warp's quarter.  Of every 8 columns lane l holds, as in
 // the accumulators of a warp-level MMA, columns 2 (l mod 4) and the next of row l / 4 (registers 4g, 4g + 1) and of row
 // l / 4 + 8 (4g + 2, 4g + 3).  A pair of neighbours makes one 32-bit word of 16-bit P, and of every 4 words lane l
-// holds word l mod 4 of the same two rows (2g, 2g + 1).  LD_64, ST_64: 64 columns; ST_P32, ST_P16: 32 and 16 words.
+// holds word l mod 4 of the same two rows (2g, 2g + 1).  LD_64, ST_64: 64 columns; ST_P32: 32 words.
 #define XKV_TMEM_LD_64(taddr, r, o)                                                                 \
   asm volatile(                                                                                     \
       "tcgen05.ld.sync.aligned.16x256b.x8.b32 {"                                                    \
@@ -390,14 +390,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b_d
         "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),                                                 \
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]),                                               \
         "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory")
-
-#define XKV_TMEM_ST_P16(taddr, r)                                                                   \
-  asm volatile(                                                                                     \
-      "tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {"                                              \
-      "%1,%2,%3,%4,%5,%6,%7,%8};"                                                                   \
-      ::"r"(taddr),                                                                                 \
-        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),                                                 \
-        "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory")
 
 // Shared-memory matrix descriptor, 128-byte swizzle, 8-row groups 1024 B apart.
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
@@ -783,11 +775,11 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           l1 = add_f2(l1, pack_f2(__bfloat162float(__float2bfloat16_rn(top1)) - top1, 0.f));
         }
         const uint32_t colP = col_t + 128 * (cnt & 1);       // (over scores of these rows only)
-        // Exponentials against the reference; P (16-bit pairs) -> TMEM.  64 columns at a time, or 32 where
-        // the producers fetch constants per token.
-        auto columns = [&](int g0, uint32_t* pk, int groups) {
+        // Exponentials against the reference; P (16-bit pairs) -> TMEM, 64 columns at a time (32: 24 layers at 4096
+        // 980 -> 1029 us, keys quantised once at 16384 3668 -> 3798, 8-bit 1481 -> 1538).
+        auto columns = [&](int g0, uint32_t* pk) {
 #pragma unroll
-          for (int g = 0; g < groups; ++g) {
+          for (int g = 0; g < 8; ++g) {
             const uint32_t* x = sc + 4 * (g0 + g);
             const uint64_t x0 = fma_f2(pack_f2(__uint_as_float(x[0]), __uint_as_float(x[1])), sc2, nm0);
             const uint64_t x1 = fma_f2(pack_f2(__uint_as_float(x[2]), __uint_as_float(x[3])), sc2, nm1);
@@ -798,16 +790,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
             pk[2 * g + 1] = kBf16 ? pack_bf2(e2, e3) : pack_h2(e2, e3);
           }
         };
-        if (ONCE) {
-          uint32_t pk[8];
-          columns(0, pk, 4);  XKV_TMEM_ST_P16(colP, pk);
-          columns(4, pk, 4);  XKV_TMEM_ST_P16(colP + 16, pk);
-          columns(8, pk, 4);  XKV_TMEM_ST_P16(colP + 32, pk);
-          columns(12, pk, 4); XKV_TMEM_ST_P16(colP + 48, pk);
-        } else {
+        {
           uint32_t pk[16];
-          columns(0, pk, 8); XKV_TMEM_ST_P32(colP, pk);
-          columns(8, pk, 8); XKV_TMEM_ST_P32(colP + 32, pk);
+          columns(0, pk); XKV_TMEM_ST_P32(colP, pk);
+          columns(8, pk); XKV_TMEM_ST_P32(colP + 32, pk);
         }
         if (jj > 0 && __any_sync(0xffffffffu, grow)) {
           // the accumulator is quiescent once the previous step's PV has completed
