@@ -626,3 +626,13 @@ def test_reset_after_a_stream_of_bad_values(xkv, bits, once):
         ea, eb = used.export(), new.export()
         assert all(np.array_equal(np.asarray(ea[key]), np.asarray(eb[key])) for key in eb), t
         assert used.xkv_poll_status() == 0 and new.xkv_poll_status() == 0
+
+
+@pytest.mark.parametrize("bits", [4, 16])
+@pytest.mark.parametrize("sizes", [(1, 1, 2), (7, 9, 8), (16, 15, 17), (33, 63, 64), (65, 127, 1), (129, 136, 40)])
+def test_attention_rows_and_columns_at_the_edges_of_a_warps_share(xkv, bits, sizes):
+    """A softmax warp takes 16 rows of a query tile and a lane two columns of every eight: query counts around 8, 16
+    and 128 and cache lengths (masked columns) around 2, 8, 64 and 128, items whole and cut between blocks."""
+    for blocks in (0, 3):
+        p = xkv.Params(n_heads=2, budget=400, max_frame_tokens=136, kv_bits=bits)
+        run_stream(xkv, p, list(sizes), 3, seed=17, max_blocks=blocks)
