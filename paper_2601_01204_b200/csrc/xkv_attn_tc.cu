@@ -640,8 +640,8 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   {
-    // Registers move from the warps that need few to the softmax warps, which keep half a row of
-    // scores in registers.  The pool is what the CTA was launched with (per scheduler 6 warps x 80
+    // Registers move from the warps that need few to the softmax warps, whose threads keep 64 scores
+    // in registers.  The pool is what the CTA was launched with (per scheduler 6 warps x 80
     // registers per lane = 480); afterwards 4 x 96 + 48 + 48 (or 56 + 40, 64 + 32 where the producers hold more)
     // of them are in use: all 480.
     if (warp < 16) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
