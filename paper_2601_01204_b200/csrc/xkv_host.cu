@@ -23,7 +23,6 @@ struct Layout {
   size_t off_kslot[2], off_ktab32, off_ktab16, off_ref, off_ring;
   int n_slots;
   size_t attn_bytes;
-  size_t zeroed;      // the bytes from the start that a stream needs zeroed
   size_t total;
 };
 
@@ -57,28 +56,11 @@ Layout make_layout(const xkv_params* p) {
   L.off_status = take(256);
   L.off_counters = take(576 * sizeof(unsigned int));
   L.off_hist = take(4 * 4096 * sizeof(unsigned int));
-  if (p->key_mode == XKV_KEYS_ONCE) {
-    // every live group holds at least one cached token, so one slot per token slot never runs out;
-    // at least the groups of two frames (the first and the one arriving) are needed in any case
-    const int least = 2 * ((max_n + 63) / 64) + 1;
-    L.n_slots = p->key_table_slots > 0 ? (p->key_table_slots > least ? p->key_table_slots : least) : L.cap;
-    L.off_ref = take((size_t)L.n_slots * sizeof(int32_t));
-  }
-  // The attention multiplies the values of masked slots by weights of 0, and reports group parameters that
-  // are out of range whether their slots are masked or not, so slots that a stream has not used yet must not
-  // hold what another one left there: parameters of 0 make codes 0, and 16-bit rows have no parameters.
-  // (Zeroing the whole workspace, 62 MB a layer for chunks of 4016 tokens at 6144, cost more: 24 layers and eight
-  // frames 7196 us, and 7002 with this much; eight frames of 261 tokens on one layer 281.4 and 276.4.)
-  for (int b = 0; b < 2; ++b) {
-    L.off_kpar[b] = take(H * (L.cap / 64) * 64 * sizeof(float2));
-    L.off_vpar[b] = take(H * L.cap * sizeof(float2));
-  }
-  if (p->kv_bits == 16)
-    for (int b = 0; b < 2; ++b) L.off_v[b] = take(H * L.cap * L.row_bytes);
-  L.zeroed = off;
   for (int b = 0; b < 2; ++b) {
     L.off_k[b] = take(H * L.cap * L.row_bytes);
-    if (p->kv_bits != 16) L.off_v[b] = take(H * L.cap * L.row_bytes);
+    L.off_kpar[b] = take(H * (L.cap / 64) * 64 * sizeof(float2));
+    L.off_v[b] = take(H * L.cap * L.row_bytes);
+    L.off_vpar[b] = take(H * L.cap * sizeof(float2));
     L.off_origin[b] = take((size_t)L.cap * sizeof(int32_t));
     L.off_kbar[b] = take((size_t)L.cap * 64 * sizeof(float));
   }
@@ -91,9 +73,14 @@ Layout make_layout(const xkv_params* p) {
   L.off_run_hi = take((size_t)(L.cap / 64) * sizeof(unsigned int));
   L.off_cand = take((size_t)L.cap * sizeof(unsigned long long));
   if (p->key_mode == XKV_KEYS_ONCE) {
+    // every live group holds at least one cached token, so one slot per token slot never runs out;
+    // at least the groups of two frames (the first and the one arriving) are needed in any case
+    const int least = 2 * ((max_n + 63) / 64) + 1;
+    L.n_slots = p->key_table_slots > 0 ? (p->key_table_slots > least ? p->key_table_slots : least) : L.cap;
     for (int b = 0; b < 2; ++b) L.off_kslot[b] = take((size_t)L.cap * sizeof(int32_t));
     L.off_ktab32 = take((size_t)L.n_slots * H * 64 * sizeof(float2));
     L.off_ktab16 = take((size_t)L.n_slots * H * 8 * 12 * sizeof(uint32_t));
+    L.off_ref = take((size_t)L.n_slots * sizeof(int32_t));
     L.off_ring = take((size_t)L.n_slots * sizeof(int32_t));
   }
   L.attn_bytes = attn_tc_scratch_bytes(p);
@@ -113,8 +100,8 @@ void after_head_means(const xkv_cache* c, cudaStream_t st) {
   if (c->kbar_done && cudaStreamWaitEvent(st, c->kbar_done, 0) != cudaSuccess) cudaGetLastError();
 }
 
-int zero_workspace(xkv_cache* c, size_t bytes, cudaStream_t st) {
-  if (cudaMemsetAsync(c->ws, 0, bytes, st) != cudaSuccess) return XKV_E_CUDA;
+int zero_workspace(xkv_cache* c, cudaStream_t st) {
+  if (cudaMemsetAsync(c->ws, 0, c->ws_bytes, st) != cudaSuccess) return XKV_E_CUDA;
   if (c->p.key_mode == XKV_KEYS_ONCE && launch_once_init(c, st) != cudaSuccess) return XKV_E_CUDA;
   return XKV_OK;
 }
@@ -195,7 +182,7 @@ int xkv_create(const xkv_params* params, void* dev_workspace, size_t bytes, xkv_
   if (cudaEventCreateWithFlags(&c->kbar_done, cudaEventDisableTiming) != cudaSuccess) {
     delete c->prof; delete c; return XKV_E_CUDA;
   }
-  const int rc = zero_workspace(c, c->ws_bytes, reinterpret_cast<cudaStream_t>(stream));
+  const int rc = zero_workspace(c, reinterpret_cast<cudaStream_t>(stream));
   if (rc != XKV_OK) { cudaEventDestroy(c->kbar_done); delete c->prof; delete c; return rc; }
   *out = c;
   return XKV_OK;
@@ -206,7 +193,7 @@ int xkv_reset(xkv_cache* c, xkv_stream stream) {
   // a head-mean kernel of the last stream step may still run on the library's stream
   after_head_means(c, reinterpret_cast<cudaStream_t>(stream));
   reset_host_state(c);
-  return zero_workspace(c, make_layout(&c->p).zeroed, reinterpret_cast<cudaStream_t>(stream));
+  return zero_workspace(c, reinterpret_cast<cudaStream_t>(stream));
 }
 
 int xkv_destroy(xkv_cache* c) {

@@ -625,8 +625,8 @@ def test_export_of_16bit_rows_may_end_anywhere(xkv, n_bytes):
 
 @pytest.mark.parametrize("bits,once", [(4, 0), (4, 1), (8, 1), (16, 0)])
 def test_reset_after_a_stream_of_bad_values(xkv, bits, once):
-    """xkv_reset zeroes what a stream needs zeroed and no more: after a stream of infinities, numbers beyond fp16 and
-    NaN, with longer frames, a cache behaves like a new one."""
+    """After a stream of infinities, numbers beyond fp16 and NaN, with longer frames, a cache that was reset behaves
+    like a new one."""
     import torch
     H, n = 2, 150
     p = xkv.Params(n_heads=H, budget=400, max_frame_tokens=n, kv_bits=bits, key_mode=once)
@@ -650,6 +650,33 @@ def test_reset_after_a_stream_of_bad_values(xkv, bits, once):
         ea, eb = used.export(), new.export()
         assert all(np.array_equal(np.asarray(ea[key]), np.asarray(eb[key])) for key in eb), t
         assert used.xkv_poll_status() == 0 and new.xkv_poll_status() == 0
+
+
+@pytest.mark.parametrize("bits,once", [(4, 0), (4, 1), (8, 1), (16, 0)])
+@pytest.mark.parametrize("between", ["nothing", "zeros", "ones"])
+def test_reset_fills_the_whole_workspace(xkv, bits, once, between):
+    """xkv_reset leaves the workspace as xkv_create does, byte for byte: nothing of the stream before is left in it, or
+    of what its owner kept there meanwhile, and the unused slots of an export are those of a new cache too."""
+    H, n = 2, 150
+    p = xkv.Params(n_heads=H, budget=400, max_frame_tokens=n, kv_bits=bits, key_mode=once)
+    used, new = xkv.Cache(p), xkv.Cache(p)
+    for t in range(5):
+        q, k, v = (to_device_bf16(b) for b in synth.gen_frame(85, 0, t, H, n, 64))
+        xkv.xkv_stream_step([used], [q], [k], [v], [q.clone()])
+    if between != "nothing":
+        used.workspace.fill_(255 if between == "ones" else 0)
+    used.xkv_reset()
+    assert used.workspace.equal(new.workspace)
+    for t in range(2):                                 # and unused slots stay as they are while the next stream starts
+        q, k, v = (to_device_bf16(b) for b in synth.gen_frame(86, 0, t, H, 40, 64))
+        outs = [q.clone(), q.clone()]
+        for c, out in zip((used, new), outs):
+            xkv.xkv_stream_step([c], [q], [k], [v], [out])
+        assert outs[0].equal(outs[1])
+        buffers = [xkv.BUF_K_CODES, xkv.BUF_K_PARAMS, xkv.BUF_V_CODES, xkv.BUF_V_PARAMS, xkv.BUF_ORIGIN, xkv.BUF_QVEC]
+        for which in buffers + ([xkv.BUF_K_SLOT, xkv.BUF_K_TABLE, xkv.BUF_K_REF] if once else []):
+            a, b = (np.asarray(c.xkv_debug_export(which, 1 << 24)) for c in (used, new))
+            assert np.array_equal(a, b), (t, which)
 
 
 @pytest.mark.parametrize("bits", [4, 16])
