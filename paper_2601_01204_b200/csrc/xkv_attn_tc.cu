@@ -664,6 +664,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     const int hf = warp >> 3;                // half of the quarter's rows
     const int lane = tid & 31;
     const int r = (warp & 3) * 32 + 16 * hf + (lane >> 2);        // rows r and r + 8 of the tile
+    const bool odd = lane & 1, second = lane & 2;
     const int cq2 = 2 * (lane & 3);          // this thread's columns: cq2 and the next of every 8
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32 + 16 * hf) << 16);
     const uint32_t col_t = lane_addr + kColTile * t;
@@ -732,13 +733,25 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           for (int i = 0; i < 64; ++i)
             if (8 * (i >> 2) + cq2 + (i & 1) >= lim) sc[i] = 0xff800000u;           // -inf: exponential 0
         }
-        float mx0 = -INFINITY, mx1 = -INFINITY;
+        float mx0 = -INFINITY, mx1 = -INFINITY, low0 = 0.f, low1 = 0.f;
 #pragma unroll
         for (int g = 0; g < 16; ++g) {
+          if (kBf16 && g == 8) {         // (16-bit caches: the two halves of the columns apart, see below)
+            low0 = mx0; low1 = mx1;
+            mx0 = mx1 = -INFINITY;
+          }
           mx0 = max3(mx0, __uint_as_float(sc[4 * g]), __uint_as_float(sc[4 * g + 1]));
           mx1 = max3(mx1, __uint_as_float(sc[4 * g + 2]), __uint_as_float(sc[4 * g + 3]));
         }
-        const float own0 = mx0, own1 = mx1;
+        float half_max = 0.f;
+        if (kBf16) {
+          // the quad's four maxima of half a row: row r in lanes 0 (columns below 64) and 1, row r + 8 in lanes 2 and 3
+          const float low = fmaxf(odd ? mx0 : low0, __shfl_xor_sync(0xffffffffu, odd ? low0 : mx0, 1));
+          const float high = fmaxf(odd ? mx1 : low1, __shfl_xor_sync(0xffffffffu, odd ? low1 : mx1, 1));
+          half_max = fmaxf(second ? high : low, __shfl_xor_sync(0xffffffffu, second ? low : high, 2));
+          mx0 = fmaxf(mx0, low0);
+          mx1 = fmaxf(mx1, low1);
+        }
 #pragma unroll
         for (int o = 1; o < 4; o <<= 1) {
           mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
@@ -767,12 +780,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
         if (kBf16) {
           // A weight rounded to bf16 and the sum that it is divided by: where one key dominates a row its
           // rounding error drops out if the sum holds the rounded weight as well.  The largest weight of
-          // these 32 columns is enough (of 64, error against float64 as with all of them: 32768 tokens 2.18e-3
-          // -> 1.92e-3, of which the rounding of the output is 1.67e-3); adding up all rounded weights
-          // cost 6 % of the step (24 layers at 32768: 7860 -> 8400 us).
-          const float top0 = fast_exp2(fmaf(own0, a.scale_log2, -m0)), top1 = fast_exp2(fmaf(own1, a.scale_log2, -m1));
-          l0 = add_f2(l0, pack_f2(__bfloat162float(__float2bfloat16_rn(top0)) - top0, 0.f));
-          l1 = add_f2(l1, pack_f2(__bfloat162float(__float2bfloat16_rn(top1)) - top1, 0.f));
+          // every 64 columns is enough (error against float64 at 32760 tokens 2.16e-3 -> 1.90e-3, of which the
+          // rounding of the output is 1.66e-3; 24 layers at 32768 7636 -> 7905 us); all rounded weights were no
+          // better and cost 6 % of the step, measured before the warps took whole rows.  Which columns go together
+          // is part of the result: a thread's own 32 instead saved 0.7 % and moved outputs by 2e-4.
+          const float top = fast_exp2(fmaf(half_max, a.scale_log2, second ? -m1 : -m0));
+          const float off = __bfloat162float(__float2bfloat16_rn(top)) - top;
+          l0 = add_f2(l0, pack_f2(second ? 0.f : off, 0.f));
+          l1 = add_f2(l1, pack_f2(second ? off : 0.f, 0.f));
         }
         const uint32_t colP = col_t + 128 * (cnt & 1);       // (over scores of these rows only)
         // Exponentials against the reference; P (16-bit pairs) -> TMEM, 64 columns at a time (32: 24 layers at 4096
