@@ -200,17 +200,19 @@ def test_single_token_frames_and_exact_budget(xkv):
 
 
 @pytest.mark.parametrize("middle", [64, 65, 128, 191])
-def test_blocks_that_leave_before_the_selection(xkv, middle):
+@pytest.mark.parametrize("n", [50, 130])
+def test_blocks_that_leave_before_the_selection(xkv, n, middle):
     """The append and the pooled query of a frame fill more blocks than the scoring and selection of its middle
     tokens; the others leave at the first barrier.  Lengths of the middle at the edges of 64-token runs, layers
-    together in a launch and one by one, three evicting steps each (the barrier's count goes on)."""
+    together in a launch and one by one, three evicting steps each (the barrier's count goes on).  Frames of 130
+    tokens evict without a selection where the middle holds fewer."""
     from xkv_testlib import compare_state, oracle_params
     from oracle import xkv_oracle as xo
-    H, n, d = 8, 130, 64
+    H, d = 8, 64
     p = xkv.Params(n_heads=H, budget=n + middle, max_frame_tokens=n, kv_bits=4)
     layers = [xkv.Cache(p) for _ in range(3)]                      # two together, one by itself
     oras = [xo.OracleLayer(oracle_params(p)) for _ in layers]
-    for t in range(5):
+    for t in range(max(5, middle // n + 4)):
         bits = [synth.gen_frame(31, l, t, H, n, d) for l in range(3)]
         q, k, v = ([to_device_bf16(b[i]) for b in bits] for i in range(3))
         out = [x.clone() for x in q]
@@ -220,7 +222,8 @@ def test_blocks_that_leave_before_the_selection(xkv, middle):
             o.step(*(synth.bf16_bits_to_f32(b) for b in bits[l]))
             compare_state(c.export(), o.export(), f"frame {t} layer {l}")
             assert c.xkv_poll_status() == 0
-    assert all(c.xkv_get_info().last_evicted > 0 for c in layers)
+    infos = [c.xkv_get_info() for c in layers]
+    assert all(i.last_prunable == max(middle, n) and i.last_kept == max(0, middle - n) for i in infos)
 
 
 def test_score_ties_are_broken_by_position(xkv):
