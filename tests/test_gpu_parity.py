@@ -682,14 +682,14 @@ def test_reset_fills_the_whole_workspace(xkv, bits, once, between):
             assert np.array_equal(a, b), (t, which)
 
 
-@pytest.mark.parametrize("bits", [4, 16])
+@pytest.mark.parametrize("bits,once,tail", [(4, 0, False), (4, 0, True), (4, 1, False), (4, 1, True), (8, 1, False), (16, 0, False)])
 @pytest.mark.parametrize("sizes", [(1, 1, 2), (7, 9, 8), (16, 15, 17), (33, 63, 64), (65, 127, 1), (129, 136, 40)])
-def test_attention_rows_and_columns_at_the_edges_of_a_warps_share(xkv, bits, sizes):
+def test_attention_rows_and_columns_at_the_edges_of_a_warps_share(xkv, bits, once, tail, sizes):
     """A softmax warp takes 16 rows of a query tile and a lane two columns of every eight: query counts around 8, 16
-    and 128 and cache lengths (masked columns) around 2, 8, 64 and 128, items whole and cut between blocks."""
+    and 128 and cache lengths (masked columns) around 2, 8, 64 and 128, items whole and cut between blocks, every form of the kernel."""
     for blocks in (0, 3):
-        p = xkv.Params(n_heads=2, budget=400, max_frame_tokens=136, kv_bits=bits)
-        run_stream(xkv, p, list(sizes), 3, seed=17, max_blocks=blocks)
+        p = xkv.Params(n_heads=2, budget=400, max_frame_tokens=136, kv_bits=bits, key_mode=once)
+        run_stream(xkv, p, list(sizes), 3, seed=17, max_blocks=blocks, tail=tail)
 
 
 def weights_as_rounded(q, k, v, halves):
