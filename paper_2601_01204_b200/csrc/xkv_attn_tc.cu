@@ -51,17 +51,20 @@ constexpr int kMaxDevices = 64;
 constexpr int kThreads = 768;
 // registers per thread after the reallocation (setmaxnreg)
 constexpr int kRegsSoftmax = 96;
-// (24 layers at 16384 tokens: tail 3535 us with 56 + 40, 3421 with 64 + 32; keys once 3688 with 56 + 40,
-// 3897 with 48 + 48)
+// (24 layers, three streams in turn: tail at 16384 4225 us with 56 + 40, 4118 with 64 + 32, 4048 with 72 + 24, which is not
+// taken up here; keys once at 16384 4515 with 48 + 48, 4329 with 56 + 40, 4326 with 64 + 32, 8-bit at 8192 2096, 1988 and
+// 1973; 4-bit at 16384 3761, 3763, 3768 and 3757 with 40, 48, 56 and 64 for the producers, within the noise.  16-bit
+// caches give the producers, who have nothing to do there, 48 as well.)
 __host__ __device__ constexpr int regs_producers(bool once, bool tail) { return tail ? 64 : once ? 56 : 48; }
 __host__ __device__ constexpr int regs_misc(bool once, bool tail) { return 96 - regs_producers(once, tail); }   // MMA issuers, copy thread
 constexpr int kQRows = 128;
 constexpr int kMaxGrid = 160;                 // CTAs the scratch is sized for (>= SM count of the part)
 constexpr uint32_t kSpinLimit = 1u << 22;
 // The reference maximum of a row moves only when the row maximum exceeds it by more than 2^kGrow
-// (log2 units).  Until then exponentials reach at most 2^14 = 16384, inside the fp16 range; the
-// decision is taken per warp, so a low threshold would make some row of the 32 trip it at every
-// few tiles.
+// (log2 units).  Until then exponentials reach at most 2^14 = 16384, inside the fp16 range.  Sums are
+// rescaled row by row, but the accumulator as soon as one of a warp's 16 rows asks for it, so a low
+// threshold would trip it at every few tiles (24 layers at 4096: 14, 8, 4 take 1018, 1034, 1058 us; at 16384
+// 3764, 3793, 3827).
 constexpr float kGrow = 14.f;
 
 constexpr uint32_t kAhead = 4;        // tiles whose constants are asked for ahead of the producers (keys quantised once)
@@ -81,7 +84,7 @@ template <> struct Cfg<8> {                    // 8-bit codes, keys quantised on
   static constexpr int kRawStage = kRawK + kRawV + kRawKP + kRawVP;
 };
 // 16-bit caches: no raw stages and no work for the producers, whose copies within shared memory (64 KB a tile, read and
-// written) cost time and, at the power cap, clock.  24 layers, 1374 tokens at 32768: 8047 -> 7887 us a step.
+// written) cost time and, at the power cap, clock.  24 layers, 1374 tokens at 32768: 7783 -> 7641 us a step.
 template <> struct Cfg<16> {                   // rows are stored as the MMA wants them (BufSet): the copies fill the
   static constexpr int kNK = 4, kNV = 4;      // operand tiles themselves
   static constexpr int kNR = 1;               // (no raw stages: two unused barriers)
@@ -657,9 +660,10 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
     // exponentials are computed.  What a row needs as a whole (its maximum, its sum) goes around the quad by
     // shuffles; no warp waits for another one.
     // (Before, warps w and w + 8 shared 32 rows, 64 columns each, and exchanged maxima through shared memory and
-    // a barrier in every step, 360 of its 2900 clk, which also kept the two in step.  Separate: one layer of
-    // 1374 tokens at 8192, all four calls, 132.3 -> 122.3 us; chunks of four frames, 24 layers, 7016 -> 6359; 24 layers
-    // at 4096 1038 -> 993, at 16384 3607 -> 3576, with the tail 4039 -> 3880; 16-bit at 32768 7481 -> 7398.)
+    // a barrier in every step, 360 of its 2900 clk, which also kept the two in step.  Separate, three streams in turn:
+    // one layer of 261 tokens at 1024 39.8 -> 38.2 us, of 1374 at 8192, all four calls, 132.2 -> 122.1; 24 layers: chunks of four
+    // frames 7024 -> 6381, at 4096 1038 -> 1026, at 16384 3862 -> 3791, with the tail 4206 -> 4142, 16-bit at 32768
+    // 8011 -> 7922; keys once 4450 -> 4588 and 8-bit 2035 -> 2059, which storing P 64 columns at a time makes up.)
     const int t = (warp >> 2) & 1;           // query tile of the pair
     const int hf = warp >> 3;                // half of the quarter's rows
     const int lane = tid & 31;
@@ -790,8 +794,9 @@ __global__ void __launch_bounds__(kThreads, 1) attn_tc_kernel(const __grid_const
           l1 = add_f2(l1, pack_f2(second ? off : 0.f, 0.f));
         }
         const uint32_t colP = col_t + 128 * (cnt & 1);       // (over scores of these rows only)
-        // Exponentials against the reference; P (16-bit pairs) -> TMEM, 64 columns at a time (32: 24 layers at 4096
-        // 980 -> 1029 us, keys quantised once at 16384 3668 -> 3798, 8-bit 1481 -> 1538).
+        // Exponentials against the reference; P (16-bit pairs) -> TMEM, 64 columns at a time (32 at a time, three streams
+        // in turn: 24 layers at 4096 1019 -> 1075 us, at 16384 3762 -> 3983, keys once 4384 -> 4547, tail 4119 -> 4273,
+        // 8-bit 1981 -> 2036).
         auto columns = [&](int g0, uint32_t* pk) {
 #pragma unroll
           for (int g = 0; g < 8; ++g) {

@@ -286,8 +286,8 @@ __device__ __forceinline__ bool grid_barrier(const MaintArgs& a, const Blocks& B
 // Of `count` blocks, those with work in the scoring and selection of r_old tokens, 64 at a time, and one more that
 // clears what the next step needs clear; the others leave at the first barrier, and the two barriers behind it are
 // among few.  (A gather, or head means, behind or beside them have work for all.)  One layer, 261 tokens at 1024: 13 of
-// 87 blocks stay, a step takes 38.0 instead of 38.8 us, eight frames from an empty cache 258.2 instead of 262.0; where
-// every block has tokens to score nothing changes (1374 tokens at 8192: 121.4 and 121.5).
+// 87 blocks stay, a step takes 38.6 instead of 38.9 us, eight frames from an empty cache 265.3 instead of 266.9; where
+// every block has tokens to score nothing changes (1374 tokens at 8192: 120.0 and 120.1).
 __host__ __device__ __forceinline__ int later_blocks(uint32_t phases, int r_old, int count) {
   const int need = (r_old + 63) / 64 + 1;
   return (phases & (kPhPack | kPhKbarNew)) || need > count ? count : need;
